@@ -13,7 +13,7 @@
 #include <cmath>
 #include <vector>
 
-#include "fft.cuh"
+#include "fxfft.cuh"
 #include "problem.h"
 #include "revolve.h"
 
@@ -39,122 +39,78 @@ struct BurgersParams {
   int ws_len;
 };
 
+// Buffers of a CTA: two transform pairs of L entries each.  The inverse transforms read their staged
+// spectra from B (and D for a second one) and leave the grid in A or B (C or D).
 struct Smem {
-  double2* A;
-  double2* B;
-  double2* C;
-  double2* D;
-  double2* S;  // spectrum staging (K)
-  double2* O;  // spectral output staging (K)
+  int A, B, C, D;
 };
 
-__device__ __forceinline__ Smem carve(const BurgersParams& P) {
-  extern __shared__ double2 sm[];
-  Smem s;
-  s.A = sm;
-  s.B = s.A + P.L;
-  s.C = s.B + P.L;
-  s.D = s.C + P.L;
-  s.S = s.D + P.L;
-  s.O = s.S + P.K;
-  return s;
-}
-
-// grid (packed) of the coefficients in S, weights (w0, w): see c2r_pre.  Result buffer returned.
-__device__ double2* c2g_packed(const BurgersParams& P, const double2* S, double2* a, double2* b, double w0,
-                               double w) {
-  c2r_pre(a, [&](int k) { return S[k]; }, P.K, P.L, P.WM, w0, w);
-  __syncthreads();
-  return cfft_smem(a, b, P.plan, P.WM, +1);
-}
-
-// forward real FFT of the packed grid in a; writes scale(k, 2 X_k) to O (k < K): the factor 1/2
-// of the real-transform unpacking is left to the scale functors.
-template <class Scale>
-__device__ void g2c_packed(const BurgersParams& P, double2* a, double2* b, double2* O, Scale scale) {
-  double2* z = cfft_smem(a, b, P.plan, P.WM, -1);
-  r2c_post2(z, [&](int k, double2 v) { O[k] = scale(k, v); }, P.K, P.L, P.WM);
-  __syncthreads();
-}
+__device__ __forceinline__ Smem carve(const BurgersParams& P) { return Smem{0, P.L, 2 * P.L, 3 * P.L}; }
 
 __device__ __forceinline__ double kwav(const BurgersParams& P, int k) { return P.kscale * k; }
 
-// O <- F(S) = -i k T[(B S)^2 / 2]
-__device__ void eval_F(const BurgersParams& P, Smem& s) {
-  double2* u = c2g_packed(P, s.S, s.A, s.B, 1.0, 1.0);
-  for (int j = threadIdx.x; j < P.L; j += blockDim.x) {
-    double2 v = u[j];
-    u[j] = make_double2(v.x * v.x, v.y * v.y);  // u^2; the 1/2 goes into the scale below
-  }
-  __syncthreads();
-  double2* other = (u == s.A) ? s.B : s.A;
-  const double q = 0.25 / P.M;  // (1/2 of u^2/2) (1/2 of the unpacking) / M
-  g2c_packed(P, u, other, s.O, [&](int k, double2 v) {
-    double kk = kwav(P, k) * q;  // -i k v / M
-    return make_double2(kk * v.y, -kk * v.x);
+// Puts F(x)_k = -i k T[(B x)^2 / 2]_k, k < K, through out(k, F_k), from the spectrum staged in B.
+template <class Out>
+__device__ __forceinline__ void eval_F(const BurgersParams& P, const Smem& s, Out out) {
+  const FxRes u = xf_c2r_staged<1, false>(s.A, s.B, FxLay{1, 1, P.L, 0}, P.plan, P.K);
+  const FxRes z = xf_r2c<1, true, false>(s.C, s.D, FxLay{1, 1, P.L, 0}, P.plan, [&](int, int, int j) {
+    const double2 v = u.at(0, 0, j);
+    return make_double2(v.x * v.x, v.y * v.y);  // u^2; the 1/2 goes into the scale below
   });
-}
-
-// From the primal spectrum S and the tangent spectrum S2: O <- F(S) (if want_F) and
-// O2 <- (dF/dX)(S) S2 = -i k T[(B S)(B S2)].
-__device__ void eval_F_and_jvp(const BurgersParams& P, Smem& s, const double2* S2, double2* O2, bool want_F) {
-  // both inverse transforms in the same FFT passes (A|B and C|D are 2L apart)
-  c2r_pre(s.A, [&](int k) { return s.S[k]; }, P.K, P.L, P.WM, 1.0, 1.0);
-  c2r_pre(s.C, [&](int k) { return S2[k]; }, P.K, P.L, P.WM, 1.0, 1.0);
-  __syncthreads();
-  cfft_smem_sets<1>(s.A, s.B, 2 * P.L, 2, P.plan, 1);
-  const bool odd = P.plan.nrad & 1;
-  double2* u = odd ? s.B : s.A;
-  double2* du = odd ? s.D : s.C;
-  double2* uo = odd ? s.A : s.B;
-  double2* duo = odd ? s.C : s.D;
-  for (int j = threadIdx.x; j < P.L; j += blockDim.x) {
-    double2 v = u[j], dv = du[j];
-    du[j] = make_double2(v.x * dv.x, v.y * dv.y);
-    u[j] = make_double2(v.x * v.x, v.y * v.y);
-  }
-  __syncthreads();
-  const double qf = 0.25 / P.M, qj = 0.5 / P.M;  // -i k (u^2/2) / M and -i k (u du) / M, unpacking 1/2 included
-  auto mikf = [&](int k, double2 v) {
-    double kk = kwav(P, k) * qf;
-    return make_double2(kk * v.y, -kk * v.x);
-  };
-  auto mikj = [&](int k, double2 v) {
-    double kk = kwav(P, k) * qj;
-    return make_double2(kk * v.y, -kk * v.x);
-  };
-  if (want_F) g2c_packed(P, u, uo, s.O, mikf);
-  g2c_packed(P, du, duo, O2, mikj);
-}
-
-// O <- (dF/dX)(S)^dagger W  with W staged in S2:  B^dagger[(B S) * T^dagger(i k W)]
-__device__ void eval_vjp(const BurgersParams& P, Smem& s, double2* S2) {
-  // S2 <- i k W / (2M) (in place, own entries only): T^dagger's weights (1/M on the real part of
-  // k = 0, 1/(2M) elsewhere) folded in, the k = 0 entry being 0
   const double q = 0.5 / P.M;
   for (int k = threadIdx.x; k < P.K; k += blockDim.x) {
-    double2 w = S2[k];
-    double kk = kwav(P, k) * q;
-    S2[k] = make_double2(-kk * w.y, kk * w.x);
+    const double2 v = z.coef(0, 0, k);
+    const double kk = kwav(P, k) * q;  // -i k v / M
+    out(k, make_double2(kk * v.y, -kk * v.x));
   }
-  __syncthreads();
-  // both inverse transforms in the same FFT passes (A|B and C|D are 2L apart)
-  c2r_pre(s.A, [&](int k) { return s.S[k]; }, P.K, P.L, P.WM, 1.0, 1.0);
-  c2r_pre(s.C, [&](int k) { return S2[k]; }, P.K, P.L, P.WM, 1.0, 1.0);
-  __syncthreads();
-  cfft_smem_sets<1>(s.A, s.B, 2 * P.L, 2, P.plan, 1);
+}
+
+// From the primal spectrum staged in B and the tangent spectrum in D: outF(k, F_k) (if want_F) and
+// outJ(k, ((dF/dX) dX)_k), (dF/dX) dX = -i k T[(B x)(B dx)].
+template <class OutF, class OutJ>
+__device__ __forceinline__ void eval_F_and_jvp(const BurgersParams& P, const Smem& s, bool want_F, OutF outF, OutJ outJ) {
+  // both inverse transforms in the same passes (A|B and C|D are 2L apart)
+  const FxRes u = xf_c2r_staged<2, false>(s.A, s.B, FxLay{2, 1, 2 * P.L, 0}, P.plan, P.K);
   const bool odd = P.plan.nrad & 1;
-  double2* u = odd ? s.B : s.A;
-  double2* v = odd ? s.D : s.C;
-  double2* vo = odd ? s.C : s.D;
-  for (int j = threadIdx.x; j < P.L; j += blockDim.x) {
-    double2 a = u[j], b = v[j];
-    v[j] = make_double2(a.x * b.x, a.y * b.y);
+  const int f0 = odd ? s.A : s.B, f1 = odd ? s.C : s.D;  // free halves
+  for (int t = want_F ? 0 : 1; t < 2; ++t) {
+    const FxRes z = xf_r2c<1, true, false>(f0, f1, FxLay{1, 1, P.L, 2}, P.plan, [&](int, int, int j) {
+      const double2 v = u.at(0, 0, j), w = t ? u.at(1, 0, j) : v;
+      return make_double2(v.x * w.x, v.y * w.y);
+    });
+    const double q = (t ? 1.0 : 0.5) / P.M;
+    for (int k = threadIdx.x; k < P.K; k += blockDim.x) {
+      const double2 v = z.coef(0, 0, k);
+      const double kk = kwav(P, k) * q;
+      const double2 o = make_double2(kk * v.y, -kk * v.x);
+      if (t) outJ(k, o);
+      else outF(k, o);
+    }
+    __syncthreads();
   }
-  __syncthreads();
-  g2c_packed(P, v, vo, s.O, [&](int k, double2 x) {  // x = 2 X_k
-    return k == 0 ? make_double2(0.5 * x.x, 0.0) : x;
+}
+
+// i k w / (2M): T^dagger's weights (1/M on the real part of k = 0, 1/(2M) elsewhere) folded in, the k = 0
+// entry being 0
+__device__ __forceinline__ double2 vjp_cotangent(const BurgersParams& P, int k, double2 w) {
+  const double kk = kwav(P, k) * (0.5 / P.M);
+  return make_double2(-kk * w.y, kk * w.x);
+}
+// From the primal spectrum staged in B and vjp_cotangent(W) in D: out(k, ((dF/dX)^dagger W)_k),
+// (dF/dX)^dagger W = B^dagger[(B x) * T^dagger(i k W)].
+template <class Out>
+__device__ __forceinline__ void eval_vjp(const BurgersParams& P, const Smem& s, Out out) {
+  const FxRes u = xf_c2r_staged<2, false>(s.A, s.B, FxLay{2, 1, 2 * P.L, 0}, P.plan, P.K);
+  const bool odd = P.plan.nrad & 1;
+  const int f0 = odd ? s.A : s.B, f1 = odd ? s.C : s.D;
+  const FxRes z = xf_r2c<1, true, false>(f0, f1, FxLay{1, 1, P.L, 0}, P.plan, [&](int, int, int j) {
+    const double2 a = u.at(0, 0, j), b = u.at(1, 0, j);
+    return make_double2(a.x * b.x, a.y * b.y);
   });
+  for (int k = threadIdx.x; k < P.K; k += blockDim.x) {
+    const double2 x = z.coef(0, 0, k);
+    out(k, k == 0 ? make_double2(x.x, 0.0) : make_double2(2.0 * x.x, 2.0 * x.y));
+  }
 }
 
 __device__ __forceinline__ const double2* row(const double* base, int b, int K) {
@@ -166,63 +122,58 @@ __device__ __forceinline__ double2* row(double* base, int b, int K) {
 
 // ---- single-shot kernels (transforms, F, JVP, VJP) ----------------------------------------
 
-__global__ void transform_kernel(BurgersParams P, int kind, const double* __restrict__ in, double* __restrict__ out) {
-  Smem s = carve(P);
-  const int b = blockIdx.x;
-  const int K = P.K, L = P.L, M = P.M;
-  if (kind == 0 || kind == 3) {  // coefficients -> grid
-    const double2* x = row(in, b, K);
-    for (int k = threadIdx.x; k < K; k += blockDim.x) s.S[k] = x[k];
-    __syncthreads();
-    double2* z = (kind == 0) ? c2g_packed(P, s.S, s.A, s.B, 1.0, 1.0)
-                             : c2g_packed(P, s.S, s.A, s.B, 1.0 / M, 0.5 / M);
-    double2* g = reinterpret_cast<double2*>(out + (size_t)b * M);
-    for (int j = threadIdx.x; j < L; j += blockDim.x) g[j] = z[j];
-  } else {  // grid -> coefficients
-    const double2* g = reinterpret_cast<const double2*>(in + (size_t)b * M);
-    for (int j = threadIdx.x; j < L; j += blockDim.x) s.A[j] = g[j];
-    __syncthreads();
-    double2* y = row(out, b, K);
-    if (kind == 1) {
-      const double halfinvM = 0.5 / M;
-      g2c_packed(P, s.A, s.B, s.O, [&](int k, double2 v) { return cscale(v, halfinvM); });
-    } else {
-      g2c_packed(P, s.A, s.B, s.O, [&](int k, double2 v) {
-        return k == 0 ? make_double2(0.5 * v.x, 0.0) : v;
-      });
-    }
-    for (int k = threadIdx.x; k < K; k += blockDim.x) y[k] = s.O[k];
+// coefficients -> grid with the weights w0 (k = 0) and w
+__global__ void __launch_bounds__(64) to_grid_kernel(const __grid_constant__ BurgersParams P, double w0, double w, const double2* __restrict__ x,
+                                                     double2* __restrict__ g) {
+  const Smem s = carve(P);
+  const double2* xr = x + (size_t)blockIdx.x * P.K;
+  double2* gr = g + (size_t)blockIdx.x * P.L;
+  const FxRes z = xf_c2r<1, true, false>(s.A, s.B, FxLay{1, 1, P.L, 0}, P.plan, P.K,
+                                         [&](int, int, int k) { return cscale(ldg128(xr + k), k == 0 ? w0 : w); });
+  for (int j = threadIdx.x; j < P.L; j += blockDim.x) stg128(gr + j, z.at(0, 0, j));
+}
+// grid -> coefficients times s0 (k = 0, real part only if re0) or s
+__global__ void __launch_bounds__(64) to_coef_kernel(const __grid_constant__ BurgersParams P, double s0, double sc, int re0,
+                                                     const double2* __restrict__ g, double2* __restrict__ y) {
+  const Smem s = carve(P);
+  const double2* gr = g + (size_t)blockIdx.x * P.L;
+  double2* yr = y + (size_t)blockIdx.x * P.K;
+  const FxRes z = xf_r2c<1, true, false>(s.A, s.B, FxLay{1, 1, P.L, 0}, P.plan, [&](int, int, int j) { return ldg128(gr + j); });
+  for (int k = threadIdx.x; k < P.K; k += blockDim.x) {
+    double2 v = cscale(z.coef(0, 0, k), k == 0 ? s0 : sc);
+    if (k == 0 && re0) v.y = 0.0;
+    stg128(yr + k, v);
   }
 }
 
-__global__ void F_kernel(BurgersParams P, int mode, const double* __restrict__ x, const double* __restrict__ d,
+__global__ void __launch_bounds__(64) F_kernel(const __grid_constant__ BurgersParams P, int mode, const double* __restrict__ x, const double* __restrict__ d,
                          double* __restrict__ out) {
-  Smem s = carve(P);
-  extern __shared__ double2 sm[];
-  double2* S2 = sm + 4 * P.L + 2 * P.K;  // second input spectrum (JVP direction / VJP cotangent)
-  double2* O2 = S2 + P.K;                // second output spectrum
+  const Smem s = carve(P);
   const int b = blockIdx.x, K = P.K;
   const double2* xr = row(x, b, K);
   double2* o = row(out, b, K);
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    s.S[k] = xr[k];
-    if (mode != 0) S2[k] = row(d, b, K)[k];
-  }
-  __syncthreads();
   if (!P.nonlinear) {
-    for (int k = threadIdx.x; k < K; k += blockDim.x) o[k] = make_double2(0.0, 0.0);
+    for (int k = threadIdx.x; k < K; k += blockDim.x) stg128(o + k, make_double2(0.0, 0.0));
     return;
   }
-  if (mode == 0) {
-    eval_F(P, s);
-    for (int k = threadIdx.x; k < K; k += blockDim.x) o[k] = s.O[k];
-  } else if (mode == 1) {
-    eval_F_and_jvp(P, s, S2, O2, false);
-    for (int k = threadIdx.x; k < K; k += blockDim.x) o[k] = O2[k];
-  } else {
-    eval_vjp(P, s, S2);
-    for (int k = threadIdx.x; k < K; k += blockDim.x) o[k] = s.O[k];
+  unsigned m0 = 0u, m1 = 0u;
+  for (int k = threadIdx.x; k < K; k += blockDim.x) {
+    const double2 v = ldg128(xr + k);
+    fx_put64(s.B + k, v);
+    m0 = fx_absmax(m0, v);
+    if (mode != 0) {
+      double2 w = ldg128(row(d, b, K) + k);
+      if (mode == 2) w = vjp_cotangent(P, k, w);
+      fx_put64(s.D + k, w);
+      m1 = fx_absmax(m1, w);
+    }
   }
+  fx_put_max(0, 1, 0, m0);
+  if (mode != 0) fx_put_max(1, 1, 0, m1);
+  auto put = [&](int k, double2 v) { stg128(o + k, v); };
+  if (mode == 0) eval_F(P, s, put);
+  else if (mode == 1) eval_F_and_jvp(P, s, false, put, put);
+  else eval_vjp(P, s, put);
 }
 
 // ---- persistent trajectory kernels ----------------------------------------------------------
@@ -294,21 +245,39 @@ __device__ __forceinline__ double2 hist_rhs(const Coef& c, const double2 (&hf)[O
 // final state (or tangent), s_out the final restart state (or its tangent), traj the states
 // X_{n_first}..X_{n_first+n_steps}.
 template <int Q, int ORD>
-__global__ void __launch_bounds__(64) trajectory_kernel(BurgersParams P, int n_first, int n_steps,
+__global__ void __launch_bounds__(64) trajectory_kernel(const __grid_constant__ BurgersParams P, int n_first, int n_steps,
                                                         const double* __restrict__ s_in, int in_blocks,
                                                         const double* __restrict__ ds_in, double* __restrict__ x_out,
                                                         double* __restrict__ s_out, double* __restrict__ traj,
                                                         int tangent) {
-  Smem s = carve(P);
-  extern __shared__ double2 sm[];
-  double2* S2 = sm + 4 * P.L + 2 * P.K;
-  double2* O2 = S2 + P.K;
+  const Smem s = carve(P);
   const int b = blockIdx.x, K = P.K, G = blockDim.x, tid = threadIdx.x;
   const int nb = gridDim.x;
   const size_t blk = (size_t)nb * 2 * K;
   const int so = P.order;
   const int nx = in_blocks > 1 ? so : 1;  // X blocks present in s_in
   double2 X[Q][ORD], F[Q][ORD], D[Q][ORD], GJ[Q][ORD];
+  unsigned mx = 0u, md = 0u;  // largest high words of the staged spectra
+  // F (and its tangent) of the staged spectra into slot 0 of the histories: thread tid owns k = tid + q G
+  auto nonlinear = [&]() {
+    fx_put_max(0, 1, 0, mx);
+    if (tangent) {
+      fx_put_max(1, 1, 0, md);
+      eval_F_and_jvp(P, s, true, [&](int k, double2 v) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) if (k == tid + q * G) F[q][0] = v;
+      }, [&](int k, double2 v) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) if (k == tid + q * G) GJ[q][0] = v;
+      });
+    } else {
+      eval_F(P, s, [&](int k, double2 v) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) if (k == tid + q * G) F[q][0] = v;
+      });
+    }
+    mx = md = 0u;
+  };
   for (int q = 0; q < Q; ++q) {
     int k = tid + q * G;
     double2 z = make_double2(0.0, 0.0);
@@ -318,28 +287,24 @@ __global__ void __launch_bounds__(64) trajectory_kernel(BurgersParams P, int n_f
 #pragma unroll
       for (int i = 0; i < ORD; ++i) {
         if (i < nx) {
-          X[q][i] = row(s_in + i * blk, b, K)[k];
-          if (tangent) D[q][i] = row(ds_in + i * blk, b, K)[k];
+          X[q][i] = ldg128(row(s_in + i * blk, b, K) + k);
+          if (tangent) D[q][i] = ldg128(row(ds_in + i * blk, b, K) + k);
         }
         if (i >= 1 && i < so && in_blocks > 1) {
-          F[q][i] = row(s_in + (so + i - 1) * blk, b, K)[k];
-          if (tangent) GJ[q][i] = row(ds_in + (so + i - 1) * blk, b, K)[k];
+          F[q][i] = ldg128(row(s_in + (so + i - 1) * blk, b, K) + k);
+          if (tangent) GJ[q][i] = ldg128(row(ds_in + (so + i - 1) * blk, b, K) + k);
         }
       }
-      s.S[k] = X[q][0];
-      if (tangent) S2[k] = D[q][0];
-      if (traj) row(traj, b, K)[k] = X[q][0];
+      fx_put64(s.B + k, X[q][0]);
+      mx = fx_absmax(mx, X[q][0]);
+      if (tangent) {
+        fx_put64(s.D + k, D[q][0]);
+        md = fx_absmax(md, D[q][0]);
+      }
+      if (traj) stg128(row(traj, b, K) + k, X[q][0]);
     }
   }
-  __syncthreads();
-  if (P.nonlinear) {
-    if (tangent) eval_F_and_jvp(P, s, S2, O2, true);
-    else eval_F(P, s);
-    for (int q = 0; q < Q; ++q) {
-      int k = tid + q * G;
-      if (k < K) { F[q][0] = s.O[k]; if (tangent) GJ[q][0] = O2[k]; }
-    }
-  }
+  if (P.nonlinear) nonlinear();
   // nu k^2 per mode and 1 / (a_0 + nu k^2), recomputed only when a_0 changes (the step order, or
   // the step size of a schedule)
   double nk2[Q], inv_m[Q];
@@ -365,36 +330,30 @@ __global__ void __launch_bounds__(64) trajectory_kernel(BurgersParams P, int n_f
 #pragma unroll
       for (int i = ORD - 1; i > 0; --i) { X[q][i] = X[q][i - 1]; F[q][i] = F[q][i - 1]; }
       X[q][0] = xn;
-      s.S[k] = xn;
-      if (traj) row(traj + (size_t)j * blk, b, K)[k] = xn;
+      fx_put64(s.B + k, xn);
+      mx = fx_absmax(mx, xn);
+      if (traj) stg128(row(traj + (size_t)j * blk, b, K) + k, xn);
       if (tangent) {
         double2 dn = cscale(hist_rhs<ORD>(c, GJ[q], D[q]), inv);
         if (k == 0) dn.y = 0.0;
 #pragma unroll
         for (int i = ORD - 1; i > 0; --i) { D[q][i] = D[q][i - 1]; GJ[q][i] = GJ[q][i - 1]; }
         D[q][0] = dn;
-        S2[k] = dn;
+        fx_put64(s.D + k, dn);
+        md = fx_absmax(md, dn);
       }
     }
-    __syncthreads();
-    if (j < n_steps && P.nonlinear) {
-      if (tangent) eval_F_and_jvp(P, s, S2, O2, true);
-      else eval_F(P, s);
-      for (int q = 0; q < Q; ++q) {
-        int k = tid + q * G;
-        if (k < K) { F[q][0] = s.O[k]; if (tangent) GJ[q][0] = O2[k]; }
-      }
-    }
+    if (j < n_steps && P.nonlinear) nonlinear();
   }
   for (int q = 0; q < Q; ++q) {
     int k = tid + q * G;
     if (k >= K) continue;
-    if (x_out) row(x_out, b, K)[k] = tangent ? D[q][0] : X[q][0];
+    if (x_out) stg128(row(x_out, b, K) + k, tangent ? D[q][0] : X[q][0]);
     if (s_out) {
 #pragma unroll
       for (int i = 0; i < ORD; ++i) {
-        if (i < so) row(s_out + i * blk, b, K)[k] = tangent ? D[q][i] : X[q][i];
-        if (i >= 1 && i < so) row(s_out + (so + i - 1) * blk, b, K)[k] = tangent ? GJ[q][i] : F[q][i];
+        if (i < so) stg128(row(s_out + i * blk, b, K) + k, tangent ? D[q][i] : X[q][i]);
+        if (i >= 1 && i < so) stg128(row(s_out + (so + i - 1) * blk, b, K) + k, tangent ? GJ[q][i] : F[q][i]);
       }
     }
   }
@@ -409,14 +368,12 @@ __global__ void __launch_bounds__(64) trajectory_kernel(BurgersParams P, int n_f
 // solve) followed by Y_1, ..., Y_{s-1} when out_blocks = s.  Cotangents injected at X_n: seeds
 // (indexed by seed_at[n], nullable) and src (nullable, at n = n_hi).
 template <int Q, int ORD>
-__global__ void __launch_bounds__(64) adjoint_kernel(BurgersParams P, int n_steps, int n_hi, int n_lo,
+__global__ void __launch_bounds__(64) adjoint_kernel(const __grid_constant__ BurgersParams P, int n_steps, int n_hi, int n_lo,
                                                      const double* __restrict__ traj, const double* __restrict__ y_final,
                                                      const double* __restrict__ carry_in, double* __restrict__ out,
                                                      int out_blocks, const int* __restrict__ seed_at,
                                                      const double* __restrict__ seeds, const double* __restrict__ src) {
-  Smem s = carve(P);
-  extern __shared__ double2 sm[];
-  double2* S2 = sm + 4 * P.L + 2 * P.K;
+  const Smem s = carve(P);
   const int b = blockIdx.x, K = P.K, G = blockDim.x, tid = threadIdx.x;
   const int nb = gridDim.x;
   const size_t stride = (size_t)nb * 2 * K;
@@ -434,14 +391,14 @@ __global__ void __launch_bounds__(64) adjoint_kernel(BurgersParams P, int n_step
   for (int q = 0; q < Q; ++q) {
     const int k = tid + q * G;
 #pragma unroll
-    for (int i = 0; i < ORD; ++i) Y[q][i] = (carry_in && i < so && k < K) ? row(carry_in + i * stride, b, K)[k] : z;
+    for (int i = 0; i < ORD; ++i) Y[q][i] = (carry_in && i < so && k < K) ? ldg128(row(carry_in + i * stride, b, K) + k) : z;
   }
   for (int n = n_hi; n >= n_lo; --n) {
     double2 lam[Q];
     if (n == n_steps) {
       for (int q = 0; q < Q; ++q) {
         int k = tid + q * G;
-        lam[q] = (k < K && y_final) ? row(y_final, b, K)[k] : z;
+        lam[q] = (k < K && y_final) ? ldg128(row(y_final, b, K) + k) : z;
       }
     } else {
       // the weights of step n+i that multiply X_n: c_i^{n+i}, a_i^{n+i} (zero past the horizon)
@@ -453,21 +410,33 @@ __global__ void __launch_bounds__(64) adjoint_kernel(BurgersParams P, int n_step
         wa[i] = ci.a[i];
       }
       const double2* xn = row(traj + (size_t)(n - n_lo) * stride, b, K);
+      unsigned mx = 0u, mw = 0u;
       for (int q = 0; q < Q; ++q) {
         int k = tid + q * G;
         if (k >= K) continue;
-        s.S[k] = xn[k];
+        const double2 x = ldg128(xn + k);
+        fx_put64(s.B + k, x);
+        mx = fx_absmax(mx, x);
         double2 w = axpby(wc[1], Y[q][0], wc[2], Y[q][1]);
 #pragma unroll
         for (int i = 3; i <= ORD; ++i) w = make_double2(w.x + wc[i] * Y[q][i - 1].x, w.y + wc[i] * Y[q][i - 1].y);
-        S2[k] = w;
+        w = vjp_cotangent(P, k, w);
+        fx_put64(s.D + k, w);
+        mw = fx_absmax(mw, w);
       }
-      __syncthreads();
-      if (P.nonlinear) eval_vjp(P, s, S2);
+      for (int q = 0; q < Q; ++q) lam[q] = z;
+      if (P.nonlinear) {
+        fx_put_max(0, 1, 0, mx);
+        fx_put_max(1, 1, 0, mw);
+        eval_vjp(P, s, [&](int k, double2 v) {
+#pragma unroll
+          for (int q = 0; q < Q; ++q) if (k == tid + q * G) lam[q] = v;
+        });
+      }
       for (int q = 0; q < Q; ++q) {
         int k = tid + q * G;
-        if (k >= K) { lam[q] = z; continue; }
-        double2 v = P.nonlinear ? s.O[k] : z;
+        if (k >= K) continue;
+        const double2 v = lam[q];
         double2 l = make_double2(v.x - wa[1] * Y[q][0].x - wa[2] * Y[q][1].x, v.y - wa[1] * Y[q][0].y - wa[2] * Y[q][1].y);
 #pragma unroll
         for (int i = 3; i <= ORD; ++i) l = make_double2(l.x - wa[i] * Y[q][i - 1].x, l.y - wa[i] * Y[q][i - 1].y);
@@ -479,23 +448,23 @@ __global__ void __launch_bounds__(64) adjoint_kernel(BurgersParams P, int n_step
       const double* sv = seeds + (size_t)seed_at[n] * nb * 2 * K;
       for (int q = 0; q < Q; ++q) {
         int k = tid + q * G;
-        if (k < K) lam[q] = cadd(lam[q], row(sv, b, K)[k]);
+        if (k < K) lam[q] = cadd(lam[q], ldg128(row(sv, b, K) + k));
       }
     }
     if (src && n == n_hi) {
       for (int q = 0; q < Q; ++q) {
         int k = tid + q * G;
-        if (k < K) lam[q] = cadd(lam[q], row(src, b, K)[k]);
+        if (k < K) lam[q] = cadd(lam[q], ldg128(row(src, b, K) + k));
       }
     }
     if (n == 0) {
       for (int q = 0; q < Q; ++q) {
         int k = tid + q * G;
         if (k >= K) continue;
-        row(out, b, K)[k] = lam[q];
+        stg128(row(out, b, K) + k, lam[q]);
 #pragma unroll
         for (int i = 1; i < ORD; ++i)
-          if (i < so && i < out_blocks) row(out + i * stride, b, K)[k] = Y[q][i - 1];
+          if (i < so && i < out_blocks) stg128(row(out + i * stride, b, K) + k, Y[q][i - 1]);
       }
       return;
     }
@@ -521,7 +490,7 @@ __global__ void __launch_bounds__(64) adjoint_kernel(BurgersParams P, int n_step
     if (k >= K) continue;
 #pragma unroll
     for (int i = 0; i < ORD; ++i)
-      if (i < so && i < out_blocks) row(out + i * stride, b, K)[k] = Y[q][i];
+      if (i < so && i < out_blocks) stg128(row(out + i * stride, b, K) + k, Y[q][i]);
   }
 }
 
@@ -600,16 +569,16 @@ struct Burgers : EqImpl {
       double th = -2.0 * M_PI * (double)m / (double)P.M;
       h[m] = make_double2(std::cos(th), std::sin(th));
     }
-    {  // the butterflies' scaled-twiddle records follow the M-table in the same buffer
-      const std::vector<double2> sct = scaled_twiddle_table(P.plan);
+    {  // the transforms' tables follow the M-table in the same buffer
+      const std::vector<double2> sct = fft_tables(P.plan);
       h.insert(h.end(), sct.begin(), sct.end());
     }
     SPADJ_CUDA_TRY(p, wm.ensure(sizeof(double2) * h.size()));
     SPADJ_CUDA_TRY(p, cudaMemcpyAsync(wm.ptr, h.data(), sizeof(double2) * h.size(), cudaMemcpyHostToDevice, p->stream));
     SPADJ_CUDA_TRY(p, cudaStreamSynchronize(p->stream));
     P.WM = wm.as<double2>();
-    bind_scaled_twiddles(P.plan, P.WM + P.M);
-    smem = sizeof(double2) * (4 * P.L + 4 * P.K);
+    fft_bind(P.plan, P.WM + P.M, P.WM);
+    smem = sizeof(double2) * 4 * P.L;
     return SPADJ_OK;
   }
 
@@ -654,7 +623,12 @@ struct Burgers : EqImpl {
 
   spadj_status transform(Problem* p, int kind, const double* in, double* out) override {
     if (kind < 0 || kind > 3) return p->fail(SPADJ_ERR_INVALID, "transform: kind must be 0..3");
-    transform_kernel<<<B, G, smem, p->stream>>>(P, kind, in, out);
+    const double2* i2 = reinterpret_cast<const double2*>(in);
+    double2* o2 = reinterpret_cast<double2*>(out);
+    if (kind == 0) to_grid_kernel<<<B, G, smem, p->stream>>>(P, 1.0, 1.0, i2, o2);
+    else if (kind == 3) to_grid_kernel<<<B, G, smem, p->stream>>>(P, 1.0 / P.M, 0.5 / P.M, i2, o2);
+    else if (kind == 1) to_coef_kernel<<<B, G, smem, p->stream>>>(P, 1.0 / P.M, 1.0 / P.M, 0, i2, o2);
+    else to_coef_kernel<<<B, G, smem, p->stream>>>(P, 1.0, 2.0, 1, i2, o2);
     return check_launch(p, "burgers transform");
   }
 

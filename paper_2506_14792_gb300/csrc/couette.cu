@@ -40,7 +40,7 @@ struct Couette : EqImpl {
   size_t npts = 0;    // grid points Mz*My*Mx
   XParams xp{};
   YParams yp{};
-  DevBuf wmx, w2y, czE, cdzE, gzF, gzTE, czTF, cdzTF, gmat, phi1F, phi1A, phi2F, phi2A, one;
+  DevBuf wmx, twy, czE, cdzE, gzF, gzTE, czTF, cdzTF, gmat, phi1F, phi1A, phi2F, phi2A, one;
   // banded factors of the step solves: [scheme order - 1][0 forward, 1 adjoint]
   struct BandDev {
     DevBuf L, U, dinv, piv, ssb;
@@ -130,20 +130,16 @@ struct Couette : EqImpl {
         hczTF[(size_t)n * Mh + j] = o.Cz[(size_t)j * N + n];
         hcdzTF[(size_t)n * Mh + j] = o.Cdz[(size_t)j * N + n];
       }
-    std::vector<double2> hwx(Mx), hwy(2 * My);
+    std::vector<double2> hwx(Mx);
     for (int m = 0; m < Mx; ++m) {
       const double th = -2.0 * M_PI * (double)m / (double)Mx;
       hwx[m] = make_double2(std::cos(th), std::sin(th));
     }
-    for (int m = 0; m < 2 * My; ++m) {
-      const double th = -2.0 * M_PI * (double)m / (double)(2 * My);
-      hwy[m] = make_double2(std::cos(th), std::sin(th));
-    }
-    {  // the butterflies' scaled-twiddle records follow each twiddle table in its buffer
-      const std::vector<double2> sx = scaled_twiddle_table(xp.plan), sy = scaled_twiddle_table(yp.plan);
+    {  // the x transforms' tables follow the M-table in the same buffer
+      const std::vector<double2> sx = fft_tables(xp.plan);
       hwx.insert(hwx.end(), sx.begin(), sx.end());
-      hwy.insert(hwy.end(), sy.begin(), sy.end());
     }
+    const std::vector<double2> hwy = fft_tables(yp.plan);
     const double hone = 1.0;
     auto up = [&](DevBuf& b, const void* h, size_t bytes) -> cudaError_t {
       cudaError_t e = b.ensure(bytes);
@@ -151,7 +147,7 @@ struct Couette : EqImpl {
       return cudaMemcpyAsync(b.ptr, h, bytes, cudaMemcpyHostToDevice, p->stream);
     };
     SPADJ_CUDA_TRY(p, up(wmx, hwx.data(), sizeof(double2) * hwx.size()));
-    SPADJ_CUDA_TRY(p, up(w2y, hwy.data(), sizeof(double2) * hwy.size()));
+    SPADJ_CUDA_TRY(p, up(twy, hwy.data(), sizeof(double2) * hwy.size()));
     SPADJ_CUDA_TRY(p, up(czE, hczE.data(), sizeof(double) * hczE.size()));
     SPADJ_CUDA_TRY(p, up(cdzE, hcdzE.data(), sizeof(double) * hcdzE.size()));
     SPADJ_CUDA_TRY(p, up(gzF, hgzF.data(), sizeof(double) * hgzF.size()));
@@ -162,9 +158,8 @@ struct Couette : EqImpl {
     SPADJ_CUDA_TRY(p, up(one, &hone, sizeof(double)));
     SPADJ_CUDA_TRY(p, cudaStreamSynchronize(p->stream));
     xp.WM = wmx.as<double2>();
-    yp.W2 = w2y.as<double2>();
-    bind_scaled_twiddles(xp.plan, xp.WM + Mx);
-    bind_scaled_twiddles(yp.plan, yp.W2 + 2 * My);
+    fft_bind(xp.plan, xp.WM + Mx, xp.WM);
+    fft_bind(yp.plan, twy.as<double2>(), nullptr);
     const size_t sb = sizeof(double2) * ns, gb = sizeof(double) * npts;
     SPADJ_CUDA_TRY(p, Zm.ensure(6 * sizeof(double2) * nzm));
     SPADJ_CUDA_TRY(p, Ym.ensure(6 * sizeof(double2) * nym));
@@ -1204,7 +1199,7 @@ struct Couette : EqImpl {
     for (auto& o2 : band)
       for (BandDev& B : o2)
         for (DevBuf* b : {&B.L, &B.U, &B.dinv, &B.piv, &B.ssb}) b->release();
-    for (DevBuf* b : {&wmx, &w2y, &czE, &cdzE, &gzF, &gzTE, &czTF, &cdzTF, &gmat, &phi1F, &phi1A, &phi2F, &phi2A, &one,
+    for (DevBuf* b : {&wmx, &twy, &czE, &cdzE, &gzF, &gzTE, &czTF, &cdzTF, &gmat, &phi1F, &phi1A, &phi2F, &phi2A, &one,
                       &Zm, &Ym, &Gf, &dGf, &Gb, &Fg, &Xr, &Fr, &dXr, &dFr, &Wr, &xbar, &src0, &partial, &edev, &sdev,
                       &Jdev, &slots, &wts, &phiRF, &phiRA, &ginv, &nrm, &g2, &htraj, &hdtraj, &dWr, &dxbar, &htmp})
       b->release();

@@ -8,7 +8,7 @@
 //   y-mixed       [Mz][My][Kx]          complex (z and y on the grid, x spectral)
 //   grid          [Mz][My][Mx]          real
 #pragma once
-#include "fft.cuh"
+#include "fxfft.cuh"
 #include "pdl.cuh"
 
 namespace spadj {
@@ -46,11 +46,10 @@ struct YParams {
   int Kx, Ny, My, TK, ntile;
   double kxs, kys;
   FFTPlan plan;
-  const double2* W2;  // exp(-2 pi i m / (2 My)), m < 2 My
 };
 
 // CTA = (z row, tile of TK adjacent kx columns, job); the TK columns are transformed together.
-__global__ void __launch_bounds__(128) yfft_kernel(const __grid_constant__ YJobs js, YParams P) {
+__global__ void __launch_bounds__(128) yfft_kernel(const __grid_constant__ YJobs js, const __grid_constant__ YParams P) {
   pdl_trigger();
   pdl_wait();
   const YJob& J = js.j[blockIdx.y];
@@ -58,20 +57,17 @@ __global__ void __launch_bounds__(128) yfft_kernel(const __grid_constant__ YJobs
   const int TK = P.TK, Kx = P.Kx, Ny = P.Ny, My = P.My;
   const int m0 = tile * TK;
   const int tk = min(TK, Kx - m0);
-  extern __shared__ double2 sy[];
-  double2* a = sy;
-  double2* b = sy + (size_t)My * TK;
+  const int a = 0, b = My * TK;
+  const FxLay lay{1, TK, My * TK, 0};
   const int tid = threadIdx.x, nt = blockDim.x;
   if (J.dir == 0) {
-    for (int idx = tid; idx < My * TK; idx += nt) a[idx] = make_double2(0.0, 0.0);
-    __syncthreads();
-    for (int idx = tid; idx < Ny * TK; idx += nt) {
-      const int q = idx / TK, c = idx - q * TK;
-      const int e = ypos(q, Ny, My);
-      if (c >= tk || e < 0) continue;
+    const FxRes r = xf_c2c<1, 1, true>(a, b, lay, P.plan, [&](int, int c, int e) {
+      // entry e holds ky row q (none between the positive and the negative wavenumbers)
+      const int q = e < Ny / 2 ? e : e - (My - Ny);
+      double2 v = make_double2(0.0, 0.0);
+      if (c >= tk || (e >= Ny / 2 && q <= Ny / 2)) return v;
       const int m = m0 + c;
       const size_t g = ((size_t)i * Ny + q) * Kx + m;
-      double2 v = make_double2(0.0, 0.0);
       for (int t = 0; t < J.nin; ++t) {
         double2 x = J.in[t][g];
         if (J.mult[t]) {
@@ -81,26 +77,21 @@ __global__ void __launch_bounds__(128) yfft_kernel(const __grid_constant__ YJobs
         v.x = fma(J.alpha[t], x.x, v.x);
         v.y = fma(J.alpha[t], x.y, v.y);
       }
-      a[e * TK + c] = v;
-    }
-    __syncthreads();
-    const double2* r = cfft_smem_batch<1>(a, b, P.plan, P.W2, TK);
+      return v;
+    });
     for (int idx = tid; idx < My * TK; idx += nt) {
       const int e = idx / TK, c = idx - e * TK;
-      if (c < tk) J.out[((size_t)i * My + e) * Kx + m0 + c] = cscale(r[idx], J.scale);
+      if (c < tk) J.out[((size_t)i * My + e) * Kx + m0 + c] = cscale(r.at(0, c, e), J.scale);
     }
   } else {
-    for (int idx = tid; idx < My * TK; idx += nt) {
-      const int e = idx / TK, c = idx - e * TK;
-      a[idx] = c < tk ? J.in[0][((size_t)i * My + e) * Kx + m0 + c] : make_double2(0.0, 0.0);
-    }
-    __syncthreads();
-    const double2* r = cfft_smem_batch<-1>(a, b, P.plan, P.W2, TK);
+    const FxRes r = xf_c2c<-1, 1, true>(a, b, lay, P.plan, [&](int, int c, int e) {
+      return c < tk ? J.in[0][((size_t)i * My + e) * Kx + m0 + c] : make_double2(0.0, 0.0);
+    });
     for (int idx = tid; idx < Ny * TK; idx += nt) {
       const int q = idx / TK, c = idx - q * TK;
       if (c >= tk) continue;
       const int e = ypos(q, Ny, My);
-      J.out[((size_t)i * Ny + q) * Kx + m0 + c] = e < 0 ? make_double2(0.0, 0.0) : cscale(r[e * TK + c], J.scale);
+      J.out[((size_t)i * Ny + q) * Kx + m0 + c] = e < 0 ? make_double2(0.0, 0.0) : cscale(r.at(0, c, e), J.scale);
     }
   }
 }

@@ -33,6 +33,13 @@ struct FFTPlan {
   int nrad;               // number of passes
   unsigned char rad[8];   // radix of each pass (product = n)
   const double2* sc[2];   // device scaled-twiddle records: [0] exp(-), [1] exp(+)
+  // fixed-point passes (fxfft.cuh): the radices a byte each from the low end, the passes' twiddles of
+  // both directions, the real transforms' unpacking factors, the passes' scalings, FP64 unpacking factors
+  unsigned long long radw;
+  const int4* fx[2];
+  const int4* fxr;
+  const int* fxs;
+  const double2* wm;
 };
 
 // double2 entries of one record (one twiddle index k of a pass) for radix R

@@ -1,0 +1,790 @@
+// Collocation FFTs in 64-bit block fixed point: the transforms' FP64 inputs and outputs, with the
+// butterflies between them on the integer pipes.
+//
+// Why: this chip issues 2 FP64 multiply-adds per clock and SM against 64 32-bit integer
+// multiply-adds, about 32 of their 32 x 32 + 64 bit form and 128 additions (measured: 1.6, 59, 25
+// and 110 a clock; a 64-bit addition costs 1/34 of an FP64 one).  A radix-4 butterfly with three
+// twiddles is 22 FP64 instructions (14 clocks per thread and SM) or 36 wide multiply-adds and
+// about 70 additions and shifts (2 clocks).
+//
+// Format.  One sequence of the transform shares one exponent: its largest input component, of
+// biased exponent emax, is placed below 2^B (B = 59; 58 for the packed real spectra), and every value is a
+// signed 64-bit integer from there on.  Twiddles are fixed point too (2^-61 resolution).  A product
+// keeps the top 64 bits of the 128: with
+//   x 2^-sg = 2^29 xh + xl / 8,   w = 2^-29 wh + 2^-61 wl     (signed 32-bit xh, xl, wh, wl)
+//   x w 2^-sg = xh wh + (xh wl + xl wh) 2^-32 + O(1/4)
+// which is three wide multiply-adds, and the cross products' high word is taken by register, not by a
+// shift; sg in 0..3 is a free scaling by 2^-sg (it only moves the split).
+//
+// Overflow.  A product's scaled operand has a complex modulus <= 2^60 (then the sums of four products stay
+// below 2^63), so a pass of radix R <= 4 leaves moduli <= 2^62.  A pass multiplies the bound of the
+// moduli by at most R, and no value ever exceeds the sum of the moduli of the pass-0 inputs times
+// the scalings so far.  Each pass scales by the smallest 2^-sg that brings the smaller of the two bounds
+// to 2^60: a peaked input (one mode, a smooth spectrum) is hardly scaled at all, a flat one by 2^-2 per
+// radix-4 pass.
+//
+// Accuracy.  The rounding is about 0.7 units of 2^-59 of the largest value in each pass, against 2^-53 of each
+// value in FP64, and the results are rounded to FP64 once: the relative 2-norm error of complex transforms
+// (n = 3..1536; flat, smooth, single-mode and 1/k inputs) is 0.4-1.3e-16 against 1.3-2.5e-16 of FP64
+// butterflies, and that of the real ones up to 2 x 768 points 0.5-2.0e-16 against 1.3-2.8e-16; the longer
+// real transforms (peaked spectra: 2.0e-16 against 2.0e-16) stay with the FP64 butterflies of fft.cuh.  Non-finite
+// input gives NaN in every output of the sequence; sequences below 2^-895 are scaled up by 2^512 first, so
+// subnormals keep their bits.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <cmath>
+#include <cstdint>
+#include <cstring>
+#include <vector>
+
+#include "fft.cuh"
+
+namespace spadj {
+
+constexpr int kFxMaxN = 2048;      // longest complex transform: 32-bit index and sum ranges
+constexpr int kFxMaxReal = 768;    // longest packed real transform (2 x 768 grid points)
+constexpr int kFxB = 59, kFxBReal = 58;  // log2 of the bound on the converted inputs' components
+constexpr int kFxSeqMax = 8;       // sequences of one call
+constexpr int kFxWarpsMax = 8;     // warps of a CTA that calls the transforms
+constexpr int kFxNaN = 1 << 20;    // scale exponent of a sequence with non-finite input
+
+struct alignas(16) fx2 {
+  long long x, y;
+};
+struct FxLimb {
+  int h, l;
+};
+
+// Memory accesses of the transforms' kernels are written out one by one (here and at fx_get / fx_put), each of
+// exactly its own width.
+__device__ __forceinline__ double2 ldg128(const double2* p) {
+  double2 v;
+  asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ void stg128(double2* p, double2 v) {
+  asm volatile("st.global.v2.f64 [%0], {%1, %2};" ::"l"(p), "d"(v.x), "d"(v.y) : "memory");
+}
+__device__ __forceinline__ int4 ldtab(const int4* p) {  // read-only tables
+  int4 v;
+  asm volatile("ld.global.nc.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+
+// ---- arithmetic (host and device: the host side is the CPU check of the same code) ----------------
+
+__host__ __device__ __forceinline__ FxLimb fx_split(long long v, int sg) {
+  const unsigned lo = (unsigned)v, hi = (unsigned)(v >> 32);
+  FxLimb r;
+  r.l = (int)(lo << (3 - sg));
+#ifdef __CUDA_ARCH__
+  r.h = (int)(__funnelshift_rc(lo, hi, 29 + sg) + ((unsigned)r.l >> 31));
+#else
+  r.h = (int)((unsigned)(((unsigned long long)hi << 32 | lo) >> (29 + sg)) + ((unsigned)r.l >> 31));
+#endif
+  return r;
+}
+__host__ __device__ __forceinline__ long long fx_mad(int a, int b, long long c) { return (long long)a * b + c; }
+// high word of a cross-product sum, sign-extended
+__host__ __device__ __forceinline__ long long fx_hi(long long c) { return (long long)(int)(c >> 32); }
+constexpr long long kFxRound = 1ll << 31;
+
+// v w 2^-sg, w = (re.h, re.l, im.h, im.l)
+__host__ __device__ __forceinline__ fx2 fx_cmul(fx2 v, int4 w, int sg) {
+  const FxLimb a = fx_split(v.x, sg), b = fx_split(v.y, sg);
+  const int nh = -w.z, nl = -w.w;
+  const long long cr = fx_mad(b.h, nl, fx_mad(b.l, nh, fx_mad(a.h, w.y, fx_mad(a.l, w.x, kFxRound))));
+  const long long ci = fx_mad(b.h, w.y, fx_mad(b.l, w.x, fx_mad(a.h, w.w, fx_mad(a.l, w.z, kFxRound))));
+  fx2 r;
+  r.x = fx_mad(a.h, w.x, fx_mad(b.h, nh, fx_hi(cr)));
+  r.y = fx_mad(a.h, w.z, fx_mad(b.h, w.x, fx_hi(ci)));
+  return r;
+}
+// v c for a real constant c = 2^-29 ch + 2^-61 cl
+__host__ __device__ __forceinline__ long long fx_rmul(long long v, int ch, int cl) {
+  const FxLimb a = fx_split(v, 0);
+  return fx_mad(a.h, ch, fx_hi(fx_mad(a.h, cl, fx_mad(a.l, ch, kFxRound))));
+}
+__host__ __device__ __forceinline__ fx2 fx_add(fx2 a, fx2 b) { return fx2{a.x + b.x, a.y + b.y}; }
+__host__ __device__ __forceinline__ fx2 fx_sub(fx2 a, fx2 b) { return fx2{a.x - b.x, a.y - b.y}; }
+__host__ __device__ __forceinline__ fx2 fx_shr(fx2 a, int sg) { return fx2{a.x >> sg, a.y >> sg}; }
+template <int SIGN>
+__host__ __device__ __forceinline__ fx2 fx_rot(fx2 a) {  // SIGN i a
+  return SIGN > 0 ? fx2{-a.y, a.x} : fx2{a.y, -a.x};
+}
+
+// Butterflies in place, scaled by 2^-sg; w: the pass's twiddles of this k (R - 1 of them), nullptr for the
+// first pass.
+template <int SIGN>
+__host__ __device__ __forceinline__ void fx_out4(fx2& v0, fx2& v1, fx2& v2, fx2& v3) {
+  const fx2 t0 = fx_add(v0, v2), t1 = fx_sub(v0, v2), t2 = fx_add(v1, v3);
+  const fx2 t3 = fx_sub(v1, v3);
+  v0 = fx_add(t0, t2);
+  v2 = fx_sub(t0, t2);
+  if (SIGN > 0) {  // t1 +- i t3
+    v1 = fx2{t1.x - t3.y, t1.y + t3.x};
+    v3 = fx2{t1.x + t3.y, t1.y - t3.x};
+  } else {
+    v1 = fx2{t1.x + t3.y, t1.y - t3.x};
+    v3 = fx2{t1.x - t3.y, t1.y + t3.x};
+  }
+}
+constexpr int kFxS3h = 464943848, kFxS3l = 1481419380;  // sqrt(3)/2 = 2^-29 h + 2^-61 l
+template <int SIGN>
+__host__ __device__ __forceinline__ void fx_out3(fx2& v0, fx2& v1, fx2& v2) {
+  const fx2 t = fx_add(v1, v2), d = fx_sub(v1, v2);
+  const fx2 m = fx_sub(v0, fx_shr(t, 1));
+  const fx2 r = fx_rot<SIGN>(fx2{fx_rmul(d.x, kFxS3h, kFxS3l), fx_rmul(d.y, kFxS3h, kFxS3l)});
+  v0 = fx_add(v0, t);
+  v1 = fx_add(m, r);
+  v2 = fx_sub(m, r);
+}
+
+// Fixed-point value of the double x: x = v 2^(emax + 1 - 1023 - B) to the last unit (toward zero), |v| < 2^B
+// for biased exponents <= emax.  emax >= 128, so that whatever has a zero exponent field vanishes.
+template <int B>
+__host__ __device__ __forceinline__ long long fx_from_double(double x, int emax) {
+#ifdef __CUDA_ARCH__
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+#else
+  unsigned long long bits;
+  std::memcpy(&bits, &x, 8);
+  const unsigned hi = (unsigned)(bits >> 32), lo = (unsigned)bits;
+#endif
+  const int d = emax - (int)((hi >> 20) & 0x7ff);
+  const unsigned long long m = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32 | lo) << (B - 53);
+  unsigned long long v;
+#ifdef __CUDA_ARCH__
+  asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"(d));  // shifts above 63 give 0
+#else
+  v = d > 63 ? 0 : m >> d;
+#endif
+  const long long s = (int)hi >> 31;
+  return ((long long)v ^ s) - s;
+}
+
+// v 2^se rounded to FP64; se >= kFxNaN / 2 marks a sequence with non-finite input.
+__host__ __device__ inline double fx_to_double_rare(long long v, int se) {
+#ifdef __CUDA_ARCH__
+  if (se >= kFxNaN / 2) return __longlong_as_double(0x7ff8000000000000ll);
+#else
+  if (se >= kFxNaN / 2) return std::nan("");
+#endif
+  return ldexp((double)v, se);  // overflow and subnormal results
+}
+__host__ __device__ __forceinline__ double fx_to_double(long long v, int se) {
+  const long long s = v >> 63;
+  const unsigned long long mag = (unsigned long long)((v ^ s) - s);
+#ifdef __CUDA_ARCH__
+  const int lz = __clzll((long long)mag);
+#else
+  const int lz = mag ? __builtin_clzll(mag) : 64;
+#endif
+  const int e = se + 1086 - lz;  // biased exponent of the leading bit
+  if ((unsigned)(e - 1) >= 2046u) return fx_to_double_rare(v, se);
+  const unsigned long long m = mag << (lz & 63);
+  // mantissa with the implicit bit at 52, rounded half up; a carry moves into the exponent
+  unsigned long long bits = (m >> 11) + ((m >> 10) & 1) + ((unsigned long long)(e - 1) << 52);
+  bits = mag ? bits : 0ull;
+  bits |= (unsigned long long)s & 0x8000000000000000ull;
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double((long long)bits);
+#else
+  double r;
+  std::memcpy(&r, &bits, 8);
+  return r;
+#endif
+}
+
+// Entries k and n - k of the packed spectrum of a half-length real transform, from x = c_k and y = c_{n-k}
+// (0 where not stored), w = exp(-i pi k / n):
+//   Z_k = e + t,  Z_{n-k} = conj(e - t),  e = x + conj(y),  t = i conj(w) (x - conj(y))
+__host__ __device__ __forceinline__ void fx_pack(fx2 x, fx2 y, int4 w, fx2& z0, fx2& z1) {
+  w.z = -w.z;
+  w.w = -w.w;
+  const fx2 t = fx_cmul(fx2{-x.y - y.y, x.x - y.x}, w, 0);
+  z0 = fx2{x.x + y.x + t.x, x.y - y.y + t.y};
+  z1 = fx2{x.x + y.x - t.x, y.y - x.y + t.y};
+}
+// A quarter of the spectrum entry ((u + conj(v)) - i w (u - conj(v))) / 2 of a real field from the entries u = Z_k, v = Z_{n-k} of
+// its packed transform.
+__host__ __device__ __forceinline__ fx2 fx_unpack(fx2 u, fx2 v, int4 w) {
+  const fx2 t = fx_cmul(fx2{u.y + v.y, v.x - u.x}, w, 3);
+  return fx2{((u.x + v.x) >> 3) + t.x, ((u.y - v.y) >> 3) + t.y};
+}
+__host__ __device__ __forceinline__ unsigned fx_l1(fx2 v) {  // >= (|x| + |y|) / 2^42
+  const int x = (int)(v.x >> 32), y = (int)(v.y >> 32);
+  return ((unsigned)(x < 0 ? -x : x) >> 10) + ((unsigned)(y < 0 ? -y : y) >> 10) + 2u;
+}
+
+// The scalings sg of the passes, two bits each from the low end, and their sum in bits 24.. : b2 = twice the
+// log2 of the bound on the pass-0 moduli, l2 = twice that of the bound on the sum of the moduli.
+__host__ __device__ inline int fx_schedule(unsigned long long radw, int b2, int l2) {
+  int bits = 0, tot = 0;
+  for (int i = 0; radw; ++i, radw >>= 8) {
+    const int sg = i > 0 && b2 > 120 ? (b2 - 119) / 2 : 0;
+    bits |= sg << (2 * i);
+    tot += sg;
+    l2 -= 2 * sg;
+    b2 += ((radw & 0xff) == 2 ? 2 : 4) - 2 * sg;
+    if (b2 > l2) b2 = l2;
+  }
+  return bits | tot << 24;
+}
+
+// ---- tables (host) ---------------------------------------------------------------------------------
+
+inline void fx_const(long double w, int* h, int* l) {
+  const long long W = llroundl(w * 2305843009213693952.0L);  // 2^61
+  const long long hh = (W + (1ll << 31)) >> 32;
+  long long ll = W - (hh << 32);
+  if (ll == -(1ll << 31)) ll += 1;  // its negative stays a 32-bit number
+  *h = (int)hh;
+  *l = (int)ll;
+}
+// exp(i pi j / n), j < 2n, from the cosines and sines of the first octant (4 | n; else all of them)
+inline std::vector<int4> fx_roots(int n) {
+  std::vector<int4> r(2 * n);
+  const long double pi = 3.14159265358979323846264338327950288L;
+  auto at = [&](int j) {
+    int4 w;
+    fx_const(cosl(pi * j / n), &w.x, &w.y);
+    fx_const(sinl(pi * j / n), &w.z, &w.w);
+    return w;
+  };
+  if (n % 4 != 0) {
+    for (int j = 0; j < 2 * n; ++j) r[j] = at(j);
+    return r;
+  }
+  for (int j = 0; j <= n / 4; ++j) r[j] = at(j);
+  for (int j = n / 4 + 1; j <= n / 2; ++j) {  // mirrored at 45 degrees
+    const int4 a = r[n / 2 - j];
+    r[j] = make_int4(a.z, a.w, a.x, a.y);
+  }
+  for (int j = n / 2 + 1; j < 2 * n; ++j) {  // quarter turns
+    const int4 a = r[j - n / 2];
+    r[j] = make_int4(-a.z, -a.w, a.x, a.y);
+  }
+  return r;
+}
+// entries of one direction's twiddles: R - 1 per (pass with Ns > 1, k)
+inline int fx_twiddle_entries(const FFTPlan& p) {
+  int e = 0, Ns = 1;
+  for (int i = 0; i < p.nrad; ++i) {
+    if (Ns > 1) e += Ns * (p.rad[i] - 1);
+    Ns *= p.rad[i];
+  }
+  return e;
+}
+// exp(-) twiddles, exp(+) twiddles in pass order, then exp(-pi i k / n), k < n (the real transforms'
+// unpacking), then the scalings of the passes by the leading zeros of the sum of the moduli (fx_schedule; 32
+// words for complex, 32 for packed real inputs), as 16-byte entries
+inline std::vector<double2> fx_table(const FFTPlan& p) {
+  const std::vector<int4> root = fx_roots(p.n);
+  const int period = 2 * p.n;
+  std::vector<int4> t;
+  for (int dir = 0; dir < 2; ++dir) {
+    int Ns = 1;
+    for (int i = 0; i < p.nrad; ++i) {
+      const int R = p.rad[i], step = period / (R * Ns);
+      if (Ns > 1)
+        for (int k = 0; k < Ns; ++k)
+          for (int m = 1; m < R; ++m) t.push_back(root[dir ? m * k * step : (period - m * k * step) % period]);
+      Ns *= R;
+    }
+  }
+  for (int k = 0; k < p.n; ++k) t.push_back(root[(period - k) % period]);
+  for (int b2 : {2 * kFxB + 1, 2 * kFxBReal + 5})
+    for (int z = 0; z < 32; z += 4) {
+      int s[4];
+      for (int q = 0; q < 4; ++q) s[q] = fx_schedule(p.radw, b2, 2 * (42 + 32 - (z + q)));
+      t.push_back(make_int4(s[0], s[1], s[2], s[3]));
+    }
+  std::vector<double2> out(t.size());
+  std::memcpy(out.data(), t.data(), sizeof(int4) * t.size());
+  return out;
+}
+// the FP64 records are built only for lengths that use them
+inline bool fx_needs_fp64(const FFTPlan& p) { return p.n > kFxMaxReal; }
+// All tables of a plan (the fixed-point ones, then the FP64 records where needed), and the plan's pointers into the device
+// copy; wm: device table of exp(-2 pi i m / 2n), m < 2n.
+inline std::vector<double2> fft_tables(FFTPlan& p) {
+  p.radw = 0;
+  for (int i = 0; i < p.nrad; ++i) p.radw |= (unsigned long long)p.rad[i] << (8 * i);
+  std::vector<double2> t = fx_table(p);
+  if (fx_needs_fp64(p)) {
+    const std::vector<double2> s = scaled_twiddle_table(p);
+    t.insert(t.end(), s.begin(), s.end());
+  }
+  return t;
+}
+inline void fft_bind(FFTPlan& p, const double2* dev, const double2* wm) {
+  const int e = fx_twiddle_entries(p);
+  const int4* t = reinterpret_cast<const int4*>(dev);
+  p.fx[0] = t;
+  p.fx[1] = t + e;
+  p.fxr = t + 2 * e;
+  p.fxs = reinterpret_cast<const int*>(p.fxr + p.n);
+  if (fx_needs_fp64(p)) bind_scaled_twiddles(p, dev + 2 * e + p.n + 16);
+  p.wm = wm;
+}
+
+// ---- device: the transform of the sequences of one CTA ------------------------------------------------
+//
+// Buffers are offsets (in 16-byte entries) into the CTA's dynamic shared memory, so that every access
+// is a shared-memory access with a 32-bit address.  Sequence
+// s = set * nb + c holds element e at [set * stride + e * nb + c] of its buffers a and b: ns sets of nb
+// interleaved sequences.  All threads of the CTA (a multiple of 32, <= 256) call.
+
+__device__ __forceinline__ double2* fx_mem64() {
+  extern __shared__ double2 fx_dyn[];
+  return fx_dyn;
+}
+// One 16-byte shared-memory access each, to entry e of the buffers (written out, so that neighbouring entries
+// are never combined into accesses that ask for more than 16-byte alignment).
+__device__ __forceinline__ unsigned fx_addr(int e) {
+  return static_cast<unsigned>(__cvta_generic_to_shared(fx_mem64())) + 16u * (unsigned)e;
+}
+__device__ __forceinline__ fx2 fx_get(int e) {
+  fx2 v;
+  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(fx_addr(e)) : "memory");
+  return v;
+}
+__device__ __forceinline__ void fx_put(int e, fx2 v) {
+  asm volatile("st.shared.v2.b64 [%0], {%1, %2};" ::"r"(fx_addr(e)), "l"(v.x), "l"(v.y) : "memory");
+}
+__device__ __forceinline__ double2 fx_get64(int e) {
+  double2 v;
+  asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(fx_addr(e)) : "memory");
+  return v;
+}
+__device__ __forceinline__ void fx_put64(int e, double2 v) {
+  asm volatile("st.shared.v2.f64 [%0], {%1, %2};" ::"r"(fx_addr(e)), "d"(v.x), "d"(v.y) : "memory");
+}
+
+// Per-warp slots: every warp reduces over its own entries, and all warps combine the slots after the
+// barrier that the data needs anyway.
+struct alignas(16) FxShared {
+  unsigned mx[kFxWarpsMax][kFxSeqMax];  // largest |high word| of the sequence's components
+  unsigned l1[kFxWarpsMax][kFxSeqMax];  // sum of the moduli, in units of 2^42
+  unsigned se[kFxWarpsMax][kFxSeqMax];  // scale exponent of the results and scalings of the passes (each
+  unsigned sch[kFxWarpsMax][kFxSeqMax]; // warp's copy)
+};
+__device__ __forceinline__ FxShared& fx_shared() {
+  __shared__ FxShared s;
+  return s;
+}
+__device__ __forceinline__ unsigned lds32(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(static_cast<unsigned>(__cvta_generic_to_shared(p))) : "memory");
+  return v;
+}
+__device__ __forceinline__ void sts32(unsigned* p, unsigned v) {
+  asm volatile("st.shared.b32 [%0], %1;" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(p))), "r"(v) : "memory");
+}
+
+struct FxLay {
+  int ns, nb, stride;  // sets, interleaved sequences per set, entries between sets
+  int s0;              // first of the call's ns * nb slots for the sequences' scales (a later call on other
+                       // slots leaves the earlier results readable)
+};
+
+__device__ __forceinline__ unsigned fx_absmax(unsigned m, double2 v) {
+  return max(m, max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu));
+}
+// Reductions over a warp by shuffles
+__device__ __forceinline__ unsigned fx_warp_max(unsigned v) {
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, d));
+  return v;
+}
+__device__ __forceinline__ unsigned fx_warp_sum(unsigned v) {
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+  return v;
+}
+// Before fx_put_max with nb > 1: the warp's slots of ns * nb sequences to zero
+__device__ __forceinline__ void fx_clear(unsigned (&slots)[kFxWarpsMax][kFxSeqMax], int s0, int nseq) {
+  const int l = threadIdx.x & 31;
+  if (l < nseq) sts32(&slots[threadIdx.x >> 5][s0 + l], 0u);
+  __syncwarp();
+}
+// The warp's largest high word of a set's sequences from each thread's m; all threads call, c = the thread's
+// sequence in the set or -1 when it saw none (nb == 1: one sequence, no clearing needed)
+__device__ __forceinline__ void fx_put_max(int set, int nb, int c, unsigned m, int s0 = 0) {
+  FxShared& S = fx_shared();
+  const int w = threadIdx.x >> 5;
+  if (nb == 1) {
+    m = fx_warp_max(m);
+    if ((threadIdx.x & 31) == 0) sts32(&S.mx[w][s0 + set], m);
+  } else if (c >= 0) {
+    atomicMax(&S.mx[w][s0 + set * nb + c], m);
+  }
+}
+__device__ __forceinline__ unsigned fx_get_max(int s) {
+  unsigned m = 0u;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = max(m, lds32(&fx_shared().mx[w][s]));
+  return m;
+}
+struct FxExp {
+  int emax;  // biased exponent of the sequence's scale, >= 128
+  bool pre;  // inputs are multiplied by 2^512 first (sequences of tiny values)
+};
+__device__ __forceinline__ FxExp fx_exponent(unsigned mx) {
+  FxExp r;
+  r.emax = (int)(mx >> 20);
+  r.pre = r.emax < 128;
+  if (r.pre) r.emax = max(r.emax, 1) + 512;
+  return r;
+}
+template <int B>
+__device__ __forceinline__ fx2 fx_load(double2 v, FxExp e) {
+  if (e.pre) {
+    v.x *= 0x1p512;
+    v.y *= 0x1p512;
+  }
+  return fx2{fx_from_double<B>(v.x, e.emax), fx_from_double<B>(v.y, e.emax)};
+}
+
+// Each warp writes its copy of the sequences' scale exponents and scalings (after a barrier that makes mx and
+// l1 final): results are v 2^exponent.  sched: the plan's table for this kind of input.
+template <int B>
+__device__ __forceinline__ void fx_make_meta(FxLay lay, const int* __restrict__ sched) {
+  FxShared& S = fx_shared();
+  const int lane = lay.s0 + (threadIdx.x & 31), w = threadIdx.x >> 5;
+  if (lane < lay.s0 + lay.ns * lay.nb) {
+    unsigned mx = 0u, l1 = 0u;
+    for (int v = 0; v < (int)(blockDim.x >> 5); ++v) {
+      mx = max(mx, lds32(&S.mx[v][lane]));
+      l1 += lds32(&S.l1[v][lane]);
+    }
+    const int sch = __ldg(sched + __clz((int)l1));
+    const FxExp e = fx_exponent(mx);
+    sts32(&S.se[w][lane], (unsigned)(mx >= 0x7ff00000u ? kFxNaN : e.emax + 1 - 1023 - B + (sch >> 24) - (e.pre ? 512 : 0)));
+    sts32(&S.sch[w][lane], (unsigned)sch);
+  }
+  __syncwarp();
+}
+__device__ __forceinline__ int fx_se(int s) { return (int)lds32(&fx_shared().se[threadIdx.x >> 5][s]); }
+__device__ __forceinline__ int fx_sch(int s) { return (int)lds32(&fx_shared().sch[threadIdx.x >> 5][s]); }
+
+// Bank-conflict-free order of the entries written by the passes with Ns <= 4 (consecutive threads store
+// 64 bytes apart there): the low three bits are exchanged by XOR with higher ones, inside groups of 8.
+__device__ __forceinline__ int fx_swz(int e) {
+  const int t = e >> 3;
+  return e ^ ((t & 3) | ((t & 2) << 1));
+}
+
+// j mod Ns (Ns a power of two, or via the multiplier inv = ceil(2^20 / Ns); j Ns < 2^20)
+__device__ __forceinline__ int fx_mod(int j, int Ns, unsigned inv) {
+  if ((Ns & (Ns - 1)) == 0) return j & (Ns - 1);
+  return j - (int)(((unsigned)j * inv) >> 20) * Ns;
+}
+
+// The butterfly passes of NS sets over the entries in a; the results are in a when the number of passes is even,
+// else in b.  On return they are visible to all threads.
+template <int SIGN, int NS>
+__device__ __forceinline__ void fx_passes(int a, int b, FxLay lay, int n, unsigned long long radw,
+                                          const int4* __restrict__ tw) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const int nb = lay.nb;
+  const bool swz = nb == 1 && (n & 7) == 0;
+  int Ns = 1;
+  bool rs = false;
+#pragma unroll 1
+  for (int pass = 0; radw; ++pass) {
+    const int R = (int)(radw & 0xff), nbf = n / R, per = nbf * nb;
+    radw >>= 8;
+    const unsigned inv = (unsigned)(((1 << 20) + Ns - 1) / Ns);
+    const bool ws = swz && radw && Ns <= 4;
+#pragma unroll 1
+    for (int i = tid; i < NS * per; i += nt) {
+      int set = 0, j = i, c = 0;
+      if (NS > 1) {
+#pragma unroll
+        for (int s = 1; s < NS; ++s)
+          if (j >= per) {
+            j -= per;
+            ++set;
+          }
+      }
+      if (nb > 1) {
+        const int q = (nb & (nb - 1)) == 0 ? j >> (__ffs(nb) - 1) : j / nb;
+        c = j - q * nb;
+        j = q;
+      }
+      const int sg = (fx_sch(lay.s0 + set * nb + c) >> (2 * pass)) & 3;
+      const int as = a + set * lay.stride + c, bs = b + set * lay.stride + c;
+      const int k = fx_mod(j, Ns, inv);
+      const int base = (j - k) * R + k;
+      auto ld = [&](int e) { return fx_get(as + (rs ? fx_swz(e) : e) * nb); };
+      auto st = [&](int e, fx2 v) { fx_put(bs + (ws ? fx_swz(e) : e) * nb, v); };
+      if (R == 4) {
+        fx2 v0 = ld(j), v1 = ld(j + nbf), v2 = ld(j + 2 * nbf), v3 = ld(j + 3 * nbf);
+        if (pass > 0) {
+          const int4* w = tw + 3 * k;
+          v0 = fx_shr(v0, sg);
+          v1 = fx_cmul(v1, ldtab(w), sg);
+          v2 = fx_cmul(v2, ldtab(w + 1), sg);
+          v3 = fx_cmul(v3, ldtab(w + 2), sg);
+        }
+        fx_out4<SIGN>(v0, v1, v2, v3);
+        st(base, v0);
+        st(base + Ns, v1);
+        st(base + 2 * Ns, v2);
+        st(base + 3 * Ns, v3);
+      } else if (R == 3) {
+        fx2 v0 = ld(j), v1 = ld(j + nbf), v2 = ld(j + 2 * nbf);
+        if (pass > 0) {
+          const int4* w = tw + 2 * k;
+          v0 = fx_shr(v0, sg);
+          v1 = fx_cmul(v1, ldtab(w), sg);
+          v2 = fx_cmul(v2, ldtab(w + 1), sg);
+        }
+        fx_out3<SIGN>(v0, v1, v2);
+        st(base, v0);
+        st(base + Ns, v1);
+        st(base + 2 * Ns, v2);
+      } else {
+        fx2 v0 = ld(j), v1 = ld(j + nbf);
+        if (pass > 0) {
+          v0 = fx_shr(v0, sg);
+          v1 = fx_cmul(v1, ldtab(tw + k), sg);
+        }
+        st(base, fx_add(v0, v1));
+        st(base + Ns, fx_sub(v0, v1));
+      }
+    }
+    __syncthreads();
+    const int t = a;
+    a = b;
+    b = t;
+    if (Ns > 1) tw += Ns * (R - 1);
+    Ns *= R;
+    rs = ws;
+  }
+}
+
+// ---- device: transforms ----------------------------------------------------------------------------------
+//
+// xf_c2c, xf_c2r and xf_r2c stage their input through load(set, c, e) (called once per entry; CF: consecutive
+// threads take consecutive sequences c of an entry, otherwise consecutive entries), run the passes and
+// return the results where FxRes reads them; buffers a and b hold lay.stride entries per set, and what load reads
+// must not lie in them.  The CTA synchronises before the buffers are used again.  Lengths above kFxMaxN run
+// the FP64 butterflies (ANY = false: the caller's lengths never do).
+
+struct FxRes {
+  int z;  // buffer that holds the results
+  FxLay lay;
+  int n;
+  const int4* fxr;
+  const double2* wm;
+  bool fixed;  // constant true where the FP64 path is not compiled in
+  __device__ __forceinline__ double2 raw64(int set, int c, int e) const {
+    return fx_get64(z + set * lay.stride + e * lay.nb + c);
+  }
+  // entry e of a complex transform, or grid pair (g_2e, g_2e+1) of an inverse real one
+  __device__ __forceinline__ double2 at(int set, int c, int e) const {
+    if (!fixed) return raw64(set, c, e);
+    const fx2 v = fx_get(z + set * lay.stride + e * lay.nb + c);
+    const int se = fx_se(lay.s0 + set * lay.nb + c);
+    return make_double2(fx_to_double(v.x, se), fx_to_double(v.y, se));
+  }
+  // spectrum entry X_k = sum_j g_j exp(-2 pi i j k / 2n) of a forward real transform
+  __device__ __forceinline__ double2 coef(int set, int c, int k) const {
+    const int kc = k == 0 ? 0 : n - k;
+    if (!fixed) return r2c_combine(raw64(set, c, k), cconj(raw64(set, c, kc)), __ldg(&wm[k]));
+    const int q = z + set * lay.stride + c;
+    const fx2 u = fx_get(q + k * lay.nb), v = fx_get(q + kc * lay.nb);
+    const int se = fx_se(lay.s0 + set * lay.nb + c);
+    const fx2 r = fx_unpack(u, v, ldtab(fxr + k));
+    return make_double2(fx_to_double(r.x, se + 2), fx_to_double(r.y, se + 2));
+  }
+};
+
+// (entry, sequence in the set) of item i among cnt entries of nb sequences
+template <bool CF>
+__device__ __forceinline__ void fx_item(int i, int cnt, int nb, int& e, int& c) {
+  c = 0;
+  e = i;
+  if (nb == 1) return;
+  if (CF) {
+    e = (nb & (nb - 1)) == 0 ? i >> (__ffs(nb) - 1) : i / nb;
+    c = i - e * nb;
+  } else {
+    while (e >= cnt) {
+      e -= cnt;
+      ++c;
+    }
+  }
+}
+
+// FP64 values of cnt entries of every sequence into dst, and the sequences' largest high words
+template <int NS, bool CF, class Load>
+__device__ __forceinline__ void fx_stage(int dst, FxLay lay, int cnt, Load load) {
+  const int nb = lay.nb;
+  unsigned m[NS];
+  int cp = -1;
+  if (nb > 1) fx_clear(fx_shared().mx, lay.s0, NS * nb);
+#pragma unroll
+  for (int s = 0; s < NS; ++s) m[s] = 0u;
+  for (int i = threadIdx.x; i < cnt * nb; i += blockDim.x) {
+    int e, c;
+    fx_item<CF>(i, cnt, nb, e, c);
+    if (c != cp && cp >= 0) {
+#pragma unroll
+      for (int s = 0; s < NS; ++s) {
+        fx_put_max(s, nb, cp, m[s], lay.s0);
+        m[s] = 0u;
+      }
+    }
+    cp = c;
+    double2 v[NS];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) v[s] = load(s, c, e);
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      fx_put64(dst + s * lay.stride + e * nb + c, v[s]);
+      m[s] = fx_absmax(m[s], v[s]);
+    }
+  }
+#pragma unroll
+  for (int s = 0; s < NS; ++s) fx_put_max(s, nb, cp, m[s], lay.s0);
+}
+
+__device__ __forceinline__ void fx_put_l1(int s0, int set, int nb, int c, unsigned s) {
+  FxShared& S = fx_shared();
+  const int w = threadIdx.x >> 5;
+  if (nb == 1) {
+    s = fx_warp_sum(s);
+    if ((threadIdx.x & 31) == 0) sts32(&S.l1[w][s0 + set], s);
+  } else if (c >= 0) {
+    atomicAdd(&S.l1[w][s0 + set * nb + c], s);
+  }
+}
+
+template <int SIGN, int NS>
+__device__ __forceinline__ FxRes fx_run(int a, int b, FxLay lay, const FFTPlan& p) {
+  fx_passes<SIGN, NS>(a, b, lay, p.n, p.radw, p.fx[SIGN > 0 ? 1 : 0]);
+  return FxRes{(p.nrad & 1) ? b : a, lay, p.n, p.fxr, p.wm, true};
+}
+template <int SIGN>
+__device__ __forceinline__ FxRes fx_run64(int a, int b, FxLay lay, int NS, const FFTPlan& p) {
+  cfft_smem_sets<SIGN>(fx_mem64() + a, fx_mem64() + b, lay.stride, NS, p, lay.nb);
+  return FxRes{(p.nrad & 1) ? b : a, lay, p.n, p.fxr, p.wm, false};
+}
+// Complex transform of length p.n, unnormalised: exp(-) for SIGN < 0, exp(+) for SIGN > 0.
+template <int SIGN, int NS, bool CF, bool ANY = true, class Load>
+__device__ __forceinline__ FxRes xf_c2c(int a, int b, FxLay lay, const FFTPlan& p, Load load,
+                                         int max_n = kFxMaxN) {
+  const int nb = lay.nb, n = p.n;
+  fx_stage<NS, CF>(a, lay, n, load);
+  if (ANY && n > max_n) {
+    __syncthreads();
+    return fx_run64<SIGN>(a, b, lay, NS, p);
+  }
+  __syncthreads();
+  if (nb > 1) fx_clear(fx_shared().l1, lay.s0, NS * nb);
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {  // each thread converts the entries it staged
+    unsigned l1 = 0u;
+    int cp = -1;
+    FxExp ex{};
+    for (int i = threadIdx.x; i < n * nb; i += blockDim.x) {
+      int e, c;
+      fx_item<CF>(i, n, nb, e, c);
+      if (c != cp) {
+        if (cp >= 0) fx_put_l1(lay.s0, s, nb, cp, l1);
+        l1 = 0u;
+        cp = c;
+        ex = fx_exponent(fx_get_max(lay.s0 + s * nb + c));
+      }
+      const int q = a + s * lay.stride + e * nb + c;
+      const fx2 v = fx_load<kFxB>(fx_get64(q), ex);
+      fx_put(q, v);
+      l1 += fx_l1(v);
+    }
+    fx_put_l1(lay.s0, s, nb, cp, l1);
+  }
+  __syncthreads();
+  fx_make_meta<kFxB>(lay, p.fxs);
+  return fx_run<SIGN, NS>(a, b, lay, p);
+}
+
+// xf_c2r (below) with the c_k of every sequence already in b as FP64 pairs and their largest high words given
+// (fx_put_max); the call starts with a barrier.
+template <int NS, bool ANY = true>
+__device__ __forceinline__ FxRes xf_c2r_staged(int a, int b, FxLay lay, const FFTPlan& p, int K) {
+  const int nb = lay.nb, n = p.n;
+  if (ANY && n > kFxMaxReal) {
+    __syncthreads();
+    for (int s = 0; s < NS; ++s)
+      for (int i = threadIdx.x; i < n * nb; i += blockDim.x) {
+        int e, c;
+        fx_item<true>(i, n, nb, e, c);
+        const double2* S = fx_mem64() + b + s * lay.stride + c;
+        fx_mem64()[a + s * lay.stride + i] =
+            c2r_entry<true>([&](int k) { return S[k * nb]; }, e, K, n, p.wm, 1.0, 1.0);
+      }
+    __syncthreads();
+    return fx_run64<1>(a, b, lay, NS, p);
+  }
+  __syncthreads();
+  const int half = n / 2 + 1;
+  if (nb > 1) fx_clear(fx_shared().l1, lay.s0, NS * nb);
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+    unsigned l1 = 0u;
+    int cp = -1;
+    FxExp ex{};
+    for (int i = threadIdx.x; i < half * nb; i += blockDim.x) {
+      int k, c;
+      fx_item<true>(i, half, nb, k, c);
+      if (c != cp) {
+        if (cp >= 0) fx_put_l1(lay.s0, s, nb, cp, l1);
+        l1 = 0u;
+        cp = c;
+        ex = fx_exponent(fx_get_max(lay.s0 + s * nb + c));
+      }
+      const int S = b + s * lay.stride + c;
+      const int kc = n - k;
+      // c_k and c_{n-k} (0 where not stored), c_0 real
+      const bool hx = k < K, hy = k > 0 && kc < K;
+      double2 sx = fx_get64(S + (hx ? k : 0) * nb), sy = fx_get64(S + (hy ? kc : 0) * nb);
+      if (!hx) sx.x = 0.0;
+      if (!hx || k == 0) sx.y = 0.0;
+      if (!hy) sy = make_double2(0.0, 0.0);
+      const fx2 x = fx_load<kFxBReal>(sx, ex), y = fx_load<kFxBReal>(sy, ex);
+      fx2 z0, z1;
+      fx_pack(x, y, ldtab(p.fxr + k), z0, z1);
+      const int A = a + s * lay.stride + c;
+      fx_put(A + k * nb, z0);
+      l1 += fx_l1(z0);
+      if (k > 0 && kc != k) {
+        fx_put(A + kc * nb, z1);
+        l1 += fx_l1(z1);
+      }
+    }
+    fx_put_l1(lay.s0, s, nb, cp, l1);
+  }
+  __syncthreads();
+  fx_make_meta<kFxBReal>(lay, p.fxs + 32);
+  return fx_run<1, NS>(a, b, lay, p);
+}
+
+// Inverse real transform: the grid values g_j = Re c_0 + 2 Re sum_{1 <= k < K} c_k exp(2 pi i j k / 2n),
+// j < 2n, from c_k = load(set, c, k) (the imaginary part of c_0 is not used).
+template <int NS, bool CF, bool ANY = true, class Load>
+__device__ __forceinline__ FxRes xf_c2r(int a, int b, FxLay lay, const FFTPlan& p, int K, Load load) {
+  fx_stage<NS, CF>(b, lay, K, load);
+  return xf_c2r_staged<NS, ANY>(a, b, lay, p, K);
+}
+
+// Forward real transform of the grid pairs (g_2j, g_2j+1) = load(set, c, j), j < n; results by FxRes::coef.
+template <int NS, bool CF, bool ANY = true, class Load>
+__device__ __forceinline__ FxRes xf_r2c(int a, int b, FxLay lay, const FFTPlan& p, Load load) {
+  return xf_c2c<-1, NS, CF, ANY>(a, b, lay, p, load, kFxMaxReal);
+}
+
+}  // namespace spadj

@@ -28,7 +28,7 @@
 #include <vector>
 
 #include "closure.cuh"
-#include "fft.cuh"
+#include "fxfft.cuh"
 #include "problem.h"
 
 namespace spadj {
@@ -49,8 +49,8 @@ struct KMember {
 
 struct KRes {
   FFTPlan px, py;
-  const double2* WMx;  // exp(-2 pi i m / M), m < M  (x real FFT through L = M/2)
-  const double2* W2M;  // exp(-2 pi i m / 2M), m < 2M (y complex FFT of length M)
+  // per (kx, ky row): 1 / |k|^2 (0 at k = 0) and 1 / (a_0 + |k|^2 / Re) for SBDF1 and SBDF2, [3][Kx][N]
+  const double* diag;
 };
 
 struct KolArgs {
@@ -58,7 +58,6 @@ struct KolArgs {
   const KMember* mem;
   KRes res[kMaxRes];
   double Re, dt;
-  double invRe;      // 1 / Re
   double kc[2][5];   // SBDF1 (row 0) and SBDF2 (row 1): a0, a1, a2 (divided by dt), c1, c2
   int CW, RW;
   int nCAtot, nBtot;
@@ -117,10 +116,8 @@ __device__ __forceinline__ Coef kcoef(int n, const double (&kc)[2][5]) {
 __device__ __forceinline__ int kyof(int q, int N) { return q < N / 2 ? q : q - N; }
 __device__ __forceinline__ int yidx(int q, int N, int M) { return q < N / 2 ? q : (q == N / 2 ? -1 : M - N + q); }
 
-// multiplier of field f (0 u, 1 v, 2 w_x, 3 w_y) applied to w(kx, ky)
-__device__ __forceinline__ double2 fmult(int f, double kx, double ky, double2 w) {
-  const double k2 = kx * kx + ky * ky;
-  const double ik2 = k2 > 0.0 ? 1.0 / k2 : 0.0;
+// multiplier of field f (0 u, 1 v, 2 w_x, 3 w_y) applied to w(kx, ky); ik2 = 1 / |k|^2 from the table
+__device__ __forceinline__ double2 fmult(int f, double kx, double ky, double ik2, double2 w) {
   double s;
   switch (f) {
     case 0: s = ky * ik2; break;    // i ky / |k|^2
@@ -148,16 +145,31 @@ __device__ void project_col(double2* x, int N, int kx) {
   __syncthreads();
 }
 
-// y-FFT of a padded column: fill a (length M) from fill(j), transform with SIGN, return result
-template <int SIGN>
-__device__ double2* col_fft(double2* a, double2* b, const KRes& R) {
-  __syncthreads();
-  return cfft_smem_t<SIGN>(a, b, R.py, R.W2M);
+// coefficient row of entry j of the length-M y-FFT (-1 for the padding)
+__device__ __forceinline__ int yrow(int j, int N, int M) { return j < N / 2 ? j : (j > M - N / 2 ? j - (M - N) : -1); }
+
+// The y-FFT input of field f (0..3; 4 = omega itself) of the column xs (rows q, wavenumber kx) at entry j
+__device__ __forceinline__ double2 field_entry(int f, const double2* xs, const double* ik2, int kx, int j, int N, int M) {
+  const int q = yrow(j, N, M);
+  if (q < 0) return make_double2(0.0, 0.0);
+  const double2 x = ldcg2(&xs[q]);
+  return f < 4 ? fmult(f, (double)kx, (double)kyof(q, N), __ldg(&ik2[q]), x) : x;
 }
 
-struct KSmem {
-  double2* buf;  // base of dynamic smem
-};
+// Inverse y transforms of the fields f0 .. f0 + NP - 1 of a column (transform pairs at fs + 2 p M, scratch + M;
+// the column is read from global memory), into dst(f)[row j].
+template <int NP, class Dst>
+__device__ __forceinline__ void fields_y(int fs, const KRes& R, int f0, const double2* xs, const double* ik2, int kx, int N,
+                                         int M, Dst dst) {
+  const FxRes r = xf_c2c<1, NP, true, false>(fs, fs + M, FxLay{NP, 1, 2 * M, 0}, R.py, [&](int p, int, int j) {
+    return field_entry(f0 + p, xs, ik2, kx, j, N, M);
+  });
+  for (int i = threadIdx.x; i < NP * M; i += blockDim.x) {
+    const int p = i >= M ? 1 : 0, j = i - p * M;
+    dst(f0 + p, j, r.at(p, 0, j));
+  }
+  __syncthreads();
+}
 
 // ---- forward CA tile --------------------------------------------------------------------------
 __device__ void ca_forward(const KolArgs& A, const KMember& m, int tile, int s) {
@@ -166,9 +178,8 @@ __device__ void ca_forward(const KolArgs& A, const KMember& m, int tile, int s) 
   const int n = A.n0 + s;           // absolute step of this stage
   const int last = A.nstage - 1;    // the launch's last stage
   const KRes& R = A.res[m.res];
-  double2* ca = ks;          // M
-  double2* cb = ca + M;      // M
-  double2* xc = cb + M;      // N
+  const int fs = 0;          // transform pairs from the start of ks
+  double2* xc = ks + 2 * M;              // N
   const int kx0 = tile * A.CW, kx1 = min(Kx, kx0 + A.CW);
   const long long S = A.state_size;
   for (int kx = kx0; kx < kx1; ++kx) {
@@ -177,18 +188,20 @@ __device__ void ca_forward(const KolArgs& A, const KMember& m, int tile, int s) 
       for (int q = threadIdx.x; q < N; q += blockDim.x) xc[q] = A.x0[col + q];
       __syncthreads();
     } else {
-      double2* r = nullptr;
-      if (A.nonlinear || A.closure) {
-        for (int j = threadIdx.x; j < M; j += blockDim.x) ca[j] = ldcg2(&A.mixB[0][m.off_mix + (long long)j * Kx + kx]);
-        r = col_fft<-1>(ca, cb, R);
-      }
+      FxRes r{};
+      if (A.nonlinear || A.closure)
+        r = xf_c2c<-1, 1, true, false>(fs, fs + M, FxLay{1, 1, M, 0}, R.py, [&](int, int, int j) {
+          return ldcg2(&A.mixB[0][m.off_mix + (long long)j * Kx + kx]);
+        });
       const Coef c = kcoef(n, A.kc);
       const double invM = 1.0 / M;
       for (int q = threadIdx.x; q < N; q += blockDim.x) {
         const int idx = yidx(q, N, M);
-        const double ky = kyof(q, N);
         double2 F = make_double2(0.0, 0.0);
-        if (idx >= 0 && (A.nonlinear || A.closure)) F = make_double2(-r[idx].x * invM, -r[idx].y * invM);
+        if (idx >= 0 && (A.nonlinear || A.closure)) {
+          const double2 v = r.at(0, 0, idx);
+          F = make_double2(-v.x * invM, -v.y * invM);
+        }
         if (A.forcing && kx == 0 && (q == 4 || q == N - 4)) F.x -= 2.0;
         if (A.fonly) {
           A.out[col + q] = F;
@@ -203,7 +216,7 @@ __device__ void ca_forward(const KolArgs& A, const KMember& m, int tile, int s) 
           num.y += c.c2 * F2.y - c.a2 * X2.y;
         }
         A.Fr[(n - 1) & 1][col + q] = F;
-        const double inv = 1.0 / (c.a0 + ((double)kx * kx + ky * ky) * A.invRe);
+        const double inv = __ldg(&R.diag[((size_t)(n <= 1 ? 1 : 2) * Kx + kx) * N + q]);
         xc[q] = make_double2(num.x * inv, num.y * inv);
       }
       __syncthreads();
@@ -216,136 +229,74 @@ __device__ void ca_forward(const KolArgs& A, const KMember& m, int tile, int s) 
       if (s == last) A.out[col + q] = xc[q];
     }
     if (s < last && (A.nonlinear || A.closure)) {
-      // the fields' inverse y transforms two at a time, sharing their passes: set p at
-      // ks + 2 p M (scratch + M); the column is read back from the state just written, its
-      // shared slot being reused
-      const int nf = A.closure ? 5 : 4;
+      // the fields' inverse y transforms two at a time, sharing their passes; the column is read back from the
+      // state just written, its shared slot being reused
       const double2* xs = A.Xr[n & 1] + col;
-      for (int f0 = 0; f0 < nf; f0 += 2) {
-        const int np = min(2, nf - f0);
-        __syncthreads();
-        for (int i = threadIdx.x; i < np * M; i += blockDim.x) {
-          const int pq = i / M;
-          ks[pq * 2 * M + (i - pq * M)] = make_double2(0.0, 0.0);
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < np * N; i += blockDim.x) {
-          const int pq = i / N, q = i - pq * N, f = f0 + pq;
-          const int idx = yidx(q, N, M);
-          if (idx < 0) continue;
-          const double2 x = ldcg2(&xs[q]);
-          ks[pq * 2 * M + idx] = f < 4 ? fmult(f, (double)kx, (double)kyof(q, N), x) : x;
-        }
-        __syncthreads();
-        cfft_smem_sets<1>(ks, ks + M, 2 * M, np, R.py, 1);
-        const double2* r = (R.py.nrad & 1) ? ks + M : ks;
-        for (int i = threadIdx.x; i < np * M; i += blockDim.x) {
-          const int pq = i / M, j = i - pq * M;
-          A.mixA[f0 + pq][m.off_mix + (long long)j * Kx + kx] = r[pq * 2 * M + j];
-        }
-      }
+      const double* ik2 = R.diag + (size_t)kx * N;
+      auto dst = [&](int f, int j, double2 v) { A.mixA[f][m.off_mix + (long long)j * Kx + kx] = v; };
+      __syncthreads();
+#pragma unroll 1
+      for (int f0 = 0; f0 < 4; f0 += 2) fields_y<2>(fs, R, f0, xs, ik2, kx, N, M, dst);
+      if (A.closure) fields_y<1>(fs, R, 4, xs, ik2, kx, N, M, dst);
     }
     __syncthreads();
   }
 }
 
-// inverse x transform of one mixed row into a packed real row (L complex) kept in dst
-__device__ void row_c2r(const double2* src, double2* dst, double2* sa, double2* sb, double2* st, const KMember& m,
-                        const KRes& R, double w0, double w) {
-  const int Kx = m.Kx, L = m.L;
-  for (int k = threadIdx.x; k < Kx; k += blockDim.x) st[k] = ldcg2(&src[k]);
-  __syncthreads();
-  c2r_pre(sa, [&](int k) { return st[k]; }, Kx, L, R.WMx, w0, w);
-  __syncthreads();
-  double2* r = cfft_smem_t<1>(sa, sb, R.px, R.WMx);
-  if (r != dst) {
-    for (int j = threadIdx.x; j < L; j += blockDim.x) dst[j] = r[j];
-  }
-  __syncthreads();
+// Inverse x transform of one mixed row (weights w0 on k = 0, w elsewhere) in the buffers a, b on scale slot s0.
+__device__ __forceinline__ FxRes row_c2r(const double2* src, int a, int b, const KMember& m, const KRes& R, double w0,
+                                         double w, int s0) {
+  return xf_c2r<1, true, false>(a, b, FxLay{1, 1, m.L, s0}, R.px, m.Kx, [&](int, int, int k) {
+    const double2 v = ldcg2(&src[k]);
+    const double f = k == 0 ? w0 : w;
+    return make_double2(v.x * f, v.y * f);
+  });
 }
 
-// forward x transform of a packed real row held in `row` (destroyed) into dst[k], k < Kx
-__device__ void row_r2c(double2* row, double2* scratch, double2* dst, const KMember& m, const KRes& R, double s0,
-                        double s) {
-  const int Kx = m.Kx, L = m.L;
-  double2* z = cfft_smem_t<-1>(row, scratch, R.px, R.WMx);
-  r2c_post2(z, [&](int k, double2 v) {  // v = 2 X_k
-    const double f = 0.5 * (k == 0 ? s0 : s);
-    double2 o = make_double2(v.x * f, v.y * f);
-    if (k == 0) o.y = 0.0;
-    dst[k] = o;
-  }, Kx, L, R.WMx);
-  __syncthreads();
-}
-
-// Inverse x transforms of nf mixed rows at once (weights 1): spectrum f (Kx entries from src(f))
-// is staged in base + (2f+1) L, its packed spectrum built in base + 2f L, and the nf FFTs share
-// their passes (more butterflies per pass than threads in one row's, one barrier per pass for
-// all).  Returns the slot of field 0's packed grid row; field f's is 2 f L further.
+// Inverse x transforms of the mixed rows src(0..3) at once (weights 1), field f in the pair base + 2 f L: the FFTs
+// share their passes (more butterflies per pass than threads in one row's, one barrier per pass for all).
 template <class Src>
-__device__ double2* rows_c2r_sets(double2* base, int nf, Src src, const KMember& m, const KRes& R) {
-  const int Kx = m.Kx, L = m.L;
-  for (int idx = threadIdx.x; idx < nf * Kx; idx += blockDim.x) {
-    const int f = idx / Kx, k = idx - f * Kx;
-    base[(2 * f + 1) * L + k] = ldcg2(&src(f)[k]);
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < nf * L; idx += blockDim.x) {
-    const int f = idx / L, k = idx - f * L;
-    const double2* S = base + (2 * f + 1) * L;
-    base[2 * f * L + k] = c2r_entry<true>([&](int i) { return S[i]; }, k, Kx, L, R.WMx, 1.0, 1.0);
-  }
-  __syncthreads();
-  cfft_smem_sets<1>(base, base + L, 2 * L, nf, R.px, 1);
-  return (R.px.nrad & 1) ? base + L : base;
+__device__ __forceinline__ FxRes rows_c2r4(int base, Src src, const KMember& m, const KRes& R) {
+  return xf_c2r<4, true, false>(base, base + m.L, FxLay{4, 1, 2 * m.L, 0}, R.px, m.Kx,
+                                [&](int f, int, int k) { return ldcg2(&src(f)[k]); });
 }
 
-// Forward x transforms of nf packed grid rows at once: row f at a + 2 f L (destroyed), scratch at
-// b + 2 f L; put(f, k, 2 X_k) for k < Kx (the unpacking's 1/2 is left to put).
-template <class Put>
-__device__ void rows_r2c_sets(double2* a, double2* b, int nf, Put put, const KMember& m, const KRes& R) {
-  const int Kx = m.Kx, L = m.L;
-  cfft_smem_sets<-1>(a, b, 2 * L, nf, R.px, 1);
-  const double2* z = (R.px.nrad & 1) ? b : a;
-  for (int idx = threadIdx.x; idx < nf * Kx; idx += blockDim.x) {
-    const int f = idx / Kx, k = idx - f * Kx;
-    const double2* Z = z + 2 * f * L;
-    put(f, k, r2c_combine2(Z[k], cconj(Z[k == 0 ? 0 : L - k]), __ldg(&R.WMx[k])));
+// Spectrum of a forward row transform into dst[k], k < Kx, times s (s0 on k = 0, real)
+__device__ __forceinline__ void put_row(const FxRes& z, int set, double2* dst, int Kx, double s0, double s) {
+  for (int k = threadIdx.x; k < Kx; k += blockDim.x) {
+    const double2 v = z.coef(set, 0, k);
+    dst[k] = k == 0 ? make_double2(v.x * s0, 0.0) : make_double2(v.x * s, v.y * s);
   }
-  __syncthreads();
 }
 
 // ---- forward B tile ---------------------------------------------------------------------------
 __device__ void b_forward(const KolArgs& A, const KMember& m, int tile) {
-  extern __shared__ double2 ks[];
   const int Kx = m.Kx, M = m.M, L = m.L;
   const KRes& R = A.res[m.res];
-  // ks[0, 8L): four transform sets (field f: slots 2f, 2f+1 of L entries); ks[8L, 8L+Kx): staging
-  double2* st = ks + 8 * L;
+  const int fs = 0;  // four transform pairs (field f: slots 2f, 2f+1 of L entries)
   const int j0 = tile * A.RW, j1 = min(M, j0 + A.RW);
   const double invM = 1.0 / M;
   for (int j = j0; j < j1; ++j) {
     if (A.closure) {
-      row_c2r(A.mixA[4] + m.off_mix + (long long)j * Kx, ks, ks, ks + L, st, m, R, 1.0, 1.0);
+      const FxRes w = row_c2r(A.mixA[4] + m.off_mix + (long long)j * Kx, fs, fs + L, m, R, 1.0, 1.0, 0);
       double2* gw = reinterpret_cast<double2*>(A.gridW + m.off_grid + (long long)j * M);
-      for (int i = threadIdx.x; i < L; i += blockDim.x) gw[i] = ks[i];
+      for (int i = threadIdx.x; i < L; i += blockDim.x) gw[i] = w.at(0, 0, i);
       __syncthreads();
     }
-    double2 *prod = ks, *scratch = ks + L;
+    double2* dst = A.mixB[0] + m.off_mix + (long long)j * Kx;
     if (A.nonlinear) {
-      // u, v, w_x, w_y on the grid row, then u w_x + v w_y into the free slot of field 0
-      const double2* r = rows_c2r_sets(ks, 4, [&](int f) { return A.mixA[f] + m.off_mix + (long long)j * Kx; }, m, R);
-      prod = (r == ks) ? ks + L : ks;
-      scratch = prod + 2 * L;
-      for (int i = threadIdx.x; i < L; i += blockDim.x) {
-        const double2 u = r[i], v = r[2 * L + i], wx = r[4 * L + i], wy = r[6 * L + i];
-        prod[i] = make_double2(fma(u.x, wx.x, v.x * wy.x), fma(u.y, wx.y, v.y * wy.y));
-      }
+      // u, v, w_x, w_y on the grid row, then u w_x + v w_y through the free slots of fields 0 and 1
+      const FxRes r = rows_c2r4(fs, [&](int f) { return A.mixA[f] + m.off_mix + (long long)j * Kx; }, m, R);
+      const int fr = (R.px.nrad & 1) ? fs : fs + L;
+      const FxRes z = xf_r2c<1, true, false>(fr, fr + 2 * L, FxLay{1, 1, L, 0}, R.px, [&](int, int, int i) {
+        const double2 u = r.at(0, 0, i), v = r.at(1, 0, i), wx = r.at(2, 0, i), wy = r.at(3, 0, i);
+        return make_double2(fma(u.x, wx.x, v.x * wy.x), fma(u.y, wx.y, v.y * wy.y));
+      });
+      put_row(z, 0, dst, Kx, invM, invM);
     } else {
-      for (int i = threadIdx.x; i < L; i += blockDim.x) prod[i] = make_double2(0.0, 0.0);
+      for (int k = threadIdx.x; k < Kx; k += blockDim.x) dst[k] = make_double2(0.0, 0.0);
     }
     __syncthreads();
-    row_r2c(prod, scratch, A.mixB[0] + m.off_mix + (long long)j * Kx, m, R, invM, invM);
   }
 }
 
@@ -356,13 +307,12 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
   extern __shared__ double2 ks[];
   const int N = m.N, Kx = m.Kx, M = m.M;
   const KRes& R = A.res[m.res];
-  // The VJP's forward y transforms run two at a time (sets at ks + 2 p M, scratch + M) when the
+  // The VJP's forward y transforms run two at a time (pairs at ks + 2 p M, scratch + M) when the
   // accumulator lam fits beside them; otherwise one at a time in ks[0, 2M).
   const bool pairs = 4 * M + N <= A.smem_entries;
-  double2* ca = ks;                             // M
-  double2* cb = ca + M;                         // M
-  double2* lam = pairs ? ks + 4 * M : cb + M;   // N
-  double2* yc = pairs ? ks + 2 * M : lam + N;   // N (used after the VJP)
+  const int fs = 0;
+  double2* lam = pairs ? ks + 4 * M : ks + 2 * M;  // N
+  double2* yc = pairs ? ks + 2 * M : lam + N;      // N (used after the VJP)
   const int kx0 = tile * A.CW, kx1 = min(Kx, kx0 + A.CW);
   const long long S = A.state_size;
   const int SN = A.S;
@@ -377,37 +327,47 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
     if (n < SN && (A.nonlinear || A.closure)) {
       // VJP: B_y^dagger of the grid cotangents, then the adjoint multipliers (identity for the
       // closure's input field)
-      const int fa = A.nonlinear ? 0 : 4, fb = A.closure ? 5 : 4, per = pairs ? 2 : 1;
-      for (int f0 = fa; f0 < fb; f0 += per) {
-        const int np = min(per, fb - f0);
-        for (int i = threadIdx.x; i < np * M; i += blockDim.x) {
-          const int pq = i / M, j = i - pq * M;
-          ks[pq * 2 * M + j] = ldcg2(&A.mixB[f0 + pq][m.off_mix + (long long)j * Kx + kx]);
-        }
-        __syncthreads();
-        cfft_smem_sets<-1>(ks, ks + M, 2 * M, np, R.py, 1);
-        const double2* r = (R.py.nrad & 1) ? ks + M : ks;
+      const double* ik2 = R.diag + (size_t)kx * N;
+      auto add = [&](int f0, int np, const FxRes& r) {
         for (int q = threadIdx.x; q < N; q += blockDim.x) {
           const int idx = yidx(q, N, M);
           if (idx < 0) continue;
           double2 l = lam[q];
           for (int pq = 0; pq < np; ++pq) {
             const int f = f0 + pq;
-            const double2 v = r[pq * 2 * M + idx];
+            const double2 v = r.at(pq, 0, idx);
             if (f == 4) {
               l.x += v.x;
               l.y += v.y;
               continue;
             }
             // adjoint of i*s is -i*s: fmult with the negated multiplier
-            const double2 fv = fmult(f, (double)kx, (double)kyof(q, N), v);
+            const double2 fv = fmult(f, (double)kx, (double)kyof(q, N), __ldg(&ik2[q]), v);
             l.x -= fv.x;
             l.y -= fv.y;
           }
           lam[q] = l;
         }
         __syncthreads();
+      };
+      auto one = [&](int f) {
+        add(f, 1, xf_c2c<-1, 1, true, false>(fs, fs + M, FxLay{1, 1, M, 0}, R.py, [&](int, int, int j) {
+              return ldcg2(&A.mixB[f][m.off_mix + (long long)j * Kx + kx]);
+            }));
+      };
+      bool per_one = false;
+      if (A.nonlinear && pairs) {
+#pragma unroll 1
+        for (int f0 = 0; f0 < 4; f0 += 2)
+          add(f0, 2, xf_c2c<-1, 2, true, false>(fs, fs + M, FxLay{2, 1, 2 * M, 0}, R.py, [&](int pq, int, int j) {
+                return ldcg2(&A.mixB[f0 + pq][m.off_mix + (long long)j * Kx + kx]);
+              }));
+      } else if (A.nonlinear) {
+        per_one = true;
       }
+      if (per_one || A.closure)
+#pragma unroll 1
+        for (int f = per_one ? 0 : 4; f < (A.closure ? 5 : 4); ++f) one(f);
     }
     const int si = A.seed_at ? A.seed_at[n] : -1;
     const Coef c1 = (n + 1 <= SN) ? kcoef(n + 1, A.kc) : Coef{0, 0, 0, 0, 0};
@@ -435,10 +395,8 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
       continue;
     }
     project_col(lam, N, kx);
-    const Coef cn = kcoef(n, A.kc);
     for (int q = threadIdx.x; q < N; q += blockDim.x) {
-      const double ky = kyof(q, N);
-      const double inv = 1.0 / (cn.a0 + ((double)kx * kx + ky * ky) * A.invRe);
+      const double inv = __ldg(&R.diag[((size_t)(n <= 1 ? 1 : 2) * Kx + kx) * N + q]);
       yc[q] = make_double2(lam[q].x * inv, lam[q].y * inv);
     }
     __syncthreads();
@@ -463,98 +421,74 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
     __syncthreads();
     if (!A.nonlinear && !A.closure) continue;
     // T_y^dagger W (inverse FFT with 1/M) -> mixA[4]
-    for (int j = threadIdx.x; j < M; j += blockDim.x) ca[j] = make_double2(0.0, 0.0);
-    __syncthreads();
-    for (int q = threadIdx.x; q < N; q += blockDim.x) {
-      const int idx = yidx(q, N, M);
-      if (idx >= 0) ca[idx] = lam[q];
-    }
     {
-      double2* r = col_fft<1>(ca, cb, R);
+      const FxRes r = xf_c2c<1, 1, true, false>(fs, fs + M, FxLay{1, 1, M, 0}, R.py, [&](int, int, int j) {
+        const int q = yrow(j, N, M);
+        return q < 0 ? make_double2(0.0, 0.0) : lam[q];
+      });
       const double invM = 1.0 / M;
-      for (int j = threadIdx.x; j < M; j += blockDim.x)
-        A.mixA[4][m.off_mix + (long long)j * Kx + kx] = make_double2(r[j].x * invM, r[j].y * invM);
+      for (int j = threadIdx.x; j < M; j += blockDim.x) {
+        const double2 v = r.at(0, 0, j);
+        A.mixA[4][m.off_mix + (long long)j * Kx + kx] = make_double2(v.x * invM, v.y * invM);
+      }
+      __syncthreads();
     }
-    // fields of X_{n-1} from the trajectory, their inverse y transforms two at a time (sets at
-    // ks + 2 p M, scratch + M; 4M <= the CTA's shared memory for every member)
+    // fields of X_{n-1} from the trajectory, their inverse y transforms two at a time (4M <= the CTA's
+    // shared memory for every member); the closure's input field goes to slot 5 (slot 4 holds T^dagger W)
     const double2* xs = A.traj + (long long)(n - 1 - A.lo) * S + col;
-    const int fa = A.nonlinear ? 0 : 4, fb = A.closure ? 5 : 4;
-    for (int f0 = fa; f0 < fb; f0 += 2) {
-      const int np = min(2, fb - f0);
-      __syncthreads();
-      for (int i = threadIdx.x; i < np * M; i += blockDim.x) {
-        const int pq = i / M;
-        ks[pq * 2 * M + (i - pq * M)] = make_double2(0.0, 0.0);
-      }
-      __syncthreads();
-      for (int i = threadIdx.x; i < np * N; i += blockDim.x) {
-        const int pq = i / N, q = i - pq * N, f = f0 + pq;
-        const int idx = yidx(q, N, M);
-        if (idx < 0) continue;
-        const double2 x = ldcg2(&xs[q]);
-        ks[pq * 2 * M + idx] = f < 4 ? fmult(f, (double)kx, (double)kyof(q, N), x) : x;
-      }
-      __syncthreads();
-      cfft_smem_sets<1>(ks, ks + M, 2 * M, np, R.py, 1);
-      const double2* r = (R.py.nrad & 1) ? ks + M : ks;
-      for (int i = threadIdx.x; i < np * M; i += blockDim.x) {
-        const int pq = i / M, j = i - pq * M, f = f0 + pq;
-        // the closure's input field goes to slot 5 (slot 4 holds T^dagger W)
-        A.mixA[f < 4 ? f : 5][m.off_mix + (long long)j * Kx + kx] = r[pq * 2 * M + j];
-      }
+    const double* ik2 = R.diag + (size_t)kx * N;
+    auto dst = [&](int f, int j, double2 v) { A.mixA[f < 4 ? f : 5][m.off_mix + (long long)j * Kx + kx] = v; };
+    if (A.nonlinear) {
+#pragma unroll 1
+      for (int f0 = 0; f0 < 4; f0 += 2) fields_y<2>(fs, R, f0, xs, ik2, kx, N, M, dst);
     }
-    __syncthreads();
+    if (A.closure) fields_y<1>(fs, R, 4, xs, ik2, kx, N, M, dst);
   }
 }
 
 // ---- adjoint B' tile --------------------------------------------------------------------------
 __device__ void b_adjoint(const KolArgs& A, const KMember& m, int tile) {
-  extern __shared__ double2 ks[];
   const int Kx = m.Kx, M = m.M, L = m.L;
   const KRes& R = A.res[m.res];
-  // ks[0, 8L): four transform sets (field f: slots 2f, 2f+1 of L entries); ks[8L, 8L+Kx): staging
-  double2* st = ks + 8 * L;
+  const int fs = 0;  // four transform pairs (field f: slots 2f, 2f+1 of L entries)
   const int j0 = tile * A.RW, j1 = min(M, j0 + A.RW);
   for (int j = j0; j < j1; ++j) {
+    double2* gw = reinterpret_cast<double2*>(A.gridW + m.off_grid + (long long)j * M);
+    double2* gg = reinterpret_cast<double2*>(A.gridG + m.off_grid + (long long)j * M);
+    auto mixed = [&](int f) { return A.mixA[f] + m.off_mix + (long long)j * Kx; };
     if (!A.nonlinear) {  // closure only: omega and the grid cotangent g, for the CNN's backward pass
       if (A.closure) {
-        row_c2r(A.mixA[4] + m.off_mix + (long long)j * Kx, ks, ks, ks + L, st, m, R, 1.0 / M, 0.5 / M);
-        row_c2r(A.mixA[5] + m.off_mix + (long long)j * Kx, ks + 2 * L, ks + 2 * L, ks + 3 * L, st, m, R, 1.0, 1.0);
-        double2* gw = reinterpret_cast<double2*>(A.gridW + m.off_grid + (long long)j * M);
-        double2* gg = reinterpret_cast<double2*>(A.gridG + m.off_grid + (long long)j * M);
-        for (int i = threadIdx.x; i < L; i += blockDim.x) { gw[i] = ks[2 * L + i]; gg[i] = ks[i]; }
+        const FxRes g = row_c2r(mixed(4), fs, fs + L, m, R, 1.0 / M, 0.5 / M, 0);
+        const FxRes w = row_c2r(mixed(5), fs + 2 * L, fs + 3 * L, m, R, 1.0, 1.0, 1);
+        for (int i = threadIdx.x; i < L; i += blockDim.x) {
+          gw[i] = w.at(0, 0, i);
+          gg[i] = g.at(0, 0, i);
+        }
         __syncthreads();
       }
       continue;
     }
-    // u, v, w_x, w_y in one set of transforms; the free slots F_f = fr + 2 f L take g (F_0, with
-    // F_1 as its scratch), the closure's omega (F_2, scratch F_3), then serve as the forward
-    // transforms' scratch
-    double2* r = rows_c2r_sets(ks, 4, [&](int f) { return A.mixA[f] + m.off_mix + (long long)j * Kx; }, m, R);
-    double2* fr = (r == ks) ? ks + L : ks;
-    row_c2r(A.mixA[4] + m.off_mix + (long long)j * Kx, fr, fr, fr + 2 * L, st, m, R, 1.0 / M, 0.5 / M);
+    // u, v, w_x, w_y in one set of transforms; the free slots F_f = fr + 2 f L take g (F_0 and F_1) and the
+    // closure's omega (F_2 and F_3), then the products
+    const FxRes r = rows_c2r4(fs, mixed, m, R);
+    const int fr = (R.px.nrad & 1) ? fs : fs + L;
+    const FxRes g = row_c2r(mixed(4), fr, fr + 2 * L, m, R, 1.0 / M, 0.5 / M, 4);
     if (A.closure) {
-      row_c2r(A.mixA[5] + m.off_mix + (long long)j * Kx, fr + 4 * L, fr + 4 * L, fr + 6 * L, st, m, R, 1.0, 1.0);
-      double2* gw = reinterpret_cast<double2*>(A.gridW + m.off_grid + (long long)j * M);
-      double2* gg = reinterpret_cast<double2*>(A.gridG + m.off_grid + (long long)j * M);
-      for (int i = threadIdx.x; i < L; i += blockDim.x) { gw[i] = fr[4 * L + i]; gg[i] = fr[i]; }
+      const FxRes w = row_c2r(mixed(5), fr + 4 * L, fr + 6 * L, m, R, 1.0, 1.0, 5);
+      for (int i = threadIdx.x; i < L; i += blockDim.x) {
+        gw[i] = w.at(0, 0, i);
+        gg[i] = g.at(0, 0, i);
+      }
       __syncthreads();
     }
-    // grid cotangents of u, v, w_x, w_y: -g w_x, -g w_y, -g u, -g v
-    for (int i = threadIdx.x; i < L; i += blockDim.x) {
-      const double2 u = r[i], v = r[2 * L + i], wx = r[4 * L + i], wy = r[6 * L + i], g = fr[i];
-      r[i] = make_double2(-g.x * wx.x, -g.y * wx.y);
-      r[2 * L + i] = make_double2(-g.x * wy.x, -g.y * wy.y);
-      r[4 * L + i] = make_double2(-g.x * u.x, -g.y * u.y);
-      r[6 * L + i] = make_double2(-g.x * v.x, -g.y * v.y);
-    }
+    // grid cotangents of u, v, w_x, w_y: -g w_x, -g w_y, -g u, -g v (entry i of g's slot is overwritten by the
+    // thread that has read it)
+    const FxRes z = xf_r2c<4, true, false>(fr, r.z, FxLay{4, 1, 2 * L, 0}, R.px, [&](int f, int, int i) {
+      const double2 a = g.at(0, 0, i), b = r.at(f ^ 2, 0, i);
+      return make_double2(-a.x * b.x, -a.y * b.y);
+    });
+    for (int f = 0; f < 4; ++f) put_row(z, f, A.mixB[f] + m.off_mix + (long long)j * Kx, Kx, 1.0, 2.0);
     __syncthreads();
-    rows_r2c_sets(r, fr, 4, [&](int f, int k, double2 v) {  // v = 2 X_k; scales 1 (k = 0), 2
-      const double sc = k == 0 ? 0.5 : 1.0;
-      double2 o = make_double2(v.x * sc, v.y * sc);
-      if (k == 0) o.y = 0.0;
-      A.mixB[f][m.off_mix + (long long)j * Kx + k] = o;
-    }, m, R);
   }
 }
 
@@ -644,28 +578,24 @@ __global__ void __launch_bounds__(kKolThreads) kol_phase(const __grid_constant__
 // closure term enters F = -P + C with P stored), mode 1 mixB[4] = B_x^dagger(grid row).
 __global__ void __launch_bounds__(kKolThreads) closure_rows_kernel(const __grid_constant__ KolArgs A, const double* grid,
                                                                   int mode) {
-  extern __shared__ double2 ks[];
   const int b = blockIdx.y;
   const KMember& m = A.mem[b];
   const int j = blockIdx.x;
   if (j >= m.M) return;
   const KRes& R = A.res[m.res];
   const int L = m.L, Kx = m.Kx;
-  double2* sa = ks;
-  double2* sb = sa + L;
-  double2* st = sb + L;
+  const int fs = 0;
   const double2* g = reinterpret_cast<const double2*>(grid + m.off_grid + (long long)j * m.M);
-  for (int i = threadIdx.x; i < L; i += blockDim.x) sa[i] = g[i];
-  __syncthreads();
+  const FxRes z = xf_r2c<1, true, false>(fs, fs + L, FxLay{1, 1, L, 0}, R.px, [&](int, int, int i) { return g[i]; });
   if (mode == 0) {
-    row_r2c(sa, sb, st, m, R, 1.0 / m.M, 1.0 / m.M);
     double2* dst = A.mixB[0] + m.off_mix + (long long)j * Kx;
+    const double s = 1.0 / m.M;
     for (int k = threadIdx.x; k < Kx; k += blockDim.x) {
-      const double2 v = dst[k];
-      dst[k] = make_double2(v.x - st[k].x, v.y - st[k].y);
+      const double2 v = dst[k], c = z.coef(0, 0, k);
+      dst[k] = make_double2(v.x - c.x * s, k == 0 ? v.y : v.y - c.y * s);
     }
   } else {
-    row_r2c(sa, sb, A.mixB[4] + m.off_mix + (long long)j * Kx, m, R, 1.0, 2.0);
+    put_row(z, 0, A.mixB[4] + m.off_mix + (long long)j * Kx, Kx, 1.0, 2.0);
   }
 }
 
@@ -772,7 +702,7 @@ struct Kol : EqImpl {
   int CW = 4, RW = 2, ctas_per_sm = 0, persistent = 1;
   unsigned spin_limit = kSpinLimit;
   int drop_signal_member = -1;
-  DevBuf dmem, tables, Xr[2], Fr[2], Yr[2], mixA, mixB, ctr, trajbuf, seedbuf, seedmap, obsbuf, obsteps, partial, Jd,
+  DevBuf dmem, tables, diag, Xr[2], Fr[2], Yr[2], mixA, mixB, ctr, trajbuf, seedbuf, seedmap, obsbuf, obsteps, partial, Jd,
       tmp;
   int n_obs = 0, obs_kmax = 32;
   std::vector<int> obs_steps_h;
@@ -843,9 +773,10 @@ struct Kol : EqImpl {
     state_size = offs;
     mix_size = offm;
     grid_size = offg;
-    // twiddle tables per resolution: WMx (M entries) then W2M (2M entries)
+    // per resolution: exp(-2 pi i m / M), the transforms' tables, and the diagonal factors (KRes::diag)
     std::vector<double2> ht;
-    std::vector<size_t> toff, soff;
+    std::vector<double> hd;
+    std::vector<size_t> toff, soff, doff;
     for (size_t i = 0; i < resN.size(); ++i) {
       const int M = 3 * resN[i] / 2;
       kres[i].px = make_plan(M / 2);
@@ -859,26 +790,30 @@ struct Kol : EqImpl {
         const double th = -2.0 * M_PI * m / M;
         ht.push_back(make_double2(std::cos(th), std::sin(th)));
       }
-      for (int m = 0; m < 2 * M; ++m) {
-        const double th = -2.0 * M_PI * m / (2.0 * M);
-        ht.push_back(make_double2(std::cos(th), std::sin(th)));
-      }
-      // the butterflies' scaled-twiddle records of the x and y plans
+      // the transforms' tables of the x and y plans
       soff.push_back(ht.size());
-      const std::vector<double2> sx = scaled_twiddle_table(kres[i].px);
+      const std::vector<double2> sx = fft_tables(kres[i].px);
       ht.insert(ht.end(), sx.begin(), sx.end());
       soff.push_back(ht.size());
-      const std::vector<double2> sy = scaled_twiddle_table(kres[i].py);
+      const std::vector<double2> sy = fft_tables(kres[i].py);
       ht.insert(ht.end(), sy.begin(), sy.end());
+      doff.push_back(hd.size());
+      const double shift[3] = {0.0, 1.0 / p->desc.dt, 1.5 / p->desc.dt};
+      for (int t = 0; t < 3; ++t)
+        for (int kx = 0; kx < N / 2; ++kx)
+          for (int q = 0; q < N; ++q) {
+            const double ky = q < N / 2 ? q : q - N, k2 = (double)kx * kx + ky * ky;
+            hd.push_back(t ? 1.0 / std::fma(k2, 1.0 / Re, shift[t]) : (k2 > 0.0 ? 1.0 / k2 : 0.0));
+          }
     }
+    SPADJ_CUDA_TRY(p, diag.ensure(sizeof(double) * hd.size()));
+    SPADJ_CUDA_TRY(p, cudaMemcpyAsync(diag.ptr, hd.data(), sizeof(double) * hd.size(), cudaMemcpyHostToDevice, p->stream));
     SPADJ_CUDA_TRY(p, tables.ensure(sizeof(double2) * ht.size()));
     SPADJ_CUDA_TRY(p, cudaMemcpyAsync(tables.ptr, ht.data(), sizeof(double2) * ht.size(), cudaMemcpyHostToDevice, p->stream));
     for (size_t i = 0; i < resN.size(); ++i) {
-      const int M = 3 * resN[i] / 2;
-      kres[i].WMx = tables.as<double2>() + toff[i];
-      kres[i].W2M = tables.as<double2>() + toff[i] + M;
-      bind_scaled_twiddles(kres[i].px, tables.as<double2>() + soff[2 * i]);
-      bind_scaled_twiddles(kres[i].py, tables.as<double2>() + soff[2 * i + 1]);
+      fft_bind(kres[i].px, tables.as<double2>() + soff[2 * i], tables.as<double2>() + toff[i]);
+      fft_bind(kres[i].py, tables.as<double2>() + soff[2 * i + 1], nullptr);
+      kres[i].diag = diag.as<double>() + doff[i];
     }
     const size_t sb = sizeof(double2) * state_size, mb = sizeof(double2) * mix_size;
     for (int i = 0; i < 2; ++i) {
@@ -988,7 +923,6 @@ struct Kol : EqImpl {
     A.mem = dmem.as<KMember>();
     for (int i = 0; i < kMaxRes; ++i) A.res[i] = kres[i];
     A.Re = Re; A.dt = dt; A.CW = CW; A.RW = RW;
-    A.invRe = 1.0 / Re;
     const double kc[2][5] = {{1.0 / dt, -1.0 / dt, 0.0, 1.0, 0.0}, {1.5 / dt, -2.0 / dt, 0.5 / dt, 2.0, -1.0}};
     for (int r = 0; r < 2; ++r)
       for (int i = 0; i < 5; ++i) A.kc[r][i] = kc[r][i];
@@ -1737,7 +1671,7 @@ struct Kol : EqImpl {
     for (DevBuf* b : {&gridW, &gridG, &corr, &xq, &hbuf[0], &hbuf[1], &hbuf[2], &dact[0], &dact[1], &dact[2], &dh, &dz, &dz2,
                       &pbuf, &wq, &bq, &part, &gp, &chunkbuf})
       b->release();
-    for (DevBuf* b : {&dmem, &tables, &Xr[0], &Xr[1], &Fr[0], &Fr[1], &Yr[0], &Yr[1], &mixA, &mixB, &ctr, &trajbuf,
+    for (DevBuf* b : {&dmem, &tables, &diag, &Xr[0], &Xr[1], &Fr[0], &Fr[1], &Yr[0], &Yr[1], &mixA, &mixB, &ctr, &trajbuf,
                       &seedbuf, &seedmap, &obsbuf, &obsteps, &partial, &Jd, &tmp, &segx0, &segbuf, &rsbuf, &cslots,
                       &obsstates, &obsidx, &cnnerr})
       b->release();

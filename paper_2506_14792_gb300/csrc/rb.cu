@@ -177,8 +177,8 @@ struct RB : EqImpl {
       const double th = -2.0 * M_PI * (double)m / (double)Mx;
       hwm[m] = make_double2(std::cos(th), std::sin(th));
     }
-    {  // the butterflies' scaled-twiddle records follow the M-table in the same buffer
-      const std::vector<double2> sct = scaled_twiddle_table(xp.plan);
+    {  // the transforms' tables follow the M-table in the same buffer
+      const std::vector<double2> sct = fft_tables(xp.plan);
       hwm.insert(hwm.end(), sct.begin(), sct.end());
     }
     auto up = [&](DevBuf& b, const void* h, size_t bytes) -> cudaError_t {
@@ -200,7 +200,7 @@ struct RB : EqImpl {
       if (s != SPADJ_OK) return s;
     }
     xp.WM = wm.as<double2>();
-    bind_scaled_twiddles(xp.plan, xp.WM + Mx);
+    fft_bind(xp.plan, xp.WM + Mx, xp.WM);
     // work buffers
     const size_t sb = sizeof(double2) * ns, mb = sizeof(double2) * nmix, gb = sizeof(double) * npts;
     for (WS& l : ws) {

@@ -12,7 +12,7 @@
 #include <algorithm>
 #include <cooperative_groups.h>
 
-#include "fft.cuh"
+#include "fxfft.cuh"
 #include "pdl.cuh"
 
 namespace spadj {
@@ -231,200 +231,84 @@ struct XParams {
   const double2* WM;
 };
 
-__global__ void __launch_bounds__(64) xfft_kernel(const __grid_constant__ XJobs js, XParams P) {
-  pdl_trigger();
-  pdl_wait();
-  const XJob& J = js.j[blockIdx.y];
-  const int row = blockIdx.x;
-  const int L = P.L, Kx = P.Kx, Mx = P.Mx;
-  extern __shared__ double2 sx[];
-  double2* A = sx;
-  double2* B = A + L;
-  double2* C = B + L;
-  double2* D = C + L;
-  double2* S = D + L;  // Kx
-  if (J.dir == 0) {
-    const double2* src = J.cin + (size_t)row * Kx;
-    for (int k = threadIdx.x; k < Kx; k += blockDim.x) {
-      double2 v = src[k];
-      if (J.cmul == 1) {  // i k v
-        const double kk = P.kscale * k;
-        v = make_double2(-kk * v.y, kk * v.x);
-      }
-      S[k] = v;
-    }
-    __syncthreads();
-    c2r_pre(A, [&](int k) { return S[k]; }, Kx, L, P.WM, J.w0, J.w);
-    __syncthreads();
-    double2* z = cfft_smem(A, B, P.plan, P.WM, +1);
-    double2* g = reinterpret_cast<double2*>(J.rout + (size_t)row * Mx);
-    for (int j = threadIdx.x; j < L; j += blockDim.x) g[j] = z[j];
-  } else {
-    if (J.nprod > 0) {
-      auto rowp = [&](const double* base, int slot) {
-        return reinterpret_cast<const double2*>(base + (size_t)slot * J.npts + (size_t)row * Mx);
-      };
-      const double2 *a0 = rowp(J.G, J.pa[0]), *b0 = rowp(J.G, J.pb[0]);
-      const double2 *a1 = rowp(J.G, J.pa[1]), *b1 = rowp(J.G, J.pb[1]);
-      const double p0 = J.ps[0], p1 = J.ps[1];
-      if (!J.dG) {
-        for (int j = threadIdx.x; j < L; j += blockDim.x) {
-          const double2 a = a0[j], b = b0[j], c = a1[j], d = b1[j];
-          A[j] = make_double2(fma(p0 * a.x, b.x, p1 * (c.x * d.x)), fma(p0 * a.y, b.y, p1 * (c.y * d.y)));
-        }
-      } else {
-        const double2 *da0 = rowp(J.dG, J.pa[0]), *db0 = rowp(J.dG, J.pb[0]);
-        const double2 *da1 = rowp(J.dG, J.pa[1]), *db1 = rowp(J.dG, J.pb[1]);
-        for (int j = threadIdx.x; j < L; j += blockDim.x) {
-          const double2 a = a0[j], b = b0[j], c = a1[j], d = b1[j];
-          const double2 da = da0[j], db = db0[j], dc = da1[j], dd = db1[j];
-          A[j] = make_double2(p0 * (da.x * b.x + a.x * db.x) + p1 * (dc.x * d.x + c.x * dd.x),
-                              p0 * (da.y * b.y + a.y * db.y) + p1 * (dc.y * d.y + c.y * dd.y));
-        }
-      }
-    } else {
-      for (int t = 0; t < J.nr; ++t) {
-        double2* a = (t == 0) ? A : C;
-        const double2* g = reinterpret_cast<const double2*>(J.rin[t] + (size_t)row * Mx);
-        for (int j = threadIdx.x; j < L; j += blockDim.x) a[j] = g[j];
-      }
-    }
-    __syncthreads();
-    double2 *z0, *z1 = nullptr;
-    if (J.nr > 1) {  // both inputs' transforms in the same passes (A|B and C|D are 2L apart)
-      cfft_smem_sets<-1>(A, B, 2 * L, 2, P.plan, 1);
-      z0 = (P.plan.nrad & 1) ? B : A;
-      z1 = (P.plan.nrad & 1) ? D : C;
-    } else {
-      z0 = cfft_smem(A, B, P.plan, P.WM, -1);
-    }
-    double2* dst = J.cout + (size_t)row * Kx;
-    // r2c post-processing for each input, combined
-    for (int k = threadIdx.x; k < Kx; k += blockDim.x) {
-      double2 acc = make_double2(0.0, 0.0);
-      for (int t = 0; t < J.nr; ++t) {
-        const double2* Z = (t == 0) ? z0 : z1;
-        double2 X = r2c_combine2(Z[k], cconj(Z[k == 0 ? 0 : L - k]), __ldg(&P.WM[k]));  // twice the entry
-        if (J.rmul[t] == 2) {  // -i k X
-          const double kk = P.kscale * k;
-          X = make_double2(kk * X.y, -kk * X.x);
-        }
-        acc = t == 0 ? X : cadd(acc, X);
-      }
-      const double sc = 0.5 * ((k == 0) ? J.s0 : J.s);
-      double2 r = cscale(acc, sc);
-      if (k == 0) r.y = 0.0;
-      dst[k] = r;
-    }
-  }
-}
-
 constexpr int kXThreadsMax = 192;
-// xfft_kernel's jobs for nb rows per CTA (nb <= 4): the rows are interleaved in shared memory
-// (element e of row c at e * nb + c) and transformed together by cfft_smem_batch, so short rows
-// keep all threads of the CTA busy in every Stockham pass and share its barriers.
-__global__ void __launch_bounds__(kXThreadsMax) xfftm_kernel(const __grid_constant__ XJobs js, XParams P, int nb, int nrows) {
+// x-transform jobs, nb rows per CTA (nb <= 4): the rows are interleaved in shared memory (element e of row c
+// at e * nb + c) and transformed together, so short rows keep all threads of the CTA busy in every
+// pass and share its barriers.  Every row has its own scale, so the results do not depend on nb.
+__global__ void __launch_bounds__(kXThreadsMax) xfft_kernel(const __grid_constant__ XJobs js,
+                                                            const __grid_constant__ XParams P, int nb, int nrows) {
   pdl_trigger();
   pdl_wait();
   const XJob& J = js.j[blockIdx.y];
   const int row0 = blockIdx.x * nb;
   const int L = P.L, Kx = P.Kx, Mx = P.Mx;
-  extern __shared__ double2 sx[];
-  double2* A = sx;
-  double2* B = A + (size_t)L * nb;
-  double2* C = B + (size_t)L * nb;
-  double2* D = C + (size_t)L * nb;
-  double2* S = D + (size_t)L * nb;  // [nb][Kx]
+  const int a = 0, b = L * nb;
   const int tid = threadIdx.x, nt = blockDim.x;
+  const double2 zero = make_double2(0.0, 0.0);
   if (J.dir == 0) {
-    for (int idx = tid; idx < nb * Kx; idx += nt) {
-      const int c = idx / Kx, k = idx - c * Kx;
-      double2 v = make_double2(0.0, 0.0);
-      if (row0 + c < nrows) {
-        v = J.cin[(size_t)(row0 + c) * Kx + k];
-        if (J.cmul == 1) {  // i k v
-          const double kk = P.kscale * k;
-          v = make_double2(-kk * v.y, kk * v.x);
-        }
+    const double2* src = J.cin + (size_t)row0 * Kx;
+    const FxRes z = xf_c2r<1, false>(a, b, FxLay{1, nb, L * nb, 0}, P.plan, Kx, [&](int, int c, int k) {
+      if (row0 + c >= nrows) return zero;
+      double2 v = src[(size_t)c * Kx + k];
+      if (J.cmul == 1) {  // i k v
+        const double kk = P.kscale * k;
+        v = make_double2(-kk * v.y, kk * v.x);
       }
-      S[idx] = v;
-    }
-    __syncthreads();
-    // packed spectrum of each real row (c2r_pre), interleaved
-    for (int idx = tid; idx < nb * L; idx += nt) {
-      const int k = idx / nb, c = idx - k * nb;
-      const double2* Sr = S + (size_t)c * Kx;
-      double2 xk = make_double2(0.0, 0.0), xc = make_double2(0.0, 0.0);
-      if (k == 0) xk = make_double2(J.w0 * Sr[0].x, 0.0);
-      else if (k < Kx) xk = cscale(Sr[k], J.w);
-      const int kc = L - k;
-      if (k > 0 && kc < Kx) xc = cconj(cscale(Sr[kc], J.w));
-      A[idx] = c2r_combine(cadd(xk, xc), csub(xk, xc), __ldg(&P.WM[k]));
-    }
-    __syncthreads();
-    const double2* z = cfft_smem_batch<1>(A, B, P.plan, P.WM, nb);
-    for (int idx = tid; idx < nb * L; idx += nt) {
-      const int c = idx / L, j = idx - c * L;
-      if (row0 + c < nrows) reinterpret_cast<double2*>(J.rout + (size_t)(row0 + c) * Mx)[j] = z[j * nb + c];
+      return cscale(v, k == 0 ? J.w0 : J.w);
+    });
+    for (int c = 0; c < nb && row0 + c < nrows; ++c) {
+      double2* g = reinterpret_cast<double2*>(J.rout + (size_t)(row0 + c) * Mx);
+      for (int j = tid; j < L; j += nt) g[j] = z.at(0, c, j);
     }
     return;
   }
-  const int nin = J.nprod > 0 ? 1 : J.nr;
-  for (int idx = tid; idx < nb * L; idx += nt) {
-    const int c = idx / L, j = idx - c * L;
-    double2 v0 = make_double2(0.0, 0.0), v1 = make_double2(0.0, 0.0);
-    if (row0 + c < nrows) {
-      const size_t ro = (size_t)(row0 + c) * Mx;
-      if (J.nprod > 0) {
-        auto at = [&](const double* base, int slot) {
-          return reinterpret_cast<const double2*>(base + (size_t)slot * J.npts + ro)[j];
-        };
-        const double2 a = at(J.G, J.pa[0]), b = at(J.G, J.pb[0]), cc = at(J.G, J.pa[1]), d = at(J.G, J.pb[1]);
-        const double p0 = J.ps[0], p1 = J.ps[1];
-        if (!J.dG) {
-          v0 = make_double2(fma(p0 * a.x, b.x, p1 * (cc.x * d.x)), fma(p0 * a.y, b.y, p1 * (cc.y * d.y)));
-        } else {
-          const double2 da = at(J.dG, J.pa[0]), db = at(J.dG, J.pb[0]), dc = at(J.dG, J.pa[1]), dd = at(J.dG, J.pb[1]);
-          v0 = make_double2(p0 * (da.x * b.x + a.x * db.x) + p1 * (dc.x * d.x + cc.x * dd.x),
-                            p0 * (da.y * b.y + a.y * db.y) + p1 * (dc.y * d.y + cc.y * dd.y));
+  auto store = [&](const FxRes& z, int nin) {
+    for (int c = 0; c < nb && row0 + c < nrows; ++c) {
+      double2* dst = J.cout + (size_t)(row0 + c) * Kx;
+      for (int k = tid; k < Kx; k += nt) {
+        double2 acc = zero;
+        for (int t = 0; t < nin; ++t) {
+          double2 X = z.coef(t, c, k);
+          if (J.rmul[t] == 2) {  // -i k X
+            const double kk = P.kscale * k;
+            X = make_double2(kk * X.y, -kk * X.x);
+          }
+          acc = t == 0 ? X : cadd(acc, X);
         }
-      } else {
-        v0 = reinterpret_cast<const double2*>(J.rin[0] + ro)[j];
-        if (nin > 1) v1 = reinterpret_cast<const double2*>(J.rin[1] + ro)[j];
+        double2 o = cscale(acc, k == 0 ? J.s0 : J.s);
+        if (k == 0) o.y = 0.0;
+        dst[k] = o;
       }
     }
-    A[j * nb + c] = v0;
-    if (nin > 1) C[j * nb + c] = v1;
+  };
+  if (J.nprod > 0) {
+    const double p0 = J.ps[0], p1 = J.ps[1];
+    store(xf_r2c<1, false>(a, b, FxLay{1, nb, L * nb, 0}, P.plan, [&](int, int c, int j) {
+      if (row0 + c >= nrows) return zero;
+      const size_t ro = (size_t)(row0 + c) * Mx;
+      auto at = [&](const double* base, int slot) {
+        return reinterpret_cast<const double2*>(base + (size_t)slot * J.npts + ro)[j];
+      };
+      const double2 x = at(J.G, J.pa[0]), y = at(J.G, J.pb[0]), u = at(J.G, J.pa[1]), v = at(J.G, J.pb[1]);
+      if (!J.dG) return make_double2(fma(p0 * x.x, y.x, p1 * (u.x * v.x)), fma(p0 * x.y, y.y, p1 * (u.y * v.y)));
+      const double2 dx = at(J.dG, J.pa[0]), dy = at(J.dG, J.pb[0]), du = at(J.dG, J.pa[1]), dv = at(J.dG, J.pb[1]);
+      return make_double2(p0 * (dx.x * y.x + x.x * dy.x) + p1 * (du.x * v.x + u.x * dv.x),
+                          p0 * (dx.y * y.y + x.y * dy.y) + p1 * (du.y * v.y + u.y * dv.y));
+    }), 1);
+    return;
   }
-  __syncthreads();
-  cfft_smem_sets<-1>(A, B, 2 * L * nb, nin, P.plan, nb);  // A|B and C|D are 2 L nb apart
-  const double2* z0 = (P.plan.nrad & 1) ? B : A;
-  const double2* z1 = (P.plan.nrad & 1) ? D : C;
-  for (int idx = tid; idx < nb * Kx; idx += nt) {
-    const int c = idx / Kx, k = idx - c * Kx;
-    if (row0 + c >= nrows) continue;
-    double2 acc = make_double2(0.0, 0.0);
-    for (int t = 0; t < nin; ++t) {
-      const double2* Z = t == 0 ? z0 : z1;
-      double2 X = r2c_combine2(Z[k * nb + c], cconj(Z[(k == 0 ? 0 : L - k) * nb + c]), __ldg(&P.WM[k]));
-      if (J.rmul[t] == 2) {  // -i k X
-        const double kk = P.kscale * k;
-        X = make_double2(kk * X.y, -kk * X.x);
-      }
-      acc = t == 0 ? X : cadd(acc, X);
-    }
-    const double sc = 0.5 * ((k == 0) ? J.s0 : J.s);
-    double2 out = cscale(acc, sc);
-    if (k == 0) out.y = 0.0;
-    J.cout[(size_t)(row0 + c) * Kx + k] = out;
-  }
+  auto row = [&](int t, int c, int j) {
+    return row0 + c < nrows ? reinterpret_cast<const double2*>(J.rin[t] + (size_t)(row0 + c) * Mx)[j] : zero;
+  };
+  if (J.nr > 1) store(xf_r2c<2, false>(a, b, FxLay{2, nb, 2 * L * nb, 0}, P.plan, row), 2);  // sets 2 L nb apart
+  else store(xf_r2c<1, false>(a, b, FxLay{1, nb, L * nb, 0}, P.plan, row), 1);
 }
 
-inline size_t xfftm_smem(int L, int Kx, int nb) { return sizeof(double2) * (size_t)nb * (4 * L + Kx); }
+inline size_t xfft_smem(int L, int nb) { return sizeof(double2) * (size_t)nb * 4 * L; }
 constexpr int kXRowsMax = 4;
 
 // Launch variant of the x transforms: rows per CTA nb (low byte) and threads per CTA nt (the
-// bits above; 0 = 64).  nb = 1 with 64 threads is xfft_kernel, everything else xfftm_kernel.
+// bits above; 0 = 64).
 // Threads per CTA that are a multiple of the butterflies of a pass keep every lane busy in
 // it: for L = 192 (radix 4, 4, 4, 3: 48, 48, 48, 64 butterflies per row) that is 96 threads
 // on two rows or 192 on four.
@@ -435,10 +319,8 @@ constexpr int xvar_threads(int xv) { return (xv >> 8) ? (xv >> 8) : 64; }
 // x-transform jobs over nrows rows in launch variant xv
 inline cudaError_t launch_xfft(bool pdl, int xv, const XJobs& js, const XParams& xp, int nrows, cudaStream_t st) {
   const int nb = xvar_rows(xv) < 1 ? 1 : xvar_rows(xv), nt = xvar_threads(xv);
-  if (nb == 1 && nt == 64)
-    return launch_kernel(pdl, xfft_kernel, dim3(nrows, js.n), dim3(64), xfftm_smem(xp.L, xp.Kx, 1), st, js, xp);
-  return launch_kernel(pdl, xfftm_kernel, dim3((nrows + nb - 1) / nb, js.n), dim3(nt), xfftm_smem(xp.L, xp.Kx, nb), st,
-                       js, xp, nb, nrows);
+  return launch_kernel(pdl, xfft_kernel, dim3((nrows + nb - 1) / nb, js.n), dim3(nt), xfft_smem(xp.L, nb), st, js, xp, nb,
+                       nrows);
 }
 
 // Launch variant for the x transforms of this problem: rows `forced` (1, 2 or 4, 64 threads)
@@ -451,13 +333,11 @@ inline int tune_xfft_rows(const XJobs& js, const XParams& xp, int nrows, cudaStr
   // row counts whose shared memory fits one CTA (raising the opt-in limit where needed)
   bool ok[kXRowsMax + 1] = {false, false, false, false, false};
   for (int nb : {1, 2, 4}) {
-    const size_t sm = xfftm_smem(xp.L, xp.Kx, nb);
-    if (sm <= 48 * 1024) {
+    const size_t sm = xfft_smem(xp.L, nb), fix = sizeof(FxShared);
+    if (sm + fix <= 48 * 1024) {
       ok[nb] = true;
-    } else if (sm <= 227 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(xfftm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      if (e == cudaSuccess && nb == 1)
-        e = cudaFuncSetAttribute(xfft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    } else if (sm + fix <= 227 * 1024) {
+      cudaError_t e = cudaFuncSetAttribute(xfft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       ok[nb] = e == cudaSuccess;
       cudaGetLastError();
     }
