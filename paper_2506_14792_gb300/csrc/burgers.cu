@@ -25,7 +25,7 @@ constexpr int kQMax = 4;  // modes per thread
 constexpr int kMaxOrder = 4;
 
 struct BurgersParams {
-  int K, L, M;
+  int K, L, M, C;  // C: entries of one transform buffer
   double nu, kscale, dt, length;
   int order, nonlinear;
   FFTPlan plan;
@@ -39,55 +39,46 @@ struct BurgersParams {
   int ws_len;
 };
 
-// Buffers of a CTA: two transform pairs of L entries each.  The inverse transforms read their staged
+// Buffers of a CTA: two transform pairs of C entries each.  The inverse transforms read their staged
 // spectra from B (and D for a second one) and leave the grid in A or B (C or D).
 struct Smem {
   int A, B, C, D;
 };
 
-__device__ __forceinline__ Smem carve(const BurgersParams& P) { return Smem{0, P.L, 2 * P.L, 3 * P.L}; }
+__device__ __forceinline__ Smem carve(const BurgersParams& P) { return Smem{0, P.C, 2 * P.C, 3 * P.C}; }
 
 __device__ __forceinline__ double kwav(const BurgersParams& P, int k) { return P.kscale * k; }
 
+// -i k v s
+__device__ __forceinline__ double2 minus_ik(const BurgersParams& P, int k, double2 v, double s) {
+  const double kk = kwav(P, k) * s;
+  return make_double2(kk * v.y, -kk * v.x);
+}
 // Puts F(x)_k = -i k T[(B x)^2 / 2]_k, k < K, through out(k, F_k), from the spectrum staged in B.
-template <class Out>
+template <int PATH, class Out>
 __device__ __forceinline__ void eval_F(const BurgersParams& P, const Smem& s, Out out) {
-  const FxRes u = xf_c2r_staged<1, false>(s.A, s.B, FxLay{1, 1, P.L, 0}, P.plan, P.K);
-  const FxRes z = xf_r2c<1, true, false>(s.C, s.D, FxLay{1, 1, P.L, 0}, P.plan, [&](int, int, int j) {
-    const double2 v = u.at(0, 0, j);
+  const auto u = xf_c2r_staged<1, PATH>(s.A, s.B, FxLay{1, P.C, 0}, P.plan, P.K);
+  const auto z = xf_r2c<1, PATH>(s.C, s.D, FxLay{1, P.C, 0}, P.plan, [&](int, int j) {
+    const double2 v = u.at(0, j);
     return make_double2(v.x * v.x, v.y * v.y);  // u^2; the 1/2 goes into the scale below
   });
-  const double q = 0.5 / P.M;
-  for (int k = threadIdx.x; k < P.K; k += blockDim.x) {
-    const double2 v = z.coef(0, 0, k);
-    const double kk = kwav(P, k) * q;  // -i k v / M
-    out(k, make_double2(kk * v.y, -kk * v.x));
-  }
+  for (int k = threadIdx.x; k < P.K; k += blockDim.x) out(k, minus_ik(P, k, z.coef(0, k), 0.5 / P.M));
 }
 
-// From the primal spectrum staged in B and the tangent spectrum in D: outF(k, F_k) (if want_F) and
-// outJ(k, ((dF/dX) dX)_k), (dF/dX) dX = -i k T[(B x)(B dx)].
-template <class OutF, class OutJ>
-__device__ __forceinline__ void eval_F_and_jvp(const BurgersParams& P, const Smem& s, bool want_F, OutF outF, OutJ outJ) {
-  // both inverse transforms in the same passes (A|B and C|D are 2L apart)
-  const FxRes u = xf_c2r_staged<2, false>(s.A, s.B, FxLay{2, 1, 2 * P.L, 0}, P.plan, P.K);
-  const bool odd = P.plan.nrad & 1;
-  const int f0 = odd ? s.A : s.B, f1 = odd ? s.C : s.D;  // free halves
-  for (int t = want_F ? 0 : 1; t < 2; ++t) {
-    const FxRes z = xf_r2c<1, true, false>(f0, f1, FxLay{1, 1, P.L, 2}, P.plan, [&](int, int, int j) {
-      const double2 v = u.at(0, 0, j), w = t ? u.at(1, 0, j) : v;
-      return make_double2(v.x * w.x, v.y * w.y);
-    });
-    const double q = (t ? 1.0 : 0.5) / P.M;
-    for (int k = threadIdx.x; k < P.K; k += blockDim.x) {
-      const double2 v = z.coef(0, 0, k);
-      const double kk = kwav(P, k) * q;
-      const double2 o = make_double2(kk * v.y, -kk * v.x);
-      if (t) outJ(k, o);
-      else outF(k, o);
-    }
-    __syncthreads();
-  }
+// From the primal spectrum staged in B and the tangent spectrum in D: out(k, F_k, ((dF/dX) dX)_k),
+// (dF/dX) dX = -i k T[(B x)(B dx)].  Both transforms of each direction share their passes (A|B and C|D are 2C
+// apart); the second ones are staged in the free halves and overwrite the grids after that.
+template <int PATH, class Out>
+__device__ __forceinline__ void eval_F_and_jvp(const BurgersParams& P, const Smem& s, Out out) {
+  const FxLay lay{2, 2 * P.C, 0};
+  const auto u = xf_c2r_staged<2, PATH>(s.A, s.B, lay, P.plan, P.K);
+  const auto z = xf_r2c<2, PATH>(u.z == s.A ? s.B : s.A, u.z, lay, P.plan, [&](int q, int j) {
+    const double2 v = u.at(0, j), w = q ? u.at(1, j) : v;
+    return make_double2(v.x * w.x, v.y * w.y);
+  });
+  for (int k = threadIdx.x; k < P.K; k += blockDim.x)
+    out(k, minus_ik(P, k, z.coef(0, k), 0.5 / P.M), minus_ik(P, k, z.coef(1, k), 1.0 / P.M));
+  __syncthreads();  // the results lie where the next spectra are staged
 }
 
 // i k w / (2M): T^dagger's weights (1/M on the real part of k = 0, 1/(2M) elsewhere) folded in, the k = 0
@@ -98,17 +89,16 @@ __device__ __forceinline__ double2 vjp_cotangent(const BurgersParams& P, int k, 
 }
 // From the primal spectrum staged in B and vjp_cotangent(W) in D: out(k, ((dF/dX)^dagger W)_k),
 // (dF/dX)^dagger W = B^dagger[(B x) * T^dagger(i k W)].
-template <class Out>
+template <int PATH, class Out>
 __device__ __forceinline__ void eval_vjp(const BurgersParams& P, const Smem& s, Out out) {
-  const FxRes u = xf_c2r_staged<2, false>(s.A, s.B, FxLay{2, 1, 2 * P.L, 0}, P.plan, P.K);
-  const bool odd = P.plan.nrad & 1;
-  const int f0 = odd ? s.A : s.B, f1 = odd ? s.C : s.D;
-  const FxRes z = xf_r2c<1, true, false>(f0, f1, FxLay{1, 1, P.L, 0}, P.plan, [&](int, int, int j) {
-    const double2 a = u.at(0, 0, j), b = u.at(1, 0, j);
+  const auto u = xf_c2r_staged<2, PATH>(s.A, s.B, FxLay{2, 2 * P.C, 0}, P.plan, P.K);
+  const int f0 = u.z == s.A ? s.B : s.A;  // free halves
+  const auto z = xf_r2c<1, PATH>(f0, f0 + 2 * P.C, FxLay{1, 2 * P.C, 0}, P.plan, [&](int, int j) {
+    const double2 a = u.at(0, j), b = u.at(1, j);
     return make_double2(a.x * b.x, a.y * b.y);
   });
   for (int k = threadIdx.x; k < P.K; k += blockDim.x) {
-    const double2 x = z.coef(0, 0, k);
+    const double2 x = z.coef(0, k);
     out(k, k == 0 ? make_double2(x.x, 0.0) : make_double2(2.0 * x.x, 2.0 * x.y));
   }
 }
@@ -120,7 +110,10 @@ __device__ __forceinline__ double2* row(double* base, int b, int K) {
   return reinterpret_cast<double2*>(base) + (size_t)b * K;
 }
 
-// ---- single-shot kernels (transforms, F, JVP, VJP) ----------------------------------------
+// ---- single-shot kernels (transforms, F, JVP, VJP) ---------------------------------------
+//
+// One call of these is all launch and latency (about 10 us), so they keep the FP64 transforms; the step loops
+// below run the fixed-point ones.
 
 // coefficients -> grid with the weights w0 (k = 0) and w
 __global__ void __launch_bounds__(64) to_grid_kernel(const __grid_constant__ BurgersParams P, double w0, double w, const double2* __restrict__ x,
@@ -128,9 +121,9 @@ __global__ void __launch_bounds__(64) to_grid_kernel(const __grid_constant__ Bur
   const Smem s = carve(P);
   const double2* xr = x + (size_t)blockIdx.x * P.K;
   double2* gr = g + (size_t)blockIdx.x * P.L;
-  const FxRes z = xf_c2r<1, true, false>(s.A, s.B, FxLay{1, 1, P.L, 0}, P.plan, P.K,
-                                         [&](int, int, int k) { return cscale(ldg128(xr + k), k == 0 ? w0 : w); });
-  for (int j = threadIdx.x; j < P.L; j += blockDim.x) stg128(gr + j, z.at(0, 0, j));
+  const auto z = xf_c2r<1, kFp64>(s.A, s.B, FxLay{1, P.C, 0}, P.plan, P.K,
+                                         [&](int, int k) { return cscale(ldg128(xr + k), k == 0 ? w0 : w); });
+  for (int j = threadIdx.x; j < P.L; j += blockDim.x) stg128(gr + j, z.at(0, j));
 }
 // grid -> coefficients times s0 (k = 0, real part only if re0) or s
 __global__ void __launch_bounds__(64) to_coef_kernel(const __grid_constant__ BurgersParams P, double s0, double sc, int re0,
@@ -138,20 +131,23 @@ __global__ void __launch_bounds__(64) to_coef_kernel(const __grid_constant__ Bur
   const Smem s = carve(P);
   const double2* gr = g + (size_t)blockIdx.x * P.L;
   double2* yr = y + (size_t)blockIdx.x * P.K;
-  const FxRes z = xf_r2c<1, true, false>(s.A, s.B, FxLay{1, 1, P.L, 0}, P.plan, [&](int, int, int j) { return ldg128(gr + j); });
+  const auto z = xf_r2c<1, kFp64>(s.A, s.B, FxLay{1, P.C, 0}, P.plan, [&](int, int j) { return ldg128(gr + j); });
   for (int k = threadIdx.x; k < P.K; k += blockDim.x) {
-    double2 v = cscale(z.coef(0, 0, k), k == 0 ? s0 : sc);
+    double2 v = cscale(z.coef(0, k), k == 0 ? s0 : sc);
     if (k == 0 && re0) v.y = 0.0;
     stg128(yr + k, v);
   }
 }
 
-__global__ void __launch_bounds__(64) F_kernel(const __grid_constant__ BurgersParams P, int mode, const double* __restrict__ x, const double* __restrict__ d,
-                         double* __restrict__ out) {
+// F (MODE 0), its JVP along d (1) or its VJP of d (2)
+template <int MODE>
+__global__ void __launch_bounds__(64) F_kernel(const __grid_constant__ BurgersParams P, const double2* __restrict__ x,
+                                               const double2* __restrict__ d, double2* __restrict__ out) {
   const Smem s = carve(P);
-  const int b = blockIdx.x, K = P.K;
-  const double2* xr = row(x, b, K);
-  double2* o = row(out, b, K);
+  const int K = P.K;
+  const double2* xr = x + (size_t)blockIdx.x * K;
+  const double2* dr = d + (size_t)blockIdx.x * K;
+  double2* o = out + (size_t)blockIdx.x * K;
   if (!P.nonlinear) {
     for (int k = threadIdx.x; k < K; k += blockDim.x) stg128(o + k, make_double2(0.0, 0.0));
     return;
@@ -161,19 +157,19 @@ __global__ void __launch_bounds__(64) F_kernel(const __grid_constant__ BurgersPa
     const double2 v = ldg128(xr + k);
     fx_put64(s.B + k, v);
     m0 = fx_absmax(m0, v);
-    if (mode != 0) {
-      double2 w = ldg128(row(d, b, K) + k);
-      if (mode == 2) w = vjp_cotangent(P, k, w);
+    if (MODE != 0) {
+      double2 w = ldg128(dr + k);
+      if (MODE == 2) w = vjp_cotangent(P, k, w);
       fx_put64(s.D + k, w);
       m1 = fx_absmax(m1, w);
     }
   }
-  fx_put_max(0, 1, 0, m0);
-  if (mode != 0) fx_put_max(1, 1, 0, m1);
+  fx_put_max(0, m0);
+  if (MODE != 0) fx_put_max(1, m1);
   auto put = [&](int k, double2 v) { stg128(o + k, v); };
-  if (mode == 0) eval_F(P, s, put);
-  else if (mode == 1) eval_F_and_jvp(P, s, false, put, put);
-  else eval_vjp(P, s, put);
+  if (MODE == 0) eval_F<kFp64>(P, s, put);
+  else if (MODE == 1) eval_F_and_jvp<kFp64>(P, s, [&](int k, double2, double2 v) { put(k, v); });
+  else eval_vjp<kFp64>(P, s, put);
 }
 
 // ---- persistent trajectory kernels ----------------------------------------------------------
@@ -260,18 +256,19 @@ __global__ void __launch_bounds__(64) trajectory_kernel(const __grid_constant__ 
   unsigned mx = 0u, md = 0u;  // largest high words of the staged spectra
   // F (and its tangent) of the staged spectra into slot 0 of the histories: thread tid owns k = tid + q G
   auto nonlinear = [&]() {
-    fx_put_max(0, 1, 0, mx);
+    fx_put_max(0, mx);
     if (tangent) {
-      fx_put_max(1, 1, 0, md);
-      eval_F_and_jvp(P, s, true, [&](int k, double2 v) {
+      fx_put_max(1, md);
+      eval_F_and_jvp<kFxOnly>(P, s, [&](int k, double2 f, double2 g) {
 #pragma unroll
-        for (int q = 0; q < Q; ++q) if (k == tid + q * G) F[q][0] = v;
-      }, [&](int k, double2 v) {
-#pragma unroll
-        for (int q = 0; q < Q; ++q) if (k == tid + q * G) GJ[q][0] = v;
+        for (int q = 0; q < Q; ++q)
+          if (k == tid + q * G) {
+            F[q][0] = f;
+            GJ[q][0] = g;
+          }
       });
     } else {
-      eval_F(P, s, [&](int k, double2 v) {
+      eval_F<kFxOnly>(P, s, [&](int k, double2 v) {
 #pragma unroll
         for (int q = 0; q < Q; ++q) if (k == tid + q * G) F[q][0] = v;
       });
@@ -426,9 +423,9 @@ __global__ void __launch_bounds__(64) adjoint_kernel(const __grid_constant__ Bur
       }
       for (int q = 0; q < Q; ++q) lam[q] = z;
       if (P.nonlinear) {
-        fx_put_max(0, 1, 0, mx);
-        fx_put_max(1, 1, 0, mw);
-        eval_vjp(P, s, [&](int k, double2 v) {
+        fx_put_max(0, mx);
+        fx_put_max(1, mw);
+        eval_vjp<kFxOnly>(P, s, [&](int k, double2 v) {
 #pragma unroll
           for (int q = 0; q < Q; ++q) if (k == tid + q * G) lam[q] = v;
         });
@@ -562,6 +559,7 @@ struct Burgers : EqImpl {
         P.wc[s][i] = kSbdfC[s][i];
       }
     P.plan = make_plan(P.L);
+    P.C = P.L;
     if (P.plan.nrad < 0) return p->fail(SPADJ_ERR_INVALID, "burgers: 3N/4 must be of the form 2^a 3^b");
     if (P.K > kQMax * G) return p->fail(SPADJ_ERR_INVALID, "burgers: n[0] too large (max 512)");
     std::vector<double2> h(P.M);
@@ -570,15 +568,15 @@ struct Burgers : EqImpl {
       h[m] = make_double2(std::cos(th), std::sin(th));
     }
     {  // the transforms' tables follow the M-table in the same buffer
-      const std::vector<double2> sct = fft_tables(P.plan);
+      const std::vector<double2> sct = fft_tables(P.plan, true, true);
       h.insert(h.end(), sct.begin(), sct.end());
     }
     SPADJ_CUDA_TRY(p, wm.ensure(sizeof(double2) * h.size()));
     SPADJ_CUDA_TRY(p, cudaMemcpyAsync(wm.ptr, h.data(), sizeof(double2) * h.size(), cudaMemcpyHostToDevice, p->stream));
     SPADJ_CUDA_TRY(p, cudaStreamSynchronize(p->stream));
     P.WM = wm.as<double2>();
-    fft_bind(P.plan, P.WM + P.M, P.WM);
-    smem = sizeof(double2) * 4 * P.L;
+    fft_bind(P.plan, true, P.WM + P.M, P.WM, true);
+    smem = sizeof(double2) * 4 * P.C;
     return SPADJ_OK;
   }
 
@@ -633,7 +631,11 @@ struct Burgers : EqImpl {
   }
 
   spadj_status eval_F(Problem* p, int mode, const double* x, const double* dx, double* out) override {
-    F_kernel<<<B, G, smem, p->stream>>>(P, mode, x, dx, out);
+    const double2 *x2 = reinterpret_cast<const double2*>(x), *d2 = reinterpret_cast<const double2*>(dx);
+    double2* o2 = reinterpret_cast<double2*>(out);
+    if (mode == 0) F_kernel<0><<<B, G, smem, p->stream>>>(P, x2, d2, o2);
+    else if (mode == 1) F_kernel<1><<<B, G, smem, p->stream>>>(P, x2, d2, o2);
+    else F_kernel<2><<<B, G, smem, p->stream>>>(P, x2, d2, o2);
     return check_launch(p, "burgers F");
   }
 

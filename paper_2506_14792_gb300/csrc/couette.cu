@@ -55,7 +55,7 @@ struct Couette : EqImpl {
   HostBuf hslots;  // host tier of the two-level checkpoint schedule
   double res_omega = 0.0;
   bool res_built = false;
-  size_t zsmem = 0, xsmem = 0, ysmem = 0;
+  size_t zsmem = 0, ysmem = 0;
   rbhost::Operators ops;
   int xnb = 1;  // x-FFT launch variant, xvar(rows per CTA, threads) (tuned at creation)
 
@@ -109,10 +109,12 @@ struct Couette : EqImpl {
     xp.Kx = Kx; xp.Mx = Mx; xp.L = L; xp.kscale = 2.0 * M_PI / Lx;
     xp.plan = make_plan(L);
     yp.Kx = Kx; yp.Ny = Ny; yp.My = My;
-    yp.TK = Kx < 8 ? Kx : 8;
+    yp.TK = Kx >= 8 ? 8 : Kx >= 4 ? 4 : Kx >= 2 ? 2 : 1;
     yp.ntile = (Kx + yp.TK - 1) / yp.TK;
     yp.kxs = 2.0 * M_PI / Lx; yp.kys = 2.0 * M_PI / Ly;
     yp.plan = make_plan(My);
+    yp.C = My;
+    xp.C = L;
     if (xp.plan.nrad < 0 || yp.plan.nrad < 0)
       return p->fail(SPADJ_ERR_INVALID, "couette: 3*n[0]/4 and 3*n[1]/2 must be of the form 2^a 3^b");
 
@@ -136,10 +138,10 @@ struct Couette : EqImpl {
       hwx[m] = make_double2(std::cos(th), std::sin(th));
     }
     {  // the x transforms' tables follow the M-table in the same buffer
-      const std::vector<double2> sx = fft_tables(xp.plan);
+      const std::vector<double2> sx = fft_tables(xp.plan, true);
       hwx.insert(hwx.end(), sx.begin(), sx.end());
     }
-    const std::vector<double2> hwy = fft_tables(yp.plan);
+    const std::vector<double2> hwy = fft_tables(yp.plan, false);
     const double hone = 1.0;
     auto up = [&](DevBuf& b, const void* h, size_t bytes) -> cudaError_t {
       cudaError_t e = b.ensure(bytes);
@@ -158,8 +160,8 @@ struct Couette : EqImpl {
     SPADJ_CUDA_TRY(p, up(one, &hone, sizeof(double)));
     SPADJ_CUDA_TRY(p, cudaStreamSynchronize(p->stream));
     xp.WM = wmx.as<double2>();
-    fft_bind(xp.plan, xp.WM + Mx, xp.WM);
-    fft_bind(yp.plan, twy.as<double2>(), nullptr);
+    fft_bind(xp.plan, true, xp.WM + Mx, xp.WM);
+    fft_bind(yp.plan, false, twy.as<double2>(), nullptr);
     const size_t sb = sizeof(double2) * ns, gb = sizeof(double) * npts;
     SPADJ_CUDA_TRY(p, Zm.ensure(6 * sizeof(double2) * nzm));
     SPADJ_CUDA_TRY(p, Ym.ensure(6 * sizeof(double2) * nym));
@@ -177,8 +179,7 @@ struct Couette : EqImpl {
     SPADJ_CUDA_TRY(p, sdev.ensure(sizeof(double) * 2));
     SPADJ_CUDA_TRY(p, Jdev.ensure(sizeof(double)));
     zsmem = (size_t)2 * 2 * (size_t)std::max(N, Mz / 2) * kTM * sizeof(double2);
-    xsmem = sizeof(double2) * (4 * L + Kx);
-    ysmem = sizeof(double2) * 2 * (size_t)My * yp.TK;
+    ysmem = sizeof(double2) * (2 * (size_t)yp.C + 1) * yp.TK;
     {  // the step-solve operators of the selected form (the other one is built on first use)
       // One warp per pencil pair runs the band sweeps: with fewer than 8 pairs per SM the warps
       // cannot keep the FP64 pipe busy and the dense Phi (a CTA per pair) is faster (measured:
@@ -250,7 +251,11 @@ struct Couette : EqImpl {
   spadj_status launch_y(Problem* p, YJobs& js) {
     const double f = js.n * (double)Mz * Kx * 5.0 * My * std::log2((double)My);
     cudaEvent_t t = p->tic();
-    SPADJ_CUDA_TRY(p, launch_kernel(p->pdl, yfft_kernel, dim3(Mz * yp.ntile, js.n), dim3(128), ysmem, p->stream, js, yp));
+    auto go = [&](auto kernel) {
+      return launch_kernel(p->pdl, kernel, dim3(Mz * yp.ntile, js.n), dim3(128), ysmem, p->stream, js, yp);
+    };
+    SPADJ_CUDA_TRY(p, yp.TK == 8 ? go(yfft_kernel<8>) : yp.TK == 4 ? go(yfft_kernel<4>) : yp.TK == 2 ? go(yfft_kernel<2>)
+                                                                                                 : go(yfft_kernel<1>));
     p->toc(t, KC_YFFT, f);
     return check_launch(p, "couette yfft");
   }

@@ -43,25 +43,27 @@ struct YJobs {
   int n;
 };
 struct YParams {
-  int Kx, Ny, My, TK, ntile;
+  int Kx, Ny, My, TK, ntile;  // TK: 1, 2, 4 or 8 columns per CTA
+  int C;                      // entries of one transform buffer
   double kxs, kys;
   FFTPlan plan;
 };
 
 // CTA = (z row, tile of TK adjacent kx columns, job); the TK columns are transformed together.
+template <int TK>
 __global__ void __launch_bounds__(128) yfft_kernel(const __grid_constant__ YJobs js, const __grid_constant__ YParams P) {
   pdl_trigger();
   pdl_wait();
   const YJob& J = js.j[blockIdx.y];
   const int i = blockIdx.x / P.ntile, tile = blockIdx.x % P.ntile;
-  const int TK = P.TK, Kx = P.Kx, Ny = P.Ny, My = P.My;
+  const int Kx = P.Kx, Ny = P.Ny, My = P.My;
   const int m0 = tile * TK;
   const int tk = min(TK, Kx - m0);
-  const int a = 0, b = My * TK;
-  const FxLay lay{1, TK, My * TK, 0};
+  const int b = P.C;
+  const FxLay lay{TK, 2 * P.C + 1, 0};  // an odd stride: the threads of one entry meet different banks
   const int tid = threadIdx.x, nt = blockDim.x;
   if (J.dir == 0) {
-    const FxRes r = xf_c2c<1, 1, true>(a, b, lay, P.plan, [&](int, int c, int e) {
+    const auto r = xf_c2c<true, TK, TK>(0, b, lay, P.plan, [&](int c, int e) {
       // entry e holds ky row q (none between the positive and the negative wavenumbers)
       const int q = e < Ny / 2 ? e : e - (My - Ny);
       double2 v = make_double2(0.0, 0.0);
@@ -81,17 +83,17 @@ __global__ void __launch_bounds__(128) yfft_kernel(const __grid_constant__ YJobs
     });
     for (int idx = tid; idx < My * TK; idx += nt) {
       const int e = idx / TK, c = idx - e * TK;
-      if (c < tk) J.out[((size_t)i * My + e) * Kx + m0 + c] = cscale(r.at(0, c, e), J.scale);
+      if (c < tk) J.out[((size_t)i * My + e) * Kx + m0 + c] = cscale(r.at(c, e), J.scale);
     }
   } else {
-    const FxRes r = xf_c2c<-1, 1, true>(a, b, lay, P.plan, [&](int, int c, int e) {
+    const auto r = xf_c2c<false, TK, TK>(0, b, lay, P.plan, [&](int c, int e) {
       return c < tk ? J.in[0][((size_t)i * My + e) * Kx + m0 + c] : make_double2(0.0, 0.0);
     });
     for (int idx = tid; idx < Ny * TK; idx += nt) {
       const int q = idx / TK, c = idx - q * TK;
       if (c >= tk) continue;
       const int e = ypos(q, Ny, My);
-      J.out[((size_t)i * Ny + q) * Kx + m0 + c] = e < 0 ? make_double2(0.0, 0.0) : cscale(r.at(0, c, e), J.scale);
+      J.out[((size_t)i * Ny + q) * Kx + m0 + c] = e < 0 ? make_double2(0.0, 0.0) : cscale(r.at(c, e), J.scale);
     }
   }
 }

@@ -33,12 +33,11 @@ struct FFTPlan {
   int nrad;               // number of passes
   unsigned char rad[8];   // radix of each pass (product = n)
   const double2* sc[2];   // device scaled-twiddle records: [0] exp(-), [1] exp(+)
-  // fixed-point passes (fxfft.cuh): the radices a byte each from the low end, the passes' twiddles of
-  // both directions, the real transforms' unpacking factors, the passes' scalings, FP64 unpacking factors
-  unsigned long long radw;
-  const int4* fx[2];
-  const int4* fxr;
+  // fixed-point transforms (fxfft.cuh): the passes (nullptr: none for this length), their twiddles, the real
+  // transforms' unpacking factors, the passes' scalings, the parity of their number, and FP64 unpacking factors
+  const int4 *fxp, *fxt, *fxr;
   const int* fxs;
+  int fxodd;
   const double2* wm;
 };
 

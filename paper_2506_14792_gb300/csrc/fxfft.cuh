@@ -17,11 +17,11 @@
 // shift; sg in 0..3 is a free scaling by 2^-sg (it only moves the split).
 //
 // Overflow.  A product's scaled operand has a complex modulus <= 2^60 (then the sums of four products stay
-// below 2^63), so a pass of radix R <= 4 leaves moduli <= 2^62.  A pass multiplies the bound of the
-// moduli by at most R, and no value ever exceeds the sum of the moduli of the pass-0 inputs times
-// the scalings so far.  Each pass scales by the smallest 2^-sg that brings the smaller of the two bounds
-// to 2^60: a peaked input (one mode, a smooth spectrum) is hardly scaled at all, a flat one by 2^-2 per
-// radix-4 pass.
+// below 2^63), so a pass of radix R <= 4 leaves moduli <= 2^62, and the differences that radix 3 multiplies by
+// sqrt(3)/2 stay below 2^62 (split at bit 31 there).  A pass multiplies the bound of the moduli by at most R,
+// and no value ever exceeds the sum of the moduli of the pass-0 inputs times the scalings so far.  Each pass
+// scales by the smallest 2^-sg that brings the smaller of the two bounds to 2^60: a peaked input (one mode, a
+// smooth spectrum) is hardly scaled at all, a flat one by 2^-2 per radix-4 pass.
 //
 // Accuracy.  The rounding is about 0.7 units of 2^-59 of the largest value in each pass, against 2^-53 of each
 // value in FP64, and the results are rounded to FP64 once: the relative 2-norm error of complex transforms
@@ -101,48 +101,36 @@ __host__ __device__ __forceinline__ fx2 fx_cmul(fx2 v, int4 w, int sg) {
   r.y = fx_mad(a.h, w.z, fx_mad(b.h, w.x, fx_hi(ci)));
   return r;
 }
-// v c for a real constant c = 2^-29 ch + 2^-61 cl
+// v c for a real constant c = 2^-31 ch + 2^-63 cl, |v| < 2^62
 __host__ __device__ __forceinline__ long long fx_rmul(long long v, int ch, int cl) {
-  const FxLimb a = fx_split(v, 0);
+  const FxLimb a = fx_split(v, 2);  // v = 2^31 h + l / 2
   return fx_mad(a.h, ch, fx_hi(fx_mad(a.h, cl, fx_mad(a.l, ch, kFxRound))));
 }
 __host__ __device__ __forceinline__ fx2 fx_add(fx2 a, fx2 b) { return fx2{a.x + b.x, a.y + b.y}; }
 __host__ __device__ __forceinline__ fx2 fx_sub(fx2 a, fx2 b) { return fx2{a.x - b.x, a.y - b.y}; }
 __host__ __device__ __forceinline__ fx2 fx_shr(fx2 a, int sg) { return fx2{a.x >> sg, a.y >> sg}; }
-template <int SIGN>
-__host__ __device__ __forceinline__ fx2 fx_rot(fx2 a) {  // SIGN i a
-  return SIGN > 0 ? fx2{-a.y, a.x} : fx2{a.y, -a.x};
-}
+__host__ __device__ __forceinline__ fx2 fx_swap(fx2 a) { return fx2{a.y, a.x}; }
 
-// Butterflies in place, scaled by 2^-sg; w: the pass's twiddles of this k (R - 1 of them), nullptr for the
-// first pass.
-template <int SIGN>
+// Forward (exp(-)) butterflies in place, outputs in order.  Inverse transforms run the forward passes on swapped
+// components: IDFT(x) = swap(DFT(swap(x))).
 __host__ __device__ __forceinline__ void fx_out4(fx2& v0, fx2& v1, fx2& v2, fx2& v3) {
-  const fx2 t0 = fx_add(v0, v2), t1 = fx_sub(v0, v2), t2 = fx_add(v1, v3);
-  const fx2 t3 = fx_sub(v1, v3);
+  const fx2 t0 = fx_add(v0, v2), t1 = fx_sub(v0, v2), t2 = fx_add(v1, v3), t3 = fx_sub(v1, v3);
   v0 = fx_add(t0, t2);
   v2 = fx_sub(t0, t2);
-  if (SIGN > 0) {  // t1 +- i t3
-    v1 = fx2{t1.x - t3.y, t1.y + t3.x};
-    v3 = fx2{t1.x + t3.y, t1.y - t3.x};
-  } else {
-    v1 = fx2{t1.x + t3.y, t1.y - t3.x};
-    v3 = fx2{t1.x - t3.y, t1.y + t3.x};
-  }
+  v1 = fx2{t1.x + t3.y, t1.y - t3.x};  // t1 -+ i t3
+  v3 = fx2{t1.x - t3.y, t1.y + t3.x};
 }
-constexpr int kFxS3h = 464943848, kFxS3l = 1481419380;  // sqrt(3)/2 = 2^-29 h + 2^-61 l
-template <int SIGN>
+constexpr int kFxS3h = 1859775393, kFxS3l = 1630710223;  // sqrt(3)/2 = 2^-31 h + 2^-63 l
 __host__ __device__ __forceinline__ void fx_out3(fx2& v0, fx2& v1, fx2& v2) {
   const fx2 t = fx_add(v1, v2), d = fx_sub(v1, v2);
   const fx2 m = fx_sub(v0, fx_shr(t, 1));
-  const fx2 r = fx_rot<SIGN>(fx2{fx_rmul(d.x, kFxS3h, kFxS3l), fx_rmul(d.y, kFxS3h, kFxS3l)});
+  const fx2 r = fx2{fx_rmul(d.y, kFxS3h, kFxS3l), -fx_rmul(d.x, kFxS3h, kFxS3l)};  // -i (sqrt3/2) d
   v0 = fx_add(v0, t);
   v1 = fx_add(m, r);
   v2 = fx_sub(m, r);
 }
-
-// Fixed-point value of the double x: x = v 2^(emax + 1 - 1023 - B) to the last unit (toward zero), |v| < 2^B
-// for biased exponents <= emax.  emax >= 128, so that whatever has a zero exponent field vanishes.
+// Fixed-point value of the double x: x = v 2^(emax + 1 - 1023 - B) to the last unit (toward zero; to the nearest for
+// the packed real spectra, whose many small entries would add up otherwise), |v| <= 2^B for biased exponents <= emax.  emax >= 128, so that whatever has a zero exponent field vanishes.
 template <int B>
 __host__ __device__ __forceinline__ long long fx_from_double(double x, int emax) {
 #ifdef __CUDA_ARCH__
@@ -153,13 +141,15 @@ __host__ __device__ __forceinline__ long long fx_from_double(double x, int emax)
   const unsigned hi = (unsigned)(bits >> 32), lo = (unsigned)bits;
 #endif
   const int d = emax - (int)((hi >> 20) & 0x7ff);
-  const unsigned long long m = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32 | lo) << (B - 53);
+  constexpr int kUp = B - 53 + (B == kFxBReal ? 1 : 0);
+  const unsigned long long m = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32 | lo) << kUp;
   unsigned long long v;
 #ifdef __CUDA_ARCH__
   asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"(d));  // shifts above 63 give 0
 #else
   v = d > 63 ? 0 : m >> d;
 #endif
+  if (B == kFxBReal) v = (v + 1) >> 1;
   const long long s = (int)hi >> 31;
   return ((long long)v ^ s) - s;
 }
@@ -207,29 +197,37 @@ __host__ __device__ __forceinline__ void fx_pack(fx2 x, fx2 y, int4 w, fx2& z0, 
   z0 = fx2{x.x + y.x + t.x, x.y - y.y + t.y};
   z1 = fx2{x.x + y.x - t.x, y.y - x.y + t.y};
 }
-// A quarter of the spectrum entry ((u + conj(v)) - i w (u - conj(v))) / 2 of a real field from the entries u = Z_k, v = Z_{n-k} of
-// its packed transform.
-__host__ __device__ __forceinline__ fx2 fx_unpack(fx2 u, fx2 v, int4 w) {
-  const fx2 t = fx_cmul(fx2{u.y + v.y, v.x - u.x}, w, 3);
-  return fx2{((u.x + v.x) >> 3) + t.x, ((u.y - v.y) >> 3) + t.y};
+// Twice the spectrum entry ((u + conj(v)) - i w (u - conj(v))) / 2 of a real field, scaled by 2^-us, from the
+// entries u = Z_k, v = Z_{n-k} of its packed transform.
+__host__ __device__ __forceinline__ fx2 fx_unpack(fx2 u, fx2 v, int4 w, int us) {
+  const fx2 t = fx_cmul(fx2{u.y + v.y, v.x - u.x}, w, us);
+  return fx2{((u.x + v.x) >> us) + t.x, ((u.y - v.y) >> us) + t.y};
 }
 __host__ __device__ __forceinline__ unsigned fx_l1(fx2 v) {  // >= (|x| + |y|) / 2^42
   const int x = (int)(v.x >> 32), y = (int)(v.y >> 32);
   return ((unsigned)(x < 0 ? -x : x) >> 10) + ((unsigned)(y < 0 ? -y : y) >> 10) + 2u;
 }
 
-// The scalings sg of the passes, two bits each from the low end, and their sum in bits 24.. : b2 = twice the
-// log2 of the bound on the pass-0 moduli, l2 = twice that of the bound on the sum of the moduli.
-__host__ __device__ inline int fx_schedule(unsigned long long radw, int b2, int l2) {
-  int bits = 0, tot = 0;
+// The scalings sg of the passes, two bits each from the low end, and their sum in bits 24.., for inputs whose sum of
+// moduli is below 2^l.  The bounds are followed in quarters of log2.  The values of a forward real transform
+// stay <= 2^61.5, and bits 16 and 17 hold the scaling of its fx_unpack.
+enum { kFxComplex = 0, kFxInvReal = 1, kFxFwdReal = 2 };
+inline int fx_schedule(unsigned long long radw, int kind, int l) {
+  // bound of the pass-0 moduli: sqrt(2) 2^B, and 4 sqrt(2) 2^B for the packed spectra
+  int bits = 0, tot = 0, b = kind == kFxInvReal ? 4 * kFxBReal + 10 : 4 * kFxB + 2;
+  l *= 4;
   for (int i = 0; radw; ++i, radw >>= 8) {
-    const int sg = i > 0 && b2 > 120 ? (b2 - 119) / 2 : 0;
+    const int R = (int)(radw & 0xff), grow = R == 4 ? 8 : R == 3 ? 7 : 4;
+    int lim = 240;  // of a scaled operand: the sums of four products fit the words
+    if (kind == kFxFwdReal && lim > 246 - grow) lim = 246 - grow;
+    const int sg = i > 0 && b > lim ? (b - lim + 3) / 4 : 0;
     bits |= sg << (2 * i);
     tot += sg;
-    l2 -= 2 * sg;
-    b2 += ((radw & 0xff) == 2 ? 2 : 4) - 2 * sg;
-    if (b2 > l2) b2 = l2;
+    l -= 4 * sg;
+    b += grow - 4 * sg;
+    if (b > l) b = l;
   }
+  if (kind == kFxFwdReal && b + 4 > 240) bits |= ((b + 4 - 240 + 3) / 4) << 16;
   return bits | tot << 24;
 }
 
@@ -268,74 +266,110 @@ inline std::vector<int4> fx_roots(int n) {
   }
   return r;
 }
-// entries of one direction's twiddles: R - 1 per (pass with Ns > 1, k)
-inline int fx_twiddle_entries(const FFTPlan& p) {
-  int e = 0, Ns = 1;
-  for (int i = 0; i < p.nrad; ++i) {
-    if (Ns > 1) e += Ns * (p.rad[i] - 1);
-    Ns *= p.rad[i];
-  }
-  return e;
+// Radices of the fixed-point passes, a byte each from the low end: the 3s first (the first pass then grows the
+// moduli least, which the packed real spectra need), then 4s, then a 2.  Radix 8 in place of the 4s needs fewer passes
+// but leaves half the lanes idle at these lengths (24 butterflies at n = 192): 16384 Burgers members of N = 256 take
+// 18.9 ms with it and 17.8 ms without.  0: no such plan (n without a factor 3, or above kFxMaxN).
+inline unsigned long long fx_radices(int n) {
+  if (n < 3 || n > kFxMaxN) return 0;
+  unsigned long long w = 0;
+  int m = n, i = 0;
+  auto push = [&](int r) {
+    w |= (unsigned long long)r << (8 * i++);
+    m /= r;
+  };
+  while (m % 3 == 0 && i < 8) push(3);
+  if (i == 0) return 0;
+  while (m % 4 == 0 && i < 8) push(4);
+  if (m % 2 == 0 && i < 8) push(2);
+  return m == 1 ? w : 0;
 }
-// exp(-) twiddles, exp(+) twiddles in pass order, then exp(-pi i k / n), k < n (the real transforms'
-// unpacking), then the scalings of the passes by the leading zeros of the sum of the moduli (fx_schedule; 32
-// words for complex, 32 for packed real inputs), as 16-byte entries
-inline std::vector<double2> fx_table(const FFTPlan& p) {
-  const std::vector<int4> root = fx_roots(p.n);
-  const int period = 2 * p.n;
-  std::vector<int4> t;
-  for (int dir = 0; dir < 2; ++dir) {
-    int Ns = 1;
-    for (int i = 0; i < p.nrad; ++i) {
-      const int R = p.rad[i], step = period / (R * Ns);
-      if (Ns > 1)
-        for (int k = 0; k < Ns; ++k)
-          for (int m = 1; m < R; ++m) t.push_back(root[dir ? m * k * step : (period - m * k * step) % period]);
-      Ns *= R;
-    }
+// One pass: butterfly j = q Ns + k of nbf reads entries j + r nbf of its input and writes q Ns R + k + r Ns;
+// mNs, mBf: 2^32 / Ns and 2^32 / nbf rounded up (division by multiplication); tw: offset of its twiddles.
+struct alignas(16) FxPass {
+  int R, Ns, nbf, tw;
+  unsigned mNs, mBf;
+  int more, pad;
+};
+inline std::vector<FxPass> fx_pass_list(int n) {
+  std::vector<FxPass> v;
+  int Ns = 1, tw = 0;
+  for (unsigned long long w = fx_radices(n); w; w >>= 8) {
+    FxPass p{};
+    p.R = (int)(w & 0xff);
+    p.Ns = Ns;
+    p.nbf = n / p.R;
+    p.more = (w >> 8) != 0;
+    p.mNs = Ns > 1 ? (unsigned)(((1ull << 32) + Ns - 1) / Ns) : 0u;
+    p.mBf = p.nbf > 1 ? (unsigned)(((1ull << 32) + p.nbf - 1) / p.nbf) : 0u;
+    p.tw = tw;
+    if (Ns > 1) tw += Ns * (p.R - 1);
+    Ns *= p.R;
+    v.push_back(p);
   }
-  for (int k = 0; k < p.n; ++k) t.push_back(root[(period - k) % period]);
-  for (int b2 : {2 * kFxB + 1, 2 * kFxBReal + 5})
-    for (int z = 0; z < 32; z += 4) {
-      int s[4];
-      for (int q = 0; q < 4; ++q) s[q] = fx_schedule(p.radw, b2, 2 * (42 + 32 - (z + q)));
-      t.push_back(make_int4(s[0], s[1], s[2], s[3]));
-    }
+  return v;
+}
+// Tables of a plan, as 16-byte entries: the passes, exp(-) twiddles in pass order (R - 1 per k), exp(-pi i k / n),
+// k < n (the real transforms' unpacking), the scalings of the passes by the leading zeros of the sum of
+// the moduli (fx_schedule; 32 words for each kind of transform), and the FP64 records where needed.
+// real: the plan is that of packed real transforms; both: the FP64 records in any case.
+inline bool fx_has_plan(int n, bool real) { return !(real && n > kFxMaxReal) && fx_radices(n) != 0; }
+inline std::vector<double2> fft_tables(const FFTPlan& p, bool real, bool both = false) {
+  std::vector<int4> t;
+  if (fx_has_plan(p.n, real)) {
+    const unsigned long long radw = fx_radices(p.n);
+    const std::vector<FxPass> ps = fx_pass_list(p.n);
+    t.resize(ps.size() * (sizeof(FxPass) / sizeof(int4)));
+    std::memcpy(t.data(), ps.data(), sizeof(FxPass) * ps.size());
+    const std::vector<int4> root = fx_roots(p.n);
+    const int period = 2 * p.n;
+    for (const FxPass& q : ps)
+      if (q.Ns > 1)
+        for (int k = 0; k < q.Ns; ++k)
+          for (int m = 1; m < q.R; ++m) t.push_back(root[(period - m * k * (period / (q.R * q.Ns)) % period) % period]);
+    for (int k = 0; k < p.n; ++k) t.push_back(root[(period - k) % period]);
+    for (int kind : {kFxComplex, kFxInvReal, kFxFwdReal})
+      for (int z = 0; z < 32; z += 4) {
+        int s[4];
+        for (int q = 0; q < 4; ++q) s[q] = fx_schedule(radw, kind, 42 + 32 - (z + q));
+        t.push_back(make_int4(s[0], s[1], s[2], s[3]));
+      }
+  }
   std::vector<double2> out(t.size());
-  std::memcpy(out.data(), t.data(), sizeof(int4) * t.size());
+  if (!t.empty()) std::memcpy(out.data(), t.data(), sizeof(int4) * t.size());
+  if (both || !fx_has_plan(p.n, real)) {
+    const std::vector<double2> s = scaled_twiddle_table(p);
+    out.insert(out.end(), s.begin(), s.end());
+  }
   return out;
 }
-// the FP64 records are built only for lengths that use them
-inline bool fx_needs_fp64(const FFTPlan& p) { return p.n > kFxMaxReal; }
-// All tables of a plan (the fixed-point ones, then the FP64 records where needed), and the plan's pointers into the device
-// copy; wm: device table of exp(-2 pi i m / 2n), m < 2n.
-inline std::vector<double2> fft_tables(FFTPlan& p) {
-  p.radw = 0;
-  for (int i = 0; i < p.nrad; ++i) p.radw |= (unsigned long long)p.rad[i] << (8 * i);
-  std::vector<double2> t = fx_table(p);
-  if (fx_needs_fp64(p)) {
-    const std::vector<double2> s = scaled_twiddle_table(p);
-    t.insert(t.end(), s.begin(), s.end());
+// The plan's pointers into the device copy of its tables; wm: device table of exp(-2 pi i m / 2n), m < 2n (the FP64
+// real transforms').
+inline void fft_bind(FFTPlan& p, bool real, const double2* dev, const double2* wm, bool both = false) {
+  p.fxp = nullptr;
+  if (fx_has_plan(p.n, real)) {
+    const std::vector<FxPass> ps = fx_pass_list(p.n);
+    int tw = 0;
+    for (const FxPass& q : ps) tw += q.Ns > 1 ? q.Ns * (q.R - 1) : 0;
+    const int np = (int)(ps.size() * (sizeof(FxPass) / sizeof(int4)));
+    const int4* t = reinterpret_cast<const int4*>(dev);
+    p.fxp = t;
+    p.fxt = t + np;
+    p.fxr = p.fxt + tw;
+    p.fxs = reinterpret_cast<const int*>(p.fxr + p.n);
+    p.fxodd = (int)ps.size() & 1;
+    if (both) bind_scaled_twiddles(p, dev + np + tw + p.n + 3 * 32 / 4);
+  } else {
+    bind_scaled_twiddles(p, dev);
   }
-  return t;
-}
-inline void fft_bind(FFTPlan& p, const double2* dev, const double2* wm) {
-  const int e = fx_twiddle_entries(p);
-  const int4* t = reinterpret_cast<const int4*>(dev);
-  p.fx[0] = t;
-  p.fx[1] = t + e;
-  p.fxr = t + 2 * e;
-  p.fxs = reinterpret_cast<const int*>(p.fxr + p.n);
-  if (fx_needs_fp64(p)) bind_scaled_twiddles(p, dev + 2 * e + p.n + 16);
   p.wm = wm;
 }
 
 // ---- device: the transform of the sequences of one CTA ------------------------------------------------
 //
-// Buffers are offsets (in 16-byte entries) into the CTA's dynamic shared memory, so that every access
-// is a shared-memory access with a 32-bit address.  Sequence
-// s = set * nb + c holds element e at [set * stride + e * nb + c] of its buffers a and b: ns sets of nb
-// interleaved sequences.  All threads of the CTA (a multiple of 32, <= 256) call.
+// Buffers are offsets (in 16-byte entries) into the CTA's dynamic shared memory.  Sequence s of a call holds its
+// entries from a + s * stride (and the other buffer from b + s * stride); every buffer has n entries.  All
+// threads of the CTA (a multiple of 32, <= 256) call.
 
 __device__ __forceinline__ double2* fx_mem64() {
   extern __shared__ double2 fx_dyn[];
@@ -385,42 +419,35 @@ __device__ __forceinline__ void sts32(unsigned* p, unsigned v) {
 }
 
 struct FxLay {
-  int ns, nb, stride;  // sets, interleaved sequences per set, entries between sets
-  int s0;              // first of the call's ns * nb slots for the sequences' scales (a later call on other
-                       // slots leaves the earlier results readable)
+  int ns, stride;  // sequences of the call, entries between their buffers
+  int s0;          // first of the ns slots for their scales (a later call on other slots leaves the earlier
+                   // results readable)
 };
 
 __device__ __forceinline__ unsigned fx_absmax(unsigned m, double2 v) {
   return max(m, max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu));
 }
-// Reductions over a warp by shuffles
+// Reductions by shuffles over the lanes that agree modulo W (W = 1: the whole warp)
+template <int W = 1>
 __device__ __forceinline__ unsigned fx_warp_max(unsigned v) {
 #pragma unroll
-  for (int d = 16; d > 0; d >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, d));
+  for (int d = 16; d >= W; d >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, d));
   return v;
 }
+template <int W = 1>
 __device__ __forceinline__ unsigned fx_warp_sum(unsigned v) {
 #pragma unroll
-  for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+  for (int d = 16; d >= W; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
   return v;
 }
-// Before fx_put_max with nb > 1: the warp's slots of ns * nb sequences to zero
-__device__ __forceinline__ void fx_clear(unsigned (&slots)[kFxWarpsMax][kFxSeqMax], int s0, int nseq) {
-  const int l = threadIdx.x & 31;
-  if (l < nseq) sts32(&slots[threadIdx.x >> 5][s0 + l], 0u);
-  __syncwarp();
+// The warp's largest high word of the sequence of slot s, from each thread's m (all threads call)
+__device__ __forceinline__ void fx_put_max(int s, unsigned m) {
+  m = fx_warp_max(m);
+  if ((threadIdx.x & 31) == 0) sts32(&fx_shared().mx[threadIdx.x >> 5][s], m);
 }
-// The warp's largest high word of a set's sequences from each thread's m; all threads call, c = the thread's
-// sequence in the set or -1 when it saw none (nb == 1: one sequence, no clearing needed)
-__device__ __forceinline__ void fx_put_max(int set, int nb, int c, unsigned m, int s0 = 0) {
-  FxShared& S = fx_shared();
-  const int w = threadIdx.x >> 5;
-  if (nb == 1) {
-    m = fx_warp_max(m);
-    if ((threadIdx.x & 31) == 0) sts32(&S.mx[w][s0 + set], m);
-  } else if (c >= 0) {
-    atomicMax(&S.mx[w][s0 + set * nb + c], m);
-  }
+__device__ __forceinline__ void fx_put_l1(int s, unsigned v) {
+  v = fx_warp_sum(v);
+  if ((threadIdx.x & 31) == 0) sts32(&fx_shared().l1[threadIdx.x >> 5][s], v);
 }
 __device__ __forceinline__ unsigned fx_get_max(int s) {
   unsigned m = 0u;
@@ -453,7 +480,7 @@ template <int B>
 __device__ __forceinline__ void fx_make_meta(FxLay lay, const int* __restrict__ sched) {
   FxShared& S = fx_shared();
   const int lane = lay.s0 + (threadIdx.x & 31), w = threadIdx.x >> 5;
-  if (lane < lay.s0 + lay.ns * lay.nb) {
+  if (lane < lay.s0 + lay.ns) {
     unsigned mx = 0u, l1 = 0u;
     for (int v = 0; v < (int)(blockDim.x >> 5); ++v) {
       mx = max(mx, lds32(&S.mx[v][lane]));
@@ -469,111 +496,84 @@ __device__ __forceinline__ void fx_make_meta(FxLay lay, const int* __restrict__ 
 __device__ __forceinline__ int fx_se(int s) { return (int)lds32(&fx_shared().se[threadIdx.x >> 5][s]); }
 __device__ __forceinline__ int fx_sch(int s) { return (int)lds32(&fx_shared().sch[threadIdx.x >> 5][s]); }
 
-// Bank-conflict-free order of the entries written by the passes with Ns <= 4 (consecutive threads store
-// 64 bytes apart there): the low three bits are exchanged by XOR with higher ones, inside groups of 8.
-__device__ __forceinline__ int fx_swz(int e) {
-  const int t = e >> 3;
-  return e ^ ((t & 3) | ((t & 2) << 1));
-}
-
-// j mod Ns (Ns a power of two, or via the multiplier inv = ceil(2^20 / Ns); j Ns < 2^20)
-__device__ __forceinline__ int fx_mod(int j, int Ns, unsigned inv) {
-  if ((Ns & (Ns - 1)) == 0) return j & (Ns - 1);
-  return j - (int)(((unsigned)j * inv) >> 20) * Ns;
-}
-
-// The butterfly passes of NS sets over the entries in a; the results are in a when the number of passes is even,
-// else in b.  On return they are visible to all threads.
-template <int SIGN, int NS>
-__device__ __forceinline__ void fx_passes(int a, int b, FxLay lay, int n, unsigned long long radw,
-                                          const int4* __restrict__ tw) {
+// The forward passes over the entries in a; the results are in a when the number of passes is even, else in b.  On
+// return they are visible to all threads.
+__device__ __forceinline__ void fx_passes(int a, int b, FxLay lay, const int4* __restrict__ passes,
+                                          const int4* __restrict__ twiddles) {
   const int tid = threadIdx.x, nt = blockDim.x;
-  const int nb = lay.nb;
-  const bool swz = nb == 1 && (n & 7) == 0;
-  int Ns = 1;
-  bool rs = false;
+  int4 d0 = ldtab(passes), d1 = ldtab(passes + 1);
+  for (int pass = 0;; ++pass) {
+    const int R = d0.x, Ns = d0.y, nbf = d0.z, more = d1.z;
+    const int4* tw = twiddles + d0.w;
+    const unsigned mNs = (unsigned)d1.x, mBf = (unsigned)d1.y;
+    if (more) {  // the next pass's parameters, before they are needed
+      passes += 2;
+      d0 = ldtab(passes);
+      d1 = ldtab(passes + 1);
+    }
+    const int total = lay.ns * nbf;
 #pragma unroll 1
-  for (int pass = 0; radw; ++pass) {
-    const int R = (int)(radw & 0xff), nbf = n / R, per = nbf * nb;
-    radw >>= 8;
-    const unsigned inv = (unsigned)(((1 << 20) + Ns - 1) / Ns);
-    const bool ws = swz && radw && Ns <= 4;
-#pragma unroll 1
-    for (int i = tid; i < NS * per; i += nt) {
-      int set = 0, j = i, c = 0;
-      if (NS > 1) {
-#pragma unroll
-        for (int s = 1; s < NS; ++s)
-          if (j >= per) {
-            j -= per;
-            ++set;
-          }
+    for (int i = tid; i < total; i += nt) {
+      int s = 0, j = i;
+      if (lay.ns > 1) {
+        s = mBf ? (int)__umulhi((unsigned)i, mBf) : i;
+        j = i - s * nbf;
       }
-      if (nb > 1) {
-        const int q = (nb & (nb - 1)) == 0 ? j >> (__ffs(nb) - 1) : j / nb;
-        c = j - q * nb;
-        j = q;
-      }
-      const int sg = (fx_sch(lay.s0 + set * nb + c) >> (2 * pass)) & 3;
-      const int as = a + set * lay.stride + c, bs = b + set * lay.stride + c;
-      const int k = fx_mod(j, Ns, inv);
-      const int base = (j - k) * R + k;
-      auto ld = [&](int e) { return fx_get(as + (rs ? fx_swz(e) : e) * nb); };
-      auto st = [&](int e, fx2 v) { fx_put(bs + (ws ? fx_swz(e) : e) * nb, v); };
+      const int q = mNs ? (int)__umulhi((unsigned)j, mNs) : j;
+      const int k = j - q * Ns;
+      const int sg = (fx_sch(lay.s0 + s) >> (2 * pass)) & 3;
+      const int rd = a + s * lay.stride + j, wr = b + s * lay.stride + q * Ns * R + k;
       if (R == 4) {
-        fx2 v0 = ld(j), v1 = ld(j + nbf), v2 = ld(j + 2 * nbf), v3 = ld(j + 3 * nbf);
-        if (pass > 0) {
-          const int4* w = tw + 3 * k;
-          v0 = fx_shr(v0, sg);
-          v1 = fx_cmul(v1, ldtab(w), sg);
-          v2 = fx_cmul(v2, ldtab(w + 1), sg);
-          v3 = fx_cmul(v3, ldtab(w + 2), sg);
-        }
-        fx_out4<SIGN>(v0, v1, v2, v3);
-        st(base, v0);
-        st(base + Ns, v1);
-        st(base + 2 * Ns, v2);
-        st(base + 3 * Ns, v3);
+        fx2 v0 = fx_get(rd), v1 = fx_get(rd + nbf), v2 = fx_get(rd + 2 * nbf), v3 = fx_get(rd + 3 * nbf);
+        const int4* w = tw + 3 * k;
+        v0 = fx_shr(v0, sg);
+        v1 = fx_cmul(v1, ldtab(w), sg);
+        v2 = fx_cmul(v2, ldtab(w + 1), sg);
+        v3 = fx_cmul(v3, ldtab(w + 2), sg);
+        fx_out4(v0, v1, v2, v3);
+        fx_put(wr, v0);
+        fx_put(wr + Ns, v1);
+        fx_put(wr + 2 * Ns, v2);
+        fx_put(wr + 3 * Ns, v3);
       } else if (R == 3) {
-        fx2 v0 = ld(j), v1 = ld(j + nbf), v2 = ld(j + 2 * nbf);
-        if (pass > 0) {
+        fx2 v0 = fx_get(rd), v1 = fx_get(rd + nbf), v2 = fx_get(rd + 2 * nbf);
+        if (pass > 0) {  // the first pass (always of radix 3) has neither twiddles nor a scaling
           const int4* w = tw + 2 * k;
           v0 = fx_shr(v0, sg);
           v1 = fx_cmul(v1, ldtab(w), sg);
           v2 = fx_cmul(v2, ldtab(w + 1), sg);
         }
-        fx_out3<SIGN>(v0, v1, v2);
-        st(base, v0);
-        st(base + Ns, v1);
-        st(base + 2 * Ns, v2);
+        fx_out3(v0, v1, v2);
+        fx_put(wr, v0);
+        fx_put(wr + Ns, v1);
+        fx_put(wr + 2 * Ns, v2);
       } else {
-        fx2 v0 = ld(j), v1 = ld(j + nbf);
-        if (pass > 0) {
-          v0 = fx_shr(v0, sg);
-          v1 = fx_cmul(v1, ldtab(tw + k), sg);
-        }
-        st(base, fx_add(v0, v1));
-        st(base + Ns, fx_sub(v0, v1));
+        fx2 v0 = fx_get(rd), v1 = fx_get(rd + nbf);
+        v0 = fx_shr(v0, sg);
+        v1 = fx_cmul(v1, ldtab(tw + k), sg);
+        fx_put(wr, fx_add(v0, v1));
+        fx_put(wr + Ns, fx_sub(v0, v1));
       }
     }
     __syncthreads();
+    if (!more) return;
     const int t = a;
     a = b;
     b = t;
-    if (Ns > 1) tw += Ns * (R - 1);
-    Ns *= R;
-    rs = ws;
   }
 }
 
 // ---- device: transforms ----------------------------------------------------------------------------------
 //
-// xf_c2c, xf_c2r and xf_r2c stage their input through load(set, c, e) (called once per entry; CF: consecutive
-// threads take consecutive sequences c of an entry, otherwise consecutive entries), run the passes and
-// return the results where FxRes reads them; buffers a and b hold lay.stride entries per set, and what load reads
-// must not lie in them.  The CTA synchronises before the buffers are used again.  Lengths above kFxMaxN run
-// the FP64 butterflies (ANY = false: the caller's lengths never do).
+// xf_c2c, xf_c2r and xf_r2c stage their input through load(s, e) (called once per entry of each of the NS
+// sequences), run the passes and return the results where FxRes reads them; what load reads must not lie in the
+// buffers.  The CTA synchronises before the buffers are used again.  Lengths without a fixed-point plan run the
+// FP64 butterflies; PATH kFxOnly: the caller's lengths never do, kFp64: all do.  W > 1 (a power of two dividing 32): NS = W
+// sequences whose entries consecutive threads take across the sequences (entry i / W of sequence i % W).
 
+enum { kFxOnly = 0, kFxAny = 1, kFp64 = 2 };
+
+template <bool INV>
 struct FxRes {
   int z;  // buffer that holds the results
   FxLay lay;
@@ -581,210 +581,167 @@ struct FxRes {
   const int4* fxr;
   const double2* wm;
   bool fixed;  // constant true where the FP64 path is not compiled in
-  __device__ __forceinline__ double2 raw64(int set, int c, int e) const {
-    return fx_get64(z + set * lay.stride + e * lay.nb + c);
-  }
+  __device__ __forceinline__ double2 raw64(int s, int e) const { return fx_get64(z + s * lay.stride + e); }
   // entry e of a complex transform, or grid pair (g_2e, g_2e+1) of an inverse real one
-  __device__ __forceinline__ double2 at(int set, int c, int e) const {
-    if (!fixed) return raw64(set, c, e);
-    const fx2 v = fx_get(z + set * lay.stride + e * lay.nb + c);
-    const int se = fx_se(lay.s0 + set * lay.nb + c);
+  __device__ __forceinline__ double2 at(int s, int e) const {
+    if (!fixed) return raw64(s, e);
+    fx2 v = fx_get(z + s * lay.stride + e);
+    if (INV) v = fx_swap(v);
+    const int se = fx_se(lay.s0 + s);
     return make_double2(fx_to_double(v.x, se), fx_to_double(v.y, se));
   }
   // spectrum entry X_k = sum_j g_j exp(-2 pi i j k / 2n) of a forward real transform
-  __device__ __forceinline__ double2 coef(int set, int c, int k) const {
+  __device__ __forceinline__ double2 coef(int s, int k) const {
     const int kc = k == 0 ? 0 : n - k;
-    if (!fixed) return r2c_combine(raw64(set, c, k), cconj(raw64(set, c, kc)), __ldg(&wm[k]));
-    const int q = z + set * lay.stride + c;
-    const fx2 u = fx_get(q + k * lay.nb), v = fx_get(q + kc * lay.nb);
-    const int se = fx_se(lay.s0 + set * lay.nb + c);
-    const fx2 r = fx_unpack(u, v, ldtab(fxr + k));
-    return make_double2(fx_to_double(r.x, se + 2), fx_to_double(r.y, se + 2));
+    if (!fixed) return r2c_combine(raw64(s, k), cconj(raw64(s, kc)), __ldg(&wm[k]));
+    const int q = z + s * lay.stride;
+    const int us = (fx_sch(lay.s0 + s) >> 16) & 3;
+    const fx2 r = fx_unpack(fx_get(q + k), fx_get(q + kc), ldtab(fxr + k), us);
+    const int se = fx_se(lay.s0 + s) + us - 1;
+    return make_double2(fx_to_double(r.x, se), fx_to_double(r.y, se));
   }
 };
 
-// (entry, sequence in the set) of item i among cnt entries of nb sequences
-template <bool CF>
-__device__ __forceinline__ void fx_item(int i, int cnt, int nb, int& e, int& c) {
-  c = 0;
-  e = i;
-  if (nb == 1) return;
-  if (CF) {
-    e = (nb & (nb - 1)) == 0 ? i >> (__ffs(nb) - 1) : i / nb;
-    c = i - e * nb;
-  } else {
-    while (e >= cnt) {
-      e -= cnt;
-      ++c;
-    }
-  }
-}
-
 // FP64 values of cnt entries of every sequence into dst, and the sequences' largest high words
-template <int NS, bool CF, class Load>
+template <int NS, int W, class Load>
 __device__ __forceinline__ void fx_stage(int dst, FxLay lay, int cnt, Load load) {
-  const int nb = lay.nb;
+  if (W > 1) {
+    const int s = threadIdx.x & (W - 1);
+    unsigned m = 0u;
+    for (int i = threadIdx.x; i < cnt * W; i += blockDim.x) {
+      const double2 v = load(s, i / W);
+      fx_put64(dst + s * lay.stride + i / W, v);
+      m = fx_absmax(m, v);
+    }
+    m = fx_warp_max<W>(m);
+    if ((threadIdx.x & 31) < W) sts32(&fx_shared().mx[threadIdx.x >> 5][lay.s0 + s], m);
+    return;
+  }
   unsigned m[NS];
-  int cp = -1;
-  if (nb > 1) fx_clear(fx_shared().mx, lay.s0, NS * nb);
 #pragma unroll
   for (int s = 0; s < NS; ++s) m[s] = 0u;
-  for (int i = threadIdx.x; i < cnt * nb; i += blockDim.x) {
-    int e, c;
-    fx_item<CF>(i, cnt, nb, e, c);
-    if (c != cp && cp >= 0) {
-#pragma unroll
-      for (int s = 0; s < NS; ++s) {
-        fx_put_max(s, nb, cp, m[s], lay.s0);
-        m[s] = 0u;
-      }
-    }
-    cp = c;
+  for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
     double2 v[NS];
 #pragma unroll
-    for (int s = 0; s < NS; ++s) v[s] = load(s, c, e);
+    for (int s = 0; s < NS; ++s) v[s] = load(s, i);
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
-      fx_put64(dst + s * lay.stride + e * nb + c, v[s]);
+      fx_put64(dst + s * lay.stride + i, v[s]);
       m[s] = fx_absmax(m[s], v[s]);
     }
   }
 #pragma unroll
-  for (int s = 0; s < NS; ++s) fx_put_max(s, nb, cp, m[s], lay.s0);
+  for (int s = 0; s < NS; ++s) fx_put_max(lay.s0 + s, m[s]);
 }
 
-__device__ __forceinline__ void fx_put_l1(int s0, int set, int nb, int c, unsigned s) {
-  FxShared& S = fx_shared();
-  const int w = threadIdx.x >> 5;
-  if (nb == 1) {
-    s = fx_warp_sum(s);
-    if ((threadIdx.x & 31) == 0) sts32(&S.l1[w][s0 + set], s);
-  } else if (c >= 0) {
-    atomicAdd(&S.l1[w][s0 + set * nb + c], s);
-  }
+template <bool INV>
+__device__ __forceinline__ FxRes<INV> fx_run(int a, int b, FxLay lay, const FFTPlan& p) {
+  fx_passes(a, b, lay, p.fxp, p.fxt);
+  return FxRes<INV>{p.fxodd ? b : a, lay, p.n, p.fxr, p.wm, true};
+}
+template <bool INV>
+__device__ __forceinline__ FxRes<INV> fx_run64(int a, int b, FxLay lay, const FFTPlan& p) {
+  cfft_smem_sets<INV ? 1 : -1>(fx_mem64() + a, fx_mem64() + b, lay.stride, lay.ns, p, 1);
+  return FxRes<INV>{(p.nrad & 1) ? b : a, lay, p.n, p.fxr, p.wm, false};
 }
 
-template <int SIGN, int NS>
-__device__ __forceinline__ FxRes fx_run(int a, int b, FxLay lay, const FFTPlan& p) {
-  fx_passes<SIGN, NS>(a, b, lay, p.n, p.radw, p.fx[SIGN > 0 ? 1 : 0]);
-  return FxRes{(p.nrad & 1) ? b : a, lay, p.n, p.fxr, p.wm, true};
-}
-template <int SIGN>
-__device__ __forceinline__ FxRes fx_run64(int a, int b, FxLay lay, int NS, const FFTPlan& p) {
-  cfft_smem_sets<SIGN>(fx_mem64() + a, fx_mem64() + b, lay.stride, NS, p, lay.nb);
-  return FxRes{(p.nrad & 1) ? b : a, lay, p.n, p.fxr, p.wm, false};
-}
-// Complex transform of length p.n, unnormalised: exp(-) for SIGN < 0, exp(+) for SIGN > 0.
-template <int SIGN, int NS, bool CF, bool ANY = true, class Load>
-__device__ __forceinline__ FxRes xf_c2c(int a, int b, FxLay lay, const FFTPlan& p, Load load,
-                                         int max_n = kFxMaxN) {
-  const int nb = lay.nb, n = p.n;
-  fx_stage<NS, CF>(a, lay, n, load);
-  if (ANY && n > max_n) {
+// Complex transform of length p.n, unnormalised: exp(-), or exp(+) for INV.  REAL: the packed grid of a forward
+// real transform.
+template <bool INV, int NS, int W = 1, int PATH = kFxAny, bool REAL = false, class Load>
+__device__ __forceinline__ FxRes<INV> xf_c2c(int a, int b, FxLay lay, const FFTPlan& p, Load load) {
+  const int n = p.n;
+  fx_stage<NS, W>(a, lay, n, load);
+  if (PATH == kFp64 || (PATH == kFxAny && !p.fxp)) {
     __syncthreads();
-    return fx_run64<SIGN>(a, b, lay, NS, p);
+    return fx_run64<INV>(a, b, lay, p);
   }
   __syncthreads();
-  if (nb > 1) fx_clear(fx_shared().l1, lay.s0, NS * nb);
-#pragma unroll
-  for (int s = 0; s < NS; ++s) {  // each thread converts the entries it staged
+  // each thread converts the entries it staged
+  auto conv = [&](int q, FxExp ex) {
+    fx2 v = fx_load<kFxB>(fx_get64(q), ex);
+    if (INV) v = fx_swap(v);
+    fx_put(q, v);
+    return fx_l1(v);
+  };
+  if (W > 1) {
+    const int s = threadIdx.x & (W - 1);
+    const FxExp ex = fx_exponent(fx_get_max(lay.s0 + s));
     unsigned l1 = 0u;
-    int cp = -1;
-    FxExp ex{};
-    for (int i = threadIdx.x; i < n * nb; i += blockDim.x) {
-      int e, c;
-      fx_item<CF>(i, n, nb, e, c);
-      if (c != cp) {
-        if (cp >= 0) fx_put_l1(lay.s0, s, nb, cp, l1);
-        l1 = 0u;
-        cp = c;
-        ex = fx_exponent(fx_get_max(lay.s0 + s * nb + c));
-      }
-      const int q = a + s * lay.stride + e * nb + c;
-      const fx2 v = fx_load<kFxB>(fx_get64(q), ex);
-      fx_put(q, v);
-      l1 += fx_l1(v);
+    for (int i = threadIdx.x; i < n * W; i += blockDim.x) l1 += conv(a + s * lay.stride + i / W, ex);
+    l1 = fx_warp_sum<W>(l1);
+    if ((threadIdx.x & 31) < W) sts32(&fx_shared().l1[threadIdx.x >> 5][lay.s0 + s], l1);
+  } else {
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const FxExp ex = fx_exponent(fx_get_max(lay.s0 + s));
+      unsigned l1 = 0u;
+      for (int i = threadIdx.x; i < n; i += blockDim.x) l1 += conv(a + s * lay.stride + i, ex);
+      fx_put_l1(lay.s0 + s, l1);
     }
-    fx_put_l1(lay.s0, s, nb, cp, l1);
   }
   __syncthreads();
-  fx_make_meta<kFxB>(lay, p.fxs);
-  return fx_run<SIGN, NS>(a, b, lay, p);
+  fx_make_meta<kFxB>(lay, p.fxs + 32 * (REAL ? kFxFwdReal : kFxComplex));
+  return fx_run<INV>(a, b, lay, p);
 }
 
 // xf_c2r (below) with the c_k of every sequence already in b as FP64 pairs and their largest high words given
 // (fx_put_max); the call starts with a barrier.
-template <int NS, bool ANY = true>
-__device__ __forceinline__ FxRes xf_c2r_staged(int a, int b, FxLay lay, const FFTPlan& p, int K) {
-  const int nb = lay.nb, n = p.n;
-  if (ANY && n > kFxMaxReal) {
-    __syncthreads();
-    for (int s = 0; s < NS; ++s)
-      for (int i = threadIdx.x; i < n * nb; i += blockDim.x) {
-        int e, c;
-        fx_item<true>(i, n, nb, e, c);
-        const double2* S = fx_mem64() + b + s * lay.stride + c;
-        fx_mem64()[a + s * lay.stride + i] =
-            c2r_entry<true>([&](int k) { return S[k * nb]; }, e, K, n, p.wm, 1.0, 1.0);
-      }
-    __syncthreads();
-    return fx_run64<1>(a, b, lay, NS, p);
-  }
+template <int NS, int PATH = kFxAny>
+__device__ __forceinline__ FxRes<true> xf_c2r_staged(int a, int b, FxLay lay, const FFTPlan& p, int K) {
+  const int n = p.n;
   __syncthreads();
+  if (PATH == kFp64 || (PATH == kFxAny && !p.fxp)) {
+    for (int s = 0; s < NS; ++s) {
+      const double2* S = fx_mem64() + b + s * lay.stride;
+      for (int i = threadIdx.x; i < n; i += blockDim.x)
+        fx_mem64()[a + s * lay.stride + i] = c2r_entry<true>([&](int k) { return S[k]; }, i, K, n, p.wm, 1.0, 1.0);
+    }
+    __syncthreads();
+    return fx_run64<true>(a, b, lay, p);
+  }
   const int half = n / 2 + 1;
-  if (nb > 1) fx_clear(fx_shared().l1, lay.s0, NS * nb);
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
+    const FxExp ex = fx_exponent(fx_get_max(lay.s0 + s));
+    const int S = b + s * lay.stride, A = a + s * lay.stride;
     unsigned l1 = 0u;
-    int cp = -1;
-    FxExp ex{};
-    for (int i = threadIdx.x; i < half * nb; i += blockDim.x) {
-      int k, c;
-      fx_item<true>(i, half, nb, k, c);
-      if (c != cp) {
-        if (cp >= 0) fx_put_l1(lay.s0, s, nb, cp, l1);
-        l1 = 0u;
-        cp = c;
-        ex = fx_exponent(fx_get_max(lay.s0 + s * nb + c));
-      }
-      const int S = b + s * lay.stride + c;
+    for (int k = threadIdx.x; k < half; k += blockDim.x) {
       const int kc = n - k;
       // c_k and c_{n-k} (0 where not stored), c_0 real
       const bool hx = k < K, hy = k > 0 && kc < K;
-      double2 sx = fx_get64(S + (hx ? k : 0) * nb), sy = fx_get64(S + (hy ? kc : 0) * nb);
+      double2 sx = fx_get64(S + (hx ? k : 0)), sy = fx_get64(S + (hy ? kc : 0));
       if (!hx) sx.x = 0.0;
       if (!hx || k == 0) sx.y = 0.0;
       if (!hy) sy = make_double2(0.0, 0.0);
       const fx2 x = fx_load<kFxBReal>(sx, ex), y = fx_load<kFxBReal>(sy, ex);
       fx2 z0, z1;
       fx_pack(x, y, ldtab(p.fxr + k), z0, z1);
-      const int A = a + s * lay.stride + c;
-      fx_put(A + k * nb, z0);
+      fx_put(A + k, fx_swap(z0));
       l1 += fx_l1(z0);
       if (k > 0 && kc != k) {
-        fx_put(A + kc * nb, z1);
+        fx_put(A + kc, fx_swap(z1));
         l1 += fx_l1(z1);
       }
     }
-    fx_put_l1(lay.s0, s, nb, cp, l1);
+    fx_put_l1(lay.s0 + s, l1);
   }
   __syncthreads();
-  fx_make_meta<kFxBReal>(lay, p.fxs + 32);
-  return fx_run<1, NS>(a, b, lay, p);
+  fx_make_meta<kFxBReal>(lay, p.fxs + 32 * kFxInvReal);
+  return fx_run<true>(a, b, lay, p);
 }
 
 // Inverse real transform: the grid values g_j = Re c_0 + 2 Re sum_{1 <= k < K} c_k exp(2 pi i j k / 2n),
-// j < 2n, from c_k = load(set, c, k) (the imaginary part of c_0 is not used).
-template <int NS, bool CF, bool ANY = true, class Load>
-__device__ __forceinline__ FxRes xf_c2r(int a, int b, FxLay lay, const FFTPlan& p, int K, Load load) {
-  fx_stage<NS, CF>(b, lay, K, load);
-  return xf_c2r_staged<NS, ANY>(a, b, lay, p, K);
+// j < 2n, from c_k = load(s, k) (the imaginary part of c_0 is not used).
+template <int NS, int PATH = kFxAny, class Load>
+__device__ __forceinline__ FxRes<true> xf_c2r(int a, int b, FxLay lay, const FFTPlan& p, int K, Load load) {
+  fx_stage<NS, 1>(b, lay, K, load);
+  return xf_c2r_staged<NS, PATH>(a, b, lay, p, K);
 }
 
-// Forward real transform of the grid pairs (g_2j, g_2j+1) = load(set, c, j), j < n; results by FxRes::coef.
-template <int NS, bool CF, bool ANY = true, class Load>
-__device__ __forceinline__ FxRes xf_r2c(int a, int b, FxLay lay, const FFTPlan& p, Load load) {
-  return xf_c2c<-1, NS, CF, ANY>(a, b, lay, p, load, kFxMaxReal);
+// Forward real transform of the grid pairs (g_2j, g_2j+1) = load(s, j), j < n; results by FxRes::coef.
+template <int NS, int PATH = kFxAny, class Load>
+__device__ __forceinline__ FxRes<false> xf_r2c(int a, int b, FxLay lay, const FFTPlan& p, Load load) {
+  return xf_c2c<false, NS, 1, PATH, true>(a, b, lay, p, load);
 }
 
 }  // namespace spadj

@@ -40,6 +40,7 @@ constexpr unsigned kSpinLimit = 1u << 26;  // x ~150 ns per probe: several secon
 
 struct KMember {
   int N, Kx, M, L, res;
+  int CM, CL;           // entries of a transform buffer of length M, L
   long long off_state;  // complex offset of the member in a state array
   long long off_mix;    // complex offset of the member in a mixed [y][kx] array
   long long off_grid;   // offset of the member in a real [y][x] grid array
@@ -156,17 +157,17 @@ __device__ __forceinline__ double2 field_entry(int f, const double2* xs, const d
   return f < 4 ? fmult(f, (double)kx, (double)kyof(q, N), __ldg(&ik2[q]), x) : x;
 }
 
-// Inverse y transforms of the fields f0 .. f0 + NP - 1 of a column (transform pairs at fs + 2 p M, scratch + M;
+// Inverse y transforms of the fields f0 .. f0 + NP - 1 of a column (transform pairs at fs + 2 p CM, scratch + CM;
 // the column is read from global memory), into dst(f)[row j].
 template <int NP, class Dst>
 __device__ __forceinline__ void fields_y(int fs, const KRes& R, int f0, const double2* xs, const double* ik2, int kx, int N,
-                                         int M, Dst dst) {
-  const FxRes r = xf_c2c<1, NP, true, false>(fs, fs + M, FxLay{NP, 1, 2 * M, 0}, R.py, [&](int p, int, int j) {
+                                         int M, int CM, Dst dst) {
+  const auto r = xf_c2c<true, NP, 1, kFxOnly>(fs, fs + CM, FxLay{NP, 2 * CM, 0}, R.py, [&](int p, int j) {
     return field_entry(f0 + p, xs, ik2, kx, j, N, M);
   });
   for (int i = threadIdx.x; i < NP * M; i += blockDim.x) {
     const int p = i >= M ? 1 : 0, j = i - p * M;
-    dst(f0 + p, j, r.at(p, 0, j));
+    dst(f0 + p, j, r.at(p, j));
   }
   __syncthreads();
 }
@@ -174,12 +175,12 @@ __device__ __forceinline__ void fields_y(int fs, const KRes& R, int f0, const do
 // ---- forward CA tile --------------------------------------------------------------------------
 __device__ void ca_forward(const KolArgs& A, const KMember& m, int tile, int s) {
   extern __shared__ double2 ks[];
-  const int N = m.N, Kx = m.Kx, M = m.M;
+  const int N = m.N, Kx = m.Kx, M = m.M, CM = m.CM;
   const int n = A.n0 + s;           // absolute step of this stage
   const int last = A.nstage - 1;    // the launch's last stage
   const KRes& R = A.res[m.res];
   const int fs = 0;          // transform pairs from the start of ks
-  double2* xc = ks + 2 * M;              // N
+  double2* xc = ks + 2 * CM;             // N
   const int kx0 = tile * A.CW, kx1 = min(Kx, kx0 + A.CW);
   const long long S = A.state_size;
   for (int kx = kx0; kx < kx1; ++kx) {
@@ -188,9 +189,9 @@ __device__ void ca_forward(const KolArgs& A, const KMember& m, int tile, int s) 
       for (int q = threadIdx.x; q < N; q += blockDim.x) xc[q] = A.x0[col + q];
       __syncthreads();
     } else {
-      FxRes r{};
+      FxRes<false> r{};
       if (A.nonlinear || A.closure)
-        r = xf_c2c<-1, 1, true, false>(fs, fs + M, FxLay{1, 1, M, 0}, R.py, [&](int, int, int j) {
+        r = xf_c2c<false, 1, 1, kFxOnly>(fs, fs + CM, FxLay{1, CM, 0}, R.py, [&](int, int j) {
           return ldcg2(&A.mixB[0][m.off_mix + (long long)j * Kx + kx]);
         });
       const Coef c = kcoef(n, A.kc);
@@ -199,7 +200,7 @@ __device__ void ca_forward(const KolArgs& A, const KMember& m, int tile, int s) 
         const int idx = yidx(q, N, M);
         double2 F = make_double2(0.0, 0.0);
         if (idx >= 0 && (A.nonlinear || A.closure)) {
-          const double2 v = r.at(0, 0, idx);
+          const double2 v = r.at(0, idx);
           F = make_double2(-v.x * invM, -v.y * invM);
         }
         if (A.forcing && kx == 0 && (q == 4 || q == N - 4)) F.x -= 2.0;
@@ -236,60 +237,60 @@ __device__ void ca_forward(const KolArgs& A, const KMember& m, int tile, int s) 
       auto dst = [&](int f, int j, double2 v) { A.mixA[f][m.off_mix + (long long)j * Kx + kx] = v; };
       __syncthreads();
 #pragma unroll 1
-      for (int f0 = 0; f0 < 4; f0 += 2) fields_y<2>(fs, R, f0, xs, ik2, kx, N, M, dst);
-      if (A.closure) fields_y<1>(fs, R, 4, xs, ik2, kx, N, M, dst);
+      for (int f0 = 0; f0 < 4; f0 += 2) fields_y<2>(fs, R, f0, xs, ik2, kx, N, M, CM, dst);
+      if (A.closure) fields_y<1>(fs, R, 4, xs, ik2, kx, N, M, CM, dst);
     }
     __syncthreads();
   }
 }
 
 // Inverse x transform of one mixed row (weights w0 on k = 0, w elsewhere) in the buffers a, b on scale slot s0.
-__device__ __forceinline__ FxRes row_c2r(const double2* src, int a, int b, const KMember& m, const KRes& R, double w0,
-                                         double w, int s0) {
-  return xf_c2r<1, true, false>(a, b, FxLay{1, 1, m.L, s0}, R.px, m.Kx, [&](int, int, int k) {
+__device__ __forceinline__ FxRes<true> row_c2r(const double2* src, int a, int b, const KMember& m, const KRes& R,
+                                               double w0, double w, int s0) {
+  return xf_c2r<1, kFxOnly>(a, b, FxLay{1, m.CL, s0}, R.px, m.Kx, [&](int, int k) {
     const double2 v = ldcg2(&src[k]);
     const double f = k == 0 ? w0 : w;
     return make_double2(v.x * f, v.y * f);
   });
 }
 
-// Inverse x transforms of the mixed rows src(0..3) at once (weights 1), field f in the pair base + 2 f L: the FFTs
+// Inverse x transforms of the mixed rows src(0..3) at once (weights 1), field f in the pair base + 2 f CL: the FFTs
 // share their passes (more butterflies per pass than threads in one row's, one barrier per pass for all).
 template <class Src>
-__device__ __forceinline__ FxRes rows_c2r4(int base, Src src, const KMember& m, const KRes& R) {
-  return xf_c2r<4, true, false>(base, base + m.L, FxLay{4, 1, 2 * m.L, 0}, R.px, m.Kx,
-                                [&](int f, int, int k) { return ldcg2(&src(f)[k]); });
+__device__ __forceinline__ FxRes<true> rows_c2r4(int base, Src src, const KMember& m, const KRes& R) {
+  return xf_c2r<4, kFxOnly>(base, base + m.CL, FxLay{4, 2 * m.CL, 0}, R.px, m.Kx,
+                          [&](int f, int k) { return ldcg2(&src(f)[k]); });
 }
 
 // Spectrum of a forward row transform into dst[k], k < Kx, times s (s0 on k = 0, real)
-__device__ __forceinline__ void put_row(const FxRes& z, int set, double2* dst, int Kx, double s0, double s) {
+__device__ __forceinline__ void put_row(const FxRes<false>& z, int set, double2* dst, int Kx, double s0, double s) {
   for (int k = threadIdx.x; k < Kx; k += blockDim.x) {
-    const double2 v = z.coef(set, 0, k);
+    const double2 v = z.coef(set, k);
     dst[k] = k == 0 ? make_double2(v.x * s0, 0.0) : make_double2(v.x * s, v.y * s);
   }
 }
 
 // ---- forward B tile ---------------------------------------------------------------------------
 __device__ void b_forward(const KolArgs& A, const KMember& m, int tile) {
-  const int Kx = m.Kx, M = m.M, L = m.L;
+  const int Kx = m.Kx, M = m.M, L = m.L, C = m.CL;
   const KRes& R = A.res[m.res];
-  const int fs = 0;  // four transform pairs (field f: slots 2f, 2f+1 of L entries)
+  const int fs = 0;  // four transform pairs (field f: slots 2f, 2f+1 of C entries)
   const int j0 = tile * A.RW, j1 = min(M, j0 + A.RW);
   const double invM = 1.0 / M;
   for (int j = j0; j < j1; ++j) {
     if (A.closure) {
-      const FxRes w = row_c2r(A.mixA[4] + m.off_mix + (long long)j * Kx, fs, fs + L, m, R, 1.0, 1.0, 0);
+      const auto w = row_c2r(A.mixA[4] + m.off_mix + (long long)j * Kx, fs, fs + C, m, R, 1.0, 1.0, 0);
       double2* gw = reinterpret_cast<double2*>(A.gridW + m.off_grid + (long long)j * M);
-      for (int i = threadIdx.x; i < L; i += blockDim.x) gw[i] = w.at(0, 0, i);
+      for (int i = threadIdx.x; i < L; i += blockDim.x) gw[i] = w.at(0, i);
       __syncthreads();
     }
     double2* dst = A.mixB[0] + m.off_mix + (long long)j * Kx;
     if (A.nonlinear) {
       // u, v, w_x, w_y on the grid row, then u w_x + v w_y through the free slots of fields 0 and 1
-      const FxRes r = rows_c2r4(fs, [&](int f) { return A.mixA[f] + m.off_mix + (long long)j * Kx; }, m, R);
-      const int fr = (R.px.nrad & 1) ? fs : fs + L;
-      const FxRes z = xf_r2c<1, true, false>(fr, fr + 2 * L, FxLay{1, 1, L, 0}, R.px, [&](int, int, int i) {
-        const double2 u = r.at(0, 0, i), v = r.at(1, 0, i), wx = r.at(2, 0, i), wy = r.at(3, 0, i);
+      const auto r = rows_c2r4(fs, [&](int f) { return A.mixA[f] + m.off_mix + (long long)j * Kx; }, m, R);
+      const int fr = R.px.fxodd ? fs : fs + C;
+      const auto z = xf_r2c<1, kFxOnly>(fr, fr + 2 * C, FxLay{1, C, 0}, R.px, [&](int, int i) {
+        const double2 u = r.at(0, i), v = r.at(1, i), wx = r.at(2, i), wy = r.at(3, i);
         return make_double2(fma(u.x, wx.x, v.x * wy.x), fma(u.y, wx.y, v.y * wy.y));
       });
       put_row(z, 0, dst, Kx, invM, invM);
@@ -305,14 +306,14 @@ __device__ void b_forward(const KolArgs& A, const KMember& m, int tile) {
 // read from the Y ring.  second: the second half (W_{n-1} and the fields of X_{n-1} for the next VJP).
 __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, bool first, bool second) {
   extern __shared__ double2 ks[];
-  const int N = m.N, Kx = m.Kx, M = m.M;
+  const int N = m.N, Kx = m.Kx, M = m.M, CM = m.CM;
   const KRes& R = A.res[m.res];
-  // The VJP's forward y transforms run two at a time (pairs at ks + 2 p M, scratch + M) when the
-  // accumulator lam fits beside them; otherwise one at a time in ks[0, 2M).
-  const bool pairs = 4 * M + N <= A.smem_entries;
+  // The VJP's forward y transforms run two at a time (pairs at ks + 2 p CM, scratch + CM) when the
+  // accumulator lam fits beside them; otherwise one at a time in ks[0, 2 CM).
+  const bool pairs = 4 * CM + N <= A.smem_entries;
   const int fs = 0;
-  double2* lam = pairs ? ks + 4 * M : ks + 2 * M;  // N
-  double2* yc = pairs ? ks + 2 * M : lam + N;      // N (used after the VJP)
+  double2* lam = pairs ? ks + 4 * CM : ks + 2 * CM;  // N
+  double2* yc = pairs ? ks + 2 * CM : lam + N;      // N (used after the VJP)
   const int kx0 = tile * A.CW, kx1 = min(Kx, kx0 + A.CW);
   const long long S = A.state_size;
   const int SN = A.S;
@@ -328,14 +329,14 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
       // VJP: B_y^dagger of the grid cotangents, then the adjoint multipliers (identity for the
       // closure's input field)
       const double* ik2 = R.diag + (size_t)kx * N;
-      auto add = [&](int f0, int np, const FxRes& r) {
+      auto add = [&](int f0, int np, const FxRes<false>& r) {
         for (int q = threadIdx.x; q < N; q += blockDim.x) {
           const int idx = yidx(q, N, M);
           if (idx < 0) continue;
           double2 l = lam[q];
           for (int pq = 0; pq < np; ++pq) {
             const int f = f0 + pq;
-            const double2 v = r.at(pq, 0, idx);
+            const double2 v = r.at(pq, idx);
             if (f == 4) {
               l.x += v.x;
               l.y += v.y;
@@ -351,7 +352,7 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
         __syncthreads();
       };
       auto one = [&](int f) {
-        add(f, 1, xf_c2c<-1, 1, true, false>(fs, fs + M, FxLay{1, 1, M, 0}, R.py, [&](int, int, int j) {
+        add(f, 1, xf_c2c<false, 1, 1, kFxOnly>(fs, fs + CM, FxLay{1, CM, 0}, R.py, [&](int, int j) {
               return ldcg2(&A.mixB[f][m.off_mix + (long long)j * Kx + kx]);
             }));
       };
@@ -359,7 +360,7 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
       if (A.nonlinear && pairs) {
 #pragma unroll 1
         for (int f0 = 0; f0 < 4; f0 += 2)
-          add(f0, 2, xf_c2c<-1, 2, true, false>(fs, fs + M, FxLay{2, 1, 2 * M, 0}, R.py, [&](int pq, int, int j) {
+          add(f0, 2, xf_c2c<false, 2, 1, kFxOnly>(fs, fs + CM, FxLay{2, 2 * CM, 0}, R.py, [&](int pq, int j) {
                 return ldcg2(&A.mixB[f0 + pq][m.off_mix + (long long)j * Kx + kx]);
               }));
       } else if (A.nonlinear) {
@@ -422,35 +423,35 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
     if (!A.nonlinear && !A.closure) continue;
     // T_y^dagger W (inverse FFT with 1/M) -> mixA[4]
     {
-      const FxRes r = xf_c2c<1, 1, true, false>(fs, fs + M, FxLay{1, 1, M, 0}, R.py, [&](int, int, int j) {
+      const auto r = xf_c2c<true, 1, 1, kFxOnly>(fs, fs + CM, FxLay{1, CM, 0}, R.py, [&](int, int j) {
         const int q = yrow(j, N, M);
         return q < 0 ? make_double2(0.0, 0.0) : lam[q];
       });
       const double invM = 1.0 / M;
       for (int j = threadIdx.x; j < M; j += blockDim.x) {
-        const double2 v = r.at(0, 0, j);
+        const double2 v = r.at(0, j);
         A.mixA[4][m.off_mix + (long long)j * Kx + kx] = make_double2(v.x * invM, v.y * invM);
       }
       __syncthreads();
     }
-    // fields of X_{n-1} from the trajectory, their inverse y transforms two at a time (4M <= the CTA's
+    // fields of X_{n-1} from the trajectory, their inverse y transforms two at a time (4 CM <= the CTA's
     // shared memory for every member); the closure's input field goes to slot 5 (slot 4 holds T^dagger W)
     const double2* xs = A.traj + (long long)(n - 1 - A.lo) * S + col;
     const double* ik2 = R.diag + (size_t)kx * N;
     auto dst = [&](int f, int j, double2 v) { A.mixA[f < 4 ? f : 5][m.off_mix + (long long)j * Kx + kx] = v; };
     if (A.nonlinear) {
 #pragma unroll 1
-      for (int f0 = 0; f0 < 4; f0 += 2) fields_y<2>(fs, R, f0, xs, ik2, kx, N, M, dst);
+      for (int f0 = 0; f0 < 4; f0 += 2) fields_y<2>(fs, R, f0, xs, ik2, kx, N, M, CM, dst);
     }
-    if (A.closure) fields_y<1>(fs, R, 4, xs, ik2, kx, N, M, dst);
+    if (A.closure) fields_y<1>(fs, R, 4, xs, ik2, kx, N, M, CM, dst);
   }
 }
 
 // ---- adjoint B' tile --------------------------------------------------------------------------
 __device__ void b_adjoint(const KolArgs& A, const KMember& m, int tile) {
-  const int Kx = m.Kx, M = m.M, L = m.L;
+  const int Kx = m.Kx, M = m.M, L = m.L, C = m.CL;
   const KRes& R = A.res[m.res];
-  const int fs = 0;  // four transform pairs (field f: slots 2f, 2f+1 of L entries)
+  const int fs = 0;  // four transform pairs (field f: slots 2f, 2f+1 of C entries)
   const int j0 = tile * A.RW, j1 = min(M, j0 + A.RW);
   for (int j = j0; j < j1; ++j) {
     double2* gw = reinterpret_cast<double2*>(A.gridW + m.off_grid + (long long)j * M);
@@ -458,33 +459,33 @@ __device__ void b_adjoint(const KolArgs& A, const KMember& m, int tile) {
     auto mixed = [&](int f) { return A.mixA[f] + m.off_mix + (long long)j * Kx; };
     if (!A.nonlinear) {  // closure only: omega and the grid cotangent g, for the CNN's backward pass
       if (A.closure) {
-        const FxRes g = row_c2r(mixed(4), fs, fs + L, m, R, 1.0 / M, 0.5 / M, 0);
-        const FxRes w = row_c2r(mixed(5), fs + 2 * L, fs + 3 * L, m, R, 1.0, 1.0, 1);
+        const auto g = row_c2r(mixed(4), fs, fs + C, m, R, 1.0 / M, 0.5 / M, 0);
+        const auto w = row_c2r(mixed(5), fs + 2 * C, fs + 3 * C, m, R, 1.0, 1.0, 1);
         for (int i = threadIdx.x; i < L; i += blockDim.x) {
-          gw[i] = w.at(0, 0, i);
-          gg[i] = g.at(0, 0, i);
+          gw[i] = w.at(0, i);
+          gg[i] = g.at(0, i);
         }
         __syncthreads();
       }
       continue;
     }
-    // u, v, w_x, w_y in one set of transforms; the free slots F_f = fr + 2 f L take g (F_0 and F_1) and the
+    // u, v, w_x, w_y in one set of transforms; the free slots F_f = fr + 2 f C take g (F_0 and F_1) and the
     // closure's omega (F_2 and F_3), then the products
-    const FxRes r = rows_c2r4(fs, mixed, m, R);
-    const int fr = (R.px.nrad & 1) ? fs : fs + L;
-    const FxRes g = row_c2r(mixed(4), fr, fr + 2 * L, m, R, 1.0 / M, 0.5 / M, 4);
+    const auto r = rows_c2r4(fs, mixed, m, R);
+    const int fr = R.px.fxodd ? fs : fs + C;
+    const auto g = row_c2r(mixed(4), fr, fr + 2 * C, m, R, 1.0 / M, 0.5 / M, 4);
     if (A.closure) {
-      const FxRes w = row_c2r(mixed(5), fr + 4 * L, fr + 6 * L, m, R, 1.0, 1.0, 5);
+      const auto w = row_c2r(mixed(5), fr + 4 * C, fr + 6 * C, m, R, 1.0, 1.0, 5);
       for (int i = threadIdx.x; i < L; i += blockDim.x) {
-        gw[i] = w.at(0, 0, i);
-        gg[i] = g.at(0, 0, i);
+        gw[i] = w.at(0, i);
+        gg[i] = g.at(0, i);
       }
       __syncthreads();
     }
     // grid cotangents of u, v, w_x, w_y: -g w_x, -g w_y, -g u, -g v (entry i of g's slot is overwritten by the
     // thread that has read it)
-    const FxRes z = xf_r2c<4, true, false>(fr, r.z, FxLay{4, 1, 2 * L, 0}, R.px, [&](int f, int, int i) {
-      const double2 a = g.at(0, 0, i), b = r.at(f ^ 2, 0, i);
+    const auto z = xf_r2c<4, kFxOnly>(fr, r.z, FxLay{4, 2 * C, 0}, R.px, [&](int f, int i) {
+      const double2 a = g.at(0, i), b = r.at(f ^ 2, i);
       return make_double2(-a.x * b.x, -a.y * b.y);
     });
     for (int f = 0; f < 4; ++f) put_row(z, f, A.mixB[f] + m.off_mix + (long long)j * Kx, Kx, 1.0, 2.0);
@@ -583,15 +584,15 @@ __global__ void __launch_bounds__(kKolThreads) closure_rows_kernel(const __grid_
   const int j = blockIdx.x;
   if (j >= m.M) return;
   const KRes& R = A.res[m.res];
-  const int L = m.L, Kx = m.Kx;
+  const int Kx = m.Kx;
   const int fs = 0;
   const double2* g = reinterpret_cast<const double2*>(grid + m.off_grid + (long long)j * m.M);
-  const FxRes z = xf_r2c<1, true, false>(fs, fs + L, FxLay{1, 1, L, 0}, R.px, [&](int, int, int i) { return g[i]; });
+  const auto z = xf_r2c<1, kFxOnly>(fs, fs + m.CL, FxLay{1, m.CL, 0}, R.px, [&](int, int i) { return g[i]; });
   if (mode == 0) {
     double2* dst = A.mixB[0] + m.off_mix + (long long)j * Kx;
     const double s = 1.0 / m.M;
     for (int k = threadIdx.x; k < Kx; k += blockDim.x) {
-      const double2 v = dst[k], c = z.coef(0, 0, k);
+      const double2 v = dst[k], c = z.coef(0, k);
       dst[k] = make_double2(v.x - c.x * s, k == 0 ? v.y : v.y - c.y * s);
     }
   } else {
@@ -696,7 +697,7 @@ struct Kol : EqImpl {
   int closure = 0;
   DevBuf gridW, gridG, corr, xq, hbuf[3], dact[3], dh, dz, dz2, pbuf, wq, bq, part, gp, chunkbuf;
   static constexpr int kWgradChunks = 8;
-  int Lmax = 0, Mmax = 0, Nmax = 0, Kxmax = 0;
+  int CLmax = 0, CMmax = 0, Nmax = 0;
   double Re = 100.0, dt = 0;
   int forcing = 1, nonlinear = 1;
   int CW = 4, RW = 2, ctas_per_sm = 0, persistent = 1;
@@ -761,6 +762,7 @@ struct Kol : EqImpl {
       }
       KMember m{};
       m.N = N; m.Kx = N / 2; m.M = 3 * N / 2; m.L = m.M / 2; m.res = r;
+      m.CM = m.M; m.CL = m.L;
       m.off_state = offs; m.off_mix = offm; m.off_grid = offg;
       offs += (long long)m.Kx * N;
       offm += (long long)m.M * m.Kx;
@@ -768,7 +770,7 @@ struct Kol : EqImpl {
       if (closure && b > 0 && N != hm[0].N)
         return p->fail(SPADJ_ERR_UNSUPPORTED, "kolmogorov: the learned closure needs one resolution for the whole batch");
       hm.push_back(m);
-      Lmax = std::max(Lmax, m.L); Mmax = std::max(Mmax, m.M); Nmax = std::max(Nmax, N); Kxmax = std::max(Kxmax, m.Kx);
+      CLmax = std::max(CLmax, m.CL); CMmax = std::max(CMmax, m.CM); Nmax = std::max(Nmax, N);
     }
     state_size = offs;
     mix_size = offm;
@@ -792,10 +794,10 @@ struct Kol : EqImpl {
       }
       // the transforms' tables of the x and y plans
       soff.push_back(ht.size());
-      const std::vector<double2> sx = fft_tables(kres[i].px);
+      const std::vector<double2> sx = fft_tables(kres[i].px, true);
       ht.insert(ht.end(), sx.begin(), sx.end());
       soff.push_back(ht.size());
-      const std::vector<double2> sy = fft_tables(kres[i].py);
+      const std::vector<double2> sy = fft_tables(kres[i].py, false);
       ht.insert(ht.end(), sy.begin(), sy.end());
       doff.push_back(hd.size());
       const double shift[3] = {0.0, 1.0 / p->desc.dt, 1.5 / p->desc.dt};
@@ -811,8 +813,8 @@ struct Kol : EqImpl {
     SPADJ_CUDA_TRY(p, tables.ensure(sizeof(double2) * ht.size()));
     SPADJ_CUDA_TRY(p, cudaMemcpyAsync(tables.ptr, ht.data(), sizeof(double2) * ht.size(), cudaMemcpyHostToDevice, p->stream));
     for (size_t i = 0; i < resN.size(); ++i) {
-      fft_bind(kres[i].px, tables.as<double2>() + soff[2 * i], tables.as<double2>() + toff[i]);
-      fft_bind(kres[i].py, tables.as<double2>() + soff[2 * i + 1], nullptr);
+      fft_bind(kres[i].px, true, tables.as<double2>() + soff[2 * i], tables.as<double2>() + toff[i]);
+      fft_bind(kres[i].py, false, tables.as<double2>() + soff[2 * i + 1], nullptr);
       kres[i].diag = diag.as<double>() + doff[i];
     }
     const size_t sb = sizeof(double2) * state_size, mb = sizeof(double2) * mix_size;
@@ -887,12 +889,12 @@ struct Kol : EqImpl {
     }
     SPADJ_CUDA_TRY(p, ctr.ensure(sizeof(int) * (2 * (size_t)nmem + 2)));
     SPADJ_CUDA_TRY(p, tmp.ensure(sb));
-    // shared memory: max over tile kinds (B and B': 8 L + Kx, four transform sets and their
-    // staging; CA': 2 M + 2 N, or 4 M + N with its VJP transforms in pairs).  The paired form's
+    // shared memory: max over tile kinds (B and B': 8 CL, four transform pairs; CA': 2 CM + 2 N, or 4 CM + N
+    // with its VJP transforms in pairs).  The paired form's
     // size is taken when it keeps as many CTAs resident per SM.
     {
-      const size_t base = sizeof(double2) * std::max<size_t>(8 * (size_t)Lmax + Kxmax, 2 * (size_t)Mmax + 2 * (size_t)Nmax);
-      const size_t ext = std::max<size_t>(base, sizeof(double2) * (4 * (size_t)Mmax + Nmax));
+      const size_t base = sizeof(double2) * std::max<size_t>({8 * (size_t)CLmax, 4 * (size_t)CMmax, 2 * (size_t)CMmax + 2 * (size_t)Nmax});
+      const size_t ext = std::max<size_t>(base, sizeof(double2) * (4 * (size_t)CMmax + Nmax));
       smem = base;
       if (ext > base && ext <= 227 * 1024) {
         int ob = 0, oe = 0;

@@ -153,6 +153,7 @@ struct RB : EqImpl {
     npts = (size_t)Mz * Mx;
     xp.Kx = Kx; xp.Mx = Mx; xp.L = L; xp.kscale = 2.0 * M_PI / Lx;
     xp.plan = make_plan(L);
+    xp.C = L;
     if (xp.plan.nrad < 0) return p->fail(SPADJ_ERR_INVALID, "rb: 3*n[0]/4 must be of the form 2^a 3^b");
 
     // host operators and solution operators
@@ -178,7 +179,7 @@ struct RB : EqImpl {
       hwm[m] = make_double2(std::cos(th), std::sin(th));
     }
     {  // the transforms' tables follow the M-table in the same buffer
-      const std::vector<double2> sct = fft_tables(xp.plan);
+      const std::vector<double2> sct = fft_tables(xp.plan, true);
       hwm.insert(hwm.end(), sct.begin(), sct.end());
     }
     auto up = [&](DevBuf& b, const void* h, size_t bytes) -> cudaError_t {
@@ -200,7 +201,7 @@ struct RB : EqImpl {
       if (s != SPADJ_OK) return s;
     }
     xp.WM = wm.as<double2>();
-    fft_bind(xp.plan, xp.WM + Mx, xp.WM);
+    fft_bind(xp.plan, true, xp.WM + Mx, xp.WM);
     // work buffers
     const size_t sb = sizeof(double2) * ns, mb = sizeof(double2) * nmix, gb = sizeof(double) * npts;
     for (WS& l : ws) {

@@ -226,49 +226,54 @@ struct XJobs {
 
 struct XParams {
   int Kx, Mx, L;
+  int C;  // entries of one transform buffer
   double kscale;
   FFTPlan plan;
   const double2* WM;
 };
 
-constexpr int kXThreadsMax = 192;
-// x-transform jobs, nb rows per CTA (nb <= 4): the rows are interleaved in shared memory (element e of row c
-// at e * nb + c) and transformed together, so short rows keep all threads of the CTA busy in every
-// pass and share its barriers.  Every row has its own scale, so the results do not depend on nb.
+constexpr int kXThreadsMax = 256;
+// x-transform jobs, NB rows per CTA: the rows are transformed together (their butterflies share every pass and its
+// barrier, so short rows keep the threads busy).  Every row has its own scale, so the results do not depend on
+// NB.  Bound by latency and instruction fetch on small grids, by the integer pipes on large ones.  The rows of a
+// CTA lie one after the other in shared memory; interleaved entry by entry, the staging, packing and unpacking
+// loops met two to four to a bank (gradient of 8 Couette steps at 128 x 64 x 64: 25.9 ms, now 24.5 ms).
+template <int NB>
 __global__ void __launch_bounds__(kXThreadsMax) xfft_kernel(const __grid_constant__ XJobs js,
-                                                            const __grid_constant__ XParams P, int nb, int nrows) {
+                                                            const __grid_constant__ XParams P, int nrows) {
   pdl_trigger();
   pdl_wait();
   const XJob& J = js.j[blockIdx.y];
-  const int row0 = blockIdx.x * nb;
-  const int L = P.L, Kx = P.Kx, Mx = P.Mx;
-  const int a = 0, b = L * nb;
+  const int row0 = blockIdx.x * NB;
+  const int L = P.L, Kx = P.Kx, Mx = P.Mx, C = P.C;
   const int tid = threadIdx.x, nt = blockDim.x;
   const double2 zero = make_double2(0.0, 0.0);
+  const FxLay lay{NB, 2 * C, 0};  // row s in the buffers 2 s C and (2 s + 1) C
   if (J.dir == 0) {
     const double2* src = J.cin + (size_t)row0 * Kx;
-    const FxRes z = xf_c2r<1, false>(a, b, FxLay{1, nb, L * nb, 0}, P.plan, Kx, [&](int, int c, int k) {
-      if (row0 + c >= nrows) return zero;
-      double2 v = src[(size_t)c * Kx + k];
+    const auto z = xf_c2r<NB>(0, C, lay, P.plan, Kx, [&](int s, int k) {
+      if (row0 + s >= nrows) return zero;
+      double2 v = src[(size_t)s * Kx + k];
       if (J.cmul == 1) {  // i k v
         const double kk = P.kscale * k;
         v = make_double2(-kk * v.y, kk * v.x);
       }
       return cscale(v, k == 0 ? J.w0 : J.w);
     });
-    for (int c = 0; c < nb && row0 + c < nrows; ++c) {
-      double2* g = reinterpret_cast<double2*>(J.rout + (size_t)(row0 + c) * Mx);
-      for (int j = tid; j < L; j += nt) g[j] = z.at(0, c, j);
+    for (int s = 0; s < NB && row0 + s < nrows; ++s) {
+      double2* g = reinterpret_cast<double2*>(J.rout + (size_t)(row0 + s) * Mx);
+      for (int j = tid; j < L; j += nt) g[j] = z.at(s, j);
     }
     return;
   }
-  auto store = [&](const FxRes& z, int nin) {
-    for (int c = 0; c < nb && row0 + c < nrows; ++c) {
-      double2* dst = J.cout + (size_t)(row0 + c) * Kx;
+  // spectra of nin inputs per row (input t of row s is sequence s + t NB), combined into the row's output
+  auto store = [&](const auto& z, int nin) {
+    for (int s = 0; s < NB && row0 + s < nrows; ++s) {
+      double2* dst = J.cout + (size_t)(row0 + s) * Kx;
       for (int k = tid; k < Kx; k += nt) {
         double2 acc = zero;
         for (int t = 0; t < nin; ++t) {
-          double2 X = z.coef(t, c, k);
+          double2 X = z.coef(s + t * NB, k);
           if (J.rmul[t] == 2) {  // -i k X
             const double kk = P.kscale * k;
             X = make_double2(kk * X.y, -kk * X.x);
@@ -283,9 +288,9 @@ __global__ void __launch_bounds__(kXThreadsMax) xfft_kernel(const __grid_constan
   };
   if (J.nprod > 0) {
     const double p0 = J.ps[0], p1 = J.ps[1];
-    store(xf_r2c<1, false>(a, b, FxLay{1, nb, L * nb, 0}, P.plan, [&](int, int c, int j) {
-      if (row0 + c >= nrows) return zero;
-      const size_t ro = (size_t)(row0 + c) * Mx;
+    store(xf_r2c<NB>(0, C, lay, P.plan, [&](int s, int j) {
+      if (row0 + s >= nrows) return zero;
+      const size_t ro = (size_t)(row0 + s) * Mx;
       auto at = [&](const double* base, int slot) {
         return reinterpret_cast<const double2*>(base + (size_t)slot * J.npts + ro)[j];
       };
@@ -297,14 +302,15 @@ __global__ void __launch_bounds__(kXThreadsMax) xfft_kernel(const __grid_constan
     }), 1);
     return;
   }
-  auto row = [&](int t, int c, int j) {
-    return row0 + c < nrows ? reinterpret_cast<const double2*>(J.rin[t] + (size_t)(row0 + c) * Mx)[j] : zero;
+  auto row = [&](int s, int j) {
+    const int t = s / NB, q = row0 + s - t * NB;
+    return q < nrows ? reinterpret_cast<const double2*>(J.rin[t] + (size_t)q * Mx)[j] : zero;
   };
-  if (J.nr > 1) store(xf_r2c<2, false>(a, b, FxLay{2, nb, 2 * L * nb, 0}, P.plan, row), 2);  // sets 2 L nb apart
-  else store(xf_r2c<1, false>(a, b, FxLay{1, nb, L * nb, 0}, P.plan, row), 1);
+  if (J.nr > 1) store(xf_r2c<2 * NB>(0, C, FxLay{2 * NB, 2 * C, 0}, P.plan, row), 2);
+  else store(xf_r2c<NB>(0, C, lay, P.plan, row), 1);
 }
 
-inline size_t xfft_smem(int L, int nb) { return sizeof(double2) * (size_t)nb * 4 * L; }
+inline size_t xfft_smem(int C, int nb) { return sizeof(double2) * (size_t)nb * 4 * C; }
 constexpr int kXRowsMax = 4;
 
 // Launch variant of the x transforms: rows per CTA nb (low byte) and threads per CTA nt (the
@@ -319,8 +325,10 @@ constexpr int xvar_threads(int xv) { return (xv >> 8) ? (xv >> 8) : 64; }
 // x-transform jobs over nrows rows in launch variant xv
 inline cudaError_t launch_xfft(bool pdl, int xv, const XJobs& js, const XParams& xp, int nrows, cudaStream_t st) {
   const int nb = xvar_rows(xv) < 1 ? 1 : xvar_rows(xv), nt = xvar_threads(xv);
-  return launch_kernel(pdl, xfft_kernel, dim3((nrows + nb - 1) / nb, js.n), dim3(nt), xfft_smem(xp.L, nb), st, js, xp, nb,
-                       nrows);
+  auto go = [&](auto kernel) {
+    return launch_kernel(pdl, kernel, dim3((nrows + nb - 1) / nb, js.n), dim3(nt), xfft_smem(xp.C, nb), st, js, xp, nrows);
+  };
+  return nb == 1 ? go(xfft_kernel<1>) : nb == 2 ? go(xfft_kernel<2>) : go(xfft_kernel<4>);
 }
 
 // Launch variant for the x transforms of this problem: rows `forced` (1, 2 or 4, 64 threads)
@@ -333,11 +341,12 @@ inline int tune_xfft_rows(const XJobs& js, const XParams& xp, int nrows, cudaStr
   // row counts whose shared memory fits one CTA (raising the opt-in limit where needed)
   bool ok[kXRowsMax + 1] = {false, false, false, false, false};
   for (int nb : {1, 2, 4}) {
-    const size_t sm = xfft_smem(xp.L, nb), fix = sizeof(FxShared);
+    const size_t sm = xfft_smem(xp.C, nb), fix = sizeof(FxShared);
     if (sm + fix <= 48 * 1024) {
       ok[nb] = true;
     } else if (sm + fix <= 227 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(xfft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      auto raise = [&](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); };
+      const cudaError_t e = nb == 1 ? raise(xfft_kernel<1>) : nb == 2 ? raise(xfft_kernel<2>) : raise(xfft_kernel<4>);
       ok[nb] = e == cudaSuccess;
       cudaGetLastError();
     }
@@ -349,7 +358,7 @@ inline int tune_xfft_rows(const XJobs& js, const XParams& xp, int nrows, cudaStr
   if ((*err = cudaEventCreate(&b)) != cudaSuccess) { cudaEventDestroy(a); return xvar(1, 64); }
   int best_xv = xvar(1, 64);
   float best = 1e30f;
-  constexpr int cand[] = {xvar(1, 64), xvar(2, 64), xvar(4, 64), xvar(2, 96), xvar(4, 96), xvar(4, 128), xvar(4, 192)};
+  constexpr int cand[] = {xvar(1, 64), xvar(1, 32), xvar(2, 64), xvar(4, 64), xvar(2, 128), xvar(4, 128), xvar(4, 256)};
   // each candidate: one untimed launch, then the median of 7 timed ones (a lucky or unlucky single
   // launch does not decide the variant)
   for (int xv : cand) {
