@@ -92,9 +92,6 @@ TRAFFIC = {
     # of the gradient (484 : 200 : 200 : 380); the working set is L2-resident, so this is the
     # cold-cache fill ncu sees after its cache flush
     ("rayleigh_benard2d_256x64_Ra1e6_rk222_2000steps", "x_fft"): 1.68e6,
-    # evp_iter_kernel, full bench launch (608 pencils, 100 iterations): 32.07 GB read + 7.4 MB
-    # written, against 35.9 GB of operator rows streamed by the algorithm (the rest hits in L2)
-    ("poiseuille_evp_N64_608pencils_Re8000_100iter", "pencil_solve"): 3.2075e10,
     # Burgers trajectory + adjoint kernels, captured at 50 steps (forward: 36 MB read + 1.650 GB of
     # trajectory written; adjoint: 1.715 GB of trajectory read + 44 MB written), trajectory bytes
     # scaled to 1000 steps by (1001 / 51), averaged over the two launches of a gradient
@@ -1276,7 +1273,7 @@ def run_gpu_evp(args, wl):
             "avg_launch_us": 1e3 * dms / dn, "flops_per_launch": dfl / dn,
             "per_kernel": per_kernel,
             "peak_note": "FP64 peak measured by the library's FMA-chain probe on this GPU; "
-                         + ("16 flops per operator entry and iteration (forward and adjoint complex matvecs)" if evp
+                         + ("8 flops per band entry of a factorisation or solve (both directions)" if evp
                             else "8 flops per operator entry and pencil solve (complex matvec), 4 per entry of "
                                  "the real Gram products")}
     launches = int(sum(v[2] for v in rep.values()))
@@ -1298,7 +1295,7 @@ def run_gpu_evp(args, wl):
             "gpu_launches": launches,
             "e2e": {"value": units / (e2e_ms / 1e3), "unit": wl.unit, "h2d_bytes_per_step": bi,
                     "d2h_bytes_per_step": bo,
-                    "note": "includes the host LU of every shifted pencil" if evp else
+                    "note": "includes the band LU of every shifted pencil" if evp else
                             "the frequency's pencil factorisations are built at the first call and kept"},
             "roofline": roof, "cpu_baseline": cpu, "clocks": clocks}
     print(json.dumps(line))

@@ -104,36 +104,6 @@ void lu_solve_multi(const std::vector<cd>& a, const std::vector<int>& piv, int n
   }
 }
 
-// Solve A^H X = B with the factors of A from lu_factor (P A = L U, so A^H = U^H L^H P):
-// forward substitution with U^H, back substitution with the unit L^H, then the row swaps
-// undone in reverse order.
-void lu_solve_h_multi(const std::vector<cd>& a, const std::vector<int>& piv, int n, std::vector<cd>& B, int nr) {
-  for (int c0 = 0; c0 < nr; c0 += kPanel) {
-    const int w = std::min(kPanel, nr - c0);
-    for (int i = 0; i < n; ++i) {
-      cd* bi = &B[(size_t)i * nr + c0];
-      for (int j = 0; j < i; ++j) {
-        const cd u = std::conj(a[(size_t)j * n + i]);
-        if (u == 0.0) continue;
-        caxpy_sub(bi, &B[(size_t)j * nr + c0], u, w);
-      }
-      const cd inv = 1.0 / std::conj(a[(size_t)i * n + i]);
-      for (int c = 0; c < w; ++c) bi[c] *= inv;
-    }
-    for (int i = n - 2; i >= 0; --i) {
-      cd* bi = &B[(size_t)i * nr + c0];
-      for (int j = i + 1; j < n; ++j) {
-        const cd l = std::conj(a[(size_t)j * n + i]);
-        if (l == 0.0) continue;
-        caxpy_sub(bi, &B[(size_t)j * nr + c0], l, w);
-      }
-    }
-  }
-  for (int k = n - 1; k >= 0; --k)
-    if (piv[k] != k)
-      for (int c = 0; c < nr; ++c) std::swap(B[(size_t)k * nr + c], B[(size_t)piv[k] * nr + c]);
-}
-
 void base_flow(const rbhost::Operators& o, int base, std::vector<double>& Umat, std::vector<double>& UPmat) {
   const int N = o.N;
   // ZS = (S1 S0 on N + 1 modes) * (z T_n in the T basis of degree N), first N rows
@@ -298,6 +268,10 @@ bool build_phi(const rbhost::Operators& o, int Kx, int Ny, double Lx, double Ly,
   return true;
 }
 
+double pressure_weight(int j) {
+  return (2.0 / (1.0 - (double)j * j)) / (2.0 / (1.0 - (double)(j + 2) * (j + 2)));
+}
+
 namespace {
 
 // Row and column orders of the banded form (couette_setup.h): perm_r[i] / perm_c[i] is the row /
@@ -321,12 +295,10 @@ void band_orders(int N, bool mean, std::vector<int>& perm_r, std::vector<int>& p
   (void)nv;
 }
 
-// The recombined, reordered pencil matrix A' (row-major nv x nv) and, for the adjoint direction,
-// J A'^H J in its place.
-void band_matrix(const rbhost::Operators& o, const std::vector<double>& ZS, const std::vector<double>& UP, double al,
-                 double be, bool mean, double nu, double a0, bool hermitian, std::vector<cd>& A, std::vector<cd>& B) {
-  const int N = o.N, nv = 4 * N + 7;
-  assemble_pencil(o, ZS, UP, al, be, mean, nu, cd(a0, 0.0), A);
+// The column recombination of the banded form, in place on the pencil matrix (or a part of it).
+template <class T>
+void recombine(int N, bool mean, std::vector<T>& A) {
+  const int nv = 4 * N + 7;
   auto col_sub = [&](int c, int c2, double w) {  // column c -= w * column c2
     for (int r = 0; r < nv; ++r) A[(size_t)r * nv + c] -= w * A[(size_t)r * nv + c2];
   };
@@ -336,11 +308,19 @@ void band_matrix(const rbhost::Operators& o, const std::vector<double>& ZS, cons
   // the pressure columns only where the gauge row reads them (the mean pencil): elsewhere the
   // recombination would raise the condition number of A' by four orders of magnitude
   for (int j = 0; mean && j + 2 < N; j += 2) {
-    const double wj = 2.0 / (1.0 - (double)j * j), wj2 = 2.0 / (1.0 - (double)(j + 2) * (j + 2));
-    col_sub(3 * N + j, 3 * N + j + 2, wj / wj2);
+    col_sub(3 * N + j, 3 * N + j + 2, pressure_weight(j));
     // int psi_j dz = 0 exactly; the gauge row's rounding residue is dropped
     A[(size_t)(4 * N + 6) * nv + 3 * N + j] = 0.0;
   }
+}
+
+// The recombined, reordered pencil matrix A' (row-major nv x nv) and, for the adjoint direction,
+// J A'^H J in its place.
+void band_matrix(const rbhost::Operators& o, const std::vector<double>& ZS, const std::vector<double>& UP, double al,
+                 double be, bool mean, double nu, double a0, bool hermitian, std::vector<cd>& A, std::vector<cd>& B) {
+  const int N = o.N, nv = 4 * N + 7;
+  assemble_pencil(o, ZS, UP, al, be, mean, nu, cd(a0, 0.0), A);
+  recombine(N, mean, A);
   std::vector<int> pr, pc;
   band_orders(N, mean, pr, pc);
   B.assign((size_t)nv * nv, cd(0.0, 0.0));
@@ -559,57 +539,69 @@ bool band_solve_host(const rbhost::Operators& o, double al, double be, double nu
   return true;
 }
 
-bool build_evp(const rbhost::Operators& o, int base, int P, const double* prm, const double* shift,
-               std::vector<double>& T, std::vector<double>& RH, std::string* err) {
-  const int N = o.N, nv = 4 * N + 7, H = 3 * N;
+void band_parts(const rbhost::Operators& o, int base, bool mean, int& kl, int& ku, std::vector<double>& E) {
+  const int N = o.N, nv = 4 * N + 7;
   std::vector<double> Um, UP;
   base_flow(o, base, Um, UP);
-  const size_t per = (size_t)nv * H * 2;
-  T.assign((size_t)P * per, 0.0);
-  RH.assign((size_t)P * per, 0.0);
-  std::vector<int> bad(P, 0);
-  auto work = [&](int p0, int p1) {
-    std::vector<cd> A, B;
-    std::vector<int> piv;
-    for (int pp = p0; pp < p1; ++pp) {
-      const double al = prm[3 * pp], be = prm[3 * pp + 1], Re = prm[3 * pp + 2];
-      const cd sigma(shift[2 * pp], shift[2 * pp + 1]);
-      assemble_pencil(o, Um, UP, al, be, al == 0.0 && be == 0.0, 1.0 / Re, sigma, A);
-      if (!lu_factor(A, piv, nv)) {
-        bad[pp] = 1;
-        continue;
+  std::vector<int> pr, pc;
+  band_orders(N, mean, pr, pc);
+  std::vector<std::vector<double>> parts(kBandParts);
+  kl = ku = 0;
+  for (int t = 0; t < kBandParts; ++t) {
+    std::vector<double> A((size_t)nv * nv, 0.0);
+    auto at = [&](int r, int c) -> double& { return A[(size_t)r * nv + c]; };
+    const int W = 2 * N, P = 3 * N, tau = 4 * N, tp = tau + 6, r0 = 4 * N;
+    for (int r = 0; r < N; ++r)
+      for (int c = 0; c < N; ++c) {
+        const double ss = o.SS[r * N + c];
+        const double diag = t == kPartShift ? ss : t == kPartVisc ? -o.DD[r * N + c] : t == kPartAlpha ? Um[r * N + c] : 0.0;
+        for (int f = 0; f < 3; ++f) at(f * N + r, f * N + c) = diag;
+        if (t == kPartConst) {
+          at(r, W + c) = UP[r * N + c];
+          at(W + r, P + c) = o.SD[r * N + c];
+          at(P + r, W + c) = o.D0[r * N + c];
+        } else if (t == kPartAlpha || t == kPartBeta) {
+          const int q = t == kPartAlpha ? 0 : N;
+          at(q + r, P + c) = ss;
+          at(P + r, q + c) = o.S0[r * N + c];
+        }
       }
-      B.assign((size_t)nv * H, cd(0.0, 0.0));
-      for (int f = 0; f < 3; ++f)
-        for (int c = 0; c < N; ++c)
-          for (int r = 0; r < N; ++r) B[(size_t)(f * N + r) * H + f * N + c] = o.SS[r * N + c];
-      lu_solve_multi(A, piv, nv, B, H);
-      double* t = &T[(size_t)pp * per];
-      for (size_t i = 0; i < (size_t)nv * H; ++i) { t[2 * i] = B[i].real(); t[2 * i + 1] = B[i].imag(); }
-      B.assign((size_t)nv * H, cd(0.0, 0.0));
-      for (int r = 0; r < H; ++r) B[(size_t)r * H + r] = 1.0;
-      lu_solve_h_multi(A, piv, nv, B, H);
-      double* rh = &RH[(size_t)pp * per];
-      for (size_t i = 0; i < (size_t)nv * H; ++i) { rh[2 * i] = B[i].real(); rh[2 * i + 1] = B[i].imag(); }
+    for (int f = 0; f < 3; ++f) {
+      if (t == kPartVisc) at(f * N + o.lift_row, tau + 2 * f) = -o.lift_val;
+      if (t == kPartConst) {
+        at(f * N + N - 1, tau + 2 * f + 1) = 1.0;
+        for (int n = 0; n < N; ++n) {
+          at(r0 + 2 * f, f * N + n) = n % 2 == 0 ? 1.0 : -1.0;
+          at(r0 + 2 * f + 1, f * N + n) = 1.0;
+        }
+      }
     }
-  };
-  unsigned nt = std::thread::hardware_concurrency();
-  if (nt == 0) nt = 1;
-  if (nt > 64) nt = 64;
-  if ((int)nt > P) nt = P;
-  std::vector<std::thread> th;
-  const int chunk = (P + nt - 1) / nt;
-  for (unsigned t = 0; t < nt; ++t) {
-    const int p0 = t * chunk, p1 = std::min(P, p0 + chunk);
-    if (p0 < p1) th.emplace_back(work, p0, p1);
+    if (t == kPartConst) {
+      at(P + N - 1, tau + 4) = 1.0;
+      if (mean) {
+        at(P, tp) = 1.0;
+        for (int n = 0; n < N; n += 2) at(r0 + 6, P + n) = 2.0 / (1.0 - (double)n * n);
+      } else {
+        at(r0 + 6, tp) = 1.0;
+      }
+    }
+    recombine(N, mean, A);
+    parts[t].assign((size_t)nv * nv, 0.0);
+    for (int i = 0; i < nv; ++i)
+      for (int k = 0; k < nv; ++k) {
+        const double v = A[(size_t)pr[i] * nv + pc[k]];
+        if (v == 0.0) continue;
+        parts[t][(size_t)i * nv + k] = v;
+        kl = std::max(kl, i - k);
+        ku = std::max(ku, k - i);
+      }
   }
-  for (auto& t : th) t.join();
-  for (int pp = 0; pp < P; ++pp)
-    if (bad[pp]) {
-      if (err) *err = "eigen: singular shifted pencil matrix at pencil " + std::to_string(pp);
-      return false;
-    }
-  return true;
+  const int w = kl + ku + 1;
+  E.assign((size_t)kBandParts * nv * w, 0.0);
+  for (int t = 0; t < kBandParts; ++t)
+    for (int i = 0; i < nv; ++i)
+      for (int k = std::max(0, i - kl); k <= std::min(nv - 1, i + ku); ++k)
+        E[((size_t)t * nv + i) * w + (k - i + kl)] = parts[t][(size_t)i * nv + k];
 }
 
 }  // namespace couhost

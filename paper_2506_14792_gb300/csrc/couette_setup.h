@@ -88,15 +88,15 @@ bool build_band(const rbhost::Operators& o, int Kx, int Ny, double Lx, double Ly
 bool band_solve_host(const rbhost::Operators& o, double al, double be, double nu, double a0, int base, bool transpose,
                      const std::complex<double>* in, std::complex<double>* out, std::string* err);
 
-// Shift-invert operators of P eigenvalue pencils (prm[p] = alpha, beta, Re; shift[p] = sigma as
-// (re, im)) of the base flow `base`: with A_p = sigma_p M + L_p (one LU per pencil),
-//   T[p]  = A_p^-1 [S1S0 on the u, v, w momentum rows]   ((4N + 7) x 3N),
-//   RH[p] = A_p^-H [e_0 .. e_{3N-1}]                      ((4N + 7) x 3N),
-// both row-major with interleaved (re, im); RH by the adjoint solve with the same factors.
-// The first 3N rows of T are the prognostic shift-invert operator Phi(sigma), and row i of RH
-// holds conj((A^-1)[r][i]) for r < 3N.  Returns false (and sets err) if a pencil is singular.
-bool build_evp(const rbhost::Operators& o, int base, int P, const double* prm, const double* shift,
-               std::vector<double>& T, std::vector<double>& RH, std::string* err);
+// The banded form A' split by its parameters, for kernels that assemble it themselves:
+//   A' = E[kPartConst] + (a0 + nu k^2) E[kPartShift] + nu E[kPartVisc]
+//        + i alpha E[kPartAlpha] + i beta E[kPartBeta],  k^2 = alpha^2 + beta^2,
+// each part real, its entry (i, k) at E[((t nv) + i) (kl + ku + 1) + k - i + kl].  mean: the
+// structure of the (0, 0) pencil (gauge row and pressure recombination).
+enum { kPartConst = 0, kPartShift, kPartVisc, kPartAlpha, kPartBeta, kBandParts };
+void band_parts(const rbhost::Operators& o, int base, bool mean, int& kl, int& ku, std::vector<double>& E);
+// weight of the mean pencil's pressure recombination: psi_j = T_j - weight T_{j+2}, even j
+double pressure_weight(int j);
 
 }  // namespace couhost
 }  // namespace spadj

@@ -3,24 +3,30 @@
 // sensitivity example).
 //
 // Pencil p has wavenumbers (alpha_p, beta_p), Reynolds number Re_p and a complex shift
-// sigma_p.  The host factorises A_p = sigma_p M + L_p once (couette_setup.cpp, build_evp) and
-// keeps T_p = A_p^-1 [S1S0 on the momentum rows] and RH_p = A_p^-H [e_0..e_{3N-1}] (the
-// adjoint solve with the same factors).  The prognostic block Phi_p (first 3N rows of T_p)
-// has eigenvalues mu = 1 / (sigma_p - lambda), so on the GPU:
+// sigma_p.  With A_p = sigma_p M + L_p, the prognostic block of Phi_p = A_p^-1 [S1S0 on the
+// momentum rows] has eigenvalues mu = 1 / (sigma_p - lambda).  On the GPU, per pencil:
 //
-//   1. shift-invert power iteration on Phi_p for the right eigenvector x and, in the same pass
-//      over Phi_p, on Phi_p^H for the left eigenvector psi (the adjoint eigenproblem); the
-//      two-sided Rayleigh quotient mu = psi^H Phi x / psi^H x gives lambda = sigma - 1/mu;
-//   2. the full eigenvectors X = T_p x (velocity, pressure, tau variables) and
-//      Y = RH_p psi, which solve (lambda M + L) X = 0 and (conj(lambda) M^H + L^H) Y = 0;
-//   3. eq. eigenvalue_sens, dlambda/dp = -<Y, dL/dp X> / <Y, M X> for p = Re, alpha, beta
+//   1. A_p and A_p^H in the banded form of couette_setup.h (recombined Chebyshev columns, ordered by mode),
+//      from real parts tabled once per problem, and their band LU with partial pivoting;
+//   2. shift-invert power iteration with the factors: x <- Phi_p x for the right eigenvector and
+//      psi <- Phi_p^H psi (the adjoint eigenproblem) side by side; the two-sided Rayleigh quotient
+//      mu = psi^H Phi x / psi^H x gives lambda = sigma - 1/mu;
+//   3. the full eigenvectors X = A^-1 [S1S0 x] (velocity, pressure, tau variables) and
+//      Y = A^-H [psi], which solve (lambda M + L) X = 0 and (conj(lambda) M^H + L^H) Y = 0;
+//   4. eq. eigenvalue_sens, dlambda/dp = -<Y, dL/dp X> / <Y, M X> for p = Re, alpha, beta
 //      (M does not depend on them), with dL/dp applied from the N x N ultraspherical blocks.
+//
+// Why banded: 96 pencils with 20 iterations at N = 48 took 22.7 ms with dense inverses (one LU and 6N solves of
+// 4N + 7 unknowns per pencil on the host's 16 cores, 21 ms of it) and take 2.2 ms now; on the GPU the
+// inverses would be 10 GFLOP, 10 ms at its FP64 rate.
+#include <algorithm>
 #include <cmath>
 #include <complex>
 #include <string>
 #include <vector>
 
 #include "couette_setup.h"
+#include "pdl.cuh"
 #include "problem.h"
 #include "rb_setup.h"
 
@@ -29,7 +35,9 @@ namespace {
 
 constexpr int kEvpThreads = 256;
 constexpr int kEvpWarps = kEvpThreads / 32;
-constexpr int kEvpMaxChunks = 12;  // 3N <= 384: N <= 128
+constexpr int kEvpMaxN = 128;      // largest N
+constexpr int kEvpMaxLower = 31;   // lower band width: a warp holds the elimination front's rows
+constexpr int kEvpMaxUpper = 64;   // width of U with its fill: two entries per lane of a warp
 constexpr int kEvpOut = 10;        // lambda, dlambda/dRe, dlambda/dalpha, dlambda/dbeta, residuals
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -38,9 +46,9 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Deterministic block sum of NV values per thread (fixed warp-then-block order); every thread
-// receives the totals.  red holds kEvpWarps * NV doubles.
-template <int NV>
+// Deterministic sum of NV values per thread over the CTA's NW warps (fixed warp-then-block order); every
+// thread receives the totals.  red holds NW * NV doubles.
+template <int NV, int NW>
 __device__ __forceinline__ void block_sum(double (&v)[NV], double* red) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -53,132 +61,400 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double* red) {
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
     double s = 0.0;
-    for (int w = 0; w < kEvpWarps; ++w) s += red[w * NV + i];
+    for (int w = 0; w < NW; ++w) s += red[w * NV + i];
     v[i] = s;
   }
 }
 
-constexpr int kRows = 4;       // rows per warp block in evp_iter_kernel (2 kRows partial sums per lane)
-constexpr int kRowsLog2V = 3;  // log2(2 kRows)
+// The banded systems of a call: system s = 2 p is A' of pencil p, s = 2 p + 1 is J A'^H J (the adjoint direction,
+// see couette_setup.h), each of nv unknowns with kl entries below and ku above the diagonal.
+struct EvpBand {
+  int N, nv, nvp, kl, ku;    // nvp: nv rounded up to whole chunks of sweep steps
+  const double *E0, *E1;     // [kBandParts][nv][kl + ku + 1] of the pencils with k != 0 and of the mean pencil
+  const double* prm;         // [P][3]: alpha, beta, Re
+  const double* shift;       // [P][2]
+  double2* B;                // [2P][nv][kl + ku + 1] assembled
+  double2* L;                // [2P][nvp][kl] multipliers by column (0 from nv on)
+  double2* U;                // [2P][nvp][kl + ku]: U_{j-1-k,j} / U_{j-1-k,j-1-k}, 0 where there is none
+  double2* dinv;             // [2P][nv]: 1 / U_jj
+  unsigned char* piv;        // [2P][nv]: pivot row - j
+  int* width;                // [2P]: largest k + 1 of a non-zero U entry
+  int* bad;                  // [P + 1]: singular pencils, and whether there is one
+  __device__ __forceinline__ bool mean(int p) const { return prm[3 * p] == 0.0 && prm[3 * p + 1] == 0.0; }
+};
 
-// Warp reduction of 2 kRows values per lane at once: a butterfly in which every exchange halves
-// the values a lane carries (offsets 16, 8, ...; the lane keeps the half selected by that bit of
-// its index) until one is left, then plain exchanges at the remaining offsets.  Every lane of the
-// group l >> (5 - kRowsLog2V) = m ends with the total of value m.  2 kRows + 1 additions per lane
-// for 2 kRows sums instead of 5 per sum; fixed order, so deterministic.
-__device__ __forceinline__ double warp_reduce_rows(double (&v)[2 * kRows], int lane) {
-  int off = 16;
-#pragma unroll
-  for (int half = kRows; half >= 1; half >>= 1, off >>= 1) {
-    const bool hi = (lane & off) != 0;
-#pragma unroll
-    for (int j = 0; j < half; ++j) {
-      const double send = hi ? v[j] : v[j + half];
-      const double keep = hi ? v[j + half] : v[j];
-      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+__global__ void __launch_bounds__(kEvpThreads) evp_assemble_kernel(const EvpBand S) {
+  const int p = blockIdx.x >> 1, dir = blockIdx.x & 1, w = S.kl + S.ku + 1;
+  const double al = S.prm[3 * p], be = S.prm[3 * p + 1], nu = 1.0 / S.prm[3 * p + 2];
+  const double* E = S.mean(p) ? S.E1 : S.E0;
+  const size_t part = (size_t)S.nv * w;
+  const double sr = S.shift[2 * p] + nu * (al * al + be * be), si = S.shift[2 * p + 1];
+  double2* B = S.B + (size_t)blockIdx.x * part;
+  for (int i = threadIdx.x; i < S.nv * w; i += blockDim.x) {
+    const int r = i / w, d = i - r * w, k = r - S.kl + d;
+    double2 v = make_double2(0.0, 0.0);
+    if (k >= 0 && k < S.nv) {
+      // entry (r, k) of J A'^H J is the conjugate of A'_{nv-1-k, nv-1-r}, on the same diagonal
+      const double* e = E + (size_t)(dir ? S.nv - 1 - k : r) * w + d;
+      const double es = __ldg(e + couhost::kPartShift * part);
+      v.x = fma(nu, __ldg(e + couhost::kPartVisc * part), fma(sr, es, __ldg(e)));
+      v.y = fma(be, __ldg(e + couhost::kPartBeta * part), fma(al, __ldg(e + couhost::kPartAlpha * part), si * es));
+      if (dir) v.y = -v.y;
     }
+    B[i] = v;
   }
-  double t = v[0];
+}
+
+__device__ __forceinline__ bool is_zero(double2 v) {
+  return (((unsigned)__double2hiint(v.x) << 1) | (unsigned)__double2loint(v.x) | ((unsigned)__double2hiint(v.y) << 1) |
+          (unsigned)__double2loint(v.y)) == 0u;
+}
+__device__ __forceinline__ double2 cinverse(double2 v) {  // 1 / v, scaled where |v|^2 could leave the range
+  double s = 1.0;
+  const unsigned e = max((unsigned)__double2hiint(v.x) & 0x7ff00000u, (unsigned)__double2hiint(v.y) & 0x7ff00000u) >> 20;
+  if (e - 600u > 800u && e != 0x7ffu && e != 0u) {
+    s = __hiloint2double((int)((2046u - e) << 20), 0);
+    v = make_double2(v.x * s, v.y * s);
+  }
+  const double q = s / fma(v.x, v.x, v.y * v.y);
+  return make_double2(v.x * q, -v.y * q);
+}
+__device__ __forceinline__ double2 csub_mul(double2 y, double2 f, double2 x) {  // y - f x
+  return make_double2(fma(-f.x, x.x, fma(f.y, x.y, y.x)), fma(-f.x, x.y, fma(-f.y, x.x, y.y)));
+}
+
+// Band LU of one system per CTA.  The kl + 1 rows of the elimination front and the next two rows sit in shared
+// memory, addressed through slot numbers (an interchange swaps two slots) with the columns modulo Wc.  Step j is
+// one barrier: warps 1.. update the columns beyond j + 1, scale and store row j of U and load a row, while warp 0
+// updates column j + 1 alone, picks its pivot, divides and publishes the multipliers of step j + 1.
+// Bound by FP64 issue: an FP64 instruction of a warp takes 64 clocks of its SM partition whatever its active
+// lanes, so warp 0's chain (update, reciprocal, multipliers: about 20 of them) runs beside the update
+// (4 per row and 32 columns, rows of zero multipliers and columns beyond the pivot row's extent skipped):
+// 0.31 ms for the 192 systems of 96 pencils at N = 48.
+__global__ void __launch_bounds__(kEvpThreads) evp_lu_kernel(const EvpBand S) {
+  const int nv = S.nv, kl = S.kl, ku = S.ku, w = kl + ku + 1, Wc = w + 1, kuf = kl + ku;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tid = threadIdx.x;
+  const double2* B = S.B + (size_t)blockIdx.x * nv * w;
+  double2* Lo = S.L + (size_t)blockIdx.x * S.nvp * kl;
+  double2* Uo = S.U + (size_t)blockIdx.x * S.nvp * kuf;
+  double2* Do = S.dinv + (size_t)blockIdx.x * nv;
+  unsigned char* Po = S.piv + (size_t)blockIdx.x * nv;
+  extern __shared__ double2 evsm[];
+  double2* ring = evsm;                                       // [kl + 3][Wc]
+  double2* mul = ring + (size_t)(kl + 3) * Wc;                // [2][32] multipliers of the step, [.][0] = 1 / pivot
+  int* slot = reinterpret_cast<int*>(mul + 64);               // [2][34]: rows j..j+kl, row j+1+kl, the free slot
+  int* ext = slot + 68;                                       // [kl + 3] last non-zero column of a slot's row
+  const double2 zero = make_double2(0.0, 0.0);
+  auto load_row = [&](int r, int s, int first, int step) {  // columns r - kl .. r + ku, and zero in the column after
+    for (int d = first; d < Wc; d += step) {
+      int c = (r - kl + d) % Wc;
+      if (c < 0) c += Wc;
+      ring[s * Wc + c] = d < w && r < nv ? __ldg(B + (size_t)r * w + d) : zero;
+    }
+    if (first == 0) ext[s] = r < nv ? min(nv - 1, r + ku) : -1;
+  };
+  // warp 0: pivot and multipliers of step j from lane k's entry a of row j + k (slot t), into buffer b
+  auto panel = [&](int j, double2 a, int t, int b) {
+    const unsigned hi = max((unsigned)__double2hiint(a.x) & 0x7fffffffu, (unsigned)__double2hiint(a.y) & 0x7fffffffu);
+    unsigned key = lane <= kl ? (hi & ~31u) | (unsigned)(31 - lane) : 0u;  // the first of the largest
 #pragma unroll
-  for (int o = 16 >> kRowsLog2V; o >= 1; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  return t;
+    for (int o = 16; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
+    const int p = 31 - (int)(key & 31u);
+    const double2 ap = make_double2(__shfl_sync(0xffffffffu, a.x, p), __shfl_sync(0xffffffffu, a.y, p));
+    const double2 a0 = make_double2(__shfl_sync(0xffffffffu, a.x, 0), __shfl_sync(0xffffffffu, a.y, 0));
+    const int tp = __shfl_sync(0xffffffffu, t, p), t0 = __shfl_sync(0xffffffffu, t, 0);
+    if (lane == p) { a = a0; t = t0; }
+    if (lane == 0) { a = ap; t = tp; }
+    const bool sing = is_zero(ap);
+    const double2 inv = sing ? zero : cinverse(ap);
+    const double2 l = make_double2(a.x * inv.x - a.y * inv.y, a.x * inv.y + a.y * inv.x);
+    if (lane <= kl) {
+      slot[b * 34 + lane] = t;
+      mul[b * 32 + lane] = lane == 0 ? inv : l;
+      if (lane > 0) Lo[(size_t)j * kl + lane - 1] = l;
+    }
+    if (lane == 0) {
+      Do[j] = inv;
+      Po[j] = (unsigned char)p;
+      if (sing) S.bad[blockIdx.x >> 1] = S.bad[gridDim.x >> 1] = 1;
+    }
+  };
+  for (int i = tid; i < (S.nvp - nv) * kl; i += blockDim.x) Lo[(size_t)nv * kl + i] = zero;
+  for (int i = tid; i < (S.nvp - nv) * kuf; i += blockDim.x) Uo[(size_t)nv * kuf + i] = zero;
+  for (int c = warp; c < min(kuf, nv); c += kEvpWarps)
+    for (int q = c + lane; q < kuf; q += 32) Uo[(size_t)c * kuf + q] = zero;
+  for (int r = warp; r < kl + 2; r += kEvpWarps) load_row(r, r, lane, 32);
+  __syncthreads();
+  if (warp == 0) {
+    panel(0, lane <= kl ? ring[lane * Wc] : zero, lane, 0);
+    if (lane == 0) { slot[kl + 1] = kl + 1; slot[kl + 2] = kl + 2; }
+  }
+  __syncthreads();
+  int jc = 0, width = 0;  // jc = j mod Wc
+  for (int j = 0; j < nv; ++j) {
+    const int b = j & 1;
+    const int* sl = slot + b * 34;
+    const double2* m = mul + b * 32;
+    const int s0 = sl[0], e0 = ext[s0];
+    const double2* piv = ring + s0 * Wc;
+    auto pos = [&](int q) { return jc + q < Wc ? jc + q : jc + q - Wc; };  // column j + q, q < Wc
+    if (warp == 0) {
+      if (j + 1 < nv) {
+        const int t = lane <= kl ? sl[lane + 1] : 0;
+        double2 a = lane <= kl ? ring[t * Wc + pos(1)] : zero;
+        if (lane < kl) a = csub_mul(a, m[lane + 1], piv[pos(1)]);
+        if (lane == 0) {
+          slot[(b ^ 1) * 34 + kl + 1] = sl[kl + 2];
+          slot[(b ^ 1) * 34 + kl + 2] = s0;
+        }
+        panel(j + 1, a, t, b ^ 1);
+      }
+    } else {
+      if (warp == 1) load_row(j + 2 + kl, sl[kl + 2], lane, 32);
+      if (warp == 2)
+        for (int q = lane; q < kuf; q += 32) {
+          const int c = j + 1 + q;
+          if (c >= nv) break;
+          double2 u = zero;
+          if (c <= e0) {
+            const double2 v = piv[pos(q + 1)], inv = m[0];
+            u = make_double2(v.x * inv.x - v.y * inv.y, v.x * inv.y + v.y * inv.x);
+          }
+          Uo[(size_t)c * kuf + q] = u;
+        }
+      if (warp == 3 && lane >= 1 && lane <= kl) {
+        const int s = sl[lane];
+        ring[s * Wc + (jc == 0 ? Wc - 1 : jc - 1)] = zero;  // column j + w of the rows that stay
+        if (!is_zero(m[lane])) ext[s] = max(ext[s], e0);
+      }
+      for (int k = warp; k <= kl; k += kEvpWarps - 1) {
+        const double2 l = m[k];
+        if (is_zero(l)) continue;
+        double2* row = ring + sl[k] * Wc;
+        for (int c = j + 2 + lane; c <= e0; c += 32) {
+          const int q = pos(c - j);
+          row[q] = csub_mul(row[q], l, piv[q]);
+        }
+      }
+      width = max(width, e0 - j);
+    }
+    __syncthreads();
+    jc = jc + 1 < Wc ? jc + 1 : 0;
+  }
+  if (tid == 32) S.width[blockIdx.x] = width;
 }
 
 struct EvpIterArgs {
-  const double2* T;      // [P][nv][H]: rows 0..H-1 are Phi
-  double2* x;            // [P][H] right iterate (in / out)
-  double2* psi;          // [P][H] left iterate (in / out)
-  const double* shift;   // [P][2]
-  double* out;           // [P][kEvpOut]
-  int H, nv, n_iter;
+  EvpBand S;
+  const double* ssb;  // [N][5]: S1S0[n][n + d]
+  const double* pw;   // [N]: the mean pencil's pressure recombination
+  double2* x;         // [P][H] right iterate (in / out)
+  double2* psi;       // [P][H] left iterate (in / out)
+  double2* XY;        // [P][2][nv]: X, Y
+  double* out;        // [P][kEvpOut]
+  int n_iter;
 };
 
-// One CTA per pencil: n_iter steps of x <- Phi x / |Phi x|, psi <- Phi^H psi / |Phi^H psi| with
-// each row of Phi read once per step for both products (warps over rows, lanes over columns,
-// coalesced), all in shared memory between steps.
-// NC = ceil(3N / 32) column chunks per lane, fixed at compile time so that only the last chunk
-// carries a bounds predicate.
-template <int NC>
-__global__ void __launch_bounds__(kEvpThreads, 2) evp_iter_kernel(const EvpIterArgs A) {
-  const int p = blockIdx.x, H = A.H;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+constexpr int kIterThreads = 128, kIterWarps = 4;
+constexpr int kChunk = 8;                 // sweep steps whose factors are copied together
+constexpr int kPadLow = 64, kPadHigh = 32;  // entries around the unknowns that steps near the ends touch
+
+// The two warps of a direction meet (one named barrier each)
+__device__ __forceinline__ void pair_sync(int dir) {
+  if (dir) asm volatile("bar.sync 2, 64;" ::: "memory");
+  else asm volatile("bar.sync 1, 64;" ::: "memory");
+}
+
+// Dynamic shared memory of evp_iter_kernel: x, psi and their images, sums, unknowns, factors, 1 / U_jj, pivots
+inline int evp_padded(int nv) { return (nv + kChunk - 1) / kChunk * kChunk; }
+inline size_t iter_smem(int N, int kuf) {
+  const size_t nvp = evp_padded(4 * N + 7);
+  return sizeof(double2) * 12 * N + sizeof(double) * (kIterWarps * 6 + 4 * (kPadLow + nvp + kPadHigh)) +
+         sizeof(double2) * (4 * (size_t)kChunk * kuf + 2 * nvp) + 2 * (nvp + kChunk);
+}
+
+// One CTA per pencil: n_iter steps of x <- Phi x / |Phi x|, psi <- Phi^H psi / |Phi^H psi|, then X and Y.  Warps 0
+// and 1 run the solves with A', warps 2 and 3 those with J A'^H J; of each pair one warp holds the real parts of
+// the unknowns and one the imaginary ones, so a sweep step is two FP64 instructions deep (128 clocks of latency).
+// Bound by that chain: 2 nv steps per solve.  The factors are copied to shared memory a chunk of steps ahead and
+// the steps of a chunk are unrolled, with entries around the unknowns so that none needs a bounds check: 96 pencils,
+// N = 48, 20 iterations 2.29 ms with factors loaded from L2 step by step, 2.08 ms copied ahead, 1.78 ms unrolled.
+__global__ void __launch_bounds__(kIterThreads) evp_iter_kernel(const EvpIterArgs A) {
+  const EvpBand& S = A.S;
+  const int p = blockIdx.x, N = S.N, H = 3 * N, nv = S.nv, nvp = S.nvp, kl = S.kl, kuf = S.kl + S.ku;
+  if (S.bad[gridDim.x]) return;  // the call fails: nothing is written
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, dir = warp >> 1, im = warp & 1, t64 = tid & 63;
+  const bool mean = S.mean(p);
+  const int orow = mean ? 0 : 1;  // position of mode 0's equations
   extern __shared__ double2 evsm[];
   double2* x = evsm;
   double2* ps = x + H;
   double2* y = ps + H;
-  double2* zp = y + H;                                    // [kEvpWarps][H] partial Phi^H psi
-  double* red = reinterpret_cast<double*>(zp + (size_t)kEvpWarps * H);
-  const double2* Tp = A.T + (size_t)p * A.nv * H;
-  for (int k = threadIdx.x; k < H; k += blockDim.x) {
+  double2* z = y + H;
+  double* red = reinterpret_cast<double*>(z + H);       // [kIterWarps * 6]
+  const int ld = kPadLow + nvp + kPadHigh;
+  double* sol = red + kIterWarps * 6 + dir * 2 * ld + kPadLow;    // this direction's unknowns: real parts,
+  double* mine = sol + im * ld;                                   // imaginary parts ld later
+  const double* other = sol + (im ^ 1) * ld;
+  double2* after = reinterpret_cast<double2*>(red + kIterWarps * 6 + 4 * ld);
+  double2* fac = after + dir * 2 * kChunk * kuf;                  // [2][kChunk][kuf] factors of two chunks of steps
+  double2* dinv = after + 4 * kChunk * kuf + dir * nvp;           // [nv]
+  unsigned char* pv = reinterpret_cast<unsigned char*>(after + 4 * kChunk * kuf + 2 * nvp) + dir * (nvp + kChunk);
+  const size_t sys = 2 * (size_t)p + dir;
+  const double2* Lp = S.L + sys * nvp * kl;
+  const double2* Up = S.U + sys * nvp * kuf;
+  const double2* Dp = S.dinv + sys * nv;
+  const unsigned char* Pp = S.piv + sys * nv;
+  const int wu = min(S.width[sys], kuf);
+  const double2 zero = make_double2(0.0, 0.0);
+  // right-hand side of this direction from v (H entries), by its 64 threads
+  auto fill = [&](const double2* v) {
+    for (int i = t64; i < 2 * ld; i += 64) sol[i - kPadLow] = 0.0;
+    pair_sync(dir);
+    for (int c = t64; c < H; c += 64) {
+      const int f = c / N, n = c - f * N;
+      double2 r = zero;
+      int q;
+      if (dir == 0) {
+        for (int d = 0; d < 5 && n + d < N; ++d) {
+          const double s = __ldg(A.ssb + n * 5 + d);
+          r.x = fma(s, v[c + d].x, r.x);
+          r.y = fma(s, v[c + d].y, r.y);
+        }
+        q = orow + 4 * n + f;
+      } else {
+        r = v[c];
+        if (n + 2 < N) r = make_double2(r.x - v[c + 2].x, r.y - v[c + 2].y);
+        q = nv - 1 - (1 + 4 * n + f);
+      }
+      sol[q] = r.x;
+      sol[ld + q] = r.y;
+    }
+    pair_sync(dir);
+  };
+  // a factor as this warp uses it: f x has the parts f.x xr - f.y xi and f.x xi + f.y xr
+  auto part = [&](double2 f) {
+    return make_double2(f.x, __hiloint2double(__double2hiint(f.y) ^ (im ? (int)0x80000000 : 0), __double2loint(f.y)));
+  };
+  // v - f x: xa is x's part of this warp, xb the other one (two dependent FP64 instructions)
+  auto sub = [&](double v, double2 f, double xa, double xb) { return fma(-f.x, xa, fma(f.y, xb, v)); };
+  // rows r0 .. r0 + n - 1 of a factor with wd entries per row into buffer b, by this direction's threads
+  auto copy = [&](const double2* src, int wd, int r0, int n, int b) {
+    double2* to = fac + b * kChunk * kuf;
+    for (int i = t64; i < n * wd; i += 64) cp_async16(to + i, src + (size_t)r0 * wd + i);
+    cp_async_commit();
+  };
+  const int chunks = nvp / kChunk;
+  auto solve = [&]() {
+    // forward: the interchange of step j + 1 is made by where step j writes its results
+    if (lane == 0 && pv[0]) {
+      const double a = mine[0];
+      mine[0] = mine[pv[0]];
+      mine[pv[0]] = a;
+    }
+    copy(Lp, kl, 0, kChunk, 0);
+    for (int c = 0; c < chunks; ++c) {
+      cp_async_wait_all();
+      pair_sync(dir);
+      if (c + 1 < chunks) copy(Lp, kl, (c + 1) * kChunk, kChunk, (c + 1) & 1);
+      const double2* F = fac + (c & 1) * kChunk * kuf + lane;
+      double* m = mine + c * kChunk;
+      const double* o = other + c * kChunk;
+      double2 f[kChunk];
+      int to[kChunk];
+#pragma unroll
+      for (int a = 0; a < kChunk; ++a) {
+        f[a] = part(lane < kl ? F[a * kl] : zero);
+        const int pc = pv[c * kChunk + a + 1];
+        to[a] = lane == 0 ? pc : lane == pc ? 0 : lane;
+      }
+#pragma unroll
+      for (int a = 0; a < kChunk; ++a) {
+        if (a > 0) pair_sync(dir);
+        const double v = sub(m[a + 1 + lane], f[a], m[a], o[a]);
+        __syncwarp();
+        m[a + 1 + to[a]] = v;
+      }
+    }
+    pair_sync(dir);
+    copy(Up, kuf, (chunks - 1) * kChunk, kChunk, 0);
+    for (int i = t64; i < nv; i += 64) {
+      const double2 d = dinv[i];
+      const double a = sol[i], c = sol[ld + i];
+      sol[i] = a * d.x - c * d.y;
+      sol[ld + i] = a * d.y + c * d.x;
+    }
+    for (int c = chunks - 1, b = 0; c >= 0; --c, b ^= 1) {
+      cp_async_wait_all();
+      pair_sync(dir);
+      if (c > 0) copy(Up, kuf, (c - 1) * kChunk, kChunk, b ^ 1);
+      const double2* F = fac + b * kChunk * kuf + lane;
+      double* m = mine + c * kChunk;
+      const double* o = other + c * kChunk;
+      double2 f[kChunk], g[kChunk];  // entries lane and lane + 32 (fill of the interchanges: few are non-zero)
+      unsigned far = 0u;
+#pragma unroll
+      for (int a = 0; a < kChunk; ++a) {
+        f[a] = part(lane < wu ? F[a * kuf] : zero);
+        g[a] = lane + 32 < wu ? F[a * kuf + 32] : zero;
+        if (!is_zero(g[a])) far |= 1u << a;
+        g[a] = part(g[a]);
+      }
+#pragma unroll
+      for (int s = 16; s > 0; s >>= 1) far |= __shfl_xor_sync(0xffffffffu, far, s);
+#pragma unroll
+      for (int a = kChunk - 1; a >= 0; --a) {
+        if (a < kChunk - 1) pair_sync(dir);
+        const double xa = m[a], xb = o[a];
+        double* e = m + a - 1 - lane;
+        e[0] = sub(e[0], f[a], xa, xb);
+        if (far >> a & 1u) e[-32] = sub(e[-32], g[a], xa, xb);
+      }
+    }
+    pair_sync(dir);
+  };
+  auto at = [&](int i) { return make_double2(sol[i], sol[ld + i]); };
+  for (int i = t64; i < nv; i += 64) dinv[i] = __ldg(Dp + i);
+  for (int i = t64; i < nvp + kChunk; i += 64) pv[i] = i < nv ? __ldg(Pp + i) : 0;
+  for (int k = tid; k < H; k += kIterThreads) {
     x[k] = A.x[(size_t)p * H + k];
     ps[k] = A.psi[(size_t)p * H + k];
   }
   double mur = 0.0, mui = 0.0, res_r = 1.0, res_l = 1.0;
   for (int it = 0; it < A.n_iter; ++it) {
     __syncthreads();
-    double2 zacc[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) zacc[c] = make_double2(0.0, 0.0);
-    // blocks of kRows rows per warp: each x chunk is read once per block, and the row sums of
-    // the block are reduced together (warp_reduce_rows) instead of one butterfly per row
-    for (int rb = warp * kRows; rb < H; rb += kRows * kEvpWarps) {
-      double acc[2 * kRows];
-      double2 pr[kRows];
-#pragma unroll
-      for (int i = 0; i < kRows; ++i) {
-        acc[2 * i] = acc[2 * i + 1] = 0.0;
-        pr[i] = rb + i < H ? ps[rb + i] : make_double2(0.0, 0.0);
-      }
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const int k = c * 32 + lane;
-        if (c < NC - 1 || k < H) {
-          const double2 xv = x[k];
-#pragma unroll
-          for (int i = 0; i < kRows; ++i) {
-            if (rb + i >= H) continue;
-            const double2 t = __ldg(&Tp[(size_t)(rb + i) * H + k]);
-            acc[2 * i] = fma(t.x, xv.x, acc[2 * i]);
-            acc[2 * i] = fma(-t.y, xv.y, acc[2 * i]);
-            acc[2 * i + 1] = fma(t.x, xv.y, acc[2 * i + 1]);
-            acc[2 * i + 1] = fma(t.y, xv.x, acc[2 * i + 1]);
-            zacc[c].x = fma(t.x, pr[i].x, zacc[c].x);  // conj(t) * psi_r
-            zacc[c].x = fma(t.y, pr[i].y, zacc[c].x);
-            zacc[c].y = fma(t.x, pr[i].y, zacc[c].y);
-            zacc[c].y = fma(-t.y, pr[i].x, zacc[c].y);
-          }
+    fill(dir == 0 ? x : ps);
+    solve();
+    for (int c = t64; c < H; c += 64) {
+      const int f = c / N, n = c - f * N;
+      if (dir == 0) {
+        double2 v = at(1 + 4 * n + f);
+        if (n >= 2) v = make_double2(v.x - sol[1 + 4 * (n - 2) + f], v.y - sol[ld + 1 + 4 * (n - 2) + f]);
+        y[c] = v;
+      } else {
+        double2 v = zero;
+        for (int d = 0; d < 5 && n - d >= 0; ++d) {
+          const double s = __ldg(A.ssb + (n - d) * 5 + d);
+          const double2 q = at(nv - 1 - (orow + 4 * (n - d) + f));
+          v.x = fma(s, q.x, v.x);
+          v.y = fma(s, q.y, v.y);
         }
+        z[c] = v;
       }
-      const double tot = warp_reduce_rows(acc, lane);
-      // lane group m = lane >> (5 - kRowsLog2V) holds value m = 2 (row - rb) + component
-      const int m = lane >> (5 - kRowsLog2V), r = rb + (m >> 1);
-      if ((lane & ((1 << (5 - kRowsLog2V)) - 1)) == 0 && r < H) reinterpret_cast<double*>(y)[2 * r + (m & 1)] = tot;
-    }
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      const int k = c * 32 + lane;
-      if (c < NC - 1 || k < H) zp[(size_t)warp * H + k] = zacc[c];
     }
     __syncthreads();
-    // z = sum of the warp partials (into zp row 0); norms and the two-sided Rayleigh quotient
+    // norms and the two-sided Rayleigh quotient
     double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int k = threadIdx.x; k < H; k += blockDim.x) {
-      double2 z = zp[k];
-      for (int w = 1; w < kEvpWarps; ++w) {
-        const double2 q = zp[(size_t)w * H + k];
-        z.x += q.x;
-        z.y += q.y;
-      }
-      zp[k] = z;
-      const double2 yk = y[k], xk = x[k], pk = ps[k];
+    for (int k = tid; k < H; k += kIterThreads) {
+      const double2 yk = y[k], zk = z[k], xk = x[k], pk = ps[k];
       v[0] = fma(yk.x, yk.x, fma(yk.y, yk.y, v[0]));
-      v[1] = fma(z.x, z.x, fma(z.y, z.y, v[1]));
+      v[1] = fma(zk.x, zk.x, fma(zk.y, zk.y, v[1]));
       v[2] += pk.x * yk.x + pk.y * yk.y;  // psi^H y
       v[3] += pk.x * yk.y - pk.y * yk.x;
       v[4] += pk.x * xk.x + pk.y * xk.y;  // psi^H x
       v[5] += pk.x * xk.y - pk.y * xk.x;
     }
-    block_sum<6>(v, red);
+    block_sum<6, kIterWarps>(v, red);
     const double dd = v[4] * v[4] + v[5] * v[5];
     if (dd > 0.0) {
       mur = (v[2] * v[4] + v[3] * v[5]) / dd;
@@ -186,71 +462,61 @@ __global__ void __launch_bounds__(kEvpThreads, 2) evp_iter_kernel(const EvpIterA
     }
     if (it + 1 == A.n_iter) {  // residuals |Phi x - mu x| / |Phi x|, |Phi^H psi - conj(mu) psi| / |Phi^H psi|
       double r2[2] = {0.0, 0.0};
-      for (int k = threadIdx.x; k < H; k += blockDim.x) {
-        const double2 yk = y[k], xk = x[k], pk = ps[k], z = zp[k];
+      for (int k = tid; k < H; k += kIterThreads) {
+        const double2 yk = y[k], xk = x[k], pk = ps[k], zk = z[k];
         const double ex = yk.x - (mur * xk.x - mui * xk.y), ey = yk.y - (mur * xk.y + mui * xk.x);
-        const double fx = z.x - (mur * pk.x + mui * pk.y), fy = z.y - (mur * pk.y - mui * pk.x);
+        const double fx = zk.x - (mur * pk.x + mui * pk.y), fy = zk.y - (mur * pk.y - mui * pk.x);
         r2[0] += ex * ex + ey * ey;
         r2[1] += fx * fx + fy * fy;
       }
-      block_sum<2>(r2, red);
+      block_sum<2, kIterWarps>(r2, red);
       res_r = v[0] > 0.0 ? sqrt(r2[0] / v[0]) : 1.0;
       res_l = v[1] > 0.0 ? sqrt(r2[1] / v[1]) : 1.0;
     }
     const double sy = v[0] > 0.0 ? 1.0 / sqrt(v[0]) : 0.0, sz = v[1] > 0.0 ? 1.0 / sqrt(v[1]) : 0.0;
-    for (int k = threadIdx.x; k < H; k += blockDim.x) {
-      const double2 yk = y[k], z = zp[k];
+    for (int k = tid; k < H; k += kIterThreads) {
+      const double2 yk = y[k], zk = z[k];
       x[k] = make_double2(yk.x * sy, yk.y * sy);
-      ps[k] = make_double2(z.x * sz, z.y * sz);
+      ps[k] = make_double2(zk.x * sz, zk.y * sz);
     }
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < H; k += blockDim.x) {
+  for (int k = tid; k < H; k += kIterThreads) {
     A.x[(size_t)p * H + k] = x[k];
     A.psi[(size_t)p * H + k] = ps[k];
   }
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     double* o = A.out + (size_t)p * kEvpOut;
     const double m2 = mur * mur + mui * mui;
     // lambda = sigma - 1/mu
-    o[0] = m2 > 0.0 ? A.shift[2 * p] - mur / m2 : 0.0;
-    o[1] = m2 > 0.0 ? A.shift[2 * p + 1] + mui / m2 : 0.0;
+    o[0] = m2 > 0.0 ? S.shift[2 * p] - mur / m2 : 0.0;
+    o[1] = m2 > 0.0 ? S.shift[2 * p + 1] + mui / m2 : 0.0;
     o[8] = res_r;
     o[9] = res_l;
   }
-}
-
-using EvpIterFn = void (*)(const EvpIterArgs);
-const EvpIterFn kEvpIter[kEvpMaxChunks] = {
-    evp_iter_kernel<1>, evp_iter_kernel<2>, evp_iter_kernel<3>, evp_iter_kernel<4>,
-    evp_iter_kernel<5>, evp_iter_kernel<6>, evp_iter_kernel<7>, evp_iter_kernel<8>,
-    evp_iter_kernel<9>, evp_iter_kernel<10>, evp_iter_kernel<11>, evp_iter_kernel<12>};
-
-// X = T x and Y = RH psi (length nv each) for every pencil: warps over rows, lanes over columns.
-__global__ void __launch_bounds__(kEvpThreads) evp_vectors_kernel(const double2* __restrict__ T,
-                                                                  const double2* __restrict__ RH,
-                                                                  const double2* __restrict__ x,
-                                                                  const double2* __restrict__ psi, int H, int nv,
-                                                                  double2* __restrict__ XY) {
-  const int p = blockIdx.x;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const double2* xp = x + (size_t)p * H;
-  const double2* pp = psi + (size_t)p * H;
-  for (int rr = warp; rr < 2 * nv; rr += kEvpWarps) {
-    const int which = rr / nv, r = rr - which * nv;
-    const double2* row = (which == 0 ? T : RH) + ((size_t)p * nv + r) * H;
-    const double2* v = which == 0 ? xp : pp;
-    double ax = 0.0, ay = 0.0;
-    for (int k = lane; k < H; k += 32) {
-      const double2 t = __ldg(&row[k]), q = __ldg(&v[k]);
-      ax = fma(t.x, q.x, ax);
-      ax = fma(-t.y, q.y, ax);
-      ay = fma(t.x, q.y, ay);
-      ay = fma(t.y, q.x, ay);
+  // X (unknowns u, v, w, p, tau_u1, ..., tau_w2, tau_p) and Y (equations u, v, w, continuity, boundary, gauge)
+  fill(dir == 0 ? x : ps);
+  solve();
+  double2* o = A.XY + sys * nv;
+  for (int i = t64; i < nv; i += 64) {
+    const int f = i / N, n = i - f * N;
+    double2 v;
+    if (dir == 0) {
+      if (f < 4) {
+        v = at(1 + 4 * n + f);
+        if (n >= 2 && (f < 3 || (mean && n % 2 == 0))) {
+          const double s = f < 3 ? 1.0 : __ldg(A.pw + n - 2);
+          const double2 u = at(1 + 4 * (n - 2) + f);
+          v = make_double2(v.x - s * u.x, v.y - s * u.y);
+        }
+      } else {
+        v = at(i == nv - 1 ? 0 : 1 + i);
+      }
+    } else {
+      const int q = f < 4 ? orow + 4 * n + f : i < nv - 1 ? orow + i : mean ? nv - 1 : 0;
+      v = at(nv - 1 - q);
     }
-    ax = warp_sum(ax);
-    ay = warp_sum(ay);
-    if (lane == 0) XY[((size_t)p * 2 + which) * nv + r] = make_double2(ax, ay);
+    o[i] = v;
   }
 }
 
@@ -259,6 +525,7 @@ struct EvpSensArgs {
   const double* prm;                 // [P][3]: alpha, beta, Re
   const double *SS, *DD, *Um, *S0;   // N x N row-major
   double* out;                       // [P][kEvpOut]
+  const int* bad;                    // non-zero: the call fails, nothing is written
   int N, nv, lift_row;
   double lift_val;
 };
@@ -270,6 +537,7 @@ struct EvpSensArgs {
 // <Y, M X> = sum over u, v, w of Y_q^H SS X_q.
 __global__ void __launch_bounds__(kEvpThreads) evp_sens_kernel(const EvpSensArgs A) {
   const int p = blockIdx.x, N = A.N, nv = A.nv;
+  if (*A.bad) return;
   extern __shared__ double2 essm[];
   double2* X = essm;
   double2* Y = X + nv;
@@ -324,7 +592,7 @@ __global__ void __launch_bounds__(kEvpThreads) evp_sens_kernel(const EvpSensArgs
       const double2 xt = X[4 * N + 2 * q];
       cjmul_add(&v[2], Y[q * N + A.lift_row], make_double2(A.lift_val * xt.x, A.lift_val * xt.y));
     }
-  block_sum<8>(v, red);
+  block_sum<8, kEvpWarps>(v, red);
   if (threadIdx.x == 0) {
     double* o = A.out + (size_t)p * kEvpOut;
     const double dr = v[0], di = v[1], dd = dr * dr + di * di;
@@ -341,7 +609,8 @@ __global__ void __launch_bounds__(kEvpThreads) evp_sens_kernel(const EvpSensArgs
 struct ShearEvp : EqImpl {
   int N = 0, H = 0, nv = 0, base = 0, Pmax = 0;
   rbhost::Operators ops;
-  DevBuf T, RH, XY, shiftd, prmd, mats;
+  int kl = 0, ku = 0;
+  DevBuf band, XY, args, mats;
 
   size_t state_len(int which) const override { return which == 0 ? (size_t)Pmax * H * 2 : 0; }
 
@@ -350,8 +619,8 @@ struct ShearEvp : EqImpl {
     N = d.n[2];
     base = (int)d.params[0];
     Pmax = d.batch;
-    if (N < 8 || 3 * N > 32 * kEvpMaxChunks)
-      return p->fail(SPADJ_ERR_INVALID, "shear evp: need 8 <= n[2] <= " + std::to_string(32 * kEvpMaxChunks / 3));
+    if (N < 8 || N > kEvpMaxN)
+      return p->fail(SPADJ_ERR_INVALID, "shear evp: need 8 <= n[2] <= " + std::to_string(kEvpMaxN));
     if ((base != 0 && base != 1) || (double)base != d.params[0])
       return p->fail(SPADJ_ERR_INVALID, "shear evp: params[0] must be 0 (plane Couette) or 1 (plane Poiseuille)");
     H = 3 * N;
@@ -364,12 +633,28 @@ struct ShearEvp : EqImpl {
     m.insert(m.end(), ops.DD.begin(), ops.DD.end());
     m.insert(m.end(), Um.begin(), Um.end());
     m.insert(m.end(), ops.S0.begin(), ops.S0.end());
+    // S1S0's band, the pressure recombination, and the parts of the banded pencil (both kinds of pencil at the same
+    // widths)
+    for (int n = 0; n < N; ++n)
+      for (int d = 0; d < 5; ++d) m.push_back(n + d < N ? ops.SS[(size_t)n * N + n + d] : 0.0);
+    for (int n = 0; n < N; ++n) m.push_back(n % 2 == 0 ? couhost::pressure_weight(n) : 0.0);
+    int l[2], u[2];
+    std::vector<double> E[2];
+    for (int k = 0; k < 2; ++k) couhost::band_parts(ops, base, k == 1, l[k], u[k], E[k]);
+    kl = std::max(l[0], l[1]);
+    ku = std::max(u[0], u[1]);
+    if (kl > kEvpMaxLower || kl + ku > kEvpMaxUpper) return p->fail(SPADJ_ERR_UNSUPPORTED, "shear evp: the pencil's band is wider than supported");
+    const int w = kl + ku + 1;
+    for (int k = 0; k < 2; ++k) {
+      const int wk = l[k] + u[k] + 1;
+      const size_t rows = E[k].size() / wk, o = m.size();
+      m.resize(o + rows * w, 0.0);
+      for (size_t r = 0; r < rows; ++r)
+        for (int d = 0; d < wk; ++d) m[o + r * w + d + kl - l[k]] = E[k][r * wk + d];
+    }
     SPADJ_CUDA_TRY(p, mats.ensure(sizeof(double) * m.size()));
     SPADJ_CUDA_TRY(p, cudaMemcpy(mats.ptr, m.data(), sizeof(double) * m.size(), cudaMemcpyHostToDevice));
-    const size_t ismem = sizeof(double2) * (size_t)(3 + kEvpWarps) * H + sizeof(double) * kEvpWarps * 6;
-    if (ismem > 48 * 1024)
-      SPADJ_CUDA_TRY(p, cudaFuncSetAttribute(kEvpIter[(H + 31) / 32 - 1],
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ismem));
+    SPADJ_CUDA_TRY(p, cudaFuncSetAttribute(evp_iter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)iter_smem(kEvpMaxN, kEvpMaxUpper)));
     return SPADJ_OK;
   }
 
@@ -380,43 +665,56 @@ struct ShearEvp : EqImpl {
     for (int i = 0; i < P; ++i)
       if (!(prm[3 * i + 2] > 0.0) || !std::isfinite(prm[3 * i]) || !std::isfinite(prm[3 * i + 1]))
         return p->fail(SPADJ_ERR_INVALID, "eigen: need finite wavenumbers and Re > 0");
-    std::vector<double> th, rh;
-    std::string err;
-    if (!couhost::build_evp(ops, base, P, prm, shift, th, rh, &err)) return p->fail(SPADJ_ERR_INVALID, err);
-    SPADJ_CUDA_TRY(p, T.ensure(sizeof(double) * th.size()));
-    SPADJ_CUDA_TRY(p, RH.ensure(sizeof(double) * rh.size()));
+    EvpBand S{};
+    S.N = N; S.nv = nv; S.nvp = evp_padded(nv); S.kl = kl; S.ku = ku;
+    const int w = kl + ku + 1, kuf = kl + ku;
+    const size_t nn = (size_t)N * N, part = (size_t)couhost::kBandParts * nv * w, ns = 2 * (size_t)P * S.nvp;
+    // per call: the arguments and flags, and the systems
+    SPADJ_CUDA_TRY(p, args.ensure(sizeof(double) * 5 * P + sizeof(int) * (3 * (size_t)P + 1)));
+    SPADJ_CUDA_TRY(p, band.ensure((sizeof(double2) * (w + kl + kuf + 1) + 1) * ns));
     SPADJ_CUDA_TRY(p, XY.ensure(sizeof(double2) * (size_t)P * 2 * nv));
-    SPADJ_CUDA_TRY(p, shiftd.ensure(sizeof(double) * 2 * P));
-    SPADJ_CUDA_TRY(p, prmd.ensure(sizeof(double) * 3 * P));
-    SPADJ_CUDA_TRY(p, cudaMemcpyAsync(T.ptr, th.data(), sizeof(double) * th.size(), cudaMemcpyHostToDevice, p->stream));
-    SPADJ_CUDA_TRY(p, cudaMemcpyAsync(RH.ptr, rh.data(), sizeof(double) * rh.size(), cudaMemcpyHostToDevice, p->stream));
-    SPADJ_CUDA_TRY(p, cudaMemcpyAsync(shiftd.ptr, shift, sizeof(double) * 2 * P, cudaMemcpyHostToDevice, p->stream));
-    SPADJ_CUDA_TRY(p, cudaMemcpyAsync(prmd.ptr, prm, sizeof(double) * 3 * P, cudaMemcpyHostToDevice, p->stream));
+    double* prmd = args.as<double>();
+    double* shiftd = prmd + 3 * P;
+    int* flags = reinterpret_cast<int*>(shiftd + 2 * P);
+    SPADJ_CUDA_TRY(p, cudaMemcpyAsync(prmd, prm, sizeof(double) * 3 * P, cudaMemcpyHostToDevice, p->stream));
+    SPADJ_CUDA_TRY(p, cudaMemcpyAsync(shiftd, shift, sizeof(double) * 2 * P, cudaMemcpyHostToDevice, p->stream));
+    SPADJ_CUDA_TRY(p, cudaMemsetAsync(flags, 0, sizeof(int) * (P + 1), p->stream));
+    const double* ssb = mats.as<double>() + 4 * nn;
+    S.E0 = ssb + 6 * N;
+    S.E1 = S.E0 + part;
+    S.prm = prmd;
+    S.shift = shiftd;
+    S.B = band.as<double2>();
+    S.L = S.B + ns * w;
+    S.U = S.L + ns * kl;
+    S.dinv = S.U + ns * kuf;
+    S.piv = reinterpret_cast<unsigned char*>(S.dinv + ns);
+    S.bad = flags;
+    S.width = flags + P + 1;
+    spadj_status s;
+    cudaEvent_t t0 = p->tic();
+    evp_assemble_kernel<<<2 * P, kEvpThreads, 0, p->stream>>>(S);
+    if ((s = check_launch(p, "evp assemble")) != SPADJ_OK) return s;
+    const size_t lsmem = sizeof(double2) * ((size_t)(kl + 3) * (w + 1) + 64) + sizeof(int) * (68 + kl + 3);
+    evp_lu_kernel<<<2 * P, kEvpThreads, lsmem, p->stream>>>(S);
+    if ((s = check_launch(p, "evp factorise")) != SPADJ_OK) return s;
     EvpIterArgs ia{};
-    ia.T = T.as<double2>();
+    ia.S = S;
+    ia.ssb = ssb;
+    ia.pw = ssb + 5 * N;
     ia.x = reinterpret_cast<double2*>(x);
     ia.psi = reinterpret_cast<double2*>(psi);
-    ia.shift = shiftd.as<double>();
+    ia.XY = XY.as<double2>();
     ia.out = out;
-    ia.H = H;
-    ia.nv = nv;
     ia.n_iter = n_iter;
-    const size_t ismem = sizeof(double2) * (size_t)(3 + kEvpWarps) * H + sizeof(double) * kEvpWarps * 6;
-    cudaEvent_t t0 = p->tic();
-    kEvpIter[(H + 31) / 32 - 1]<<<P, kEvpThreads, ismem, p->stream>>>(ia);
-    // two complex matvecs per step over the 3N x 3N block: 16 flops per entry
-    p->toc(t0, KC_SOLVE, 16.0 * (double)H * H * P * n_iter);
-    spadj_status s = check_launch(p, "evp iterate");
-    if (s != SPADJ_OK) return s;
-    cudaEvent_t t1 = p->tic();
-    evp_vectors_kernel<<<P, kEvpThreads, 0, p->stream>>>(T.as<double2>(), RH.as<double2>(), ia.x, ia.psi, H, nv,
-                                                         XY.as<double2>());
-    p->toc(t1, KC_OBJECTIVE, 16.0 * (double)nv * H * P);
-    if ((s = check_launch(p, "evp vectors")) != SPADJ_OK) return s;
+    evp_iter_kernel<<<P, kIterThreads, iter_smem(N, kuf), p->stream>>>(ia);
+    // two factorisations, and two banded solves per step and for the eigenvectors, 8 flops per factor entry
+    p->toc(t0, KC_SOLVE, 16.0 * nv * ((double)kl * (kl + ku) + (kl + ku + 1.0) * (n_iter + 1)) * P);
+    if ((s = check_launch(p, "evp iterate")) != SPADJ_OK) return s;
     EvpSensArgs sa{};
     sa.XY = XY.as<double2>();
-    sa.prm = prmd.as<double>();
-    const size_t nn = (size_t)N * N;
+    sa.prm = prmd;
+    sa.bad = flags + P;
     sa.SS = mats.as<double>();
     sa.DD = sa.SS + nn;
     sa.Um = sa.DD + nn;
@@ -431,8 +729,11 @@ struct ShearEvp : EqImpl {
     evp_sens_kernel<<<P, kEvpThreads, ssmem, p->stream>>>(sa);
     p->toc(t2, KC_OBJECTIVE, (12.0 * 4.0 * N * N + 64.0 * N) * P);
     if ((s = check_launch(p, "evp sensitivity")) != SPADJ_OK) return s;
-    // the host operator buffers must outlive the asynchronous copies
+    std::vector<int> bad(P + 1);
+    SPADJ_CUDA_TRY(p, cudaMemcpyAsync(bad.data(), flags, sizeof(int) * (P + 1), cudaMemcpyDeviceToHost, p->stream));
     SPADJ_CUDA_TRY(p, cudaStreamSynchronize(p->stream));
+    for (int i = 0; i < P; ++i)
+      if (bad[i]) return p->fail(SPADJ_ERR_INVALID, "eigen: singular shifted pencil matrix at pencil " + std::to_string(i));
     return SPADJ_OK;
   }
 
