@@ -37,7 +37,7 @@ struct FFTPlan {
   // transforms' unpacking factors, the passes' scalings, the parity of their number, and FP64 unpacking factors
   const int4 *fxp, *fxt, *fxr;
   const int* fxs;
-  int fxodd;
+  int fxodd, fxr0;  // whether the number of passes is odd, radix of the first one
   const double2* wm;
 };
 

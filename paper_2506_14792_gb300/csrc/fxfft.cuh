@@ -129,6 +129,19 @@ __host__ __device__ __forceinline__ void fx_out3(fx2& v0, fx2& v1, fx2& v2) {
   v1 = fx_add(m, r);
   v2 = fx_sub(m, r);
 }
+// Radix 6 as 2 x 3 (prime factors: no twiddles)
+__host__ __device__ __forceinline__ void fx_out6(fx2 (&v)[6]) {
+  fx2 a0 = v[0], a1 = v[2], a2 = v[4], b0 = v[3], b1 = v[5], b2 = v[1];
+  fx_out3(a0, a1, a2);
+  fx_out3(b0, b1, b2);
+  v[0] = fx_add(a0, b0);
+  v[3] = fx_sub(a0, b0);
+  v[4] = fx_add(a1, b1);
+  v[1] = fx_sub(a1, b1);
+  v[2] = fx_add(a2, b2);
+  v[5] = fx_sub(a2, b2);
+}
+
 // Fixed-point value of the double x: x = v 2^(emax + 1 - 1023 - B) to the last unit (toward zero; to the nearest for
 // the packed real spectra, whose many small entries would add up otherwise), |v| <= 2^B for biased exponents <= emax.  emax >= 128, so that whatever has a zero exponent field vanishes.
 template <int B>
@@ -217,10 +230,11 @@ inline int fx_schedule(unsigned long long radw, int kind, int l) {
   int bits = 0, tot = 0, b = kind == kFxInvReal ? 4 * kFxBReal + 10 : 4 * kFxB + 2;
   l *= 4;
   for (int i = 0; radw; ++i, radw >>= 8) {
-    const int R = (int)(radw & 0xff), grow = R == 4 ? 8 : R == 3 ? 7 : 4;
+    const int R = (int)(radw & 0xff), grow = R == 6 ? 11 : R == 4 ? 8 : R == 3 ? 7 : 4;
     int lim = 240;  // of a scaled operand: the sums of four products fit the words
     if (kind == kFxFwdReal && lim > 246 - grow) lim = 246 - grow;
-    const int sg = i > 0 && b > lim ? (b - lim + 3) / 4 : 0;
+    // pass 0 has no products: only its results have to fit (six times a packed real spectrum's bound may not)
+    const int sg = i > 0 ? (b > lim ? (b - lim + 3) / 4 : 0) : (b + grow < l ? b + grow : l) > 251 ? 1 : 0;
     bits |= sg << (2 * i);
     tot += sg;
     l -= 4 * sg;
@@ -266,10 +280,11 @@ inline std::vector<int4> fx_roots(int n) {
   }
   return r;
 }
-// Radices of the fixed-point passes, a byte each from the low end: the 3s first (the first pass then grows the
-// moduli least, which the packed real spectra need), then 4s, then a 2.  Radix 8 in place of the 4s needs fewer passes
-// but leaves half the lanes idle at these lengths (24 butterflies at n = 192): 16384 Burgers members of N = 256 take
-// 18.9 ms with it and 17.8 ms without.  0: no such plan (n without a factor 3, or above kFxMaxN).
+// Radices of the fixed-point passes, a byte each from the low end: a 6 (when the power of 2 is odd) or a 3 first,
+// without twiddles and with the least growth of the moduli, which the packed real spectra need; then the other 3s,
+// then 4s.  Radix 8 in place of the 4s needs fewer passes but leaves half the lanes idle at these lengths (24
+// butterflies at n = 192): 16384 Burgers members of N = 256 take 18.9 ms with it and 17.8 ms without.  0: no such
+// plan (n without a factor 3, or above kFxMaxN).
 inline unsigned long long fx_radices(int n) {
   if (n < 3 || n > kFxMaxN) return 0;
   unsigned long long w = 0;
@@ -278,18 +293,21 @@ inline unsigned long long fx_radices(int n) {
     w |= (unsigned long long)r << (8 * i++);
     m /= r;
   };
+  if (m % 3 != 0) return 0;
+  int two = 0;
+  for (int q = m; q % 2 == 0; q /= 2) ++two;
+  if (two % 2 == 1 && n != 6) push(6);
   while (m % 3 == 0 && i < 8) push(3);
-  if (i == 0) return 0;
   while (m % 4 == 0 && i < 8) push(4);
-  if (m % 2 == 0 && i < 8) push(2);
+  if (m % 2 == 0 && i < 8) push(2);  // n = 6: a single pass would leave too large values to unpack
   return m == 1 ? w : 0;
 }
 // One pass: butterfly j = q Ns + k of nbf reads entries j + r nbf of its input and writes q Ns R + k + r Ns;
-// mNs, mBf: 2^32 / Ns and 2^32 / nbf rounded up (division by multiplication); tw: offset of its twiddles.
+// mNs: 2^32 / Ns rounded up (division by multiplication); tw: offset of its twiddles.
 struct alignas(16) FxPass {
   int R, Ns, nbf, tw;
-  unsigned mNs, mBf;
-  int more, pad;
+  unsigned mNs;
+  int pad0, more, pad1;
 };
 inline std::vector<FxPass> fx_pass_list(int n) {
   std::vector<FxPass> v;
@@ -301,7 +319,6 @@ inline std::vector<FxPass> fx_pass_list(int n) {
     p.nbf = n / p.R;
     p.more = (w >> 8) != 0;
     p.mNs = Ns > 1 ? (unsigned)(((1ull << 32) + Ns - 1) / Ns) : 0u;
-    p.mBf = p.nbf > 1 ? (unsigned)(((1ull << 32) + p.nbf - 1) / p.nbf) : 0u;
     p.tw = tw;
     if (Ns > 1) tw += Ns * (p.R - 1);
     Ns *= p.R;
@@ -358,6 +375,7 @@ inline void fft_bind(FFTPlan& p, bool real, const double2* dev, const double2* w
     p.fxr = p.fxt + tw;
     p.fxs = reinterpret_cast<const int*>(p.fxr + p.n);
     p.fxodd = (int)ps.size() & 1;
+    p.fxr0 = ps[0].R;
     if (both) bind_scaled_twiddles(p, dev + np + tw + p.n + 3 * 32 / 4);
   } else {
     bind_scaled_twiddles(p, dev);
@@ -369,7 +387,7 @@ inline void fft_bind(FFTPlan& p, bool real, const double2* dev, const double2* w
 //
 // Buffers are offsets (in 16-byte entries) into the CTA's dynamic shared memory.  Sequence s of a call holds its
 // entries from a + s * stride (and the other buffer from b + s * stride); every buffer has n entries.  All
-// threads of the CTA (a multiple of 32, <= 256) call.
+// threads of the CTA (a multiple of 32, <= 256, divisible by the call's sequences: 1, 2, 4 or 8) call.
 
 __device__ __forceinline__ double2* fx_mem64() {
   extern __shared__ double2 fx_dyn[];
@@ -427,31 +445,55 @@ struct FxLay {
 __device__ __forceinline__ unsigned fx_absmax(unsigned m, double2 v) {
   return max(m, max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu));
 }
-// Reductions by shuffles over the lanes that agree modulo W (W = 1: the whole warp)
-template <int W = 1>
-__device__ __forceinline__ unsigned fx_warp_max(unsigned v) {
-#pragma unroll
-  for (int d = 16; d >= W; d >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, d));
-  return v;
+// The threads of a CTA share out over the NS sequences of a call: thread l of the T threads of sequence s, so that
+// whatever depends on the sequence (base, scale, scalings) is computed once per thread and call.  The T
+// threads are consecutive, or (W > 1: W = NS) every W-th one, for callers whose sequences are adjacent in memory.
+struct FxGroup {
+  int s, l, T;
+};
+template <int NS, int W>
+__device__ __forceinline__ FxGroup fx_group() {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  if (W > 1) return FxGroup{tid & (W - 1), tid / W, nt / W};
+  if (NS == 1) return FxGroup{0, tid, nt};
+  const int T = nt / NS, s = tid >> (31 - __clz(T));
+  return FxGroup{s, tid - s * T, T};
 }
-template <int W = 1>
-__device__ __forceinline__ unsigned fx_warp_sum(unsigned v) {
+// warps that hold threads of sequence s: first and one past the last
+template <int NS, int W>
+__device__ __forceinline__ int2 fx_warps(int s) {
+  const int nt = blockDim.x;
+  if (W > 1 || NS == 1) return make_int2(0, nt >> 5);
+  const int T = nt / NS, w = (s * T) >> 5;
+  return make_int2(w, max(w + 1, ((s + 1) * T) >> 5));
+}
+// Reductions by shuffles over the lanes of a sequence; its first lane writes the warp's value to the slot
+// (v[warp][s0 + s])
+template <int W>
+__device__ __forceinline__ void fx_reduce_max(FxGroup g, int s0, unsigned m) {
 #pragma unroll
-  for (int d = 16; d >= W; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-  return v;
+  for (int d = 16; d >= W; d >>= 1)
+    if (W > 1 || d < g.T) m = max(m, __shfl_xor_sync(0xffffffffu, m, d));
+  const int lane = threadIdx.x & 31;
+  if (W > 1 ? lane < W : (g.l & 31) == 0) sts32(&fx_shared().mx[threadIdx.x >> 5][s0 + g.s], m);
+}
+template <int W>
+__device__ __forceinline__ void fx_reduce_l1(FxGroup g, int s0, unsigned v) {
+#pragma unroll
+  for (int d = 16; d >= W; d >>= 1)
+    if (W > 1 || d < g.T) v += __shfl_xor_sync(0xffffffffu, v, d);
+  const int lane = threadIdx.x & 31;
+  if (W > 1 ? lane < W : (g.l & 31) == 0) sts32(&fx_shared().l1[threadIdx.x >> 5][s0 + g.s], v);
 }
 // The warp's largest high word of the sequence of slot s, from each thread's m (all threads call)
 __device__ __forceinline__ void fx_put_max(int s, unsigned m) {
-  m = fx_warp_max(m);
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, d));
   if ((threadIdx.x & 31) == 0) sts32(&fx_shared().mx[threadIdx.x >> 5][s], m);
 }
-__device__ __forceinline__ void fx_put_l1(int s, unsigned v) {
-  v = fx_warp_sum(v);
-  if ((threadIdx.x & 31) == 0) sts32(&fx_shared().l1[threadIdx.x >> 5][s], v);
-}
-__device__ __forceinline__ unsigned fx_get_max(int s) {
+__device__ __forceinline__ unsigned fx_get_max(int s, int2 warps) {
   unsigned m = 0u;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = max(m, lds32(&fx_shared().mx[w][s]));
+  for (int w = warps.x; w < warps.y; ++w) m = max(m, lds32(&fx_shared().mx[w][s]));
   return m;
 }
 struct FxExp {
@@ -475,54 +517,78 @@ __device__ __forceinline__ fx2 fx_load(double2 v, FxExp e) {
 }
 
 // Each warp writes its copy of the sequences' scale exponents and scalings (after a barrier that makes mx and
-// l1 final): results are v 2^exponent.  sched: the plan's table for this kind of input.
-template <int B>
+// l1 final): results are v 2^exponent.  sched: the plan's table for this kind of input; EVERY: all warps hold
+// maxima (fx_put_max).
+template <int B, int NS, int W, bool EVERY>
 __device__ __forceinline__ void fx_make_meta(FxLay lay, const int* __restrict__ sched) {
   FxShared& S = fx_shared();
-  const int lane = lay.s0 + (threadIdx.x & 31), w = threadIdx.x >> 5;
-  if (lane < lay.s0 + lay.ns) {
-    unsigned mx = 0u, l1 = 0u;
-    for (int v = 0; v < (int)(blockDim.x >> 5); ++v) {
-      mx = max(mx, lds32(&S.mx[v][lane]));
-      l1 += lds32(&S.l1[v][lane]);
-    }
+  const int s = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (s < NS) {
+    const int2 own = fx_warps<NS, W>(s);
+    unsigned l1 = 0u;
+    for (int v = own.x; v < own.y; ++v) l1 += lds32(&S.l1[v][lay.s0 + s]);
+    const unsigned mx = fx_get_max(lay.s0 + s, EVERY ? make_int2(0, (int)(blockDim.x >> 5)) : own);
     const int sch = __ldg(sched + __clz((int)l1));
     const FxExp e = fx_exponent(mx);
-    sts32(&S.se[w][lane], (unsigned)(mx >= 0x7ff00000u ? kFxNaN : e.emax + 1 - 1023 - B + (sch >> 24) - (e.pre ? 512 : 0)));
-    sts32(&S.sch[w][lane], (unsigned)sch);
+    sts32(&S.se[w][lay.s0 + s], (unsigned)(mx >= 0x7ff00000u ? kFxNaN : e.emax + 1 - 1023 - B + (sch >> 24) - (e.pre ? 512 : 0)));
+    sts32(&S.sch[w][lay.s0 + s], (unsigned)sch);
   }
   __syncwarp();
 }
 __device__ __forceinline__ int fx_se(int s) { return (int)lds32(&fx_shared().se[threadIdx.x >> 5][s]); }
 __device__ __forceinline__ int fx_sch(int s) { return (int)lds32(&fx_shared().sch[threadIdx.x >> 5][s]); }
 
-// The forward passes over the entries in a; the results are in a when the number of passes is even, else in b.  On
-// return they are visible to all threads.
-__device__ __forceinline__ void fx_passes(int a, int b, FxLay lay, const int4* __restrict__ passes,
-                                          const int4* __restrict__ twiddles) {
-  const int tid = threadIdx.x, nt = blockDim.x;
-  int4 d0 = ldtab(passes), d1 = ldtab(passes + 1);
-  for (int pass = 0;; ++pass) {
-    const int R = d0.x, Ns = d0.y, nbf = d0.z, more = d1.z;
-    const int4* tw = twiddles + d0.w;
-    const unsigned mNs = (unsigned)d1.x, mBf = (unsigned)d1.y;
-    if (more) {  // the next pass's parameters, before they are needed
-      passes += 2;
-      d0 = ldtab(passes);
-      d1 = ldtab(passes + 1);
-    }
-    const int total = lay.ns * nbf;
+// Pass 0 of a sequence: butterfly j of n / R takes the entries j + r n / R through get and writes R j + r from b on.
+template <class Get>
+__device__ __forceinline__ void fx_first(int b, FxGroup g, int n, int R, Get get) {
+  if (R == 6) {
+    const int m = n / 6;
 #pragma unroll 1
-    for (int i = tid; i < total; i += nt) {
-      int s = 0, j = i;
-      if (lay.ns > 1) {
-        s = mBf ? (int)__umulhi((unsigned)i, mBf) : i;
-        j = i - s * nbf;
-      }
-      const int q = mNs ? (int)__umulhi((unsigned)j, mNs) : j;
-      const int k = j - q * Ns;
-      const int sg = (fx_sch(lay.s0 + s) >> (2 * pass)) & 3;
-      const int rd = a + s * lay.stride + j, wr = b + s * lay.stride + q * Ns * R + k;
+    for (int j = g.l; j < m; j += g.T) {
+      fx2 v[6];
+#pragma unroll
+      for (int r = 0; r < 6; ++r) v[r] = get(j + r * m);
+      fx_out6(v);
+#pragma unroll
+      for (int r = 0; r < 6; ++r) fx_put(b + 6 * j + r, v[r]);
+    }
+  } else {
+    const int m = n / 3;
+#pragma unroll 1
+    for (int j = g.l; j < m; j += g.T) {
+      fx2 v0 = get(j), v1 = get(j + m), v2 = get(j + 2 * m);
+      fx_out3(v0, v1, v2);
+      fx_put(b + 3 * j, v0);
+      fx_put(b + 3 * j + 1, v1);
+      fx_put(b + 3 * j + 2, v2);
+    }
+  }
+}
+// The other passes of this thread's sequence, from the results of pass 0 in a (b: the other buffer; sch: the
+// scalings); the threads meet after each.
+struct FxDesc {
+  int4 d0, d1;
+};
+__device__ __forceinline__ FxDesc fx_desc(const int4* passes) { return FxDesc{ldtab(passes), ldtab(passes + 1)}; }
+// AHEAD: next holds pass 1's parameters, and those of each later pass are loaded a pass ahead too: for kernels
+// that run one transform and find the tables in L2 (the Rayleigh-Benard pieces at 64 x 32 take 178 us with
+// it, 192 us without); the step loops find them in L1 and need the registers (16384 Burgers members: 16.8 and 15.7 ms).
+template <bool AHEAD>
+__device__ __forceinline__ void fx_rest(int a, int b, FxGroup g, int sch, FxDesc next, const int4* __restrict__ passes,
+                                        const int4* __restrict__ twiddles) {
+  const int tid = g.l, nt = g.T;
+  for (;;) {
+    sch >>= 2;
+    if (!AHEAD) next = fx_desc(passes);
+    const int R = next.d0.x, Ns = next.d0.y, nbf = next.d0.z, more = next.d1.z, sg = sch & 3;
+    const int4* tw = twiddles + next.d0.w;
+    const unsigned mNs = (unsigned)next.d1.x;
+    passes += 2;
+    if (AHEAD && more) next = fx_desc(passes);
+#pragma unroll 1
+    for (int j = tid; j < nbf; j += nt) {
+      const int q = (int)__umulhi((unsigned)j, mNs), k = j - q * Ns;
+      const int rd = a + j, wr = b + q * Ns * R + k;
       if (R == 4) {
         fx2 v0 = fx_get(rd), v1 = fx_get(rd + nbf), v2 = fx_get(rd + 2 * nbf), v3 = fx_get(rd + 3 * nbf);
         const int4* w = tw + 3 * k;
@@ -536,21 +602,16 @@ __device__ __forceinline__ void fx_passes(int a, int b, FxLay lay, const int4* _
         fx_put(wr + 2 * Ns, v2);
         fx_put(wr + 3 * Ns, v3);
       } else if (R == 3) {
-        fx2 v0 = fx_get(rd), v1 = fx_get(rd + nbf), v2 = fx_get(rd + 2 * nbf);
-        if (pass > 0) {  // the first pass (always of radix 3) has neither twiddles nor a scaling
-          const int4* w = tw + 2 * k;
-          v0 = fx_shr(v0, sg);
-          v1 = fx_cmul(v1, ldtab(w), sg);
-          v2 = fx_cmul(v2, ldtab(w + 1), sg);
-        }
+        const int4* w = tw + 2 * k;
+        fx2 v0 = fx_shr(fx_get(rd), sg);
+        fx2 v1 = fx_cmul(fx_get(rd + nbf), ldtab(w), sg);
+        fx2 v2 = fx_cmul(fx_get(rd + 2 * nbf), ldtab(w + 1), sg);
         fx_out3(v0, v1, v2);
         fx_put(wr, v0);
         fx_put(wr + Ns, v1);
         fx_put(wr + 2 * Ns, v2);
       } else {
-        fx2 v0 = fx_get(rd), v1 = fx_get(rd + nbf);
-        v0 = fx_shr(v0, sg);
-        v1 = fx_cmul(v1, ldtab(tw + k), sg);
+        const fx2 v0 = fx_shr(fx_get(rd), sg), v1 = fx_cmul(fx_get(rd + nbf), ldtab(tw + k), sg);
         fx_put(wr, fx_add(v0, v1));
         fx_put(wr + Ns, fx_sub(v0, v1));
       }
@@ -568,8 +629,7 @@ __device__ __forceinline__ void fx_passes(int a, int b, FxLay lay, const int4* _
 // xf_c2c, xf_c2r and xf_r2c stage their input through load(s, e) (called once per entry of each of the NS
 // sequences), run the passes and return the results where FxRes reads them; what load reads must not lie in the
 // buffers.  The CTA synchronises before the buffers are used again.  Lengths without a fixed-point plan run the
-// FP64 butterflies; PATH kFxOnly: the caller's lengths never do, kFp64: all do.  W > 1 (a power of two dividing 32): NS = W
-// sequences whose entries consecutive threads take across the sequences (entry i / W of sequence i % W).
+// FP64 butterflies; PATH kFxOnly: the caller's lengths never do, kFp64: all do.  W: see FxGroup.
 
 enum { kFxOnly = 0, kFxAny = 1, kFp64 = 2 };
 
@@ -605,38 +665,22 @@ struct FxRes {
 // FP64 values of cnt entries of every sequence into dst, and the sequences' largest high words
 template <int NS, int W, class Load>
 __device__ __forceinline__ void fx_stage(int dst, FxLay lay, int cnt, Load load) {
-  if (W > 1) {
-    const int s = threadIdx.x & (W - 1);
-    unsigned m = 0u;
-    for (int i = threadIdx.x; i < cnt * W; i += blockDim.x) {
-      const double2 v = load(s, i / W);
-      fx_put64(dst + s * lay.stride + i / W, v);
-      m = fx_absmax(m, v);
-    }
-    m = fx_warp_max<W>(m);
-    if ((threadIdx.x & 31) < W) sts32(&fx_shared().mx[threadIdx.x >> 5][lay.s0 + s], m);
-    return;
+  const FxGroup g = fx_group<NS, W>();
+  const int q = dst + g.s * lay.stride;
+  unsigned m = 0u;
+  for (int e = g.l; e < cnt; e += g.T) {
+    const double2 v = load(g.s, e);
+    fx_put64(q + e, v);
+    m = fx_absmax(m, v);
   }
-  unsigned m[NS];
-#pragma unroll
-  for (int s = 0; s < NS; ++s) m[s] = 0u;
-  for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
-    double2 v[NS];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) v[s] = load(s, i);
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      fx_put64(dst + s * lay.stride + i, v[s]);
-      m[s] = fx_absmax(m[s], v[s]);
-    }
-  }
-#pragma unroll
-  for (int s = 0; s < NS; ++s) fx_put_max(lay.s0 + s, m[s]);
+  fx_reduce_max<W>(g, lay.s0, m);
 }
 
-template <bool INV>
-__device__ __forceinline__ FxRes<INV> fx_run(int a, int b, FxLay lay, const FFTPlan& p) {
-  fx_passes(a, b, lay, p.fxp, p.fxt);
+// The passes after pass 0 (whose results are in b)
+template <bool INV, bool AHEAD>
+__device__ __forceinline__ FxRes<INV> fx_run(int a, int b, FxLay lay, FxGroup g, const FFTPlan& p, FxDesc next) {
+  if (p.fxr0 != p.n)
+    fx_rest<AHEAD>(b + g.s * lay.stride, a + g.s * lay.stride, g, fx_sch(lay.s0 + g.s), next, p.fxp + 2, p.fxt);
   return FxRes<INV>{p.fxodd ? b : a, lay, p.n, p.fxr, p.wm, true};
 }
 template <bool INV>
@@ -645,48 +689,41 @@ __device__ __forceinline__ FxRes<INV> fx_run64(int a, int b, FxLay lay, const FF
   return FxRes<INV>{(p.nrad & 1) ? b : a, lay, p.n, p.fxr, p.wm, false};
 }
 
+// xf_c2c (below) with the entries of every sequence already in a as FP64 pairs and their largest high words given
+// (EVERY: by fx_put_max in all warps); the call starts with a barrier.
+template <bool INV, int NS, int W = 1, int PATH = kFxAny, bool REAL = false, bool EVERY = true>
+__device__ __forceinline__ FxRes<INV> xf_c2c_staged(int a, int b, FxLay lay, const FFTPlan& p) {
+  __syncthreads();
+  if (PATH == kFp64 || (PATH == kFxAny && !p.fxp)) return fx_run64<INV>(a, b, lay, p);
+  // pass 0 converts its inputs
+  const FxGroup g = fx_group<NS, W>();
+  FxDesc next{};
+  if (PATH == kFxAny && p.fxr0 != p.n) next = fx_desc(p.fxp + 2);
+  const FxExp ex = fx_exponent(fx_get_max(lay.s0 + g.s, EVERY ? make_int2(0, (int)(blockDim.x >> 5)) : fx_warps<NS, W>(g.s)));
+  const int A = a + g.s * lay.stride;
+  unsigned l1 = 0u;
+  fx_first(b + g.s * lay.stride, g, p.n, p.fxr0, [&](int e) {
+    const fx2 v = fx_load<kFxB>(fx_get64(A + e), ex);
+    l1 += fx_l1(v);
+    return INV ? fx_swap(v) : v;
+  });
+  fx_reduce_l1<W>(g, lay.s0, l1);
+  __syncthreads();
+  fx_make_meta<kFxB, NS, W, EVERY>(lay, p.fxs + 32 * (REAL ? kFxFwdReal : kFxComplex));
+  return fx_run<INV, PATH == kFxAny>(a, b, lay, g, p, next);
+}
+
 // Complex transform of length p.n, unnormalised: exp(-), or exp(+) for INV.  REAL: the packed grid of a forward
 // real transform.
 template <bool INV, int NS, int W = 1, int PATH = kFxAny, bool REAL = false, class Load>
 __device__ __forceinline__ FxRes<INV> xf_c2c(int a, int b, FxLay lay, const FFTPlan& p, Load load) {
-  const int n = p.n;
-  fx_stage<NS, W>(a, lay, n, load);
-  if (PATH == kFp64 || (PATH == kFxAny && !p.fxp)) {
-    __syncthreads();
-    return fx_run64<INV>(a, b, lay, p);
-  }
-  __syncthreads();
-  // each thread converts the entries it staged
-  auto conv = [&](int q, FxExp ex) {
-    fx2 v = fx_load<kFxB>(fx_get64(q), ex);
-    if (INV) v = fx_swap(v);
-    fx_put(q, v);
-    return fx_l1(v);
-  };
-  if (W > 1) {
-    const int s = threadIdx.x & (W - 1);
-    const FxExp ex = fx_exponent(fx_get_max(lay.s0 + s));
-    unsigned l1 = 0u;
-    for (int i = threadIdx.x; i < n * W; i += blockDim.x) l1 += conv(a + s * lay.stride + i / W, ex);
-    l1 = fx_warp_sum<W>(l1);
-    if ((threadIdx.x & 31) < W) sts32(&fx_shared().l1[threadIdx.x >> 5][lay.s0 + s], l1);
-  } else {
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      const FxExp ex = fx_exponent(fx_get_max(lay.s0 + s));
-      unsigned l1 = 0u;
-      for (int i = threadIdx.x; i < n; i += blockDim.x) l1 += conv(a + s * lay.stride + i, ex);
-      fx_put_l1(lay.s0 + s, l1);
-    }
-  }
-  __syncthreads();
-  fx_make_meta<kFxB>(lay, p.fxs + 32 * (REAL ? kFxFwdReal : kFxComplex));
-  return fx_run<INV>(a, b, lay, p);
+  fx_stage<NS, W>(a, lay, p.n, load);
+  return xf_c2c_staged<INV, NS, W, PATH, REAL, false>(a, b, lay, p);
 }
 
 // xf_c2r (below) with the c_k of every sequence already in b as FP64 pairs and their largest high words given
-// (fx_put_max); the call starts with a barrier.
-template <int NS, int PATH = kFxAny>
+// (EVERY: by fx_put_max in all warps); the call starts with a barrier.
+template <int NS, int PATH = kFxAny, bool EVERY = true>
 __device__ __forceinline__ FxRes<true> xf_c2r_staged(int a, int b, FxLay lay, const FFTPlan& p, int K) {
   const int n = p.n;
   __syncthreads();
@@ -699,35 +736,37 @@ __device__ __forceinline__ FxRes<true> xf_c2r_staged(int a, int b, FxLay lay, co
     __syncthreads();
     return fx_run64<true>(a, b, lay, p);
   }
-  const int half = n / 2 + 1;
-#pragma unroll
-  for (int s = 0; s < NS; ++s) {
-    const FxExp ex = fx_exponent(fx_get_max(lay.s0 + s));
-    const int S = b + s * lay.stride, A = a + s * lay.stride;
-    unsigned l1 = 0u;
-    for (int k = threadIdx.x; k < half; k += blockDim.x) {
-      const int kc = n - k;
-      // c_k and c_{n-k} (0 where not stored), c_0 real
-      const bool hx = k < K, hy = k > 0 && kc < K;
-      double2 sx = fx_get64(S + (hx ? k : 0)), sy = fx_get64(S + (hy ? kc : 0));
-      if (!hx) sx.x = 0.0;
-      if (!hx || k == 0) sx.y = 0.0;
-      if (!hy) sy = make_double2(0.0, 0.0);
-      const fx2 x = fx_load<kFxBReal>(sx, ex), y = fx_load<kFxBReal>(sy, ex);
-      fx2 z0, z1;
-      fx_pack(x, y, ldtab(p.fxr + k), z0, z1);
-      fx_put(A + k, fx_swap(z0));
-      l1 += fx_l1(z0);
-      if (k > 0 && kc != k) {
-        fx_put(A + kc, fx_swap(z1));
-        l1 += fx_l1(z1);
-      }
+  const FxGroup g = fx_group<NS, 1>();
+  FxDesc next{};
+  if (PATH == kFxAny && p.fxr0 != p.n) next = fx_desc(p.fxp + 2);
+  const int half = n / 2 + 1, S = b + g.s * lay.stride, A = a + g.s * lay.stride;
+  const FxExp ex = fx_exponent(fx_get_max(lay.s0 + g.s, EVERY ? make_int2(0, (int)(blockDim.x >> 5)) : fx_warps<NS, 1>(g.s)));
+  unsigned l1 = 0u;
+  for (int k = g.l; k < half; k += g.T) {
+    const int kc = n - k;
+    // c_k and c_{n-k} (0 where not stored), c_0 real
+    const bool hx = k < K, hy = k > 0 && kc < K;
+    double2 sx = fx_get64(S + (hx ? k : 0)), sy = fx_get64(S + (hy ? kc : 0));
+    if (!hx) sx.x = 0.0;
+    if (!hx || k == 0) sx.y = 0.0;
+    if (!hy) sy = make_double2(0.0, 0.0);
+    const fx2 x = fx_load<kFxBReal>(sx, ex), y = fx_load<kFxBReal>(sy, ex);
+    fx2 z0, z1;
+    fx_pack(x, y, ldtab(p.fxr + k), z0, z1);
+    fx_put(A + k, fx_swap(z0));
+    l1 += fx_l1(z0);
+    if (k > 0 && kc != k) {
+      fx_put(A + kc, fx_swap(z1));
+      l1 += fx_l1(z1);
     }
-    fx_put_l1(lay.s0 + s, l1);
   }
+  fx_reduce_l1<1>(g, lay.s0, l1);
   __syncthreads();
-  fx_make_meta<kFxBReal>(lay, p.fxs + 32 * kFxInvReal);
-  return fx_run<true>(a, b, lay, p);
+  fx_make_meta<kFxBReal, NS, 1, EVERY>(lay, p.fxs + 32 * kFxInvReal);
+  const int sg = fx_sch(lay.s0 + g.s) & 3;
+  fx_first(S, g, n, p.fxr0, [&](int e) { return fx_shr(fx_get(A + e), sg); });
+  __syncthreads();
+  return fx_run<true, PATH == kFxAny>(a, b, lay, g, p, next);
 }
 
 // Inverse real transform: the grid values g_j = Re c_0 + 2 Re sum_{1 <= k < K} c_k exp(2 pi i j k / 2n),
@@ -735,7 +774,7 @@ __device__ __forceinline__ FxRes<true> xf_c2r_staged(int a, int b, FxLay lay, co
 template <int NS, int PATH = kFxAny, class Load>
 __device__ __forceinline__ FxRes<true> xf_c2r(int a, int b, FxLay lay, const FFTPlan& p, int K, Load load) {
   fx_stage<NS, 1>(b, lay, K, load);
-  return xf_c2r_staged<NS, PATH>(a, b, lay, p, K);
+  return xf_c2r_staged<NS, PATH, false>(a, b, lay, p, K);
 }
 
 // Forward real transform of the grid pairs (g_2j, g_2j+1) = load(s, j), j < n; results by FxRes::coef.

@@ -484,10 +484,19 @@ __device__ void b_adjoint(const KolArgs& A, const KMember& m, int tile) {
     }
     // grid cotangents of u, v, w_x, w_y: -g w_x, -g w_y, -g u, -g v (entry i of g's slot is overwritten by the
     // thread that has read it)
-    const auto z = xf_r2c<4, kFxOnly>(fr, r.z, FxLay{4, 2 * C, 0}, R.px, [&](int f, int i) {
-      const double2 a = g.at(0, i), b = r.at(f ^ 2, i);
-      return make_double2(-a.x * b.x, -a.y * b.y);
-    });
+    unsigned mx[4] = {0u, 0u, 0u, 0u};
+    for (int i = threadIdx.x; i < L; i += blockDim.x) {
+      const double2 a = g.at(0, i);
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        const double2 b = r.at(f ^ 2, i), v = make_double2(-a.x * b.x, -a.y * b.y);
+        fx_put64(fr + 2 * f * C + i, v);
+        mx[f] = fx_absmax(mx[f], v);
+      }
+    }
+#pragma unroll
+    for (int f = 0; f < 4; ++f) fx_put_max(f, mx[f]);
+    const auto z = xf_c2c_staged<false, 4, 1, kFxOnly, true>(fr, r.z, FxLay{4, 2 * C, 0}, R.px);
     for (int f = 0; f < 4; ++f) put_row(z, f, A.mixB[f] + m.off_mix + (long long)j * Kx, Kx, 1.0, 2.0);
     __syncthreads();
   }

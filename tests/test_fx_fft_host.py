@@ -44,20 +44,20 @@ static std::vector<fx2> passes(std::vector<fx2> a, const FFTPlan& p, int sch) {
     for (int j = 0; j < q.nbf; ++j) {
       const int blk = q.mNs ? (int)(((unsigned long long)j * q.mNs) >> 32) : j, k = j - blk * q.Ns;
       if (blk != j / q.Ns) std::abort();
-      fx2 v[4];
+      fx2 v[6];
       for (int r = 0; r < q.R; ++r) v[r] = a.at(j + r * q.nbf);
-      if (ps > 0) {
+      if (ps == 0) {
+        for (int r = 0; r < q.R; ++r) v[r] = fx_shr(v[r], sg);
+      } else {
         v[0] = fx_shr(v[0], sg);
         for (int r = 1; r < q.R; ++r) v[r] = fx_cmul(v[r], tw[q.tw + (q.R - 1) * k + r - 1], sg);
       }
-      if (q.R == 4) fx_out4(v[0], v[1], v[2], v[3]);
+      if (q.R == 6) fx_out6(v);
+      else if (q.R == 4) fx_out4(v[0], v[1], v[2], v[3]);
       else if (q.R == 3) fx_out3(v[0], v[1], v[2]);
       else { const fx2 t = fx_add(v[0], v[1]); v[1] = fx_sub(v[0], v[1]); v[0] = t; }
       for (int r = 0; r < q.R; ++r) { see(v[r]); b.at(blk * q.Ns * q.R + k + r * q.Ns) = v[r]; }
     }
-    for (int s = 0; s < 8 && q.mBf; ++s)  // the division that tells the sequences apart
-      for (int j : {0, q.nbf - 1})
-        if ((int)(((unsigned long long)(s * q.nbf + j) * q.mBf) >> 32) != s) std::abort();
     a = b;
     ++ps;
   }
