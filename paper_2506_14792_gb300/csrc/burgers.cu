@@ -49,24 +49,26 @@ __device__ __forceinline__ Smem carve(const BurgersParams& P) { return Smem{0, P
 
 __device__ __forceinline__ double kwav(const BurgersParams& P, int k) { return P.kscale * k; }
 
-// -i k v s
-__device__ __forceinline__ double2 minus_ik(const BurgersParams& P, int k, double2 v, double s) {
-  const double kk = kwav(P, k) * s;
-  return make_double2(kk * v.y, -kk * v.x);
-}
-// Puts F(x)_k = -i k T[(B x)^2 / 2]_k, k < K, through out(k, F_k), from the spectrum staged in B.
+// -i f v and i f v
+__device__ __forceinline__ double2 minus_i(double f, double2 v) { return make_double2(f * v.y, -f * v.x); }
+__device__ __forceinline__ double2 plus_i(double f, double2 v) { return make_double2(-f * v.y, f * v.x); }
+// k / (2M): the factor of F_k = -i k / (2M) sum (B x)^2 exp(-i k x_j) and of T^dagger's argument i k w / (2M).  The
+// step loops keep it per mode (an FP64 instruction holds the pipe of an SM partition for 64 clocks).
+__device__ __forceinline__ double half_k(const BurgersParams& P, int k) { return kwav(P, k) * (0.5 / P.M); }
+
+// Puts the sums T_k, F(x)_k = -i half_k T_k, k < K, through out(k, T_k), from the spectrum staged in B.
 template <int PATH, class Out>
 __device__ __forceinline__ void eval_F(const BurgersParams& P, const Smem& s, Out out) {
   const auto u = xf_c2r_staged<1, PATH>(s.A, s.B, FxLay{1, P.C, 0}, P.plan, P.K);
   const auto z = xf_r2c<1, PATH>(s.C, s.D, FxLay{1, P.C, 0}, P.plan, [&](int, int j) {
     const double2 v = u.at(0, j);
-    return make_double2(v.x * v.x, v.y * v.y);  // u^2; the 1/2 goes into the scale below
+    return make_double2(v.x * v.x, v.y * v.y);
   });
-  for (int k = threadIdx.x; k < P.K; k += blockDim.x) out(k, minus_ik(P, k, z.coef(0, k), 0.5 / P.M));
+  for (int k = threadIdx.x; k < P.K; k += blockDim.x) out(k, z.coef(0, k));
 }
 
-// From the primal spectrum staged in B and the tangent spectrum in D: out(k, F_k, ((dF/dX) dX)_k),
-// (dF/dX) dX = -i k T[(B x)(B dx)].  Both transforms of each direction share their passes (A|B and C|D are 2C
+// From the primal spectrum staged in B and the tangent spectrum in D: out(k, T_k, dT_k), ((dF/dX) dX)_k =
+// -i half_k dT_k = -i k T[(B x)(B dx)].  Both transforms of each direction share their passes (A|B and C|D are 2C
 // apart); the second ones are staged in the free halves and overwrite the grids after that.
 template <int PATH, class Out>
 __device__ __forceinline__ void eval_F_and_jvp(const BurgersParams& P, const Smem& s, Out out) {
@@ -76,18 +78,12 @@ __device__ __forceinline__ void eval_F_and_jvp(const BurgersParams& P, const Sme
     const double2 v = u.at(0, j), w = q ? u.at(1, j) : v;
     return make_double2(v.x * w.x, v.y * w.y);
   });
-  for (int k = threadIdx.x; k < P.K; k += blockDim.x)
-    out(k, minus_ik(P, k, z.coef(0, k), 0.5 / P.M), minus_ik(P, k, z.coef(1, k), 1.0 / P.M));
+  for (int k = threadIdx.x; k < P.K; k += blockDim.x) out(k, z.coef(0, k), z.coef(1, k, 1));
   __syncthreads();  // the results lie where the next spectra are staged
 }
 
-// i k w / (2M): T^dagger's weights (1/M on the real part of k = 0, 1/(2M) elsewhere) folded in, the k = 0
-// entry being 0
-__device__ __forceinline__ double2 vjp_cotangent(const BurgersParams& P, int k, double2 w) {
-  const double kk = kwav(P, k) * (0.5 / P.M);
-  return make_double2(-kk * w.y, kk * w.x);
-}
-// From the primal spectrum staged in B and vjp_cotangent(W) in D: out(k, ((dF/dX)^dagger W)_k),
+// From the primal spectrum staged in B and i half_k W_k in D (T^dagger's weights, 1/M on the real part of k = 0 and
+// 1/(2M) elsewhere, folded in, the k = 0 entry being 0): out(k, ((dF/dX)^dagger W)_k),
 // (dF/dX)^dagger W = B^dagger[(B x) * T^dagger(i k W)].
 template <int PATH, class Out>
 __device__ __forceinline__ void eval_vjp(const BurgersParams& P, const Smem& s, Out out) {
@@ -98,8 +94,9 @@ __device__ __forceinline__ void eval_vjp(const BurgersParams& P, const Smem& s, 
     return make_double2(a.x * b.x, a.y * b.y);
   });
   for (int k = threadIdx.x; k < P.K; k += blockDim.x) {
-    const double2 x = z.coef(0, k);
-    out(k, k == 0 ? make_double2(x.x, 0.0) : make_double2(2.0 * x.x, 2.0 * x.y));
+    double2 x = z.coef(0, k, k == 0 ? 0 : 1);
+    if (k == 0) x.y = 0.0;
+    out(k, x);
   }
 }
 
@@ -159,7 +156,7 @@ __global__ void __launch_bounds__(64) F_kernel(const __grid_constant__ BurgersPa
     m0 = fx_absmax(m0, v);
     if (MODE != 0) {
       double2 w = ldg128(dr + k);
-      if (MODE == 2) w = vjp_cotangent(P, k, w);
+      if (MODE == 2) w = plus_i(half_k(P, k), w);
       fx_put64(s.D + k, w);
       m1 = fx_absmax(m1, w);
     }
@@ -167,8 +164,8 @@ __global__ void __launch_bounds__(64) F_kernel(const __grid_constant__ BurgersPa
   fx_put_max(0, m0);
   if (MODE != 0) fx_put_max(1, m1);
   auto put = [&](int k, double2 v) { stg128(o + k, v); };
-  if (MODE == 0) eval_F<kFp64>(P, s, put);
-  else if (MODE == 1) eval_F_and_jvp<kFp64>(P, s, [&](int k, double2, double2 v) { put(k, v); });
+  if (MODE == 0) eval_F<kFp64>(P, s, [&](int k, double2 v) { put(k, minus_i(half_k(P, k), v)); });
+  else if (MODE == 1) eval_F_and_jvp<kFp64>(P, s, [&](int k, double2, double2 v) { put(k, minus_i(half_k(P, k), v)); });
   else eval_vjp<kFp64>(P, s, put);
 }
 
@@ -179,6 +176,8 @@ __global__ void __launch_bounds__(64) F_kernel(const __grid_constant__ BurgersPa
 // weights (divided by dt), c: extrapolation weights of F; entries beyond s are zero.
 struct Coef {
   double a[kMaxOrder + 1], c[kMaxOrder + 1];
+  // whether term i has a weight (weights are never tiny: the high words tell)
+  __device__ __forceinline__ bool used(int i) const { return ((__double2hiint(a[i]) | __double2hiint(c[i])) << 1) != 0; }
 };
 constexpr double kSbdfA[kMaxOrder][kMaxOrder + 1] = {{1.0, -1.0, 0.0, 0.0, 0.0},
                                                      {1.5, -2.0, 0.5, 0.0, 0.0},
@@ -226,7 +225,7 @@ __device__ __forceinline__ double2 hist_rhs(const Coef& c, const double2 (&hf)[O
   double2 r = axpby(c.c[1], hf[0], -c.a[1], hx[0]);
 #pragma unroll
   for (int i = 2; i <= ORD; ++i)
-    if (c.c[i] != 0.0 || c.a[i] != 0.0)
+    if (c.used(i))
       r = make_double2(r.x + c.c[i] * hf[i - 1].x - c.a[i] * hx[i - 1].x,
                        r.y + c.c[i] * hf[i - 1].y - c.a[i] * hx[i - 1].y);
   return r;
@@ -254,6 +253,8 @@ __global__ void __launch_bounds__(64) trajectory_kernel(const __grid_constant__ 
   const int nx = in_blocks > 1 ? so : 1;  // X blocks present in s_in
   double2 X[Q][ORD], F[Q][ORD], D[Q][ORD], GJ[Q][ORD];
   unsigned mx = 0u, md = 0u;  // largest high words of the staged spectra
+  double hk[Q];
+  for (int q = 0; q < Q; ++q) hk[q] = half_k(P, tid + q * G);
   // F (and its tangent) of the staged spectra into slot 0 of the histories: thread tid owns k = tid + q G
   auto nonlinear = [&]() {
     fx_put_max(0, mx);
@@ -263,14 +264,14 @@ __global__ void __launch_bounds__(64) trajectory_kernel(const __grid_constant__ 
 #pragma unroll
         for (int q = 0; q < Q; ++q)
           if (k == tid + q * G) {
-            F[q][0] = f;
-            GJ[q][0] = g;
+            F[q][0] = minus_i(hk[q], f);
+            GJ[q][0] = minus_i(hk[q], g);
           }
       });
     } else {
       eval_F<kFxOnly>(P, s, [&](int k, double2 v) {
 #pragma unroll
-        for (int q = 0; q < Q; ++q) if (k == tid + q * G) F[q][0] = v;
+        for (int q = 0; q < Q; ++q) if (k == tid + q * G) F[q][0] = minus_i(hk[q], v);
       });
     }
     mx = md = 0u;
@@ -314,7 +315,7 @@ __global__ void __launch_bounds__(64) trajectory_kernel(const __grid_constant__ 
   for (int j = 1; j <= n_steps; ++j) {
     const int n = n_first + j;
     Coef c = step_coef(P, n);
-    if (c.a[0] != a0_prev) {
+    if (__double_as_longlong(c.a[0]) != __double_as_longlong(a0_prev)) {
       for (int q = 0; q < Q; ++q) inv_m[q] = 1.0 / (c.a[0] + nk2[q]);
       a0_prev = c.a[0];
     }
@@ -377,6 +378,8 @@ __global__ void __launch_bounds__(64) adjoint_kernel(const __grid_constant__ Bur
   const int so = P.order;
   double2 Y[Q][ORD];  // Y_{n+1}, ..., Y_{n+ORD}
   const double2 z = make_double2(0.0, 0.0);
+  double hk[Q];
+  for (int q = 0; q < Q; ++q) hk[q] = half_k(P, tid + q * G);
   // nu k^2 per mode and 1 / (a_0 + nu k^2) of the current step, recomputed when a_0 changes
   double nk2[Q], inv_m[Q];
   for (int q = 0; q < Q; ++q) {
@@ -417,7 +420,7 @@ __global__ void __launch_bounds__(64) adjoint_kernel(const __grid_constant__ Bur
         double2 w = axpby(wc[1], Y[q][0], wc[2], Y[q][1]);
 #pragma unroll
         for (int i = 3; i <= ORD; ++i) w = make_double2(w.x + wc[i] * Y[q][i - 1].x, w.y + wc[i] * Y[q][i - 1].y);
-        w = vjp_cotangent(P, k, w);
+        w = plus_i(hk[q], w);
         fx_put64(s.D + k, w);
         mw = fx_absmax(mw, w);
       }
@@ -467,7 +470,7 @@ __global__ void __launch_bounds__(64) adjoint_kernel(const __grid_constant__ Bur
     }
     {
       const Coef c = step_coef(P, n);
-      if (c.a[0] != a0_prev) {
+      if (__double_as_longlong(c.a[0]) != __double_as_longlong(a0_prev)) {
         for (int q = 0; q < Q; ++q) inv_m[q] = 1.0 / (c.a[0] + nk2[q]);
         a0_prev = c.a[0];
       }

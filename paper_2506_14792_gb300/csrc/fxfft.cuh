@@ -650,14 +650,17 @@ struct FxRes {
     const int se = fx_se(lay.s0 + s);
     return make_double2(fx_to_double(v.x, se), fx_to_double(v.y, se));
   }
-  // spectrum entry X_k = sum_j g_j exp(-2 pi i j k / 2n) of a forward real transform
-  __device__ __forceinline__ double2 coef(int s, int k) const {
+  // spectrum entry X_k = sum_j g_j exp(-2 pi i j k / 2n) of a forward real transform, times 2^e (e: 0 or 1)
+  __device__ __forceinline__ double2 coef(int s, int k, int e = 0) const {
     const int kc = k == 0 ? 0 : n - k;
-    if (!fixed) return r2c_combine(raw64(s, k), cconj(raw64(s, kc)), __ldg(&wm[k]));
+    if (!fixed) {
+      const double2 x = r2c_combine(raw64(s, k), cconj(raw64(s, kc)), __ldg(&wm[k]));
+      return e ? make_double2(2.0 * x.x, 2.0 * x.y) : x;
+    }
     const int q = z + s * lay.stride;
     const int us = (fx_sch(lay.s0 + s) >> 16) & 3;
     const fx2 r = fx_unpack(fx_get(q + k), fx_get(q + kc), ldtab(fxr + k), us);
-    const int se = fx_se(lay.s0 + s) + us - 1;
+    const int se = fx_se(lay.s0 + s) + us - 1 + e;
     return make_double2(fx_to_double(r.x, se), fx_to_double(r.y, se));
   }
 };
