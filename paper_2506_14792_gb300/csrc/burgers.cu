@@ -239,8 +239,9 @@ __device__ __forceinline__ double2 hist_rhs(const Coef& c, const double2 (&hf)[O
 // (a full restart state); ds_in the same blocks of the tangent.  Outputs (each nullable): x_out the
 // final state (or tangent), s_out the final restart state (or its tangent), traj the states
 // X_{n_first}..X_{n_first+n_steps}.
-template <int Q, int ORD>
-__global__ void __launch_bounds__(64) trajectory_kernel(const __grid_constant__ BurgersParams P, int n_first, int n_steps,
+// MB: CTAs per SM that the registers have to leave room for (see Burgers::dispatchQ).
+template <int Q, int ORD, int MB>
+__global__ void __launch_bounds__(64, MB) trajectory_kernel(const __grid_constant__ BurgersParams P, int n_first, int n_steps,
                                                         const double* __restrict__ s_in, int in_blocks,
                                                         const double* __restrict__ ds_in, double* __restrict__ x_out,
                                                         double* __restrict__ s_out, double* __restrict__ traj,
@@ -365,8 +366,8 @@ __global__ void __launch_bounds__(64) trajectory_kernel(const __grid_constant__ 
 // (out_blocks = s) or, when n_lo = 0, dJ/dX_0 in its first block (the right-hand side at n = 0, with no
 // solve) followed by Y_1, ..., Y_{s-1} when out_blocks = s.  Cotangents injected at X_n: seeds
 // (indexed by seed_at[n], nullable) and src (nullable, at n = n_hi).
-template <int Q, int ORD>
-__global__ void __launch_bounds__(64) adjoint_kernel(const __grid_constant__ BurgersParams P, int n_steps, int n_hi, int n_lo,
+template <int Q, int ORD, int MB>
+__global__ void __launch_bounds__(64, MB) adjoint_kernel(const __grid_constant__ BurgersParams P, int n_steps, int n_hi, int n_lo,
                                                      const double* __restrict__ traj, const double* __restrict__ y_final,
                                                      const double* __restrict__ carry_in, double* __restrict__ out,
                                                      int out_blocks, const int* __restrict__ seed_at,
@@ -527,6 +528,7 @@ struct Burgers : EqImpl {
   BurgersParams P{};
   int B = 1;
   int G = 64;
+  int sms = 0;
   DevBuf wm, traj, seed, Jd;
   size_t smem = 0;
 
@@ -580,6 +582,9 @@ struct Burgers : EqImpl {
     P.WM = wm.as<double2>();
     fft_bind(P.plan, true, P.WM + P.M, P.WM, true);
     smem = sizeof(double2) * 4 * P.C;
+    int dev = 0;
+    SPADJ_CUDA_TRY(p, cudaGetDevice(&dev));
+    SPADJ_CUDA_TRY(p, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     return SPADJ_OK;
   }
 
@@ -642,14 +647,26 @@ struct Burgers : EqImpl {
     return check_launch(p, "burgers F");
   }
 
-  // modes per thread Q and register history length (2 for SBDF1/2, 4 for SBDF3/4)
+  // Modes per thread Q, register history length (2 for SBDF1/2, 4 for SBDF3/4) and CTAs per SM MB.  Full batches hide
+  // their latencies better with 8 CTAs per SM, spilling where Q ORD > 4 (30 steps and the adjoint, MB = 1 against 8: 2000
+  // members N = 256 SBDF4 2286 and 1864 us, N = 512 4560 and 3800; 16384 members N = 256 SBDF2, 40 steps,
+  // 15385 and 14873); a few members do not have them (one, N = 512: 1065 and 1293).  Q = 1: SBDF4 of 2000 members at
+  // N = 128 1637 and 1147; SBDF2 of 4000 is fastest with the compiler's own choice (0: 1852, 1: 2181, 8: 2075).
   template <class Fn>
   spadj_status dispatchQ(Problem* p, Fn fn) {
     int Q = (P.K + G - 1) / G;
     auto byQ = [&](auto ord) {
-      if (Q <= 1) fn(std::integral_constant<int, 1>(), ord);
-      else if (Q == 2) fn(std::integral_constant<int, 2>(), ord);
-      else fn(std::integral_constant<int, 4>(), ord);
+      std::integral_constant<int, 1> one;
+      std::integral_constant<int, 8> eight;
+      constexpr int O = decltype(ord)::value;
+      if (Q <= 1) fn(one, ord, std::integral_constant<int, O == 2 ? 0 : 8>());
+      else if (Q == 2) {
+        if (O == 2 || B > 4 * sms) fn(std::integral_constant<int, 2>(), ord, eight);
+        else fn(std::integral_constant<int, 2>(), ord, one);
+      } else {
+        if (B > 4 * sms) fn(std::integral_constant<int, 4>(), ord, eight);
+        else fn(std::integral_constant<int, 4>(), ord, one);
+      }
     };
     if (P.order <= 2) byQ(std::integral_constant<int, 2>());
     else byQ(std::integral_constant<int, 4>());
@@ -664,8 +681,8 @@ struct Burgers : EqImpl {
   spadj_status launch_traj(Problem* p, int n_first, int n_steps, const double* s_in, int in_blocks, const double* ds_in,
                            double* x_out, double* s_out, double* trj, int tangent) {
     cudaEvent_t t = p->tic();
-    spadj_status s = dispatchQ(p, [&](auto q, auto o) {
-      trajectory_kernel<decltype(q)::value, decltype(o)::value><<<B, G, smem, p->stream>>>(
+    spadj_status s = dispatchQ(p, [&](auto q, auto o, auto m) {
+      trajectory_kernel<decltype(q)::value, decltype(o)::value, decltype(m)::value><<<B, G, smem, p->stream>>>(
           P, n_first, n_steps, s_in, in_blocks, ds_in, x_out, s_out, trj, tangent);
     });
     p->toc(t, KC_FUSED, (double)B * n_steps * ((tangent ? 3 : 2) * fft_flops() + P.M + 10.0 * P.K));
@@ -675,8 +692,8 @@ struct Burgers : EqImpl {
                           const double* carry_in, double* out, int out_blocks, const int* seed_at, const double* seeds,
                           const double* src) {
     cudaEvent_t t = p->tic();
-    spadj_status s = dispatchQ(p, [&](auto q, auto o) {
-      adjoint_kernel<decltype(q)::value, decltype(o)::value><<<B, G, smem, p->stream>>>(
+    spadj_status s = dispatchQ(p, [&](auto q, auto o, auto m) {
+      adjoint_kernel<decltype(q)::value, decltype(o)::value, decltype(m)::value><<<B, G, smem, p->stream>>>(
           P, n_steps, n_hi, n_lo, trj, y_final, carry_in, out, out_blocks, seed_at, seeds, src);
     });
     p->toc(t, KC_FUSED, (double)B * (n_hi - n_lo + 1) * (3 * fft_flops() + 2.0 * P.M + 12.0 * P.K));

@@ -35,6 +35,7 @@ namespace spadj {
 namespace {
 
 constexpr int kKolThreads = 128;
+constexpr int kKolThreadsFew = 256;  // of kol_persistent when there are few tiles (Kol::threads)
 constexpr int kMaxRes = 4;
 constexpr unsigned kSpinLimit = 1u << 26;  // x ~150 ns per probe: several seconds
 
@@ -546,7 +547,7 @@ __device__ bool wait_ge(int* ctr, int target, int* err, unsigned limit) {
   return ok != 0;
 }
 
-__global__ void __launch_bounds__(kKolThreads) kol_persistent(const __grid_constant__ KolArgs A) {
+__global__ void __launch_bounds__(kKolThreadsFew) kol_persistent(const __grid_constant__ KolArgs A) {
   __shared__ int item;
   const int per = A.nCAtot + A.nBtot;
   const int nrun = A.nrun > 0 ? A.nrun : A.nstage;
@@ -954,6 +955,22 @@ struct Kol : EqImpl {
     return A;
   }
 
+  int nt_persistent = kKolThreads;
+  // Threads per CTA of kol_persistent.  The four row transforms of a tile have CL butterflies per radix-4 pass; with more
+  // of them than kKolThreads and too few tiles to fill the SMs, twice the threads finish a tile sooner (8-step
+  // gradients, 128 against 256 threads: N = 192 3196 and 2504 us, 512 6551 and 4546, four of 256 3862 and 2954,
+  // 16 of 96 and 192 (3456 grid rows) 3949 and 3846); 12 of 256 (4608 rows) 5167 and 5274, 16 of 128 (CL = 96) 2677
+  // and 3115, one of 96 1853 and 1936.
+  int threads(int sms) const {
+    long long rows = 0;
+    int cl = 0;
+    for (auto& m : hm) {
+      rows += m.M;
+      cl = std::max(cl, m.CL);
+    }
+    return !closure && cl > kKolThreads && rows <= 24LL * sms ? kKolThreadsFew : kKolThreads;
+  }
+
   spadj_status launch(Problem* p, KolArgs& A) {
     const int per = A.nCAtot + A.nBtot;
     if (persistent) {
@@ -963,13 +980,14 @@ struct Kol : EqImpl {
         int dev = 0, sms = 0, occ = 0;
         SPADJ_CUDA_TRY(p, cudaGetDevice(&dev));
         SPADJ_CUDA_TRY(p, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        SPADJ_CUDA_TRY(p, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kol_persistent, kKolThreads, smem));
+        SPADJ_CUDA_TRY(p, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kol_persistent, threads(sms), smem));
         if (occ < 1) return p->fail(SPADJ_ERR_INVALID, "kolmogorov: kernel does not fit on an SM");
         const int per_sm = ctas_per_sm > 0 ? std::min(ctas_per_sm, occ) : occ;
         grid_persistent = sms * per_sm;
+        nt_persistent = threads(sms);
       }
       if (!closure) {
-        kol_persistent<<<grid_persistent, kKolThreads, smem, p->stream>>>(A);
+        kol_persistent<<<grid_persistent, nt_persistent, smem, p->stream>>>(A);
         spadj_status s = check_launch(p, "kolmogorov persistent");
         p->toc(t, KC_FUSED, work_flops(A));
         return s;
@@ -982,7 +1000,7 @@ struct Kol : EqImpl {
         if (st > 0) SPADJ_CUDA_TRY(p, cudaMemsetAsync(ctr.ptr, 0, sizeof(int), p->stream));  // the item queue only
         A.stage0 = st;
         A.nrun = 1;
-        kol_persistent<<<grid_persistent, kKolThreads, smem, p->stream>>>(A);
+        kol_persistent<<<grid_persistent, nt_persistent, smem, p->stream>>>(A);
         spadj_status s = check_launch(p, "kolmogorov persistent step");
         if (s != SPADJ_OK) return s;
         p->toc(ts, KC_FUSED, st + 1 < A.nstage ? per_stage : 0.0);
