@@ -188,12 +188,17 @@ struct RB : EqImpl {
       return cudaMemcpyAsync(b.ptr, h, bytes, cudaMemcpyHostToDevice, p->stream);
     };
     SPADJ_CUDA_TRY(p, up(wm, hwm.data(), sizeof(double2) * hwm.size()));
-    SPADJ_CUDA_TRY(p, up(czE, hczE.data(), sizeof(double) * hczE.size()));
-    SPADJ_CUDA_TRY(p, up(cdzE, hcdzE.data(), sizeof(double) * hcdzE.size()));
-    SPADJ_CUDA_TRY(p, up(gzF, hgzF.data(), sizeof(double) * hgzF.size()));
-    SPADJ_CUDA_TRY(p, up(gzTE, hgzTE.data(), sizeof(double) * hgzTE.size()));
-    SPADJ_CUDA_TRY(p, up(czTF, hczTF.data(), sizeof(double) * hczTF.size()));
-    SPADJ_CUDA_TRY(p, up(cdzTF, hcdzTF.data(), sizeof(double) * hcdzTF.size()));
+    auto upz = [&](DevBuf& b, const std::vector<double>& h, int rows, int cols) -> cudaError_t {
+      const std::vector<double> z = z_table(h, rows, cols);
+      cudaError_t e = b.ensure(sizeof(double) * z.size());
+      return e != cudaSuccess ? e : cudaMemcpy(b.ptr, z.data(), sizeof(double) * z.size(), cudaMemcpyHostToDevice);
+    };
+    SPADJ_CUDA_TRY(p, upz(czE, hczE, Mh, N));
+    SPADJ_CUDA_TRY(p, upz(cdzE, hcdzE, Mh, N));
+    SPADJ_CUDA_TRY(p, upz(gzF, hgzF, N, Mh));
+    SPADJ_CUDA_TRY(p, upz(gzTE, hgzTE, Mh, N));
+    SPADJ_CUDA_TRY(p, upz(czTF, hczTF, N, Mh));
+    SPADJ_CUDA_TRY(p, upz(cdzTF, hcdzTF, N, Mh));
     SPADJ_CUDA_TRY(p, up(gmat, o.G.data(), sizeof(double) * o.G.size()));
     SPADJ_CUDA_TRY(p, cudaStreamSynchronize(p->stream));
     {

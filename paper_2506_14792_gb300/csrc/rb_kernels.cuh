@@ -32,7 +32,7 @@ constexpr int kXMaxJobs = 12;
 // deriv_t = 1 when mat_t has the reflection parity of a z-derivative (-(-1)^n).
 struct ZJob {
   const double2* in[2];
-  const double* mat[2];
+  const double* mat[2];  // z_table
   double alpha[2];
   int deriv[2];
   int mult[2];
@@ -78,12 +78,103 @@ __device__ __forceinline__ double2 zmult(const ZJobs& js, int type, int m, doubl
 // 2*N threads per column.
 constexpr int kTM = 1;  // columns per CTA
 
-__host__ __device__ inline int zmm_threads(int expand, int I) { return 2 * (expand ? I / 2 : I); }
+__host__ __device__ inline int zmm_threads(int expand, int I) {  // whole warps
+  return (2 * (expand ? I / 2 : I) + 31) / 32 * 32;
+}
+
+// The products run in fixed point on the integer pipes.  This chip issues under 2 FP64 multiply-adds per clock and
+// SM against about 25 32 x 32 + 64 bit integer ones, three of which make a product of the format below: the
+// kernel was bound by its FP64 instructions and by matrix rows read one line per lane.  With the products in fixed
+// point and the limbs in the threads' order, explicit terms of 256 x 64 Rayleigh-Benard take 37 us (51 before),
+// gradients of 8 Couette steps at 128 x 64 x 64 19.1 ms (24.2 before; 23.9 with the products alone).  Reading the limbs
+// before the wait for the predecessor hides their latency where CTAs are few (RK443 at 96 x 40: 5.2 ms without, 4.7 with).
+//
+// Format.  Column k of a matrix is scaled by a power of two, 2^-e_k, so that its largest entry is in [1/2, 1), and stored
+// as 2^-57 (2^28 wh + wl); the staged entries x_k 2^(e_k) share one exponent per term, component and (fold) symmetry,
+// the largest below 2^56, and are split into 2^28 xh + xl.  A sum of products is
+//   (sum xh wh + 2^-28 (sum xh wl + xl wh) + O(1/4)) / 2  in units of the entries,
+// all sums exact in 64 bits (a lane's at most 48 terms of 2^57; sums of sums are halved).  The dropped and rounded
+// parts are random, about 0.3 units of 2^-57 of the largest entry per product; FP64 rounds every product and partial
+// sum to 2^-53 of itself.  Relative 2-norm errors against extended sums, N = 8..128, columns like 1/n^2 or exp(-0.4 n):
+// 0.6-1.2e-16 against 0.8-5.1e-16 of FP64; flat columns 0.5-0.9e-16 against 0.7-3.7e-16 (the derivative's expansion
+// 1.1-2.4e-16 against 1.0-2.8e-16); columns graded by exp(-12 (k mod 5)) 0.6-0.9e-16 against 0.7-2.7e-16, only there
+// the derivative's expansion loses (2.9e-16 against 1.9e-16).  A column with a non-finite entry gives NaN; entries
+// below 2^-1022 count as zero.
+struct ZLimb {
+  int h, l;
+};
+__host__ __device__ __forceinline__ ZLimb z_limbs(long long v) {  // |v| < 2^59
+  ZLimb r;
+  r.l = (int)((unsigned)v << 4) >> 4;
+  r.h = (int)((v - r.l) >> 28);
+  return r;
+}
+// x 2^(e) as a fixed-point number below 2^56 for biased exponents (of x 2^e) <= emax
+__host__ __device__ __forceinline__ long long z_fixed(double x, int e, int emax) {
+#ifdef __CUDA_ARCH__
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+#else
+  unsigned long long bits;
+  std::memcpy(&bits, &x, 8);
+  const unsigned hi = (unsigned)(bits >> 32), lo = (unsigned)bits;
+#endif
+  const int ex = (int)((hi >> 20) & 0x7ff), d = emax - (ex + e);
+  if (ex == 0 || d > 57) return 0;
+  const long long m = (long long)(((unsigned long long)((hi & 0xfffff) | 0x100000) << 32 | lo) << 3);
+  const long long v = (m + (d > 0 ? 1ll << (d - 1) : 0)) >> d;
+  return (int)hi < 0 ? -v : v;
+}
+// The device form of a z matrix (rows x cols): its entries, the limbs (wh, wl) of every entry, and e_k per column
+// (as 32-bit integers), all in 8-byte units.  The limbs are ordered as zmm_kernel's threads read them: entry kk of
+// row r's half hf (columns hf (cols / 2) + kk) at (kk rows + r) 2 + hf, so that a warp reads 256 consecutive bytes
+// (row by row, a load of a warp touched 32 lines, and that, not the arithmetic, was the kernel's time).
+__host__ __device__ inline size_t z_limb_entries(int rows, int cols) { return 2 * (size_t)rows * ((cols + 1) / 2); }
+inline std::vector<double> z_table(const std::vector<double>& A, int rows, int cols) {
+  std::vector<double> t(A);
+  t.resize((size_t)rows * cols + z_limb_entries(rows, cols) + (cols + 1) / 2, 0.0);
+  for (int k = 0; k < cols; ++k) {
+    double m = 0.0;
+    for (int r = 0; r < rows; ++r) m = std::max(m, std::fabs(A[(size_t)r * cols + k]));
+    int e = 0;
+    std::frexp(m, &e);
+    for (int r = 0; r < rows; ++r) {
+      const ZLimb w = z_limbs(std::llround(std::ldexp(A[(size_t)r * cols + k], 57 - e)));
+      const int2 v = make_int2(w.h, w.l);
+      const int hf = k >= cols / 2, kk = k - hf * (cols / 2);
+      std::memcpy(&t[(size_t)rows * cols + 2 * ((size_t)kk * rows + r) + hf], &v, 8);
+    }
+    std::memcpy(reinterpret_cast<char*>(&t[(size_t)rows * cols + z_limb_entries(rows, cols)]) + 4 * k, &e, 4);
+  }
+  return t;
+}
+struct ZAcc {  // sum xh wh, sum (xh wl + xl wh)
+  long long a = 0, c = 0;
+  __host__ __device__ __forceinline__ void add(int xh, int xl, int2 w) {
+    a = fx_mad(xh, w.x, a);
+    c = fx_mad(xl, w.x, fx_mad(xh, w.y, c));
+  }
+  __host__ __device__ __forceinline__ long long sum() const { return a + ((c + (1ll << 27)) >> 28); }
+};
+// (a + b) / 2
+__host__ __device__ __forceinline__ long long z_half(long long a, long long b) { return (a >> 1) + (b >> 1) + (a & b & 1); }
+constexpr int kZSlots = 8;  // maxima of a warp: term (2) x symmetry (2) x component (2)
 
 __global__ void __launch_bounds__(256) zmm_kernel(const __grid_constant__ ZJobs js) {
   pdl_trigger();
-  pdl_wait();
   const ZJob& J = js.j[blockIdx.y];
+  const int rows = js.expand ? J.I / 2 : J.I;  // of the matrices
+  {  // one word of every line of the limbs and exponents: they are in L1 when the column has arrived
+    const int cols = js.expand ? J.K : J.K / 2;
+    const int lines = (int)((8 * (z_limb_entries(rows, cols) + (cols + 1) / 2) + 127) / 128);
+    for (int t = 0; t < J.nterm; ++t) {
+      const char* a = reinterpret_cast<const char*>(J.mat[t] + (size_t)rows * cols);
+      for (int i = threadIdx.x; i < lines; i += blockDim.x) {
+        int v;
+        asm volatile("ld.global.nc.s32 %0, [%1];" : "=r"(v) : "l"(a + 128 * i));
+      }
+    }
+  }
+  pdl_wait();
   const int m = blockIdx.x;
   extern __shared__ double2 sb[];
   const int tid = threadIdx.x, nt = blockDim.x;
@@ -101,19 +192,58 @@ __global__ void __launch_bounds__(256) zmm_kernel(const __grid_constant__ ZJobs 
     }
     return v;
   };
+  const int nsym = js.expand ? 1 : 2;
+  __shared__ int zmax[kZSlots * 8];
+  const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
   for (int t = 0; t < J.nterm; ++t) {
     double2* s = sb + (size_t)t * 2 * Kh;
+    const int* ex = reinterpret_cast<const int*>(J.mat[t] + (size_t)rows * Kh + z_limb_entries(rows, Kh));
+    int mx[4] = {-4096, -4096, -4096, -4096};
+    auto put = [&](int y, int k, double2 v) {
+      s[y * Kh + k] = v;
+      const int e = __ldg(ex + k), a = (__double2hiint(v.x) >> 20) & 0x7ff, b = (__double2hiint(v.y) >> 20) & 0x7ff;
+      if (a) mx[2 * y] = max(mx[2 * y], a == 0x7ff ? 8192 : a + e);
+      if (b) mx[2 * y + 1] = max(mx[2 * y + 1], b == 0x7ff ? 8192 : b + e);
+    };
     for (int k = tid; k < Kh; k += nt) {
       const double2 v = comb(t, k);
       if (js.expand) {
-        s[k] = v;
+        put(0, k, v);
       } else {
         const double2 v2 = comb(t, K - 1 - k);
-        s[k] = make_double2(v.x + v2.x, v.y + v2.y);       // s_j
-        s[Kh + k] = make_double2(v.x - v2.x, v.y - v2.y);  // d_j
+        put(0, k, make_double2(v.x + v2.x, v.y + v2.y));  // s_j
+        put(1, k, make_double2(v.x - v2.x, v.y - v2.y));  // d_j
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      if (c >= 2 * nsym) break;
+      mx[c] = __reduce_max_sync(0xffffffffu, mx[c]);
+      if (lane == 0) zmax[warp * kZSlots + 4 * t + c] = mx[c];
+    }
+  }
+  __syncthreads();
+  // largest biased exponent of component c (0, 1) of symmetry y of term t
+  auto emax_of = [&](int t, int y, int c) {
+    int m = -4096;
+    for (int w = 0; w < nw; ++w) m = max(m, zmax[w * kZSlots + 4 * t + 2 * y + c]);
+    return m;
+  };
+  for (int t = 0; t < J.nterm; ++t) {
+    const int* ex = reinterpret_cast<const int*>(J.mat[t] + (size_t)rows * Kh + z_limb_entries(rows, Kh));
+    for (int y = 0; y < nsym; ++y) {
+      const int e0 = emax_of(t, y, 0), e1 = emax_of(t, y, 1);
+      double2* s = sb + (size_t)t * 2 * Kh + y * Kh;
+      for (int k = tid; k < Kh; k += nt) {
+        const double2 v = s[k];
+        const int e = __ldg(ex + k);
+        const ZLimb a = z_limbs(z_fixed(v.x, e, e0)), b = z_limbs(z_fixed(v.y, e, e1));
+        *reinterpret_cast<int4*>(&s[k]) = make_int4(a.h, a.l, b.h, b.l);
       }
     }
   }
+  // value of a sum of the term's scale
+  auto value = [](long long v, int emax) { return fx_to_double(v, emax >= 6000 ? kFxNaN : emax - 1079); };
   __syncthreads();
   const int u = tid >> 1, hf = tid & 1;
   if (js.expand) {
@@ -122,25 +252,29 @@ __global__ void __launch_bounds__(256) zmm_kernel(const __grid_constant__ ZJobs 
     const int k0 = hf * (K / 2), k1 = hf ? K : K / 2;  // K even: both halves start on an even k
     double2 lo = make_double2(0.0, 0.0), hi = make_double2(0.0, 0.0);
     for (int t = 0; t < J.nterm; ++t) {
-      const double* a = J.mat[t] + (size_t)u * K;
-      const double2* s = sb + (size_t)t * 2 * Kh;
-      double2 E = make_double2(0.0, 0.0), O = make_double2(0.0, 0.0);
+      const int2* a = reinterpret_cast<const int2*>(J.mat[t] + (size_t)rows * K) + tid;
+      const int4* s = reinterpret_cast<const int4*>(sb + (size_t)t * 2 * Kh);
+      ZAcc ex, ey, ox, oy;
 #pragma unroll 4
-      for (int k = k0; k < k1; k += 2) {
-        const double ae = __ldg(a + k), ao = __ldg(a + k + 1);
-        const double2 ve = s[k], vo = s[k + 1];
-        E.x = fma(ae, ve.x, E.x); E.y = fma(ae, ve.y, E.y);
-        O.x = fma(ao, vo.x, O.x); O.y = fma(ao, vo.y, O.y);
+      for (int k = k0; k < k1; k += 2, a += 4 * rows) {
+        const int2 ae = __ldg(a), ao = __ldg(a + 2 * rows);
+        const int4 ve = s[k], vo = s[k + 1];
+        ex.add(ve.x, ve.y, ae);
+        ey.add(ve.z, ve.w, ae);
+        ox.add(vo.x, vo.y, ao);
+        oy.add(vo.z, vo.w, ao);
       }
-      E.x += __shfl_xor_sync(__activemask(), E.x, 1);
-      E.y += __shfl_xor_sync(__activemask(), E.y, 1);
-      O.x += __shfl_xor_sync(__activemask(), O.x, 1);
-      O.y += __shfl_xor_sync(__activemask(), O.y, 1);
+      long long Ex = ex.sum(), Ey = ey.sum(), Ox = ox.sum(), Oy = oy.sum();
+      Ex = z_half(Ex, __shfl_xor_sync(__activemask(), Ex, 1));
+      Ey = z_half(Ey, __shfl_xor_sync(__activemask(), Ey, 1));
+      Ox = z_half(Ox, __shfl_xor_sync(__activemask(), Ox, 1));
+      Oy = z_half(Oy, __shfl_xor_sync(__activemask(), Oy, 1));
+      const int e0 = emax_of(t, 0, 0) + 2, e1 = emax_of(t, 0, 1) + 2;
       const double al = J.alpha[t];
       // out_j = E + O ; out_{Mz-1-j} = E - O (parity (-1)^n) or -E + O (derivative parity)
-      const double se = J.deriv[t] ? -1.0 : 1.0;
-      lo.x = fma(al, E.x + O.x, lo.x); lo.y = fma(al, E.y + O.y, lo.y);
-      hi.x = fma(al, se * (E.x - O.x), hi.x); hi.y = fma(al, se * (E.y - O.y), hi.y);
+      lo.x = fma(al, value(z_half(Ex, Ox), e0), lo.x); lo.y = fma(al, value(z_half(Ey, Oy), e1), lo.y);
+      hi.x = fma(al, value(J.deriv[t] ? z_half(Ox, -Ex) : z_half(Ex, -Ox), e0), hi.x);
+      hi.y = fma(al, value(J.deriv[t] ? z_half(Oy, -Ey) : z_half(Ey, -Oy), e1), hi.y);
     }
     if (hf == 0) {
       const size_t o1 = (size_t)u * J.oi + (size_t)m * J.om;
@@ -159,27 +293,22 @@ __global__ void __launch_bounds__(256) zmm_kernel(const __grid_constant__ ZJobs 
     const int k0 = hf * (Kf / 2), k1 = hf ? Kf : Kf / 2;
     double2 acc = make_double2(0.0, 0.0);
     for (int t = 0; t < J.nterm; ++t) {
-      const double* a = J.mat[t] + (size_t)u * Kf;
+      const int2* a = reinterpret_cast<const int2*>(J.mat[t] + (size_t)rows * Kf) + tid;
       // even rows pair with s for parity (-1)^n, with d for derivative parity
-      const bool use_s = ((u & 1) == 0) != (J.deriv[t] != 0);
-      const double2* s = sb + (size_t)t * 2 * Kh + (use_s ? 0 : Kh);
-      double2 v0 = make_double2(0.0, 0.0), v1 = make_double2(0.0, 0.0);
-      int k = k0;
+      const int y = ((u & 1) == 0) != (J.deriv[t] != 0) ? 0 : 1;
+      const int4* s = reinterpret_cast<const int4*>(sb + (size_t)t * 2 * Kh + y * Kh);
+      ZAcc sx, sy;
 #pragma unroll 4
-      for (; k + 1 < k1; k += 2) {
-        const double a0 = __ldg(a + k), a1 = __ldg(a + k + 1);
-        const double2 x0 = s[k], x1 = s[k + 1];
-        v0.x = fma(a0, x0.x, v0.x); v0.y = fma(a0, x0.y, v0.y);
-        v1.x = fma(a1, x1.x, v1.x); v1.y = fma(a1, x1.y, v1.y);
+      for (int k = k0; k < k1; ++k, a += 2 * rows) {
+        const int2 w = __ldg(a);
+        const int4 v = s[k];
+        sx.add(v.x, v.y, w);
+        sy.add(v.z, v.w, w);
       }
-      if (k < k1) {
-        const double a0 = __ldg(a + k);
-        const double2 x0 = s[k];
-        v0.x = fma(a0, x0.x, v0.x); v0.y = fma(a0, x0.y, v0.y);
-      }
-      double vx = v0.x + v1.x, vy = v0.y + v1.y;
-      vx += __shfl_xor_sync(__activemask(), vx, 1);
-      vy += __shfl_xor_sync(__activemask(), vy, 1);
+      long long Sx = sx.sum(), Sy = sy.sum();
+      Sx = z_half(Sx, __shfl_xor_sync(__activemask(), Sx, 1));
+      Sy = z_half(Sy, __shfl_xor_sync(__activemask(), Sy, 1));
+      const double vx = value(Sx, emax_of(t, y, 0) + 1), vy = value(Sy, emax_of(t, y, 1) + 1);
       acc.x = fma(J.alpha[t], vx, acc.x); acc.y = fma(J.alpha[t], vy, acc.y);
     }
     if (hf == 0) {
