@@ -109,7 +109,7 @@ __device__ __forceinline__ double2* row(double* base, int b, int K) {
 
 // ---- single-shot kernels (transforms, F, JVP, VJP) ---------------------------------------
 //
-// One call of these is all launch and latency (about 10 us), so they keep the FP64 transforms; the step loops
+// One call of these is all launch and latency, so they keep the FP64 transforms; the step loops
 // below run the fixed-point ones.
 
 // coefficients -> grid with the weights w0 (k = 0) and w
