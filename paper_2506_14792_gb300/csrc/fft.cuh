@@ -1,4 +1,5 @@
-// FP64 shared-memory FFTs for the collocation transforms (Methods, "Spectral transforms").
+// FP64 shared-memory FFTs for the collocation transforms (Methods, "Spectral transforms"), run by the lengths and
+// calls that do not take the fixed-point ones (fxfft.cuh).
 //
 // A real field of M = 2L grid points is transformed through one complex FFT of length
 // L on the packed sequence z_j = g_{2j} + i g_{2j+1} (the classic half-length real FFT),
@@ -176,9 +177,6 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 }
 __device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
 __device__ __forceinline__ double2 cscale(double2 a, double s) { return make_double2(a.x * s, a.y * s); }
-// multiply by i*s (s = +-1)
-__device__ __forceinline__ double2 cmul_i(double2 a, double s) { return make_double2(-s * a.y, s * a.x); }
-
 // Packed-spectrum entry of a real inverse transform, e + i d conj(w), written as two multiply-add
 // chains (the FP64 pipe is the binding resource: 8 instructions per entry instead of 10).
 __device__ __forceinline__ double2 c2r_combine(double2 e, double2 d, double2 w) {
@@ -315,15 +313,12 @@ __device__ __forceinline__ void stockham_bfly(int R, int Ns, int j, int nbf, con
   }
 }
 
-// Complex FFT of length p.n held in buffer a (b is scratch of the same size).  SIGN = -1:
-// forward exp(-), SIGN = +1: inverse exp(+) (unnormalised).  Returns the buffer holding
-// the result (a or b).  All threads of the CTA must call it; it synchronises internally
-// and on return the result is visible to every thread.  The WM argument is unused (the
-// butterflies read the plan's scaled-twiddle records); it stays for the callers' symmetry
-// with the real pre/post-processing.
+// Complex FFTs of length p.n (SIGN = -1: forward exp(-), SIGN = +1: inverse exp(+), unnormalised) of ns sequences,
+// sequence s held in a + s * stride with scratch b + s * stride: their butterflies share every pass and its
+// barrier.  The results are in a (+ s * stride) when p.nrad is even, else in b, and visible to every thread.  All
+// threads of the CTA must call it.
 template <int SIGN>
-static __device__ __noinline__ double2* cfft_smem_t(double2* a, double2* b, const FFTPlan p,
-                                                    const double2* __restrict__ WM) {
+static __device__ __noinline__ void cfft_smem_sets(double2* a, double2* b, int stride, int ns, const FFTPlan p) {
   const int n = p.n;
   const int tid = threadIdx.x, nt = blockDim.x;
   int Ns = 1;
@@ -331,64 +326,11 @@ static __device__ __noinline__ double2* cfft_smem_t(double2* a, double2* b, cons
   for (int pass = 0; pass < p.nrad; ++pass) {
     const int R = p.rad[pass];
     const int nbf = n / R;
-    for (int j = tid; j < nbf; j += nt)
-      stockham_bfly<SIGN>(R, Ns, j, nbf, rec, [&](int e) { return a[e]; }, [&](int e, double2 v) { b[e] = v; });
-    __syncthreads();
-    double2* tmp = a; a = b; b = tmp;
-    rec += sc_pass_entries(R, Ns);
-    Ns *= R;
-  }
-  return a;
-}
-
-// nb interleaved complex FFTs of length p.n: element e of sequence c at a[e * nb + c] (the
-// layout of a tile of nb adjacent columns).  Same passes as cfft_smem_t; threads stride over
-// (butterfly, sequence) pairs so consecutive threads touch consecutive sequences.
-template <int SIGN>
-static __device__ __noinline__ double2* cfft_smem_batch(double2* a, double2* b, const FFTPlan p,
-                                                        const double2* __restrict__ WM, int nb) {
-  const int n = p.n;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  int Ns = 1;
-  const double2* __restrict__ rec = p.sc[SIGN > 0 ? 1 : 0];
-  for (int pass = 0; pass < p.nrad; ++pass) {
-    const int R = p.rad[pass];
-    const int nbf = n / R;
-    for (int idx = tid; idx < nbf * nb; idx += nt) {
-      const int j = idx / nb, c = idx - j * nb;
-      stockham_bfly<SIGN>(R, Ns, j, nbf, rec, [&](int e) { return a[e * nb + c]; },
-                          [&](int e, double2 v) { b[e * nb + c] = v; });
-    }
-    __syncthreads();
-    double2* tmp = a; a = b; b = tmp;
-    rec += sc_pass_entries(R, Ns);
-    Ns *= R;
-  }
-  return a;
-}
-
-// ns sets of nb interleaved complex FFTs of length p.n (the layout of cfft_smem_batch), set s
-// held in a + s * stride with scratch b + s * stride: the sets' butterflies share every pass and
-// its barrier, and together fill more lanes than one set.  The results are in a (+ s * stride)
-// when p.nrad is even, else in b.
-template <int SIGN>
-static __device__ __noinline__ void cfft_smem_sets(double2* a, double2* b, int stride, int ns, const FFTPlan p,
-                                                   int nb) {
-  const int n = p.n;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  int Ns = 1;
-  const double2* __restrict__ rec = p.sc[SIGN > 0 ? 1 : 0];
-  for (int pass = 0; pass < p.nrad; ++pass) {
-    const int R = p.rad[pass];
-    const int nbf = n / R;
-    const int per = nbf * nb;
-    for (int idx = tid; idx < per * ns; idx += nt) {
-      const int set = idx / per, i = idx - set * per;
-      const int j = i / nb, c = i - j * nb;
+    for (int idx = tid; idx < nbf * ns; idx += nt) {
+      const int set = idx / nbf, j = idx - set * nbf;
       const double2* as = a + set * stride;
       double2* bs = b + set * stride;
-      stockham_bfly<SIGN>(R, Ns, j, nbf, rec, [&](int e) { return as[e * nb + c]; },
-                          [&](int e, double2 v) { bs[e * nb + c] = v; });
+      stockham_bfly<SIGN>(R, Ns, j, nbf, rec, [&](int e) { return as[e]; }, [&](int e, double2 v) { bs[e] = v; });
     }
     __syncthreads();
     double2* tmp = a; a = b; b = tmp;
@@ -396,20 +338,13 @@ static __device__ __noinline__ void cfft_smem_sets(double2* a, double2* b, int s
     Ns *= R;
   }
 }
-
-__device__ __forceinline__ double2* cfft_smem(double2* a, double2* b, const FFTPlan p, const double2* __restrict__ WM,
-                                              int sign) {
-  return sign > 0 ? cfft_smem_t<1>(a, b, p, WM) : cfft_smem_t<-1>(a, b, p, WM);
-}
-
 
 // ---- real transforms on the packed half-length sequence ---------------------------------
 //
 // c2r: coefficients c_k (k < K, read through get(k)) of a real field, g_j = sum over the
 // Hermitian-completed spectrum with weights w0 (k = 0, real part only) and w (k >= 1):
 //   g_j = w0 Re c_0 + w * 2 Re sum_{k=1}^{K-1} c_k e^{2 pi i k j / M}
-// Fills Z (length L) so that the inverse L-point FFT of Z is z_j = g_{2j} + i g_{2j+1}.
-// Entry k (< L) of the packed spectrum described below (UNIT: w0 = w = 1).
+// Entry k (< L) of the packed spectrum Z whose inverse L-point FFT is z_j = g_{2j} + i g_{2j+1} (UNIT: w0 = w = 1).
 template <bool UNIT, class Get>
 __device__ __forceinline__ double2 c2r_entry(Get get, int k, int K, int L, const double2* __restrict__ WM, double w0,
                                              double w) {
@@ -423,31 +358,4 @@ __device__ __forceinline__ double2 c2r_entry(Get get, int k, int K, int L, const
   if (k > 0 && kc < K) xc = cconj(UNIT ? get(kc) : cscale(get(kc), w));
   return c2r_combine(cadd(xk, xc), csub(xk, xc), __ldg(&WM[k]));  // e + i (xk - xc) exp(+2 pi i k / M)
 }
-template <bool UNIT, class Get>
-__device__ __forceinline__ void c2r_pre_t(double2* Z, Get get, int K, int L, const double2* __restrict__ WM,
-                                          double w0, double w) {
-  for (int k = threadIdx.x; k < L; k += blockDim.x) Z[k] = c2r_entry<UNIT>(get, k, K, L, WM, w0, w);
-}
-template <class Get>
-__device__ __forceinline__ void c2r_pre(double2* Z, Get get, int K, int L, const double2* __restrict__ WM,
-                                        double w0, double w) {
-  if (w0 == 1.0 && w == 1.0) c2r_pre_t<true>(Z, get, K, L, WM, w0, w);
-  else c2r_pre_t<false>(Z, get, K, L, WM, w0, w);
-}
-
-// r2c post: z = forward L-point FFT of the packed real field; returns
-//   X_k = sum_j g_j e^{-2 pi i k j / M}  for k < K  (via put(k, X_k)).
-// r2c_post2: the same with put(k, 2 X_k), for callers that fold the factor 1/2 into their own
-// scaling.
-template <class Put>
-__device__ __forceinline__ void r2c_post2(const double2* Z, Put put, int K, int L, const double2* __restrict__ WM) {
-  for (int k = threadIdx.x; k < K; k += blockDim.x)
-    put(k, r2c_combine2(Z[k], cconj(Z[k == 0 ? 0 : L - k]), __ldg(&WM[k])));
-}
-template <class Put>
-__device__ __forceinline__ void r2c_post(const double2* Z, Put put, int K, int L, const double2* __restrict__ WM) {
-  for (int k = threadIdx.x; k < K; k += blockDim.x)
-    put(k, r2c_combine(Z[k], cconj(Z[k == 0 ? 0 : L - k]), __ldg(&WM[k])));
-}
-
 }  // namespace spadj

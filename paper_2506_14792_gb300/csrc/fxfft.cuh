@@ -25,9 +25,9 @@
 //
 // Accuracy.  The rounding is about 0.7 units of 2^-59 of the largest value in each pass, against 2^-53 of each
 // value in FP64, and the results are rounded to FP64 once: the relative 2-norm error of complex transforms
-// (n = 3..1536; flat, smooth, single-mode and 1/k inputs) is 0.4-1.3e-16 against 1.3-2.5e-16 of FP64
-// butterflies, and that of the real ones up to 2 x 768 points 0.5-2.0e-16 against 1.3-2.8e-16; the longer
-// real transforms (peaked spectra: 2.0e-16 against 2.0e-16) stay with the FP64 butterflies of fft.cuh.  Non-finite
+// (n = 3..1536; flat, smooth, single-mode, 1/k and low-pass inputs) is at most 1.5e-16 against 2.5e-16 of FP64
+// butterflies, and that of the real ones up to 2 x 768 points at most 1.6e-16 against 3.3e-16; longer real transforms
+// (peaked spectra: 2.0e-16 against 2.0e-16) stay with the FP64 butterflies of fft.cuh.  Non-finite
 // input gives NaN in every output of the sequence; sequences below 2^-895 are scaled up by 2^512 first, so
 // subnormals keep their bits.
 #pragma once
@@ -688,7 +688,7 @@ __device__ __forceinline__ FxRes<INV> fx_run(int a, int b, FxLay lay, FxGroup g,
 }
 template <bool INV>
 __device__ __forceinline__ FxRes<INV> fx_run64(int a, int b, FxLay lay, const FFTPlan& p) {
-  cfft_smem_sets<INV ? 1 : -1>(fx_mem64() + a, fx_mem64() + b, lay.stride, lay.ns, p, 1);
+  cfft_smem_sets<INV ? 1 : -1>(fx_mem64() + a, fx_mem64() + b, lay.stride, lay.ns, p);
   return FxRes<INV>{(p.nrad & 1) ? b : a, lay, p.n, p.fxr, p.wm, false};
 }
 
