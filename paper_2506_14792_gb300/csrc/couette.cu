@@ -110,7 +110,6 @@ struct Couette : EqImpl {
     xp.plan = make_plan(L);
     yp.Kx = Kx; yp.Ny = Ny; yp.My = My;
     yp.TK = Kx >= 8 ? 8 : Kx >= 4 ? 4 : Kx >= 2 ? 2 : 1;
-    yp.ntile = (Kx + yp.TK - 1) / yp.TK;
     yp.kxs = 2.0 * M_PI / Lx; yp.kys = 2.0 * M_PI / Ly;
     yp.plan = make_plan(My);
     yp.C = My;
@@ -184,7 +183,18 @@ struct Couette : EqImpl {
     SPADJ_CUDA_TRY(p, sdev.ensure(sizeof(double) * 2));
     SPADJ_CUDA_TRY(p, Jdev.ensure(sizeof(double)));
     zsmem = (size_t)2 * 2 * (size_t)std::max(N, Mz / 2) * kTM * sizeof(double2);
-    ysmem = sizeof(double2) * (2 * (size_t)yp.C + 1) * yp.TK;
+    // The y transforms' buffers pass 48 KB from n[1] = 128 on (with 8 columns per CTA): more needs the kernel's consent,
+    // and fewer columns where even that is not enough.  Sizes that fit with none are refused by the launch.
+    constexpr size_t kOptIn = 227 * 1024 - sizeof(FxShared);
+    auto ybytes = [&](int tk) { return sizeof(double2) * (2 * (size_t)My + 1) * tk; };
+    while (yp.TK > 1 && ybytes(yp.TK) > kOptIn) yp.TK /= 2;
+    yp.ntile = (Kx + yp.TK - 1) / yp.TK;
+    ysmem = ybytes(yp.TK);
+    if (ysmem > 48 * 1024 - sizeof(FxShared) && ysmem <= kOptIn)
+      SPADJ_CUDA_TRY(p, with_yfft([](auto kernel) {
+        // the largest size, so that no other problem's creation lowers it
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOptIn);
+      }));
     {  // the step-solve operators of the selected form (the other one is built on first use)
       // One warp per pencil pair runs the band sweeps: with fewer than 8 pairs per SM the warps
       // cannot keep the FP64 pipe busy and the dense Phi (a CTA per pair) is faster (measured:
@@ -253,14 +263,17 @@ struct Couette : EqImpl {
     j.dir = 1; j.in[0] = in; j.alpha[0] = 1.0; j.nin = 1; j.scale = scale; j.out = out;
     return j;
   }
+  template <class Fn>
+  cudaError_t with_yfft(Fn go) {
+    return yp.TK == 8 ? go(yfft_kernel<8>) : yp.TK == 4 ? go(yfft_kernel<4>) : yp.TK == 2 ? go(yfft_kernel<2>)
+                                                                                          : go(yfft_kernel<1>);
+  }
   spadj_status launch_y(Problem* p, YJobs& js) {
     const double f = js.n * (double)Mz * Kx * 5.0 * My * std::log2((double)My);
     cudaEvent_t t = p->tic();
-    auto go = [&](auto kernel) {
+    SPADJ_CUDA_TRY(p, with_yfft([&](auto kernel) {
       return launch_kernel(p->pdl, kernel, dim3(Mz * yp.ntile, js.n), dim3(128), ysmem, p->stream, js, yp);
-    };
-    SPADJ_CUDA_TRY(p, yp.TK == 8 ? go(yfft_kernel<8>) : yp.TK == 4 ? go(yfft_kernel<4>) : yp.TK == 2 ? go(yfft_kernel<2>)
-                                                                                                 : go(yfft_kernel<1>));
+    }));
     p->toc(t, KC_YFFT, f);
     return check_launch(p, "couette yfft");
   }
