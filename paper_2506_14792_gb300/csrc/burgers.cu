@@ -295,10 +295,10 @@ __global__ void __launch_bounds__(64, MB) trajectory_kernel(const __grid_constan
         }
       }
       fx_put64(s.B + k, X[q][0]);
-      mx = fx_absmax(mx, X[q][0]);
+      mx = fx_absmax(mx, fx_c0(k, X[q][0]));
       if (tangent) {
         fx_put64(s.D + k, D[q][0]);
-        md = fx_absmax(md, D[q][0]);
+        md = fx_absmax(md, fx_c0(k, D[q][0]));
       }
       if (traj) stg128(row(traj, b, K) + k, X[q][0]);
     }
@@ -417,13 +417,13 @@ __global__ void __launch_bounds__(64, MB) adjoint_kernel(const __grid_constant__
         if (k >= K) continue;
         const double2 x = ldg128(xn + k);
         fx_put64(s.B + k, x);
-        mx = fx_absmax(mx, x);
+        mx = fx_absmax(mx, fx_c0(k, x));
         double2 w = axpby(wc[1], Y[q][0], wc[2], Y[q][1]);
 #pragma unroll
         for (int i = 3; i <= ORD; ++i) w = make_double2(w.x + wc[i] * Y[q][i - 1].x, w.y + wc[i] * Y[q][i - 1].y);
         w = plus_i(hk[q], w);
         fx_put64(s.D + k, w);
-        mw = fx_absmax(mw, w);
+        mw = fx_absmax(mw, fx_c0(k, w));
       }
       for (int q = 0; q < Q; ++q) lam[q] = z;
       if (P.nonlinear) {

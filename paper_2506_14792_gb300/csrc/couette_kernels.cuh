@@ -79,6 +79,8 @@ __global__ void __launch_bounds__(128) yfft_kernel(const __grid_constant__ YJobs
         v.x = fma(J.alpha[t], x.x, v.x);
         v.y = fma(J.alpha[t], x.y, v.y);
       }
+      // the imaginary part of the mean reaches only what the x transform leaves out: not into the column's scale
+      if (m == 0 && q == 0) v.y = 0.0;
       return v;
     });
     for (int idx = tid; idx < My * TK; idx += nt) {

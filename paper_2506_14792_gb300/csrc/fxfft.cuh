@@ -665,6 +665,10 @@ struct FxRes {
   }
 };
 
+// Entry k of a real field's spectrum without Im c_0, which the inverse transforms do not use: it must not take part in the
+// sequence's scale either (a large one would cost the other coefficients their bits, a non-finite one the row).
+__device__ __forceinline__ double2 fx_c0(int k, double2 v) { return k == 0 ? make_double2(v.x, 0.0) : v; }
+
 // FP64 values of cnt entries of every sequence into dst, and the sequences' largest high words
 template <int NS, int W, class Load>
 __device__ __forceinline__ void fx_stage(int dst, FxLay lay, int cnt, Load load) {
@@ -724,8 +728,8 @@ __device__ __forceinline__ FxRes<INV> xf_c2c(int a, int b, FxLay lay, const FFTP
   return xf_c2c_staged<INV, NS, W, PATH, REAL, false>(a, b, lay, p);
 }
 
-// xf_c2r (below) with the c_k of every sequence already in b as FP64 pairs and their largest high words given
-// (EVERY: by fx_put_max in all warps); the call starts with a barrier.
+// xf_c2r (below) with the c_k of every sequence already in b as FP64 pairs and their largest high words, of c_0 the real
+// part's (fx_c0), given (EVERY: by fx_put_max in all warps); the call starts with a barrier.
 template <int NS, int PATH = kFxAny, bool EVERY = true>
 __device__ __forceinline__ FxRes<true> xf_c2r_staged(int a, int b, FxLay lay, const FFTPlan& p, int K) {
   const int n = p.n;
@@ -747,7 +751,7 @@ __device__ __forceinline__ FxRes<true> xf_c2r_staged(int a, int b, FxLay lay, co
   unsigned l1 = 0u;
   for (int k = g.l; k < half; k += g.T) {
     const int kc = n - k;
-    // c_k and c_{n-k} (0 where not stored), c_0 real
+    // c_k and c_{n-k} (0 where not stored), c_0's real part
     const bool hx = k < K, hy = k > 0 && kc < K;
     double2 sx = fx_get64(S + (hx ? k : 0)), sy = fx_get64(S + (hy ? kc : 0));
     if (!hx) sx.x = 0.0;
@@ -776,7 +780,7 @@ __device__ __forceinline__ FxRes<true> xf_c2r_staged(int a, int b, FxLay lay, co
 // j < 2n, from c_k = load(s, k) (the imaginary part of c_0 is not used).
 template <int NS, int PATH = kFxAny, class Load>
 __device__ __forceinline__ FxRes<true> xf_c2r(int a, int b, FxLay lay, const FFTPlan& p, int K, Load load) {
-  fx_stage<NS, 1>(b, lay, K, load);
+  fx_stage<NS, 1>(b, lay, K, [&](int s, int k) { return fx_c0(k, load(s, k)); });
   return xf_c2r_staged<NS, PATH, false>(a, b, lay, p, K);
 }
 

@@ -155,6 +155,8 @@ __device__ __forceinline__ double2 field_entry(int f, const double2* xs, const d
   const int q = yrow(j, N, M);
   if (q < 0) return make_double2(0.0, 0.0);
   const double2 x = ldcg2(&xs[q]);
+  // (the imaginary part of omega's mean reaches only what the x transform leaves out: not into the sequence's scale)
+  if (f == 4 && kx == 0 && q == 0) return make_double2(x.x, 0.0);
   return f < 4 ? fmult(f, (double)kx, (double)kyof(q, N), __ldg(&ik2[q]), x) : x;
 }
 
