@@ -149,10 +149,10 @@ struct Couette : EqImpl {
     };
     SPADJ_CUDA_TRY(p, up(wmx, hwx.data(), sizeof(double2) * hwx.size()));
     SPADJ_CUDA_TRY(p, up(twy, hwy.data(), sizeof(double2) * hwy.size()));
+    std::vector<std::vector<double>> tables;  // kept until the copies on the problem's stream are done
     auto upz = [&](DevBuf& b, const std::vector<double>& h, int rows, int cols) -> cudaError_t {
-      const std::vector<double> z = z_table(h, rows, cols);
-      cudaError_t e = b.ensure(sizeof(double) * z.size());
-      return e != cudaSuccess ? e : cudaMemcpy(b.ptr, z.data(), sizeof(double) * z.size(), cudaMemcpyHostToDevice);
+      tables.push_back(z_table(h, rows, cols));
+      return up(b, tables.back().data(), sizeof(double) * tables.back().size());
     };
     SPADJ_CUDA_TRY(p, upz(czE, hczE, Mh, N));
     SPADJ_CUDA_TRY(p, upz(cdzE, hcdzE, Mh, N));
