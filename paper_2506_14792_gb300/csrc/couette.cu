@@ -182,7 +182,7 @@ struct Couette : EqImpl {
     SPADJ_CUDA_TRY(p, edev.ensure(sizeof(double) * 2));
     SPADJ_CUDA_TRY(p, sdev.ensure(sizeof(double) * 2));
     SPADJ_CUDA_TRY(p, Jdev.ensure(sizeof(double)));
-    zsmem = (size_t)2 * 2 * (size_t)std::max(N, Mz / 2) * kTM * sizeof(double2);
+    zsmem = zmm_smem(std::max(N, Mz / 2));
     // The y transforms' buffers pass 48 KB from n[1] = 128 on (with 8 columns per CTA): more needs the kernel's consent,
     // and fewer columns where even that is not enough.  Sizes that fit with none are refused by the launch.
     constexpr size_t kOptIn = 227 * 1024 - sizeof(FxShared);

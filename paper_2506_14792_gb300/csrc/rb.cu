@@ -243,7 +243,7 @@ struct RB : EqImpl {
     SPADJ_CUDA_TRY(p, Jdev.ensure(sizeof(double)));
     SPADJ_CUDA_TRY(p, errbuf.ensure(sizeof(int)));
     SPADJ_CUDA_TRY(p, cudaMemsetAsync(errbuf.ptr, 0, sizeof(int), p->stream));
-    zsmem = (size_t)2 * 2 * (size_t)std::max(N, Mz / 2) * kTM * sizeof(double2);
+    zsmem = zmm_smem(std::max(N, Mz / 2));
     xsmem = sizeof(double2) * (4 * L + Kx);
     const int H = 3 * (N / 2);
     ssmem = sizeof(double2) * (H + 4 * solve_rows(H)) + sizeof(double) * (size_t)H * solve_rows(H);

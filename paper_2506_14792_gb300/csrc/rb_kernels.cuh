@@ -76,30 +76,28 @@ __device__ __forceinline__ double2 zmult(const ZJobs& js, int type, int m, doubl
 // One CTA per (column, job); the reduction of every output is split over the two lanes of a
 // lane pair and combined with a shuffle, so an expand job runs 2*Mz/2 threads and a fold job
 // 2*N threads per column.
-constexpr int kTM = 1;  // columns per CTA
-
 __host__ __device__ inline int zmm_threads(int expand, int I) {  // whole warps
   return (2 * (expand ? I / 2 : I) + 31) / 32 * 32;
 }
 
 // The products run in fixed point on the integer pipes.  This chip issues under 2 FP64 multiply-adds per clock and
-// SM against about 25 32 x 32 + 64 bit integer ones, three of which make a product of the format below: the
+// SM against about 25 32 x 32 + 64 bit integer ones, six of which make a product of the format below: the
 // kernel was bound by its FP64 instructions and by matrix rows read one line per lane.  With the products in fixed
-// point and the limbs in the threads' order, explicit terms of 256 x 64 Rayleigh-Benard take 37 us (51 before),
-// gradients of 8 Couette steps at 128 x 64 x 64 19.1 ms (24.2 before; 23.9 with the products alone).  Reading the limbs
-// before the wait for the predecessor hides their latency where CTAs are few (RK443 at 96 x 40: 5.2 ms without, 4.7 with).
+// point and the limbs in the threads' order, gradients of 8 Couette steps at 128 x 64 x 64 take 20.3 ms (24.2 with FP64
+// products; 19.0 with two limbs, too few of them, see below), 40 steps of 256 x 64 Rayleigh-Benard 14.0 ms (14.9; 13.7).
+// An expansion is bound by the integer multiply-adds now (75 % of their rate).  Reading the limbs before the wait for the
+// predecessor hides their latency where CTAs are few (RK443 at 96 x 40: 5.2 ms without, 4.7 with two limbs).
 //
 // Format.  Column k of a matrix is scaled by a power of two, 2^-e_k, so that its largest entry is in [1/2, 1), and stored
-// as 2^-57 (2^28 wh + wl); the staged entries x_k 2^(e_k) share one exponent per term, component and (fold) symmetry,
-// the largest below 2^56, and are split into 2^28 xh + xl.  A sum of products is
-//   (sum xh wh + 2^-28 (sum xh wl + xl wh) + O(1/4)) / 2  in units of the entries,
-// all sums exact in 64 bits (a lane's at most 48 terms of 2^57; sums of sums are halved).  The dropped and rounded
-// parts are random, about 0.3 units of 2^-57 of the largest entry per product; FP64 rounds every product and partial
-// sum to 2^-53 of itself.  Relative 2-norm errors against extended sums, N = 8..128, columns like 1/n^2 or exp(-0.4 n):
-// 0.6-1.2e-16 against 0.8-5.1e-16 of FP64; flat columns 0.5-0.9e-16 against 0.7-3.7e-16 (the derivative's expansion
-// 1.1-2.4e-16 against 1.0-2.8e-16); columns graded by exp(-12 (k mod 5)) 0.6-0.9e-16 against 0.7-2.7e-16, only there
-// the derivative's expansion loses (2.9e-16 against 1.9e-16).  A column with a non-finite entry gives NaN; entries
-// below 2^-1022 count as zero.
+// as 2^-57 (2^28 wh + wl + 2^-28 wt); the staged entries x_k 2^(e_k) share one exponent per term, component and (fold)
+// symmetry, the largest below 2^56, and are split into 2^28 xh + xl + 2^-28 xt.  A sum of products is
+//   (sum xh wh + 2^-28 (sum xh wl + xl wh) + 2^-56 (sum xh wt + xl wl + xt wh) + O(2^-56)) / 2  in units of the entries,
+// all sums exact in 64 bits (a lane's at most 48 terms of 2^57; sums of sums are halved).  The third limbs are there for
+// rows far below their columns' largest entries: the derivative's column at the wall spans 1 to N^2, and two limbs
+// left the adjoint's low modes with errors of 1.4e-14 (N = 64) to 1e-13 (N = 128) of sum |a||x| where FP64 sums have
+// 2e-16.  With them every entry of a table is exact (entries span less than 2^32 of a column), a staged entry has 53 bits
+// down to 2^-31 of the largest and its leading ones down to 2^-84, and every row of every product is a rounding or two
+// of 2^-53 from the exact sum.  A column with a non-finite entry gives NaN.
 struct ZLimb {
   int h, l;
 };
@@ -118,30 +116,53 @@ __host__ __device__ __forceinline__ long long z_fixed(double x, int e, int emax)
   std::memcpy(&bits, &x, 8);
   const unsigned hi = (unsigned)(bits >> 32), lo = (unsigned)bits;
 #endif
-  const int ex = (int)((hi >> 20) & 0x7ff), d = emax - (ex + e);
-  if (ex == 0 || d > 57) return 0;
-  const long long m = (long long)(((unsigned long long)((hi & 0xfffff) | 0x100000) << 32 | lo) << 3);
+  const int ex = (int)((hi >> 20) & 0x7ff), d = emax - ((ex ? ex : 1) + e);
+  if (d > 57) return 0;
+  const long long m = (long long)(((unsigned long long)((hi & 0xfffff) | (ex ? 0x100000 : 0)) << 32 | lo) << 3);
   const long long v = (m + (d > 0 ? 1ll << (d - 1) : 0)) >> d;
   return (int)hi < 0 ? -v : v;
 }
-// The device form of a z matrix (rows x cols): its entries, the limbs (wh, wl) of every entry, and e_k per column
-// (as 32-bit integers), all in 8-byte units.  The limbs are ordered as zmm_kernel's threads read them: entry kk of
+// what z_fixed rounded off, in units of 2^-28, |t| <= 2^27
+__host__ __device__ __forceinline__ int z_tail(double x, int e, int emax) {
+#ifdef __CUDA_ARCH__
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+#else
+  unsigned long long bits;
+  std::memcpy(&bits, &x, 8);
+  const unsigned hi = (unsigned)(bits >> 32), lo = (unsigned)bits;
+#endif
+  const int ex = (int)((hi >> 20) & 0x7ff), d = emax - ((ex ? ex : 1) + e);
+  if (d <= 0 || d > 90) return 0;
+  const unsigned long long m = ((unsigned long long)((hi & 0xfffff) | (ex ? 0x100000 : 0)) << 32 | lo) << 3;
+  // the d low bits of m as a signed fraction (one half and more were rounded up), or all of m below 2^-1
+  const int t = d <= 57 ? (int)((long long)(m << (64 - d)) >> 36) : (int)(m >> (d - 28));
+  return (int)hi < 0 ? -t : t;
+}
+// The device form of a z matrix (rows x cols): its entries, the limbs (wh, wl) of every entry, e_k per column
+// (as 32-bit integers), all in 8-byte units, and the third limbs as 32-bit integers in the order of the others.  The limbs are ordered as zmm_kernel's threads read them: entry kk of
 // row r's half hf (columns hf (cols / 2) + kk) at (kk rows + r) 2 + hf, so that a warp reads 256 consecutive bytes
 // (row by row, a load of a warp touched 32 lines, and that, not the arithmetic, was the kernel's time).
 __host__ __device__ inline size_t z_limb_entries(int rows, int cols) { return 2 * (size_t)rows * ((cols + 1) / 2); }
+__host__ __device__ inline size_t z_tail_offset(int rows, int cols) {  // of the third limbs, in 8-byte units
+  return (size_t)rows * cols + z_limb_entries(rows, cols) + (cols + 1) / 2;
+}
 inline std::vector<double> z_table(const std::vector<double>& A, int rows, int cols) {
   std::vector<double> t(A);
-  t.resize((size_t)rows * cols + z_limb_entries(rows, cols) + (cols + 1) / 2, 0.0);
+  t.resize(z_tail_offset(rows, cols) + z_limb_entries(rows, cols) / 2, 0.0);
   for (int k = 0; k < cols; ++k) {
     double m = 0.0;
     for (int r = 0; r < rows; ++r) m = std::max(m, std::fabs(A[(size_t)r * cols + k]));
     int e = 0;
     std::frexp(m, &e);
     for (int r = 0; r < rows; ++r) {
-      const ZLimb w = z_limbs(std::llround(std::ldexp(A[(size_t)r * cols + k], 57 - e)));
+      const double a = std::ldexp(A[(size_t)r * cols + k], 57 - e);
+      const long long n = std::llround(a);
+      const ZLimb w = z_limbs(n);
       const int2 v = make_int2(w.h, w.l);
-      const int hf = k >= cols / 2, kk = k - hf * (cols / 2);
-      std::memcpy(&t[(size_t)rows * cols + 2 * ((size_t)kk * rows + r) + hf], &v, 8);
+      const int hf = k >= cols / 2, kk = k - hf * (cols / 2), tail = (int)std::lround(std::ldexp(a - (double)n, 28));
+      const size_t at = 2 * ((size_t)kk * rows + r) + hf;
+      std::memcpy(&t[(size_t)rows * cols + at], &v, 8);
+      std::memcpy(reinterpret_cast<char*>(&t[z_tail_offset(rows, cols)]) + 4 * at, &tail, 4);
     }
     std::memcpy(reinterpret_cast<char*>(&t[(size_t)rows * cols + z_limb_entries(rows, cols)]) + 4 * k, &e, 4);
   }
@@ -157,15 +178,64 @@ struct ZAcc {  // sum xh wh, sum (xh wl + xl wh)
 };
 // (a + b) / 2
 __host__ __device__ __forceinline__ long long z_half(long long a, long long b) { return (a >> 1) + (b >> 1) + (a & b & 1); }
+// h + 2^-56 f, |f| < 2^58
+struct ZWide {
+  long long h, f;
+};
+__host__ __device__ __forceinline__ ZWide z_neg(ZWide a) { return ZWide{-a.h, -a.f}; }
+__host__ __device__ __forceinline__ ZWide z_half(ZWide a, ZWide b) {
+  return ZWide{z_half(a.h, b.h), ((a.f + b.f) >> 1) + (((a.h ^ b.h) & 1) << 55)};
+}
+struct ZAcc3 : ZAcc {  // with the third limbs: sum (xh wt + xl wl + xt wh)
+  long long d = 0;
+  __host__ __device__ __forceinline__ void add(int xh, int xl, int xt, int2 w, int wt) {
+    ZAcc::add(xh, xl, w);
+    d = fx_mad(xh, wt, fx_mad(xl, w.y, fx_mad(xt, w.x, d)));
+  }
+  __host__ __device__ __forceinline__ ZWide wide() const {
+    const long long m = c + (d >> 28);  // in units of 2^-28, and what is left of d below it
+    return ZWide{a + (m >> 28), (m & ((1ll << 28) - 1)) << 28 | (d & ((1ll << 28) - 1))};
+  }
+};
+// (h + 2^-56 f) 2^se rounded to FP64 (se >= kFxNaN / 2: NaN)
+__host__ __device__ inline double z_to_double(ZWide v, int se) {
+  long long h = v.h + (v.f >> 56);
+  unsigned long long l = (unsigned long long)v.f << 8;  // 64 bits below h
+  const bool neg = h < 0;
+  if (neg) {
+    l = 0 - l;
+    h = ~h + (l == 0);
+  }
+  // the leading 63 bits: fx_to_double rounds them as it would the whole number
+#ifdef __CUDA_ARCH__
+  const int z = h ? __clzll(h) - 1 : 63;
+#else
+  const int z = h ? __builtin_clzll((unsigned long long)h) - 1 : 63;
+#endif
+  const long long t = z > 0 ? (long long)((unsigned long long)h << z | l >> (64 - z)) : h;
+  return fx_to_double(neg ? -t : t, se - z);
+}
+// Places of a staged column: entry k of symmetry y at y ld + k, and gap further in the second half, so that the up to four
+// entries that a warp reads at once (two halves, two symmetries) lie in different banks (20.65 ms without).
+struct ZPlaces {
+  int half, gap, ld;
+  __host__ __device__ __forceinline__ explicit ZPlaces(int Kh)
+      : half(Kh / 2), gap((2 - Kh / 2) & 7), ld(Kh + gap + ((4 - Kh - gap) & 7)) {}
+  __host__ __device__ __forceinline__ int at(int y, int k) const { return y * ld + k + (k >= half ? gap : 0); }
+};
+constexpr int kZPad = 14;  // most entries that ZPlaces adds to a symmetry
+// dynamic shared memory of zmm_kernel: two terms of two symmetries of at most Kmax entries, and their third limbs
+inline size_t zmm_smem(int Kmax) { return (size_t)2 * 2 * (Kmax + kZPad) * (sizeof(double2) + sizeof(int2)); }
 constexpr int kZSlots = 8;  // maxima of a warp: term (2) x symmetry (2) x component (2)
 
-__global__ void __launch_bounds__(256) zmm_kernel(const __grid_constant__ ZJobs js) {
+// Three CTAs of 256 threads per SM: 80 registers; left alone the compiler takes 64 and spills (RK443 at 96 x 40: 4.85 ms against 5.08).
+__global__ void __launch_bounds__(256, 3) zmm_kernel(const __grid_constant__ ZJobs js) {
   pdl_trigger();
   const ZJob& J = js.j[blockIdx.y];
   const int rows = js.expand ? J.I / 2 : J.I;  // of the matrices
-  {  // one word of every line of the limbs and exponents: they are in L1 when the column has arrived
+  {  // one word of every line of the limbs, exponents and third limbs: they are in L1 when the column has arrived
     const int cols = js.expand ? J.K : J.K / 2;
-    const int lines = (int)((8 * (z_limb_entries(rows, cols) + (cols + 1) / 2) + 127) / 128);
+    const int lines = (int)((12 * z_limb_entries(rows, cols) + 8 * ((cols + 1) / 2) + 127) / 128);
     for (int t = 0; t < J.nterm; ++t) {
       const char* a = reinterpret_cast<const char*>(J.mat[t] + (size_t)rows * cols);
       for (int i = threadIdx.x; i < lines; i += blockDim.x) {
@@ -193,17 +263,23 @@ __global__ void __launch_bounds__(256) zmm_kernel(const __grid_constant__ ZJobs 
     return v;
   };
   const int nsym = js.expand ? 1 : 2;
+  const ZPlaces pl(Kh);
+  int2* tails = reinterpret_cast<int2*>(sb + J.nterm * 2 * pl.ld);  // the staged entries' third limbs
   __shared__ int zmax[kZSlots * 8];
   const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
   for (int t = 0; t < J.nterm; ++t) {
-    double2* s = sb + (size_t)t * 2 * Kh;
+    double2* s = sb + t * 2 * pl.ld;
     const int* ex = reinterpret_cast<const int*>(J.mat[t] + (size_t)rows * Kh + z_limb_entries(rows, Kh));
     int mx[4] = {-4096, -4096, -4096, -4096};
     auto put = [&](int y, int k, double2 v) {
-      s[y * Kh + k] = v;
-      const int e = __ldg(ex + k), a = (__double2hiint(v.x) >> 20) & 0x7ff, b = (__double2hiint(v.y) >> 20) & 0x7ff;
-      if (a) mx[2 * y] = max(mx[2 * y], a == 0x7ff ? 8192 : a + e);
-      if (b) mx[2 * y + 1] = max(mx[2 * y + 1], b == 0x7ff ? 8192 : b + e);
+      s[pl.at(y, k)] = v;
+      const int e = __ldg(ex + k);
+      auto top = [&](int& m, double q) {
+        const int hi = __double2hiint(q), a = (hi >> 20) & 0x7ff;
+        if ((hi << 1) | __double2loint(q)) m = max(m, a == 0x7ff ? 8192 : max(a, 1) + e);
+      };
+      top(mx[2 * y], v.x);
+      top(mx[2 * y + 1], v.y);
     };
     for (int k = tid; k < Kh; k += nt) {
       const double2 v = comb(t, k);
@@ -233,92 +309,95 @@ __global__ void __launch_bounds__(256) zmm_kernel(const __grid_constant__ ZJobs 
     const int* ex = reinterpret_cast<const int*>(J.mat[t] + (size_t)rows * Kh + z_limb_entries(rows, Kh));
     for (int y = 0; y < nsym; ++y) {
       const int e0 = emax_of(t, y, 0), e1 = emax_of(t, y, 1);
-      double2* s = sb + (size_t)t * 2 * Kh + y * Kh;
+      double2* s = sb + t * 2 * pl.ld;
       for (int k = tid; k < Kh; k += nt) {
-        const double2 v = s[k];
+        const int q = pl.at(y, k);
+        const double2 v = s[q];
         const int e = __ldg(ex + k);
         const ZLimb a = z_limbs(z_fixed(v.x, e, e0)), b = z_limbs(z_fixed(v.y, e, e1));
-        *reinterpret_cast<int4*>(&s[k]) = make_int4(a.h, a.l, b.h, b.l);
+        *reinterpret_cast<int4*>(&s[q]) = make_int4(a.h, a.l, b.h, b.l);
+        tails[t * 2 * pl.ld + q] = make_int2(z_tail(v.x, e, e0), z_tail(v.y, e, e1));
       }
     }
   }
   // value of a sum of the term's scale
-  auto value = [](long long v, int emax) { return fx_to_double(v, emax >= 6000 ? kFxNaN : emax - 1079); };
-  __syncthreads();
+  auto value = [](ZWide v, int emax) { return z_to_double(v, emax >= 6000 ? kFxNaN : emax - 1079); };
   const int u = tid >> 1, hf = tid & 1;
+  // half of the sums over both lanes of the pair: the first lane goes on with the real parts, the second with the
+  // imaginary ones
+  auto pair = [&](ZWide x, ZWide y) {
+    const unsigned m = __activemask();
+    const ZWide mine = hf ? y : x, other = hf ? x : y;
+    return z_half(mine, ZWide{__shfl_xor_sync(m, other.h, 1), __shfl_xor_sync(m, other.f, 1)});
+  };
+  auto part = [&](const double2* p, size_t o) { return reinterpret_cast<const double*>(p)[2 * o + hf]; };
+  double* const out = reinterpret_cast<double*>(J.out) + hf;
+  __syncthreads();
   if (js.expand) {
     const int Ih = I / 2;
     if (u >= Ih) return;
     const int k0 = hf * (K / 2), k1 = hf ? K : K / 2;  // K even: both halves start on an even k
-    double2 lo = make_double2(0.0, 0.0), hi = make_double2(0.0, 0.0);
+    double lo = 0.0, hi = 0.0;
     for (int t = 0; t < J.nterm; ++t) {
       const int2* a = reinterpret_cast<const int2*>(J.mat[t] + (size_t)rows * K) + tid;
-      const int4* s = reinterpret_cast<const int4*>(sb + (size_t)t * 2 * Kh);
-      ZAcc ex, ey, ox, oy;
+      const int* at = reinterpret_cast<const int*>(J.mat[t] + z_tail_offset(rows, K)) + tid;
+      const int o = t * 2 * pl.ld + hf * pl.gap;
+      const int4* s = reinterpret_cast<const int4*>(sb + o);
+      const int2* st = tails + o;
+      ZAcc3 ex, ey, ox, oy;
 #pragma unroll 4
-      for (int k = k0; k < k1; k += 2, a += 4 * rows) {
+      for (int k = k0; k < k1; k += 2, a += 4 * rows, at += 4 * rows) {
         const int2 ae = __ldg(a), ao = __ldg(a + 2 * rows);
+        const int te = __ldg(at), to = __ldg(at + 2 * rows);
         const int4 ve = s[k], vo = s[k + 1];
-        ex.add(ve.x, ve.y, ae);
-        ey.add(ve.z, ve.w, ae);
-        ox.add(vo.x, vo.y, ao);
-        oy.add(vo.z, vo.w, ao);
+        const int2 ue = st[k], uo = st[k + 1];
+        ex.add(ve.x, ve.y, ue.x, ae, te);
+        ey.add(ve.z, ve.w, ue.y, ae, te);
+        ox.add(vo.x, vo.y, uo.x, ao, to);
+        oy.add(vo.z, vo.w, uo.y, ao, to);
       }
-      long long Ex = ex.sum(), Ey = ey.sum(), Ox = ox.sum(), Oy = oy.sum();
-      Ex = z_half(Ex, __shfl_xor_sync(__activemask(), Ex, 1));
-      Ey = z_half(Ey, __shfl_xor_sync(__activemask(), Ey, 1));
-      Ox = z_half(Ox, __shfl_xor_sync(__activemask(), Ox, 1));
-      Oy = z_half(Oy, __shfl_xor_sync(__activemask(), Oy, 1));
-      const int e0 = emax_of(t, 0, 0) + 2, e1 = emax_of(t, 0, 1) + 2;
-      const double al = J.alpha[t];
+      const ZWide E = pair(ex.wide(), ey.wide()), O = pair(ox.wide(), oy.wide());
+      const int e = emax_of(t, 0, hf) + 2;
       // out_j = E + O ; out_{Mz-1-j} = E - O (parity (-1)^n) or -E + O (derivative parity)
-      lo.x = fma(al, value(z_half(Ex, Ox), e0), lo.x); lo.y = fma(al, value(z_half(Ey, Oy), e1), lo.y);
-      hi.x = fma(al, value(J.deriv[t] ? z_half(Ox, -Ex) : z_half(Ex, -Ox), e0), hi.x);
-      hi.y = fma(al, value(J.deriv[t] ? z_half(Oy, -Ey) : z_half(Ey, -Oy), e1), hi.y);
+      lo = fma(J.alpha[t], value(z_half(E, O), e), lo);
+      hi = fma(J.alpha[t], value(J.deriv[t] ? z_half(O, z_neg(E)) : z_half(E, z_neg(O)), e), hi);
     }
-    if (hf == 0) {
-      const size_t o1 = (size_t)u * J.oi + (size_t)m * J.om;
-      const size_t o2 = (size_t)(I - 1 - u) * J.oi + (size_t)m * J.om;
-      for (int a = 0; a < J.nadd; ++a) {
-        const double2 p = J.add[a][o1], q = J.add[a][o2];
-        lo.x = fma(J.beta[a], p.x, lo.x); lo.y = fma(J.beta[a], p.y, lo.y);
-        hi.x = fma(J.beta[a], q.x, hi.x); hi.y = fma(J.beta[a], q.y, hi.y);
-      }
-      J.out[o1] = lo;
-      J.out[o2] = hi;
+    const size_t o1 = (size_t)u * J.oi + (size_t)m * J.om;
+    const size_t o2 = (size_t)(I - 1 - u) * J.oi + (size_t)m * J.om;
+    for (int a = 0; a < J.nadd; ++a) {
+      lo = fma(J.beta[a], part(J.add[a], o1), lo);
+      hi = fma(J.beta[a], part(J.add[a], o2), hi);
     }
+    out[2 * o1] = lo;
+    out[2 * o2] = hi;
   } else {
     if (u >= I) return;
     const int Kf = K / 2;
     const int k0 = hf * (Kf / 2), k1 = hf ? Kf : Kf / 2;
-    double2 acc = make_double2(0.0, 0.0);
+    double acc = 0.0;
     for (int t = 0; t < J.nterm; ++t) {
       const int2* a = reinterpret_cast<const int2*>(J.mat[t] + (size_t)rows * Kf) + tid;
       // even rows pair with s for parity (-1)^n, with d for derivative parity
       const int y = ((u & 1) == 0) != (J.deriv[t] != 0) ? 0 : 1;
-      const int4* s = reinterpret_cast<const int4*>(sb + (size_t)t * 2 * Kh + y * Kh);
-      ZAcc sx, sy;
+      const int* at = reinterpret_cast<const int*>(J.mat[t] + z_tail_offset(rows, Kf)) + tid;
+      const int o = (2 * t + y) * pl.ld + hf * pl.gap;
+      const int4* s = reinterpret_cast<const int4*>(sb + o);
+      const int2* st = tails + o;
+      ZAcc3 sx, sy;
 #pragma unroll 4
-      for (int k = k0; k < k1; ++k, a += 2 * rows) {
+      for (int k = k0; k < k1; ++k, a += 2 * rows, at += 2 * rows) {
         const int2 w = __ldg(a);
+        const int wt = __ldg(at);
         const int4 v = s[k];
-        sx.add(v.x, v.y, w);
-        sy.add(v.z, v.w, w);
+        const int2 u = st[k];
+        sx.add(v.x, v.y, u.x, w, wt);
+        sy.add(v.z, v.w, u.y, w, wt);
       }
-      long long Sx = sx.sum(), Sy = sy.sum();
-      Sx = z_half(Sx, __shfl_xor_sync(__activemask(), Sx, 1));
-      Sy = z_half(Sy, __shfl_xor_sync(__activemask(), Sy, 1));
-      const double vx = value(Sx, emax_of(t, y, 0) + 1), vy = value(Sy, emax_of(t, y, 1) + 1);
-      acc.x = fma(J.alpha[t], vx, acc.x); acc.y = fma(J.alpha[t], vy, acc.y);
+      acc = fma(J.alpha[t], value(pair(sx.wide(), sy.wide()), emax_of(t, y, hf) + 1), acc);
     }
-    if (hf == 0) {
-      const size_t o = (size_t)u * J.oi + (size_t)m * J.om;
-      for (int a = 0; a < J.nadd; ++a) {
-        const double2 p = J.add[a][o];
-        acc.x = fma(J.beta[a], p.x, acc.x); acc.y = fma(J.beta[a], p.y, acc.y);
-      }
-      J.out[o] = acc;
-    }
+    const size_t o = (size_t)u * J.oi + (size_t)m * J.om;
+    for (int a = 0; a < J.nadd; ++a) acc = fma(J.beta[a], part(J.add[a], o), acc);
+    out[2 * o] = acc;
   }
 }
 
