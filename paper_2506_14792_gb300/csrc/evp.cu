@@ -273,7 +273,8 @@ inline size_t iter_smem(int N, int kuf) {
          sizeof(double2) * (4 * (size_t)kChunk * kuf + 2 * nvp) + 2 * (nvp + kChunk);
 }
 
-// One CTA per pencil: n_iter steps of x <- Phi x / |Phi x|, psi <- Phi^H psi / |Phi^H psi|, then X and Y.  Warps 0
+// One CTA per pencil: n_iter steps of x <- Phi x / |Phi x|, psi <- Phi^H psi / |Phi^H psi|, then X and Y (n_iter = 0: of x
+// and psi as they are, which another kernel has iterated).  Warps 0
 // and 1 run the solves with A', warps 2 and 3 those with J A'^H J; of each pair one warp holds the real parts of
 // the unknowns and one the imaginary ones, so a sweep step is two FP64 instructions deep (128 clocks of latency).
 // Bound by that chain: 2 nv steps per solve.  The factors are copied to shared memory a chunk of steps ahead and
@@ -481,11 +482,11 @@ __global__ void __launch_bounds__(kIterThreads) evp_iter_kernel(const EvpIterArg
     }
   }
   __syncthreads();
-  for (int k = tid; k < H; k += kIterThreads) {
+  for (int k = tid; k < H && A.n_iter > 0; k += kIterThreads) {
     A.x[(size_t)p * H + k] = x[k];
     A.psi[(size_t)p * H + k] = ps[k];
   }
-  if (tid == 0) {
+  if (tid == 0 && A.n_iter > 0) {
     double* o = A.out + (size_t)p * kEvpOut;
     const double m2 = mur * mur + mui * mui;
     // lambda = sigma - 1/mu
@@ -519,6 +520,291 @@ __global__ void __launch_bounds__(kIterThreads) evp_iter_kernel(const EvpIterArg
     o[i] = v;
   }
 }
+
+// ---- iterations with the dense Phi ------------------------------------------------------------------------
+//
+// A step of the banded iteration is a chain of 2 nv dependent sweep steps however few the pencils; with the 3N x 3N
+// operator itself it is one matrix-vector product per direction.  Where enough steps pay for the operator's columns (3N
+// banded solves per pencil), it is built and iterated with (ShearEvp::dense_iterations).
+
+// Column c of Phi_p = (A_p^-1 [S1S0 e_c]) on u, v, w, one warp per column: a lane per row below the pivot (or above it, in
+// the back substitution), factors loaded a chunk of steps ahead.  Bound by FP64 issue when all partitions have
+// a warp (4 instructions a step), by the chain of 2 nv steps when there are fewer columns.
+constexpr int kPhiWarps = 4;
+inline size_t phi_smem(int nvp) { return sizeof(double) * 2 * kPhiWarps * (size_t)(kPadLow + nvp + kPadHigh); }
+__global__ void __launch_bounds__(32 * kPhiWarps) evp_phi_kernel(const EvpBand S, int P, const double* __restrict__ ssb,
+                                                                double2* __restrict__ phi) {
+  const int N = S.N, H = 3 * N, nv = S.nv, nvp = S.nvp, kl = S.kl, kuf = S.kl + S.ku;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, blocks = (H + kPhiWarps - 1) / kPhiWarps;
+  const int p = blockIdx.x / blocks, col = (blockIdx.x - p * blocks) * kPhiWarps + warp;
+  if (S.bad[P] || col >= H) return;  // (the warps do not meet)
+  extern __shared__ double2 evsm[];
+  const int ld = kPadLow + nvp + kPadHigh;
+  double* re = reinterpret_cast<double*>(evsm) + 2 * warp * ld + kPadLow;
+  double* im = re + ld;
+  const size_t sys = 2 * (size_t)p;
+  const double2* Lp = S.L + sys * nvp * kl;
+  const double2* Up = S.U + sys * nvp * kuf;
+  const double2* Dp = S.dinv + sys * nv;
+  const unsigned char* Pp = S.piv + sys * nv;
+  const int wu = min(S.width[sys], kuf), orow = S.mean(p) ? 0 : 1;
+  const double2 zero = make_double2(0.0, 0.0);
+  for (int i = lane; i < 2 * ld; i += 32) re[i - kPadLow] = 0.0;
+  __syncwarp();
+  const int f0 = col / N, n0 = col - f0 * N;
+  if (lane < 5 && n0 >= lane) re[orow + 4 * (n0 - lane) + f0] = __ldg(ssb + (n0 - lane) * 5 + lane);
+  __syncwarp();
+  if (lane == 0 && Pp[0]) {
+    const int q = Pp[0];
+    const double a = re[0], b = im[0];
+    re[0] = re[q]; im[0] = im[q];
+    re[q] = a; im[q] = b;
+  }
+  __syncwarp();
+  // v - f x
+  auto sub = [](double2 v, double2 f, double2 x) { return csub_mul(v, f, x); };
+  double2 f[kChunk], g[kChunk];
+  int to[kChunk];
+  auto loadL = [&](int j0) {
+#pragma unroll
+    for (int a = 0; a < kChunk; ++a) {
+      f[a] = lane < kl ? __ldg(Lp + (size_t)(j0 + a) * kl + lane) : zero;
+      const int pc = j0 + a + 1 < nv ? __ldg(Pp + j0 + a + 1) : 0;
+      to[a] = lane == 0 ? pc : lane == pc ? 0 : lane;  // the next step's interchange, made by where this one writes
+    }
+  };
+  loadL(0);
+  for (int j0 = 0; j0 < nvp; j0 += kChunk) {
+    double2 h[kChunk];
+    int th[kChunk];
+#pragma unroll
+    for (int a = 0; a < kChunk; ++a) { h[a] = f[a]; th[a] = to[a]; }
+    if (j0 + kChunk < nvp) loadL(j0 + kChunk);
+#pragma unroll
+    for (int a = 0; a < kChunk; ++a) {
+      const int j = j0 + a;
+      const double2 v = sub(make_double2(re[j + 1 + lane], im[j + 1 + lane]), h[a], make_double2(re[j], im[j]));
+      __syncwarp();
+      re[j + 1 + th[a]] = v.x;
+      im[j + 1 + th[a]] = v.y;
+      __syncwarp();
+    }
+  }
+  auto loadU = [&](int j0) {
+#pragma unroll
+    for (int a = 0; a < kChunk; ++a) {
+      f[a] = lane < wu ? __ldg(Up + (size_t)(j0 + a) * kuf + lane) : zero;
+      g[a] = lane + 32 < wu ? __ldg(Up + (size_t)(j0 + a) * kuf + lane + 32) : zero;
+    }
+  };
+  loadU(nvp - kChunk);
+  for (int i = lane; i < nv; i += 32) {
+    const double2 d = __ldg(Dp + i);
+    const double a = re[i], b = im[i];
+    re[i] = a * d.x - b * d.y;
+    im[i] = a * d.y + b * d.x;
+  }
+  __syncwarp();
+  for (int j0 = nvp - kChunk; j0 >= 0; j0 -= kChunk) {
+    double2 h[kChunk], w[kChunk];
+    unsigned far = 0u;
+#pragma unroll
+    for (int a = 0; a < kChunk; ++a) {
+      h[a] = f[a];
+      w[a] = g[a];
+      if (__any_sync(0xffffffffu, !is_zero(w[a]))) far |= 1u << a;
+    }
+    if (j0 > 0) loadU(j0 - kChunk);
+#pragma unroll
+    for (int a = kChunk - 1; a >= 0; --a) {
+      const int j = j0 + a, e = j - 1 - lane;
+      const double2 x = make_double2(re[j], im[j]);
+      const double2 v = sub(make_double2(re[e], im[e]), h[a], x);
+      re[e] = v.x;
+      im[e] = v.y;
+      if (far >> a & 1u) {
+        const double2 u = sub(make_double2(re[e - 32], im[e - 32]), w[a], x);
+        re[e - 32] = u.x;
+        im[e - 32] = u.y;
+      }
+      __syncwarp();
+    }
+  }
+  double2* o = phi + (size_t)p * H * H + col;
+  for (int r = lane; r < H; r += 32) {
+    const int q = r / N, n = r - q * N, i = 1 + 4 * n + q;
+    o[(size_t)r * H] = n >= 2 ? make_double2(re[i] - re[i - 8], im[i] - im[i - 8]) : make_double2(re[i], im[i]);
+  }
+}
+
+constexpr int kRows = 4;       // rows per warp block in evp_dense_kernel (2 kRows partial sums per lane)
+constexpr int kRowsLog2V = 3;  // log2(2 kRows)
+
+// Warp reduction of 2 kRows values per lane at once: a butterfly in which every exchange halves
+// the values a lane carries (offsets 16, 8, ...; the lane keeps the half selected by that bit of
+// its index) until one is left, then plain exchanges at the remaining offsets.  Every lane of the
+// group l >> (5 - kRowsLog2V) = m ends with the total of value m.  2 kRows + 1 additions per lane
+// for 2 kRows sums instead of 5 per sum; fixed order, so deterministic.
+__device__ __forceinline__ double warp_reduce_rows(double (&v)[2 * kRows], int lane) {
+  int off = 16;
+#pragma unroll
+  for (int half = kRows; half >= 1; half >>= 1, off >>= 1) {
+    const bool hi = (lane & off) != 0;
+#pragma unroll
+    for (int j = 0; j < half; ++j) {
+      const double send = hi ? v[j] : v[j + half];
+      const double keep = hi ? v[j + half] : v[j];
+      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+    }
+  }
+  double t = v[0];
+#pragma unroll
+  for (int o = 16 >> kRowsLog2V; o >= 1; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
+}
+
+struct EvpDenseArgs {
+  const double2* phi;    // [P][H][H]
+  double2* x;            // [P][H] right iterate (in / out)
+  double2* psi;          // [P][H] left iterate (in / out)
+  const double* shift;   // [P][2]
+  const int* bad;        // [P + 1]
+  double* out;           // [P][kEvpOut]
+  int H, n_iter;
+};
+
+// One CTA per pencil: n_iter steps of x <- Phi x / |Phi x|, psi <- Phi^H psi / |Phi^H psi| with
+// each row of Phi read once per step for both products (warps over rows, lanes over columns,
+// coalesced), all in shared memory between steps.
+// NC = ceil(3N / 32) column chunks per lane, fixed at compile time so that only the last chunk
+// carries a bounds predicate.
+template <int NC>
+__global__ void __launch_bounds__(kEvpThreads, 2) evp_dense_kernel(const EvpDenseArgs A) {
+  const int p = blockIdx.x, H = A.H;
+  if (A.bad[gridDim.x]) return;  // the call fails: nothing is written
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  extern __shared__ double2 evsm[];
+  double2* x = evsm;
+  double2* ps = x + H;
+  double2* y = ps + H;
+  double2* zp = y + H;                                    // [kEvpWarps][H] partial Phi^H psi
+  double* red = reinterpret_cast<double*>(zp + (size_t)kEvpWarps * H);
+  const double2* Tp = A.phi + (size_t)p * H * H;
+  for (int k = threadIdx.x; k < H; k += blockDim.x) {
+    x[k] = A.x[(size_t)p * H + k];
+    ps[k] = A.psi[(size_t)p * H + k];
+  }
+  double mur = 0.0, mui = 0.0, res_r = 1.0, res_l = 1.0;
+  for (int it = 0; it < A.n_iter; ++it) {
+    __syncthreads();
+    double2 zacc[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) zacc[c] = make_double2(0.0, 0.0);
+    // blocks of kRows rows per warp: each x chunk is read once per block, and the row sums of
+    // the block are reduced together (warp_reduce_rows) instead of one butterfly per row
+    for (int rb = warp * kRows; rb < H; rb += kRows * kEvpWarps) {
+      double acc[2 * kRows];
+      double2 pr[kRows];
+#pragma unroll
+      for (int i = 0; i < kRows; ++i) {
+        acc[2 * i] = acc[2 * i + 1] = 0.0;
+        pr[i] = rb + i < H ? ps[rb + i] : make_double2(0.0, 0.0);
+      }
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        const int k = c * 32 + lane;
+        if (c < NC - 1 || k < H) {
+          const double2 xv = x[k];
+#pragma unroll
+          for (int i = 0; i < kRows; ++i) {
+            if (rb + i >= H) continue;
+            const double2 t = __ldg(&Tp[(size_t)(rb + i) * H + k]);
+            acc[2 * i] = fma(t.x, xv.x, acc[2 * i]);
+            acc[2 * i] = fma(-t.y, xv.y, acc[2 * i]);
+            acc[2 * i + 1] = fma(t.x, xv.y, acc[2 * i + 1]);
+            acc[2 * i + 1] = fma(t.y, xv.x, acc[2 * i + 1]);
+            zacc[c].x = fma(t.x, pr[i].x, zacc[c].x);  // conj(t) * psi_r
+            zacc[c].x = fma(t.y, pr[i].y, zacc[c].x);
+            zacc[c].y = fma(t.x, pr[i].y, zacc[c].y);
+            zacc[c].y = fma(-t.y, pr[i].x, zacc[c].y);
+          }
+        }
+      }
+      const double tot = warp_reduce_rows(acc, lane);
+      // lane group m = lane >> (5 - kRowsLog2V) holds value m = 2 (row - rb) + component
+      const int m = lane >> (5 - kRowsLog2V), r = rb + (m >> 1);
+      if ((lane & ((1 << (5 - kRowsLog2V)) - 1)) == 0 && r < H) reinterpret_cast<double*>(y)[2 * r + (m & 1)] = tot;
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const int k = c * 32 + lane;
+      if (c < NC - 1 || k < H) zp[(size_t)warp * H + k] = zacc[c];
+    }
+    __syncthreads();
+    // z = sum of the warp partials (into zp row 0); norms and the two-sided Rayleigh quotient
+    double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int k = threadIdx.x; k < H; k += blockDim.x) {
+      double2 z = zp[k];
+      for (int w = 1; w < kEvpWarps; ++w) {
+        const double2 q = zp[(size_t)w * H + k];
+        z.x += q.x;
+        z.y += q.y;
+      }
+      zp[k] = z;
+      const double2 yk = y[k], xk = x[k], pk = ps[k];
+      v[0] = fma(yk.x, yk.x, fma(yk.y, yk.y, v[0]));
+      v[1] = fma(z.x, z.x, fma(z.y, z.y, v[1]));
+      v[2] += pk.x * yk.x + pk.y * yk.y;  // psi^H y
+      v[3] += pk.x * yk.y - pk.y * yk.x;
+      v[4] += pk.x * xk.x + pk.y * xk.y;  // psi^H x
+      v[5] += pk.x * xk.y - pk.y * xk.x;
+    }
+    block_sum<6, kEvpWarps>(v, red);
+    const double dd = v[4] * v[4] + v[5] * v[5];
+    if (dd > 0.0) {
+      mur = (v[2] * v[4] + v[3] * v[5]) / dd;
+      mui = (v[3] * v[4] - v[2] * v[5]) / dd;
+    }
+    if (it + 1 == A.n_iter) {  // residuals |Phi x - mu x| / |Phi x|, |Phi^H psi - conj(mu) psi| / |Phi^H psi|
+      double r2[2] = {0.0, 0.0};
+      for (int k = threadIdx.x; k < H; k += blockDim.x) {
+        const double2 yk = y[k], xk = x[k], pk = ps[k], z = zp[k];
+        const double ex = yk.x - (mur * xk.x - mui * xk.y), ey = yk.y - (mur * xk.y + mui * xk.x);
+        const double fx = z.x - (mur * pk.x + mui * pk.y), fy = z.y - (mur * pk.y - mui * pk.x);
+        r2[0] += ex * ex + ey * ey;
+        r2[1] += fx * fx + fy * fy;
+      }
+      block_sum<2, kEvpWarps>(r2, red);
+      res_r = v[0] > 0.0 ? sqrt(r2[0] / v[0]) : 1.0;
+      res_l = v[1] > 0.0 ? sqrt(r2[1] / v[1]) : 1.0;
+    }
+    const double sy = v[0] > 0.0 ? 1.0 / sqrt(v[0]) : 0.0, sz = v[1] > 0.0 ? 1.0 / sqrt(v[1]) : 0.0;
+    for (int k = threadIdx.x; k < H; k += blockDim.x) {
+      const double2 yk = y[k], z = zp[k];
+      x[k] = make_double2(yk.x * sy, yk.y * sy);
+      ps[k] = make_double2(z.x * sz, z.y * sz);
+    }
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < H; k += blockDim.x) {
+    A.x[(size_t)p * H + k] = x[k];
+    A.psi[(size_t)p * H + k] = ps[k];
+  }
+  if (threadIdx.x == 0) {
+    double* o = A.out + (size_t)p * kEvpOut;
+    const double m2 = mur * mur + mui * mui;
+    // lambda = sigma - 1/mu
+    o[0] = m2 > 0.0 ? A.shift[2 * p] - mur / m2 : 0.0;
+    o[1] = m2 > 0.0 ? A.shift[2 * p + 1] + mui / m2 : 0.0;
+    o[8] = res_r;
+    o[9] = res_l;
+  }
+}
+
+using EvpDenseFn = void (*)(const EvpDenseArgs);
+constexpr int kDenseMaxN = 64;
+const EvpDenseFn kEvpDense[3 * kDenseMaxN / 32] = {evp_dense_kernel<1>, evp_dense_kernel<2>, evp_dense_kernel<3>,
+                                                   evp_dense_kernel<4>, evp_dense_kernel<5>, evp_dense_kernel<6>};
 
 struct EvpSensArgs {
   const double2* XY;                 // [P][2][nv]: X, Y
@@ -610,7 +896,8 @@ struct ShearEvp : EqImpl {
   int N = 0, H = 0, nv = 0, base = 0, Pmax = 0;
   rbhost::Operators ops;
   int kl = 0, ku = 0;
-  DevBuf band, XY, args, mats;
+  int sms = 0;
+  DevBuf band, XY, args, mats, phi;
 
   size_t state_len(int which) const override { return which == 0 ? (size_t)Pmax * H * 2 : 0; }
 
@@ -654,8 +941,21 @@ struct ShearEvp : EqImpl {
     }
     SPADJ_CUDA_TRY(p, mats.ensure(sizeof(double) * m.size()));
     SPADJ_CUDA_TRY(p, cudaMemcpy(mats.ptr, m.data(), sizeof(double) * m.size(), cudaMemcpyHostToDevice));
+    int dev = 0;
+    SPADJ_CUDA_TRY(p, cudaGetDevice(&dev));
+    SPADJ_CUDA_TRY(p, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     SPADJ_CUDA_TRY(p, cudaFuncSetAttribute(evp_iter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)iter_smem(kEvpMaxN, kEvpMaxUpper)));
     return SPADJ_OK;
+  }
+
+  // Whether the iterations run with the dense Phi.  Measured (us): a step of up to 152 pencils takes 12.9, 18, 31, 60 and
+  // 88 at N = 8, 16, 32, 48, 64 with it and 21.6, 34, 58, 85 and 107 banded (N = 96: 182 and 158), and it costs about
+  // 1.8 N + 0.0054 P N^2 to build: one pencil of N = 16 with 30 steps 834 and 1247, 96 of N = 48 with 20 3067 and 2260, with
+  // 60 5489 and 5653.  With more pencils than SMs the banded CTAs share an SM better: 200 pencils 34 and 43 a step at
+  // N = 16, 61 and 74 at 32, 118 and 106 at 48; 400 of N = 24 78 and 81, for 1400 to build.
+  bool dense_iterations(int P, int n_iter) const {
+    if (P > sms) return N <= 32 && 4ll * n_iter >= 5ll * P;
+    return N <= kDenseMaxN && n_iter >= 5.0 + 0.1 * N + 3e-4 * P * N * N;
   }
 
   spadj_status eigen(Problem* p, int P, const double* prm, const double* shift, int n_iter, double* x, double* psi,
@@ -707,6 +1007,20 @@ struct ShearEvp : EqImpl {
     ia.XY = XY.as<double2>();
     ia.out = out;
     ia.n_iter = n_iter;
+    if (dense_iterations(P, n_iter)) {
+      if (phi.ensure(sizeof(double2) * (size_t)P * H * H) == cudaSuccess) {
+        const int blocks = (H + kPhiWarps - 1) / kPhiWarps;
+        evp_phi_kernel<<<P * blocks, 32 * kPhiWarps, phi_smem(S.nvp), p->stream>>>(S, P, ssb, phi.as<double2>());
+        if ((s = check_launch(p, "evp operator")) != SPADJ_OK) return s;
+        EvpDenseArgs da{phi.as<double2>(), ia.x, ia.psi, shiftd, flags, out, H, n_iter};
+        const size_t dsmem = sizeof(double2) * (size_t)(3 + kEvpWarps) * H + sizeof(double) * kEvpWarps * 6;
+        kEvpDense[(H + 31) / 32 - 1]<<<P, kEvpThreads, dsmem, p->stream>>>(da);
+        if ((s = check_launch(p, "evp dense iterate")) != SPADJ_OK) return s;
+        ia.n_iter = 0;
+      } else {
+        cudaGetLastError();  // no memory for the operators: the banded iterations need none
+      }
+    }
     evp_iter_kernel<<<P, kIterThreads, iter_smem(N, kuf), p->stream>>>(ia);
     // two factorisations, and two banded solves per step and for the eigenvectors, 8 flops per factor entry
     p->toc(t0, KC_SOLVE, 16.0 * nv * ((double)kl * (kl + ku) + (kl + ku + 1.0) * (n_iter + 1)) * P);
