@@ -899,6 +899,10 @@ struct ShearEvp : EqImpl {
   int sms = 0;
   DevBuf band, XY, args, mats, phi;
 
+  ~ShearEvp() override {
+    for (DevBuf* b : {&band, &XY, &args, &mats, &phi}) b->release();
+  }
+
   size_t state_len(int which) const override { return which == 0 ? (size_t)Pmax * H * 2 : 0; }
 
   spadj_status init(Problem* p) {
