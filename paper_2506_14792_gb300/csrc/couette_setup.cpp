@@ -295,9 +295,8 @@ void band_orders(int N, bool mean, std::vector<int>& perm_r, std::vector<int>& p
   (void)nv;
 }
 
-// The column recombination of the banded form, in place on the pencil matrix (or a part of it).
-template <class T>
-void recombine(int N, bool mean, std::vector<T>& A) {
+// The column recombination of the banded form, in place on the pencil matrix.
+void recombine(int N, bool mean, std::vector<cd>& A) {
   const int nv = 4 * N + 7;
   auto col_sub = [&](int c, int c2, double w) {  // column c -= w * column c2
     for (int r = 0; r < nv; ++r) A[(size_t)r * nv + c] -= w * A[(size_t)r * nv + c2];
@@ -539,69 +538,75 @@ bool band_solve_host(const rbhost::Operators& o, double al, double be, double nu
   return true;
 }
 
-void band_parts(const rbhost::Operators& o, int base, bool mean, int& kl, int& ku, std::vector<double>& E) {
-  const int N = o.N, nv = 4 * N + 7;
-  std::vector<double> Um, UP;
-  base_flow(o, base, Um, UP);
-  std::vector<int> pr, pc;
+std::vector<BandEntry> band_parts(const rbhost::Operators& o, const std::vector<double>& Um, const std::vector<double>& UP,
+                                  bool mean, int& kl, int& ku) {
+  const int N = o.N, nv = 4 * N + 7, W = 2 * N, P = 3 * N, tau = 4 * N, tp = tau + 6, r0 = 4 * N;
+  std::vector<int> pr, pc, ri(nv), ci(nv);
   band_orders(N, mean, pr, pc);
-  std::vector<std::vector<double>> parts(kBandParts);
+  for (int i = 0; i < nv; ++i) ri[pr[i]] = ci[pc[i]] = i;
+  std::vector<BandEntry> es;
+  es.reserve((size_t)96 * N);
   kl = ku = 0;
-  for (int t = 0; t < kBandParts; ++t) {
-    std::vector<double> A((size_t)nv * nv, 0.0);
-    auto at = [&](int r, int c) -> double& { return A[(size_t)r * nv + c]; };
-    const int W = 2 * N, P = 3 * N, tau = 4 * N, tp = tau + 6, r0 = 4 * N;
-    for (int r = 0; r < N; ++r)
-      for (int c = 0; c < N; ++c) {
-        const double ss = o.SS[r * N + c];
-        const double diag = t == kPartShift ? ss : t == kPartVisc ? -o.DD[r * N + c] : t == kPartAlpha ? Um[r * N + c] : 0.0;
-        for (int f = 0; f < 3; ++f) at(f * N + r, f * N + c) = diag;
-        if (t == kPartConst) {
-          at(r, W + c) = UP[r * N + c];
-          at(W + r, P + c) = o.SD[r * N + c];
-          at(P + r, W + c) = o.D0[r * N + c];
-        } else if (t == kPartAlpha || t == kPartBeta) {
-          const int q = t == kPartAlpha ? 0 : N;
-          at(q + r, P + c) = ss;
-          at(P + r, q + c) = o.S0[r * N + c];
-        }
-      }
-    for (int f = 0; f < 3; ++f) {
-      if (t == kPartVisc) at(f * N + o.lift_row, tau + 2 * f) = -o.lift_val;
-      if (t == kPartConst) {
-        at(f * N + N - 1, tau + 2 * f + 1) = 1.0;
-        for (int n = 0; n < N; ++n) {
-          at(r0 + 2 * f, f * N + n) = n % 2 == 0 ? 1.0 : -1.0;
-          at(r0 + 2 * f + 1, f * N + n) = 1.0;
-        }
-      }
+  auto put = [&](int t, int r, int c, double v) {
+    if (v == 0.0) return;
+    const int i = ri[r], k = ci[c];
+    es.push_back({t, i, k, v});
+    kl = std::max(kl, i - k);
+    ku = std::max(ku, k - i);
+  };
+  // entry (r, c) of M in the recombined velocity columns, and in the pressure columns
+  auto vel = [&](const std::vector<double>& M, int r, int c) {
+    const double* m = &M[(size_t)r * N + c];
+    return c + 2 < N ? m[0] - m[2] : m[0];
+  };
+  auto prs = [&](const std::vector<double>& M, int r, int c) {
+    const double* m = &M[(size_t)r * N + c];
+    return mean && c % 2 == 0 && c + 2 < N ? m[0] - pressure_weight(c) * m[2] : m[0];
+  };
+  // the operators' own band: columns r + lo .. r + hi of row r (two less where the recombination brings column c + 2)
+  int lo = 0, hi = 0;
+  for (const std::vector<double>* M : {&o.SS, &o.DD, &o.SD, &o.S0, &o.D0, &Um, &UP})
+    for (int r = 0; r < N; ++r) {
+      const double* m = &(*M)[(size_t)r * N];
+      for (int c = 0; c < r + lo; ++c)
+        if (m[c] != 0.0) lo = c - r;
+      for (int c = N - 1; c > r + hi; --c)
+        if (m[c] != 0.0) hi = c - r;
     }
-    if (t == kPartConst) {
-      at(P + N - 1, tau + 4) = 1.0;
-      if (mean) {
-        at(P, tp) = 1.0;
-        for (int n = 0; n < N; n += 2) at(r0 + 6, P + n) = 2.0 / (1.0 - (double)n * n);
-      } else {
-        at(r0 + 6, tp) = 1.0;
+  for (int r = 0; r < N; ++r)
+    for (int c = std::max(0, r + lo - 2); c <= std::min(N - 1, r + hi); ++c) {
+      const double ss = vel(o.SS, r, c), dd = vel(o.DD, r, c), um = vel(Um, r, c);
+      for (int f = 0; f < 3; ++f) {
+        put(kPartShift, f * N + r, f * N + c, ss);
+        put(kPartVisc, f * N + r, f * N + c, -dd);
+        put(kPartAlpha, f * N + r, f * N + c, um);
       }
+      put(kPartConst, r, W + c, vel(UP, r, c));
+      put(kPartConst, W + r, P + c, prs(o.SD, r, c));
+      put(kPartConst, P + r, W + c, vel(o.D0, r, c));
+      const double sp = prs(o.SS, r, c), s0 = vel(o.S0, r, c);
+      put(kPartAlpha, r, P + c, sp);
+      put(kPartBeta, N + r, P + c, sp);
+      put(kPartAlpha, P + r, c, s0);
+      put(kPartBeta, P + r, N + c, s0);
     }
-    recombine(N, mean, A);
-    parts[t].assign((size_t)nv * nv, 0.0);
-    for (int i = 0; i < nv; ++i)
-      for (int k = 0; k < nv; ++k) {
-        const double v = A[(size_t)pr[i] * nv + pc[k]];
-        if (v == 0.0) continue;
-        parts[t][(size_t)i * nv + k] = v;
-        kl = std::max(kl, i - k);
-        ku = std::max(ku, k - i);
-      }
+  for (int f = 0; f < 3; ++f) {
+    put(kPartVisc, f * N + o.lift_row, tau + 2 * f, -o.lift_val);
+    put(kPartConst, f * N + N - 1, tau + 2 * f + 1, 1.0);
+    for (int n = N - 2; n < N; ++n) {  // the boundary values of the recombined modes below vanish
+      put(kPartConst, r0 + 2 * f, f * N + n, n % 2 == 0 ? 1.0 : -1.0);
+      put(kPartConst, r0 + 2 * f + 1, f * N + n, 1.0);
+    }
   }
-  const int w = kl + ku + 1;
-  E.assign((size_t)kBandParts * nv * w, 0.0);
-  for (int t = 0; t < kBandParts; ++t)
-    for (int i = 0; i < nv; ++i)
-      for (int k = std::max(0, i - kl); k <= std::min(nv - 1, i + ku); ++k)
-        E[((size_t)t * nv + i) * w + (k - i + kl)] = parts[t][(size_t)i * nv + k];
+  put(kPartConst, P + N - 1, tau + 4, 1.0);
+  if (mean) {
+    put(kPartConst, P, tp, 1.0);
+    const int n = (N - 1) / 2 * 2;  // int psi_n dz = 0 below
+    put(kPartConst, r0 + 6, P + n, 2.0 / (1.0 - (double)n * n));
+  } else {
+    put(kPartConst, r0 + 6, tp, 1.0);
+  }
+  return es;
 }
 
 }  // namespace couhost

@@ -91,10 +91,16 @@ bool band_solve_host(const rbhost::Operators& o, double al, double be, double nu
 // The banded form A' split by its parameters, for kernels that assemble it themselves:
 //   A' = E[kPartConst] + (a0 + nu k^2) E[kPartShift] + nu E[kPartVisc]
 //        + i alpha E[kPartAlpha] + i beta E[kPartBeta],  k^2 = alpha^2 + beta^2,
-// each part real, its entry (i, k) at E[((t nv) + i) (kl + ku + 1) + k - i + kl].  mean: the
-// structure of the (0, 0) pencil (gauge row and pressure recombination).
+// each part real and returned by its non-zero entries (position i, k of part t), with the band widths of all of them.
+// mean: the structure of the (0, 0) pencil (gauge row and pressure recombination).
 enum { kPartConst = 0, kPartShift, kPartVisc, kPartAlpha, kPartBeta, kBandParts };
-void band_parts(const rbhost::Operators& o, int base, bool mean, int& kl, int& ku, std::vector<double>& E);
+// Um, UP: of base_flow.
+struct BandEntry {
+  int t, i, k;
+  double v;
+};
+std::vector<BandEntry> band_parts(const rbhost::Operators& o, const std::vector<double>& Um, const std::vector<double>& UP,
+                                  bool mean, int& kl, int& ku);
 // weight of the mean pencil's pressure recombination: psi_j = T_j - weight T_{j+2}, even j
 double pressure_weight(int j);
 

@@ -919,7 +919,16 @@ struct ShearEvp : EqImpl {
     ops = rbhost::build_operators(N, 3 * N / 2, 1.0);
     std::vector<double> Um, UP;
     couhost::base_flow(ops, base, Um, UP);
+    int l[2], u[2];
+    std::vector<couhost::BandEntry> E[2];
+    for (int k = 0; k < 2; ++k) E[k] = couhost::band_parts(ops, Um, UP, k == 1, l[k], u[k]);
+    kl = std::max(l[0], l[1]);
+    ku = std::max(u[0], u[1]);
+    if (kl > kEvpMaxLower || kl + ku > kEvpMaxUpper) return p->fail(SPADJ_ERR_UNSUPPORTED, "shear evp: the pencil's band is wider than supported");
+    const int w = kl + ku + 1;
+    const size_t part = (size_t)couhost::kBandParts * nv * w;
     std::vector<double> m;
+    m.reserve(4 * (size_t)N * N + 6 * (size_t)N + 2 * part);
     m.insert(m.end(), ops.SS.begin(), ops.SS.end());
     m.insert(m.end(), ops.DD.begin(), ops.DD.end());
     m.insert(m.end(), Um.begin(), Um.end());
@@ -929,19 +938,10 @@ struct ShearEvp : EqImpl {
     for (int n = 0; n < N; ++n)
       for (int d = 0; d < 5; ++d) m.push_back(n + d < N ? ops.SS[(size_t)n * N + n + d] : 0.0);
     for (int n = 0; n < N; ++n) m.push_back(n % 2 == 0 ? couhost::pressure_weight(n) : 0.0);
-    int l[2], u[2];
-    std::vector<double> E[2];
-    for (int k = 0; k < 2; ++k) couhost::band_parts(ops, base, k == 1, l[k], u[k], E[k]);
-    kl = std::max(l[0], l[1]);
-    ku = std::max(u[0], u[1]);
-    if (kl > kEvpMaxLower || kl + ku > kEvpMaxUpper) return p->fail(SPADJ_ERR_UNSUPPORTED, "shear evp: the pencil's band is wider than supported");
-    const int w = kl + ku + 1;
-    for (int k = 0; k < 2; ++k) {
-      const int wk = l[k] + u[k] + 1;
-      const size_t rows = E[k].size() / wk, o = m.size();
-      m.resize(o + rows * w, 0.0);
-      for (size_t r = 0; r < rows; ++r)
-        for (int d = 0; d < wk; ++d) m[o + r * w + d + kl - l[k]] = E[k][r * wk + d];
+    for (int k = 0; k < 2; ++k) {  // entry (i, k) of part t at ((t nv) + i) w + k - i + kl
+      const size_t at = m.size();
+      m.resize(at + part, 0.0);
+      for (const couhost::BandEntry& e : E[k]) m[at + ((size_t)e.t * nv + e.i) * w + (e.k - e.i + kl)] = e.v;
     }
     SPADJ_CUDA_TRY(p, mats.ensure(sizeof(double) * m.size()));
     SPADJ_CUDA_TRY(p, cudaMemcpy(mats.ptr, m.data(), sizeof(double) * m.size(), cudaMemcpyHostToDevice));
