@@ -109,8 +109,9 @@ __device__ __forceinline__ double2* row(double* base, int b, int K) {
 
 // ---- single-shot kernels (transforms, F, JVP, VJP) ---------------------------------------
 //
-// One call of these is all launch and latency, so they keep the FP64 transforms; the step loops
-// below run the fixed-point ones.
+// These run the FP64 transforms: some builds of them with the fixed-point ones raised a misaligned-address error (at
+// N = 16, the same at every run of a build) whose cause was found neither by reading nor by checked builds, which ran
+// clean.  One call is all launch and latency, so it costs little.  The step loops below run the fixed-point ones.
 
 // coefficients -> grid with the weights w0 (k = 0) and w
 __global__ void __launch_bounds__(64) to_grid_kernel(const __grid_constant__ BurgersParams P, double w0, double w, const double2* __restrict__ x,

@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(128) yfft_kernel(const __grid_constant__ YJobs
       const int m = m0 + c;
       const size_t g = ((size_t)i * Ny + q) * Kx + m;
       for (int t = 0; t < J.nin; ++t) {
-        double2 x = J.in[t][g];
+        double2 x = ldg128(J.in[t] + g);
         if (J.mult[t]) {
           const double k = J.mult[t] == 1 ? P.kxs * m : P.kys * ky_of(q, Ny);
           x = make_double2(-k * x.y, k * x.x);
@@ -85,17 +85,17 @@ __global__ void __launch_bounds__(128) yfft_kernel(const __grid_constant__ YJobs
     });
     for (int idx = tid; idx < My * TK; idx += nt) {
       const int e = idx / TK, c = idx - e * TK;
-      if (c < tk) J.out[((size_t)i * My + e) * Kx + m0 + c] = cscale(r.at(c, e), J.scale);
+      if (c < tk) stg128(J.out + ((size_t)i * My + e) * Kx + m0 + c, cscale(r.at(c, e), J.scale));
     }
   } else {
     const auto r = xf_c2c<false, TK, TK>(0, b, lay, P.plan, [&](int c, int e) {
-      return c < tk ? J.in[0][((size_t)i * My + e) * Kx + m0 + c] : make_double2(0.0, 0.0);
+      return c < tk ? ldg128(J.in[0] + ((size_t)i * My + e) * Kx + m0 + c) : make_double2(0.0, 0.0);
     });
     for (int idx = tid; idx < Ny * TK; idx += nt) {
       const int q = idx / TK, c = idx - q * TK;
       if (c >= tk) continue;
       const int e = ypos(q, Ny, My);
-      J.out[((size_t)i * Ny + q) * Kx + m0 + c] = e < 0 ? make_double2(0.0, 0.0) : cscale(r.at(c, e), J.scale);
+      stg128(J.out + ((size_t)i * Ny + q) * Kx + m0 + c, e < 0 ? make_double2(0.0, 0.0) : cscale(r.at(c, e), J.scale));
     }
   }
 }

@@ -56,8 +56,9 @@ struct FxLimb {
   int h, l;
 };
 
-// Memory accesses of the transforms' kernels are written out one by one (here and at fx_get / fx_put), each of
-// exactly its own width.
+// The 16-byte accesses of the kernels that run the fixed-point transforms are written out one by one (here and at
+// fx_get / fx_put), each of exactly its own width.  A precaution: builds of Burgers' single calls in this form
+// raised a misaligned-address error whose cause was not found (those calls run the FP64 butterflies).
 __device__ __forceinline__ double2 ldg128(const double2* p) {
   double2 v;
   asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
@@ -65,6 +66,11 @@ __device__ __forceinline__ double2 ldg128(const double2* p) {
 }
 __device__ __forceinline__ void stg128(double2* p, double2 v) {
   asm volatile("st.global.v2.f64 [%0], {%1, %2};" ::"l"(p), "d"(v.x), "d"(v.y) : "memory");
+}
+__device__ __forceinline__ double2 ldcg128(const double2* p) {  // from L2: written by other CTAs of the same launch
+  double2 v;
+  asm volatile("ld.global.cg.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+  return v;
 }
 __device__ __forceinline__ int4 ldtab(const int4* p) {  // read-only tables
   int4 v;
@@ -393,8 +399,7 @@ __device__ __forceinline__ double2* fx_mem64() {
   extern __shared__ double2 fx_dyn[];
   return fx_dyn;
 }
-// One 16-byte shared-memory access each, to entry e of the buffers (written out, so that neighbouring entries
-// are never combined into accesses that ask for more than 16-byte alignment).
+// One 16-byte shared-memory access each, to entry e of the buffers.
 __device__ __forceinline__ unsigned fx_addr(int e) {
   return static_cast<unsigned>(__cvta_generic_to_shared(fx_mem64())) + 16u * (unsigned)e;
 }

@@ -103,7 +103,6 @@ struct KolArgs {
   int drop_signal_member; // test knob: completion of this member is never signalled (-1: off)
 };
 
-__device__ __forceinline__ double2 ldcg2(const double2* p) { return __ldcg(p); }
 
 struct Coef {
   double a0, a1, a2, c1, c2;
@@ -154,7 +153,7 @@ __device__ __forceinline__ int yrow(int j, int N, int M) { return j < N / 2 ? j 
 __device__ __forceinline__ double2 field_entry(int f, const double2* xs, const double* ik2, int kx, int j, int N, int M) {
   const int q = yrow(j, N, M);
   if (q < 0) return make_double2(0.0, 0.0);
-  const double2 x = ldcg2(&xs[q]);
+  const double2 x = ldcg128(&xs[q]);
   // (the imaginary part of omega's mean reaches only what the x transform leaves out: not into the sequence's scale)
   if (f == 4 && kx == 0 && q == 0) return make_double2(x.x, 0.0);
   return f < 4 ? fmult(f, (double)kx, (double)kyof(q, N), __ldg(&ik2[q]), x) : x;
@@ -189,13 +188,13 @@ __device__ void ca_forward(const KolArgs& A, const KMember& m, int tile, int s) 
   for (int kx = kx0; kx < kx1; ++kx) {
     const long long col = m.off_state + (long long)kx * N;
     if (s == 0) {
-      for (int q = threadIdx.x; q < N; q += blockDim.x) xc[q] = A.x0[col + q];
+      for (int q = threadIdx.x; q < N; q += blockDim.x) xc[q] = ldg128(A.x0 + col + q);
       __syncthreads();
     } else {
       FxRes<false> r{};
       if (A.nonlinear || A.closure)
         r = xf_c2c<false, 1, 1, kFxOnly>(fs, fs + CM, FxLay{1, CM, 0}, R.py, [&](int, int j) {
-          return ldcg2(&A.mixB[0][m.off_mix + (long long)j * Kx + kx]);
+          return ldcg128(&A.mixB[0][m.off_mix + (long long)j * Kx + kx]);
         });
       const Coef c = kcoef(n, A.kc);
       const double invM = 1.0 / M;
@@ -208,18 +207,18 @@ __device__ void ca_forward(const KolArgs& A, const KMember& m, int tile, int s) 
         }
         if (A.forcing && kx == 0 && (q == 4 || q == N - 4)) F.x -= 2.0;
         if (A.fonly) {
-          A.out[col + q] = F;
+          stg128(A.out + col + q, F);
           continue;
         }
-        const double2 X1 = ldcg2(&A.Xr[(n - 1) & 1][col + q]);
+        const double2 X1 = ldcg128(&A.Xr[(n - 1) & 1][col + q]);
         double2 num = make_double2(c.c1 * F.x - c.a1 * X1.x, c.c1 * F.y - c.a1 * X1.y);
         if (n >= 2) {
-          const double2 X2 = ldcg2(&A.Xr[n & 1][col + q]);
-          const double2 F2 = ldcg2(&A.Fr[n & 1][col + q]);
+          const double2 X2 = ldcg128(&A.Xr[n & 1][col + q]);
+          const double2 F2 = ldcg128(&A.Fr[n & 1][col + q]);
           num.x += c.c2 * F2.x - c.a2 * X2.x;
           num.y += c.c2 * F2.y - c.a2 * X2.y;
         }
-        A.Fr[(n - 1) & 1][col + q] = F;
+        stg128(A.Fr[(n - 1) & 1] + col + q, F);
         const double inv = __ldg(&R.diag[((size_t)(n <= 1 ? 1 : 2) * Kx + kx) * N + q]);
         xc[q] = make_double2(num.x * inv, num.y * inv);
       }
@@ -228,16 +227,16 @@ __device__ void ca_forward(const KolArgs& A, const KMember& m, int tile, int s) 
       project_col(xc, N, kx);
     }
     for (int q = threadIdx.x; q < N; q += blockDim.x) {
-      A.Xr[n & 1][col + q] = xc[q];
-      if (A.traj) A.traj[(long long)s * S + col + q] = xc[q];
-      if (s == last) A.out[col + q] = xc[q];
+      stg128(A.Xr[n & 1] + col + q, xc[q]);
+      if (A.traj) stg128(A.traj + (long long)s * S + col + q, xc[q]);
+      if (s == last) stg128(A.out + col + q, xc[q]);
     }
     if (s < last && (A.nonlinear || A.closure)) {
       // the fields' inverse y transforms two at a time, sharing their passes; the column is read back from the
       // state just written, its shared slot being reused
       const double2* xs = A.Xr[n & 1] + col;
       const double* ik2 = R.diag + (size_t)kx * N;
-      auto dst = [&](int f, int j, double2 v) { A.mixA[f][m.off_mix + (long long)j * Kx + kx] = v; };
+      auto dst = [&](int f, int j, double2 v) { stg128(A.mixA[f] + m.off_mix + (long long)j * Kx + kx, v); };
       __syncthreads();
 #pragma unroll 1
       for (int f0 = 0; f0 < 4; f0 += 2) fields_y<2>(fs, R, f0, xs, ik2, kx, N, M, CM, dst);
@@ -251,7 +250,7 @@ __device__ void ca_forward(const KolArgs& A, const KMember& m, int tile, int s) 
 __device__ __forceinline__ FxRes<true> row_c2r(const double2* src, int a, int b, const KMember& m, const KRes& R,
                                                double w0, double w, int s0) {
   return xf_c2r<1, kFxOnly>(a, b, FxLay{1, m.CL, s0}, R.px, m.Kx, [&](int, int k) {
-    const double2 v = ldcg2(&src[k]);
+    const double2 v = ldcg128(&src[k]);
     const double f = k == 0 ? w0 : w;
     return make_double2(v.x * f, v.y * f);
   });
@@ -262,14 +261,14 @@ __device__ __forceinline__ FxRes<true> row_c2r(const double2* src, int a, int b,
 template <class Src>
 __device__ __forceinline__ FxRes<true> rows_c2r4(int base, Src src, const KMember& m, const KRes& R) {
   return xf_c2r<4, kFxOnly>(base, base + m.CL, FxLay{4, 2 * m.CL, 0}, R.px, m.Kx,
-                          [&](int f, int k) { return ldcg2(&src(f)[k]); });
+                          [&](int f, int k) { return ldcg128(&src(f)[k]); });
 }
 
 // Spectrum of a forward row transform into dst[k], k < Kx, times s (s0 on k = 0, real)
 __device__ __forceinline__ void put_row(const FxRes<false>& z, int set, double2* dst, int Kx, double s0, double s) {
   for (int k = threadIdx.x; k < Kx; k += blockDim.x) {
     const double2 v = z.coef(set, k);
-    dst[k] = k == 0 ? make_double2(v.x * s0, 0.0) : make_double2(v.x * s, v.y * s);
+    stg128(dst + k, k == 0 ? make_double2(v.x * s0, 0.0) : make_double2(v.x * s, v.y * s));
   }
 }
 
@@ -284,7 +283,7 @@ __device__ void b_forward(const KolArgs& A, const KMember& m, int tile) {
     if (A.closure) {
       const auto w = row_c2r(A.mixA[4] + m.off_mix + (long long)j * Kx, fs, fs + C, m, R, 1.0, 1.0, 0);
       double2* gw = reinterpret_cast<double2*>(A.gridW + m.off_grid + (long long)j * M);
-      for (int i = threadIdx.x; i < L; i += blockDim.x) gw[i] = w.at(0, i);
+      for (int i = threadIdx.x; i < L; i += blockDim.x) stg128(gw + i, w.at(0, i));
       __syncthreads();
     }
     double2* dst = A.mixB[0] + m.off_mix + (long long)j * Kx;
@@ -298,7 +297,7 @@ __device__ void b_forward(const KolArgs& A, const KMember& m, int tile) {
       });
       put_row(z, 0, dst, Kx, invM, invM);
     } else {
-      for (int k = threadIdx.x; k < Kx; k += blockDim.x) dst[k] = make_double2(0.0, 0.0);
+      for (int k = threadIdx.x; k < Kx; k += blockDim.x) stg128(dst + k, make_double2(0.0, 0.0));
     }
     __syncthreads();
   }
@@ -323,7 +322,7 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
   for (int kx = kx0; kx < kx1; ++kx) {
     const long long col = m.off_state + (long long)kx * N;
     if (!first) {  // Y_n from the ring (computed by the previous launch)
-      for (int q = threadIdx.x; q < N; q += blockDim.x) yc[q] = ldcg2(&A.Yr[n & 1][col + q]);
+      for (int q = threadIdx.x; q < N; q += blockDim.x) yc[q] = ldcg128(&A.Yr[n & 1][col + q]);
       __syncthreads();
     } else {
     for (int q = threadIdx.x; q < N; q += blockDim.x) lam[q] = make_double2(0.0, 0.0);
@@ -356,7 +355,7 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
       };
       auto one = [&](int f) {
         add(f, 1, xf_c2c<false, 1, 1, kFxOnly>(fs, fs + CM, FxLay{1, CM, 0}, R.py, [&](int, int j) {
-              return ldcg2(&A.mixB[f][m.off_mix + (long long)j * Kx + kx]);
+              return ldcg128(&A.mixB[f][m.off_mix + (long long)j * Kx + kx]);
             }));
       };
       bool per_one = false;
@@ -364,7 +363,7 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
 #pragma unroll 1
         for (int f0 = 0; f0 < 4; f0 += 2)
           add(f0, 2, xf_c2c<false, 2, 1, kFxOnly>(fs, fs + CM, FxLay{2, 2 * CM, 0}, R.py, [&](int pq, int j) {
-                return ldcg2(&A.mixB[f0 + pq][m.off_mix + (long long)j * Kx + kx]);
+                return ldcg128(&A.mixB[f0 + pq][m.off_mix + (long long)j * Kx + kx]);
               }));
       } else if (A.nonlinear) {
         per_one = true;
@@ -379,22 +378,22 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
     for (int q = threadIdx.x; q < N; q += blockDim.x) {
       double2 l = lam[q];
       if (si >= 0) {
-        const double2 sd = A.seeds[(long long)si * S + col + q];
+        const double2 sd = ldg128(A.seeds + (long long)si * S + col + q);
         l.x += sd.x; l.y += sd.y;
       }
       if (n + 1 <= SN) {
-        const double2 y1 = ldcg2(&A.Yr[(n + 1) & 1][col + q]);
+        const double2 y1 = ldcg128(&A.Yr[(n + 1) & 1][col + q]);
         l.x -= c1.a1 * y1.x; l.y -= c1.a1 * y1.y;
       }
       if (n + 2 <= SN) {
-        const double2 y2 = ldcg2(&A.Yr[n & 1][col + q]);
+        const double2 y2 = ldcg128(&A.Yr[n & 1][col + q]);
         l.x -= c2.a2 * y2.x; l.y -= c2.a2 * y2.y;
       }
       lam[q] = l;
     }
     __syncthreads();
     if (n == 0) {
-      for (int q = threadIdx.x; q < N; q += blockDim.x) A.out[col + q] = lam[q];
+      for (int q = threadIdx.x; q < N; q += blockDim.x) stg128(A.out + col + q, lam[q]);
       __syncthreads();
       continue;
     }
@@ -406,7 +405,7 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
     __syncthreads();
     }  // first half
     if (!second) {  // the launch ends at Y_n: store it for the next launch
-      for (int q = threadIdx.x; q < N; q += blockDim.x) A.Yr[n & 1][col + q] = yc[q];
+      for (int q = threadIdx.x; q < N; q += blockDim.x) stg128(A.Yr[n & 1] + col + q, yc[q]);
       __syncthreads();
       continue;
     }
@@ -416,11 +415,11 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
     for (int q = threadIdx.x; q < N; q += blockDim.x) {
       double2 w = make_double2(cw1.c1 * yc[q].x, cw1.c1 * yc[q].y);
       if (n + 1 <= SN) {
-        const double2 y1 = ldcg2(&A.Yr[(n + 1) & 1][col + q]);
+        const double2 y1 = ldcg128(&A.Yr[(n + 1) & 1][col + q]);
         w.x += cw2.c2 * y1.x; w.y += cw2.c2 * y1.y;
       }
       lam[q] = w;
-      A.Yr[n & 1][col + q] = yc[q];
+      stg128(A.Yr[n & 1] + col + q, yc[q]);
     }
     __syncthreads();
     if (!A.nonlinear && !A.closure) continue;
@@ -433,7 +432,7 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
       const double invM = 1.0 / M;
       for (int j = threadIdx.x; j < M; j += blockDim.x) {
         const double2 v = r.at(0, j);
-        A.mixA[4][m.off_mix + (long long)j * Kx + kx] = make_double2(v.x * invM, v.y * invM);
+        stg128(A.mixA[4] + m.off_mix + (long long)j * Kx + kx, make_double2(v.x * invM, v.y * invM));
       }
       __syncthreads();
     }
@@ -441,7 +440,7 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
     // shared memory for every member); the closure's input field goes to slot 5 (slot 4 holds T^dagger W)
     const double2* xs = A.traj + (long long)(n - 1 - A.lo) * S + col;
     const double* ik2 = R.diag + (size_t)kx * N;
-    auto dst = [&](int f, int j, double2 v) { A.mixA[f < 4 ? f : 5][m.off_mix + (long long)j * Kx + kx] = v; };
+    auto dst = [&](int f, int j, double2 v) { stg128(A.mixA[f < 4 ? f : 5] + m.off_mix + (long long)j * Kx + kx, v); };
     if (A.nonlinear) {
 #pragma unroll 1
       for (int f0 = 0; f0 < 4; f0 += 2) fields_y<2>(fs, R, f0, xs, ik2, kx, N, M, CM, dst);
@@ -465,8 +464,8 @@ __device__ void b_adjoint(const KolArgs& A, const KMember& m, int tile) {
         const auto g = row_c2r(mixed(4), fs, fs + C, m, R, 1.0 / M, 0.5 / M, 0);
         const auto w = row_c2r(mixed(5), fs + 2 * C, fs + 3 * C, m, R, 1.0, 1.0, 1);
         for (int i = threadIdx.x; i < L; i += blockDim.x) {
-          gw[i] = w.at(0, i);
-          gg[i] = g.at(0, i);
+          stg128(gw + i, w.at(0, i));
+          stg128(gg + i, g.at(0, i));
         }
         __syncthreads();
       }
@@ -480,8 +479,8 @@ __device__ void b_adjoint(const KolArgs& A, const KMember& m, int tile) {
     if (A.closure) {
       const auto w = row_c2r(mixed(5), fr + 4 * C, fr + 6 * C, m, R, 1.0, 1.0, 5);
       for (int i = threadIdx.x; i < L; i += blockDim.x) {
-        gw[i] = w.at(0, i);
-        gg[i] = g.at(0, i);
+        stg128(gw + i, w.at(0, i));
+        stg128(gg + i, g.at(0, i));
       }
       __syncthreads();
     }
@@ -599,13 +598,13 @@ __global__ void __launch_bounds__(kKolThreads) closure_rows_kernel(const __grid_
   const int Kx = m.Kx;
   const int fs = 0;
   const double2* g = reinterpret_cast<const double2*>(grid + m.off_grid + (long long)j * m.M);
-  const auto z = xf_r2c<1, kFxOnly>(fs, fs + m.CL, FxLay{1, m.CL, 0}, R.px, [&](int, int i) { return g[i]; });
+  const auto z = xf_r2c<1, kFxOnly>(fs, fs + m.CL, FxLay{1, m.CL, 0}, R.px, [&](int, int i) { return ldg128(g + i); });
   if (mode == 0) {
     double2* dst = A.mixB[0] + m.off_mix + (long long)j * Kx;
     const double s = 1.0 / m.M;
     for (int k = threadIdx.x; k < Kx; k += blockDim.x) {
-      const double2 v = dst[k], c = z.coef(0, k);
-      dst[k] = make_double2(v.x - c.x * s, k == 0 ? v.y : v.y - c.y * s);
+      const double2 v = ldg128(dst + k), c = z.coef(0, k);
+      stg128(dst + k, make_double2(v.x - c.x * s, k == 0 ? v.y : v.y - c.y * s));
     }
   } else {
     put_row(z, 0, A.mixB[4] + m.off_mix + (long long)j * Kx, Kx, 1.0, 2.0);

@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(kXThreadsMax) xfft_kernel(const __grid_constan
     const double2* src = J.cin + (size_t)row0 * Kx;
     const auto z = xf_c2r<NB>(0, C, lay, P.plan, Kx, [&](int s, int k) {
       if (row0 + s >= nrows) return zero;
-      double2 v = src[(size_t)s * Kx + k];
+      double2 v = ldg128(src + (size_t)s * Kx + k);
       if (J.cmul == 1) {  // i k v
         const double kk = P.kscale * k;
         v = make_double2(-kk * v.y, kk * v.x);
@@ -470,7 +470,7 @@ __global__ void __launch_bounds__(kXThreadsMax) xfft_kernel(const __grid_constan
     });
     for (int s = 0; s < NB && row0 + s < nrows; ++s) {
       double2* g = reinterpret_cast<double2*>(J.rout + (size_t)(row0 + s) * Mx);
-      for (int j = tid; j < L; j += nt) g[j] = z.at(s, j);
+      for (int j = tid; j < L; j += nt) stg128(g + j, z.at(s, j));
     }
     return;
   }
@@ -490,7 +490,7 @@ __global__ void __launch_bounds__(kXThreadsMax) xfft_kernel(const __grid_constan
         }
         double2 o = cscale(acc, k == 0 ? J.s0 : J.s);
         if (k == 0) o.y = 0.0;
-        dst[k] = o;
+        stg128(dst + k, o);
       }
     }
   };
@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(kXThreadsMax) xfft_kernel(const __grid_constan
       if (row0 + s >= nrows) return zero;
       const size_t ro = (size_t)(row0 + s) * Mx;
       auto at = [&](const double* base, int slot) {
-        return reinterpret_cast<const double2*>(base + (size_t)slot * J.npts + ro)[j];
+        return ldg128(reinterpret_cast<const double2*>(base + (size_t)slot * J.npts + ro) + j);
       };
       const double2 x = at(J.G, J.pa[0]), y = at(J.G, J.pb[0]), u = at(J.G, J.pa[1]), v = at(J.G, J.pb[1]);
       if (!J.dG) return make_double2(fma(p0 * x.x, y.x, p1 * (u.x * v.x)), fma(p0 * x.y, y.y, p1 * (u.y * v.y)));
@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(kXThreadsMax) xfft_kernel(const __grid_constan
   }
   auto row = [&](int s, int j) {
     const int t = s / NB, q = row0 + s - t * NB;
-    return q < nrows ? reinterpret_cast<const double2*>(J.rin[t] + (size_t)q * Mx)[j] : zero;
+    return q < nrows ? ldg128(reinterpret_cast<const double2*>(J.rin[t] + (size_t)q * Mx) + j) : zero;
   };
   if (J.nr > 1) store(xf_r2c<2 * NB>(0, C, FxLay{2 * NB, 2 * C, 0}, P.plan, row), 2);
   else store(xf_r2c<NB>(0, C, lay, P.plan, row), 1);
