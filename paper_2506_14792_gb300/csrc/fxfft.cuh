@@ -693,6 +693,8 @@ template <bool INV, bool AHEAD>
 __device__ __forceinline__ FxRes<INV> fx_run(int a, int b, FxLay lay, FxGroup g, const FFTPlan& p, FxDesc next) {
   if (p.fxr0 != p.n)
     fx_rest<AHEAD>(b + g.s * lay.stride, a + g.s * lay.stride, g, fx_sch(lay.s0 + g.s), next, p.fxp + 2, p.fxt);
+  else
+    __syncthreads();  // a single pass (n = 3): a later call writes the slots that fx_make_meta reads
   return FxRes<INV>{p.fxodd ? b : a, lay, p.n, p.fxr, p.wm, true};
 }
 template <bool INV>
