@@ -191,10 +191,7 @@ struct Couette : EqImpl {
     yp.ntile = (Kx + yp.TK - 1) / yp.TK;
     ysmem = ybytes(yp.TK);
     if (ysmem > 48 * 1024 - sizeof(FxShared) && ysmem <= kOptIn)
-      SPADJ_CUDA_TRY(p, with_yfft([](auto kernel) {
-        // the largest size, so that no other problem's creation lowers it
-        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOptIn);
-      }));
+      SPADJ_CUDA_TRY(p, with_yfft([&](auto kernel) { return raise_smem(kernel, ysmem); }));
     {  // the step-solve operators of the selected form (the other one is built on first use)
       // One warp per pencil pair runs the band sweeps: with fewer than 8 pairs per SM the warps
       // cannot keep the FP64 pipe busy and the dense Phi (a CTA per pair) is faster (measured:

@@ -948,7 +948,7 @@ struct ShearEvp : EqImpl {
     int dev = 0;
     SPADJ_CUDA_TRY(p, cudaGetDevice(&dev));
     SPADJ_CUDA_TRY(p, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    SPADJ_CUDA_TRY(p, cudaFuncSetAttribute(evp_iter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)iter_smem(kEvpMaxN, kEvpMaxUpper)));
+    SPADJ_CUDA_TRY(p, raise_smem(evp_iter_kernel, iter_smem(kEvpMaxN, kEvpMaxUpper)));
     return SPADJ_OK;
   }
 

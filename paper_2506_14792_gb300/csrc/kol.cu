@@ -882,16 +882,13 @@ struct Kol : EqImpl {
         SPADJ_CUDA_TRY(p, cudaGetDevice(&dev));
         SPADJ_CUDA_TRY(p, cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev));
       }
-      SPADJ_CUDA_TRY(p, cudaFuncSetAttribute(cnn::conv32_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)cnn::kTcSmem));
+      SPADJ_CUDA_TRY(p, raise_smem(cnn::conv32_tc_kernel, cnn::kTcSmem));
       // the halo-staged forms need two staging buffers of the grid's halo range: up to a 764-point
       // grid they fit one CTA; larger grids use the per-tap forms
       halo_fits = cnn::wgrad_halo_smem(hm[0].M) <= kHaloSmemMax && cnn::halo_smem(hm[0].M) <= kHaloSmemMax;
       if (halo_fits) {
-        SPADJ_CUDA_TRY(p, cudaFuncSetAttribute(cnn::conv32_halo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)cnn::halo_smem(hm[0].M)));
-        SPADJ_CUDA_TRY(p, cudaFuncSetAttribute(cnn::wgrad32_halo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)cnn::wgrad_halo_smem(hm[0].M)));
+        SPADJ_CUDA_TRY(p, raise_smem(cnn::conv32_halo_kernel, cnn::halo_smem(hm[0].M)));
+        SPADJ_CUDA_TRY(p, raise_smem(cnn::wgrad32_halo_kernel, cnn::wgrad_halo_smem(hm[0].M)));
       }
       SPADJ_CUDA_TRY(p, cudaMemsetAsync(pbuf.ptr, 0, sizeof(double) * np, p->stream));
       cnn::convert_kernel<<<64, 256, 0, p->stream>>>(pbuf.as<double>(), wq.as<__nv_bfloat16>(), bq.as<float>());
@@ -909,14 +906,14 @@ struct Kol : EqImpl {
       smem = base;
       if (ext > base && ext <= 227 * 1024) {
         int ob = 0, oe = 0;
-        SPADJ_CUDA_TRY(p, cudaFuncSetAttribute(kol_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ext));
+        SPADJ_CUDA_TRY(p, raise_smem(kol_persistent, ext));
         SPADJ_CUDA_TRY(p, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ob, kol_persistent, kKolThreads, base));
         SPADJ_CUDA_TRY(p, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&oe, kol_persistent, kKolThreads, ext));
         if (oe >= ob) smem = ext;
       }
     }
-    SPADJ_CUDA_TRY(p, cudaFuncSetAttribute(kol_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    SPADJ_CUDA_TRY(p, cudaFuncSetAttribute(kol_phase, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SPADJ_CUDA_TRY(p, raise_smem(kol_persistent, smem));
+    SPADJ_CUDA_TRY(p, raise_smem(kol_phase, smem));
     layout();
     SPADJ_CUDA_TRY(p, dmem.ensure(sizeof(KMember) * nmem));
     SPADJ_CUDA_TRY(p, cudaMemcpyAsync(dmem.ptr, hm.data(), sizeof(KMember) * nmem, cudaMemcpyHostToDevice, p->stream));

@@ -10,6 +10,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <mutex>
 #include <utility>
 
 namespace spadj {
@@ -69,6 +70,18 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsig
   }
   if (err) atomicExch(err, 1);
   return false;
+}
+
+// Raise a kernel's limit of dynamic shared memory to `bytes`.  The limit belongs to the kernel, not to a problem, so it is
+// never lowered: a problem with larger buffers may be in use.
+template <typename Kernel>
+inline cudaError_t raise_smem(Kernel kernel, size_t bytes) {
+  static std::mutex m;
+  std::lock_guard<std::mutex> lock(m);
+  cudaFuncAttributes a{};
+  const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+  if (e != cudaSuccess || (size_t)a.maxDynamicSharedSizeBytes >= bytes) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 // Launch `kernel` on `st`, with the programmatic stream-serialisation attribute when pdl.

@@ -251,8 +251,8 @@ struct RB : EqImpl {
     ctsmem = colstepT_smem(N, Mz);
     fused = nonlinear && !generic && std::max(csmem, ctsmem) <= 200 * 1024;
     if (fused) {
-      SPADJ_CUDA_TRY(p, cudaFuncSetAttribute(rb_colstep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem));
-      SPADJ_CUDA_TRY(p, cudaFuncSetAttribute(rb_colstepT_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctsmem));
+      SPADJ_CUDA_TRY(p, raise_smem(rb_colstep_kernel, csmem));
+      SPADJ_CUDA_TRY(p, raise_smem(rb_colstepT_kernel, ctsmem));
     }
     {  // x-FFT rows per CTA, timed on the eight inverse transforms of one F evaluation
       SPADJ_CUDA_TRY(p, cudaMemsetAsync(w->Z.ptr, 0, w->Z.bytes, p->stream));
@@ -261,7 +261,7 @@ struct RB : EqImpl {
       SPADJ_CUDA_TRY(p, e);
     }
     if (ssmem > 48 * 1024)
-      SPADJ_CUDA_TRY(p, cudaFuncSetAttribute(solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem));
+      SPADJ_CUDA_TRY(p, raise_smem(solve_kernel, ssmem));
     return SPADJ_OK;
   }
 

@@ -553,7 +553,7 @@ inline int tune_xfft_rows(const XJobs& js, const XParams& xp, int nrows, cudaStr
     if (sm + fix <= 48 * 1024) {
       ok[nb] = true;
     } else if (sm + fix <= 227 * 1024) {
-      auto raise = [&](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); };
+      auto raise = [&](auto kernel) { return raise_smem(kernel, sm); };
       const cudaError_t e = nb == 1 ? raise(xfft_kernel<1>) : nb == 2 ? raise(xfft_kernel<2>) : raise(xfft_kernel<4>);
       ok[nb] = e == cudaSuccess;
       cudaGetLastError();
