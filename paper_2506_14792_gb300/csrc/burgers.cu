@@ -25,7 +25,7 @@ constexpr int kQMax = 4;  // modes per thread
 constexpr int kMaxOrder = 4;
 
 struct BurgersParams {
-  int K, L, M, C;  // C: entries of one transform buffer
+  int K, L, M;
   double nu, kscale, dt, length;
   int order, nonlinear;
   FFTPlan plan;
@@ -39,13 +39,13 @@ struct BurgersParams {
   int ws_len;
 };
 
-// Buffers of a CTA: two transform pairs of C entries each.  The inverse transforms read their staged
+// Buffers of a CTA: two transform pairs of L entries each.  The inverse transforms read their staged
 // spectra from B (and D for a second one) and leave the grid in A or B (C or D).
 struct Smem {
   int A, B, C, D;
 };
 
-__device__ __forceinline__ Smem carve(const BurgersParams& P) { return Smem{0, P.C, 2 * P.C, 3 * P.C}; }
+__device__ __forceinline__ Smem carve(const BurgersParams& P) { return Smem{0, P.L, 2 * P.L, 3 * P.L}; }
 
 __device__ __forceinline__ double kwav(const BurgersParams& P, int k) { return P.kscale * k; }
 
@@ -59,8 +59,8 @@ __device__ __forceinline__ double half_k(const BurgersParams& P, int k) { return
 // Puts the sums T_k, F(x)_k = -i half_k T_k, k < K, through out(k, T_k), from the spectrum staged in B.
 template <int PATH, class Out>
 __device__ __forceinline__ void eval_F(const BurgersParams& P, const Smem& s, Out out) {
-  const auto u = xf_c2r_staged<1, PATH>(s.A, s.B, FxLay{1, P.C, 0}, P.plan, P.K);
-  const auto z = xf_r2c<1, PATH>(s.C, s.D, FxLay{1, P.C, 0}, P.plan, [&](int, int j) {
+  const auto u = xf_c2r_staged<1, PATH>(s.A, s.B, FxLay{1, P.L, 0}, P.plan, P.K);
+  const auto z = xf_r2c<1, PATH>(s.C, s.D, FxLay{1, P.L, 0}, P.plan, [&](int, int j) {
     const double2 v = u.at(0, j);
     return make_double2(v.x * v.x, v.y * v.y);
   });
@@ -68,11 +68,11 @@ __device__ __forceinline__ void eval_F(const BurgersParams& P, const Smem& s, Ou
 }
 
 // From the primal spectrum staged in B and the tangent spectrum in D: out(k, T_k, dT_k), ((dF/dX) dX)_k =
-// -i half_k dT_k = -i k T[(B x)(B dx)].  Both transforms of each direction share their passes (A|B and C|D are 2C
+// -i half_k dT_k = -i k T[(B x)(B dx)].  Both transforms of each direction share their passes (A|B and C|D are 2L
 // apart); the second ones are staged in the free halves and overwrite the grids after that.
 template <int PATH, class Out>
 __device__ __forceinline__ void eval_F_and_jvp(const BurgersParams& P, const Smem& s, Out out) {
-  const FxLay lay{2, 2 * P.C, 0};
+  const FxLay lay{2, 2 * P.L, 0};
   const auto u = xf_c2r_staged<2, PATH>(s.A, s.B, lay, P.plan, P.K);
   const auto z = xf_r2c<2, PATH>(u.z == s.A ? s.B : s.A, u.z, lay, P.plan, [&](int q, int j) {
     const double2 v = u.at(0, j), w = q ? u.at(1, j) : v;
@@ -87,9 +87,9 @@ __device__ __forceinline__ void eval_F_and_jvp(const BurgersParams& P, const Sme
 // (dF/dX)^dagger W = B^dagger[(B x) * T^dagger(i k W)].
 template <int PATH, class Out>
 __device__ __forceinline__ void eval_vjp(const BurgersParams& P, const Smem& s, Out out) {
-  const auto u = xf_c2r_staged<2, PATH>(s.A, s.B, FxLay{2, 2 * P.C, 0}, P.plan, P.K);
+  const auto u = xf_c2r_staged<2, PATH>(s.A, s.B, FxLay{2, 2 * P.L, 0}, P.plan, P.K);
   const int f0 = u.z == s.A ? s.B : s.A;  // free halves
-  const auto z = xf_r2c<1, PATH>(f0, f0 + 2 * P.C, FxLay{1, 2 * P.C, 0}, P.plan, [&](int, int j) {
+  const auto z = xf_r2c<1, PATH>(f0, f0 + 2 * P.L, FxLay{1, 2 * P.L, 0}, P.plan, [&](int, int j) {
     const double2 a = u.at(0, j), b = u.at(1, j);
     return make_double2(a.x * b.x, a.y * b.y);
   });
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(64) to_grid_kernel(const __grid_constant__ Bur
   const Smem s = carve(P);
   const double2* xr = x + (size_t)blockIdx.x * P.K;
   double2* gr = g + (size_t)blockIdx.x * P.L;
-  const auto z = xf_c2r<1, kFp64>(s.A, s.B, FxLay{1, P.C, 0}, P.plan, P.K,
+  const auto z = xf_c2r<1, kFp64>(s.A, s.B, FxLay{1, P.L, 0}, P.plan, P.K,
                                          [&](int, int k) { return cscale(ldg128(xr + k), k == 0 ? w0 : w); });
   for (int j = threadIdx.x; j < P.L; j += blockDim.x) stg128(gr + j, z.at(0, j));
 }
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(64) to_coef_kernel(const __grid_constant__ Bur
   const Smem s = carve(P);
   const double2* gr = g + (size_t)blockIdx.x * P.L;
   double2* yr = y + (size_t)blockIdx.x * P.K;
-  const auto z = xf_r2c<1, kFp64>(s.A, s.B, FxLay{1, P.C, 0}, P.plan, [&](int, int j) { return ldg128(gr + j); });
+  const auto z = xf_r2c<1, kFp64>(s.A, s.B, FxLay{1, P.L, 0}, P.plan, [&](int, int j) { return ldg128(gr + j); });
   for (int k = threadIdx.x; k < P.K; k += blockDim.x) {
     double2 v = cscale(z.coef(0, k), k == 0 ? s0 : sc);
     if (k == 0 && re0) v.y = 0.0;
@@ -150,20 +150,14 @@ __global__ void __launch_bounds__(64) F_kernel(const __grid_constant__ BurgersPa
     for (int k = threadIdx.x; k < K; k += blockDim.x) stg128(o + k, make_double2(0.0, 0.0));
     return;
   }
-  unsigned m0 = 0u, m1 = 0u;
   for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    const double2 v = ldg128(xr + k);
-    fx_put64(s.B + k, v);
-    m0 = fx_absmax(m0, v);
+    fx_put64(s.B + k, ldg128(xr + k));
     if (MODE != 0) {
       double2 w = ldg128(dr + k);
       if (MODE == 2) w = plus_i(half_k(P, k), w);
       fx_put64(s.D + k, w);
-      m1 = fx_absmax(m1, w);
     }
   }
-  fx_put_max(0, m0);
-  if (MODE != 0) fx_put_max(1, m1);
   auto put = [&](int k, double2 v) { stg128(o + k, v); };
   if (MODE == 0) eval_F<kFp64>(P, s, [&](int k, double2 v) { put(k, minus_i(half_k(P, k), v)); });
   else if (MODE == 1) eval_F_and_jvp<kFp64>(P, s, [&](int k, double2, double2 v) { put(k, minus_i(half_k(P, k), v)); });
@@ -565,7 +559,6 @@ struct Burgers : EqImpl {
         P.wc[s][i] = kSbdfC[s][i];
       }
     P.plan = make_plan(P.L);
-    P.C = P.L;
     if (P.plan.nrad < 0) return p->fail(SPADJ_ERR_INVALID, "burgers: 3N/4 must be of the form 2^a 3^b");
     if (P.K > kQMax * G) return p->fail(SPADJ_ERR_INVALID, "burgers: n[0] too large (max 512)");
     std::vector<double2> h(P.M);
@@ -582,7 +575,7 @@ struct Burgers : EqImpl {
     SPADJ_CUDA_TRY(p, cudaStreamSynchronize(p->stream));
     P.WM = wm.as<double2>();
     fft_bind(P.plan, true, P.WM + P.M, P.WM, true);
-    smem = sizeof(double2) * 4 * P.C;
+    smem = sizeof(double2) * 4 * P.L;
     int dev = 0;
     SPADJ_CUDA_TRY(p, cudaGetDevice(&dev));
     SPADJ_CUDA_TRY(p, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));

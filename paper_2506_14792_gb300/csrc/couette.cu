@@ -112,8 +112,6 @@ struct Couette : EqImpl {
     yp.TK = Kx >= 8 ? 8 : Kx >= 4 ? 4 : Kx >= 2 ? 2 : 1;
     yp.kxs = 2.0 * M_PI / Lx; yp.kys = 2.0 * M_PI / Ly;
     yp.plan = make_plan(My);
-    yp.C = My;
-    xp.C = L;
     if (xp.plan.nrad < 0 || yp.plan.nrad < 0)
       return p->fail(SPADJ_ERR_INVALID, "couette: 3*n[0]/4 and 3*n[1]/2 must be of the form 2^a 3^b");
 

@@ -44,7 +44,6 @@ struct YJobs {
 };
 struct YParams {
   int Kx, Ny, My, TK, ntile;  // TK: 1, 2, 4 or 8 columns per CTA
-  int C;                      // entries of one transform buffer
   double kxs, kys;
   FFTPlan plan;
 };
@@ -59,11 +58,10 @@ __global__ void __launch_bounds__(128) yfft_kernel(const __grid_constant__ YJobs
   const int Kx = P.Kx, Ny = P.Ny, My = P.My;
   const int m0 = tile * TK;
   const int tk = min(TK, Kx - m0);
-  const int b = P.C;
-  const FxLay lay{TK, 2 * P.C + 1, 0};  // an odd stride: the threads of one entry meet different banks
+  const FxLay lay{TK, 2 * My + 1, 0};  // an odd stride: the threads of one entry meet different banks
   const int tid = threadIdx.x, nt = blockDim.x;
   if (J.dir == 0) {
-    const auto r = xf_c2c<true, TK, TK>(0, b, lay, P.plan, [&](int c, int e) {
+    const auto r = xf_c2c<true, TK, TK>(0, My, lay, P.plan, [&](int c, int e) {
       // entry e holds ky row q (none between the positive and the negative wavenumbers)
       const int q = e < Ny / 2 ? e : e - (My - Ny);
       double2 v = make_double2(0.0, 0.0);
@@ -88,7 +86,7 @@ __global__ void __launch_bounds__(128) yfft_kernel(const __grid_constant__ YJobs
       if (c < tk) stg128(J.out + ((size_t)i * My + e) * Kx + m0 + c, cscale(r.at(c, e), J.scale));
     }
   } else {
-    const auto r = xf_c2c<false, TK, TK>(0, b, lay, P.plan, [&](int c, int e) {
+    const auto r = xf_c2c<false, TK, TK>(0, My, lay, P.plan, [&](int c, int e) {
       return c < tk ? ldg128(J.in[0] + ((size_t)i * My + e) * Kx + m0 + c) : make_double2(0.0, 0.0);
     });
     for (int idx = tid; idx < Ny * TK; idx += nt) {

@@ -25,11 +25,14 @@
 //
 // Accuracy.  The rounding is about 0.7 units of 2^-59 of the largest value in each pass, against 2^-53 of each
 // value in FP64, and the results are rounded to FP64 once: the relative 2-norm error of complex transforms
-// (n = 3..1536; flat, smooth, single-mode, 1/k and low-pass inputs) is at most 1.5e-16 against 2.5e-16 of FP64
-// butterflies, and that of the real ones up to 2 x 768 points at most 1.6e-16 against 3.3e-16; longer real transforms
-// (peaked spectra: 2.0e-16 against 2.0e-16) stay with the FP64 butterflies of fft.cuh.  Non-finite
-// input gives NaN in every output of the sequence; sequences below 2^-895 are scaled up by 2^512 first, so
-// subnormals keep their bits.
+// (n = 3..1536; flat, smooth, single-mode, 1/k, low-pass and alternating inputs at scales 1e-300, 1 and 1e290) is at most
+// 1.5e-16 against 3.3e-16 of FP64 butterflies, and that of the real ones up to 2 x 768 points at most 1.7e-16 against
+// 3.3e-16; a single mode, where FP64 happens to be nearly exact, can be up to 8 % above it at 8e-17.  Longer real transforms
+// (peaked spectra: 2.0e-16 against 2.0e-16) stay with the FP64 butterflies of fft.cuh.  Every output is a sum of all
+// inputs with factors of modulus 1, so what counts is the error against the sequence's largest entries: entries 2^-6 and
+// more below the largest are held with fewer than 53 bits, and below 2^-59 of it they vanish, as they all but do in an FP64
+// sum with it.  Non-finite input gives NaN in every output of the sequence; sequences below 2^-895 are scaled up by
+// 2^512 first, so subnormals keep their bits.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -313,7 +316,7 @@ inline unsigned long long fx_radices(int n) {
 struct alignas(16) FxPass {
   int R, Ns, nbf, tw;
   unsigned mNs;
-  int pad0, more, pad1;
+  int more;  // whether another pass follows
 };
 inline std::vector<FxPass> fx_pass_list(int n) {
   std::vector<FxPass> v;
@@ -585,7 +588,7 @@ __device__ __forceinline__ void fx_rest(int a, int b, FxGroup g, int sch, FxDesc
   for (;;) {
     sch >>= 2;
     if (!AHEAD) next = fx_desc(passes);
-    const int R = next.d0.x, Ns = next.d0.y, nbf = next.d0.z, more = next.d1.z, sg = sch & 3;
+    const int R = next.d0.x, Ns = next.d0.y, nbf = next.d0.z, more = next.d1.y, sg = sch & 3;
     const int4* tw = twiddles + next.d0.w;
     const unsigned mNs = (unsigned)next.d1.x;
     passes += 2;

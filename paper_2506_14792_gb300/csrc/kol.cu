@@ -41,7 +41,6 @@ constexpr unsigned kSpinLimit = 1u << 26;  // x ~150 ns per probe: several secon
 
 struct KMember {
   int N, Kx, M, L, res;
-  int CM, CL;           // entries of a transform buffer of length M, L
   long long off_state;  // complex offset of the member in a state array
   long long off_mix;    // complex offset of the member in a mixed [y][kx] array
   long long off_grid;   // offset of the member in a real [y][x] grid array
@@ -159,12 +158,12 @@ __device__ __forceinline__ double2 field_entry(int f, const double2* xs, const d
   return f < 4 ? fmult(f, (double)kx, (double)kyof(q, N), __ldg(&ik2[q]), x) : x;
 }
 
-// Inverse y transforms of the fields f0 .. f0 + NP - 1 of a column (transform pairs at fs + 2 p CM, scratch + CM;
+// Inverse y transforms of the fields f0 .. f0 + NP - 1 of a column (transform pairs at fs + 2 p M, scratch + M;
 // the column is read from global memory), into dst(f)[row j].
 template <int NP, class Dst>
 __device__ __forceinline__ void fields_y(int fs, const KRes& R, int f0, const double2* xs, const double* ik2, int kx, int N,
-                                         int M, int CM, Dst dst) {
-  const auto r = xf_c2c<true, NP, 1, kFxOnly>(fs, fs + CM, FxLay{NP, 2 * CM, 0}, R.py, [&](int p, int j) {
+                                         int M, Dst dst) {
+  const auto r = xf_c2c<true, NP, 1, kFxOnly>(fs, fs + M, FxLay{NP, 2 * M, 0}, R.py, [&](int p, int j) {
     return field_entry(f0 + p, xs, ik2, kx, j, N, M);
   });
   for (int i = threadIdx.x; i < NP * M; i += blockDim.x) {
@@ -177,12 +176,12 @@ __device__ __forceinline__ void fields_y(int fs, const KRes& R, int f0, const do
 // ---- forward CA tile --------------------------------------------------------------------------
 __device__ void ca_forward(const KolArgs& A, const KMember& m, int tile, int s) {
   extern __shared__ double2 ks[];
-  const int N = m.N, Kx = m.Kx, M = m.M, CM = m.CM;
+  const int N = m.N, Kx = m.Kx, M = m.M;
   const int n = A.n0 + s;           // absolute step of this stage
   const int last = A.nstage - 1;    // the launch's last stage
   const KRes& R = A.res[m.res];
   const int fs = 0;          // transform pairs from the start of ks
-  double2* xc = ks + 2 * CM;             // N
+  double2* xc = ks + 2 * M;             // N
   const int kx0 = tile * A.CW, kx1 = min(Kx, kx0 + A.CW);
   const long long S = A.state_size;
   for (int kx = kx0; kx < kx1; ++kx) {
@@ -193,7 +192,7 @@ __device__ void ca_forward(const KolArgs& A, const KMember& m, int tile, int s) 
     } else {
       FxRes<false> r{};
       if (A.nonlinear || A.closure)
-        r = xf_c2c<false, 1, 1, kFxOnly>(fs, fs + CM, FxLay{1, CM, 0}, R.py, [&](int, int j) {
+        r = xf_c2c<false, 1, 1, kFxOnly>(fs, fs + M, FxLay{1, M, 0}, R.py, [&](int, int j) {
           return ldcg128(&A.mixB[0][m.off_mix + (long long)j * Kx + kx]);
         });
       const Coef c = kcoef(n, A.kc);
@@ -239,8 +238,8 @@ __device__ void ca_forward(const KolArgs& A, const KMember& m, int tile, int s) 
       auto dst = [&](int f, int j, double2 v) { stg128(A.mixA[f] + m.off_mix + (long long)j * Kx + kx, v); };
       __syncthreads();
 #pragma unroll 1
-      for (int f0 = 0; f0 < 4; f0 += 2) fields_y<2>(fs, R, f0, xs, ik2, kx, N, M, CM, dst);
-      if (A.closure) fields_y<1>(fs, R, 4, xs, ik2, kx, N, M, CM, dst);
+      for (int f0 = 0; f0 < 4; f0 += 2) fields_y<2>(fs, R, f0, xs, ik2, kx, N, M, dst);
+      if (A.closure) fields_y<1>(fs, R, 4, xs, ik2, kx, N, M, dst);
     }
     __syncthreads();
   }
@@ -249,18 +248,18 @@ __device__ void ca_forward(const KolArgs& A, const KMember& m, int tile, int s) 
 // Inverse x transform of one mixed row (weights w0 on k = 0, w elsewhere) in the buffers a, b on scale slot s0.
 __device__ __forceinline__ FxRes<true> row_c2r(const double2* src, int a, int b, const KMember& m, const KRes& R,
                                                double w0, double w, int s0) {
-  return xf_c2r<1, kFxOnly>(a, b, FxLay{1, m.CL, s0}, R.px, m.Kx, [&](int, int k) {
+  return xf_c2r<1, kFxOnly>(a, b, FxLay{1, m.L, s0}, R.px, m.Kx, [&](int, int k) {
     const double2 v = ldcg128(&src[k]);
     const double f = k == 0 ? w0 : w;
     return make_double2(v.x * f, v.y * f);
   });
 }
 
-// Inverse x transforms of the mixed rows src(0..3) at once (weights 1), field f in the pair base + 2 f CL: the FFTs
+// Inverse x transforms of the mixed rows src(0..3) at once (weights 1), field f in the pair base + 2 f L: the FFTs
 // share their passes (more butterflies per pass than threads in one row's, one barrier per pass for all).
 template <class Src>
 __device__ __forceinline__ FxRes<true> rows_c2r4(int base, Src src, const KMember& m, const KRes& R) {
-  return xf_c2r<4, kFxOnly>(base, base + m.CL, FxLay{4, 2 * m.CL, 0}, R.px, m.Kx,
+  return xf_c2r<4, kFxOnly>(base, base + m.L, FxLay{4, 2 * m.L, 0}, R.px, m.Kx,
                           [&](int f, int k) { return ldcg128(&src(f)[k]); });
 }
 
@@ -274,14 +273,14 @@ __device__ __forceinline__ void put_row(const FxRes<false>& z, int set, double2*
 
 // ---- forward B tile ---------------------------------------------------------------------------
 __device__ void b_forward(const KolArgs& A, const KMember& m, int tile) {
-  const int Kx = m.Kx, M = m.M, L = m.L, C = m.CL;
+  const int Kx = m.Kx, M = m.M, L = m.L;
   const KRes& R = A.res[m.res];
-  const int fs = 0;  // four transform pairs (field f: slots 2f, 2f+1 of C entries)
+  const int fs = 0;  // four transform pairs (field f: slots 2f, 2f+1 of L entries)
   const int j0 = tile * A.RW, j1 = min(M, j0 + A.RW);
   const double invM = 1.0 / M;
   for (int j = j0; j < j1; ++j) {
     if (A.closure) {
-      const auto w = row_c2r(A.mixA[4] + m.off_mix + (long long)j * Kx, fs, fs + C, m, R, 1.0, 1.0, 0);
+      const auto w = row_c2r(A.mixA[4] + m.off_mix + (long long)j * Kx, fs, fs + L, m, R, 1.0, 1.0, 0);
       double2* gw = reinterpret_cast<double2*>(A.gridW + m.off_grid + (long long)j * M);
       for (int i = threadIdx.x; i < L; i += blockDim.x) stg128(gw + i, w.at(0, i));
       __syncthreads();
@@ -290,8 +289,8 @@ __device__ void b_forward(const KolArgs& A, const KMember& m, int tile) {
     if (A.nonlinear) {
       // u, v, w_x, w_y on the grid row, then u w_x + v w_y through the free slots of fields 0 and 1
       const auto r = rows_c2r4(fs, [&](int f) { return A.mixA[f] + m.off_mix + (long long)j * Kx; }, m, R);
-      const int fr = R.px.fxodd ? fs : fs + C;
-      const auto z = xf_r2c<1, kFxOnly>(fr, fr + 2 * C, FxLay{1, C, 0}, R.px, [&](int, int i) {
+      const int fr = R.px.fxodd ? fs : fs + L;
+      const auto z = xf_r2c<1, kFxOnly>(fr, fr + 2 * L, FxLay{1, L, 0}, R.px, [&](int, int i) {
         const double2 u = r.at(0, i), v = r.at(1, i), wx = r.at(2, i), wy = r.at(3, i);
         return make_double2(fma(u.x, wx.x, v.x * wy.x), fma(u.y, wx.y, v.y * wy.y));
       });
@@ -308,14 +307,14 @@ __device__ void b_forward(const KolArgs& A, const KMember& m, int tile) {
 // read from the Y ring.  second: the second half (W_{n-1} and the fields of X_{n-1} for the next VJP).
 __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, bool first, bool second) {
   extern __shared__ double2 ks[];
-  const int N = m.N, Kx = m.Kx, M = m.M, CM = m.CM;
+  const int N = m.N, Kx = m.Kx, M = m.M;
   const KRes& R = A.res[m.res];
-  // The VJP's forward y transforms run two at a time (pairs at ks + 2 p CM, scratch + CM) when the
-  // accumulator lam fits beside them; otherwise one at a time in ks[0, 2 CM).
-  const bool pairs = 4 * CM + N <= A.smem_entries;
+  // The VJP's forward y transforms run two at a time (pairs at ks + 2 p M, scratch + M) when the
+  // accumulator lam fits beside them; otherwise one at a time in ks[0, 2 M).
+  const bool pairs = 4 * M + N <= A.smem_entries;
   const int fs = 0;
-  double2* lam = pairs ? ks + 4 * CM : ks + 2 * CM;  // N
-  double2* yc = pairs ? ks + 2 * CM : lam + N;      // N (used after the VJP)
+  double2* lam = pairs ? ks + 4 * M : ks + 2 * M;  // N
+  double2* yc = pairs ? ks + 2 * M : lam + N;      // N (used after the VJP)
   const int kx0 = tile * A.CW, kx1 = min(Kx, kx0 + A.CW);
   const long long S = A.state_size;
   const int SN = A.S;
@@ -354,7 +353,7 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
         __syncthreads();
       };
       auto one = [&](int f) {
-        add(f, 1, xf_c2c<false, 1, 1, kFxOnly>(fs, fs + CM, FxLay{1, CM, 0}, R.py, [&](int, int j) {
+        add(f, 1, xf_c2c<false, 1, 1, kFxOnly>(fs, fs + M, FxLay{1, M, 0}, R.py, [&](int, int j) {
               return ldcg128(&A.mixB[f][m.off_mix + (long long)j * Kx + kx]);
             }));
       };
@@ -362,7 +361,7 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
       if (A.nonlinear && pairs) {
 #pragma unroll 1
         for (int f0 = 0; f0 < 4; f0 += 2)
-          add(f0, 2, xf_c2c<false, 2, 1, kFxOnly>(fs, fs + CM, FxLay{2, 2 * CM, 0}, R.py, [&](int pq, int j) {
+          add(f0, 2, xf_c2c<false, 2, 1, kFxOnly>(fs, fs + M, FxLay{2, 2 * M, 0}, R.py, [&](int pq, int j) {
                 return ldcg128(&A.mixB[f0 + pq][m.off_mix + (long long)j * Kx + kx]);
               }));
       } else if (A.nonlinear) {
@@ -425,7 +424,7 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
     if (!A.nonlinear && !A.closure) continue;
     // T_y^dagger W (inverse FFT with 1/M) -> mixA[4]
     {
-      const auto r = xf_c2c<true, 1, 1, kFxOnly>(fs, fs + CM, FxLay{1, CM, 0}, R.py, [&](int, int j) {
+      const auto r = xf_c2c<true, 1, 1, kFxOnly>(fs, fs + M, FxLay{1, M, 0}, R.py, [&](int, int j) {
         const int q = yrow(j, N, M);
         return q < 0 ? make_double2(0.0, 0.0) : lam[q];
       });
@@ -436,24 +435,24 @@ __device__ void ca_adjoint(const KolArgs& A, const KMember& m, int tile, int n, 
       }
       __syncthreads();
     }
-    // fields of X_{n-1} from the trajectory, their inverse y transforms two at a time (4 CM <= the CTA's
+    // fields of X_{n-1} from the trajectory, their inverse y transforms two at a time (4 M <= the CTA's
     // shared memory for every member); the closure's input field goes to slot 5 (slot 4 holds T^dagger W)
     const double2* xs = A.traj + (long long)(n - 1 - A.lo) * S + col;
     const double* ik2 = R.diag + (size_t)kx * N;
     auto dst = [&](int f, int j, double2 v) { stg128(A.mixA[f < 4 ? f : 5] + m.off_mix + (long long)j * Kx + kx, v); };
     if (A.nonlinear) {
 #pragma unroll 1
-      for (int f0 = 0; f0 < 4; f0 += 2) fields_y<2>(fs, R, f0, xs, ik2, kx, N, M, CM, dst);
+      for (int f0 = 0; f0 < 4; f0 += 2) fields_y<2>(fs, R, f0, xs, ik2, kx, N, M, dst);
     }
-    if (A.closure) fields_y<1>(fs, R, 4, xs, ik2, kx, N, M, CM, dst);
+    if (A.closure) fields_y<1>(fs, R, 4, xs, ik2, kx, N, M, dst);
   }
 }
 
 // ---- adjoint B' tile --------------------------------------------------------------------------
 __device__ void b_adjoint(const KolArgs& A, const KMember& m, int tile) {
-  const int Kx = m.Kx, M = m.M, L = m.L, C = m.CL;
+  const int Kx = m.Kx, M = m.M, L = m.L;
   const KRes& R = A.res[m.res];
-  const int fs = 0;  // four transform pairs (field f: slots 2f, 2f+1 of C entries)
+  const int fs = 0;  // four transform pairs (field f: slots 2f, 2f+1 of L entries)
   const int j0 = tile * A.RW, j1 = min(M, j0 + A.RW);
   for (int j = j0; j < j1; ++j) {
     double2* gw = reinterpret_cast<double2*>(A.gridW + m.off_grid + (long long)j * M);
@@ -461,8 +460,8 @@ __device__ void b_adjoint(const KolArgs& A, const KMember& m, int tile) {
     auto mixed = [&](int f) { return A.mixA[f] + m.off_mix + (long long)j * Kx; };
     if (!A.nonlinear) {  // closure only: omega and the grid cotangent g, for the CNN's backward pass
       if (A.closure) {
-        const auto g = row_c2r(mixed(4), fs, fs + C, m, R, 1.0 / M, 0.5 / M, 0);
-        const auto w = row_c2r(mixed(5), fs + 2 * C, fs + 3 * C, m, R, 1.0, 1.0, 1);
+        const auto g = row_c2r(mixed(4), fs, fs + L, m, R, 1.0 / M, 0.5 / M, 0);
+        const auto w = row_c2r(mixed(5), fs + 2 * L, fs + 3 * L, m, R, 1.0, 1.0, 1);
         for (int i = threadIdx.x; i < L; i += blockDim.x) {
           stg128(gw + i, w.at(0, i));
           stg128(gg + i, g.at(0, i));
@@ -471,13 +470,13 @@ __device__ void b_adjoint(const KolArgs& A, const KMember& m, int tile) {
       }
       continue;
     }
-    // u, v, w_x, w_y in one set of transforms; the free slots F_f = fr + 2 f C take g (F_0 and F_1) and the
+    // u, v, w_x, w_y in one set of transforms; the free slots F_f = fr + 2 f L take g (F_0 and F_1) and the
     // closure's omega (F_2 and F_3), then the products
     const auto r = rows_c2r4(fs, mixed, m, R);
-    const int fr = R.px.fxodd ? fs : fs + C;
-    const auto g = row_c2r(mixed(4), fr, fr + 2 * C, m, R, 1.0 / M, 0.5 / M, 4);
+    const int fr = R.px.fxodd ? fs : fs + L;
+    const auto g = row_c2r(mixed(4), fr, fr + 2 * L, m, R, 1.0 / M, 0.5 / M, 4);
     if (A.closure) {
-      const auto w = row_c2r(mixed(5), fr + 4 * C, fr + 6 * C, m, R, 1.0, 1.0, 5);
+      const auto w = row_c2r(mixed(5), fr + 4 * L, fr + 6 * L, m, R, 1.0, 1.0, 5);
       for (int i = threadIdx.x; i < L; i += blockDim.x) {
         stg128(gw + i, w.at(0, i));
         stg128(gg + i, g.at(0, i));
@@ -492,13 +491,13 @@ __device__ void b_adjoint(const KolArgs& A, const KMember& m, int tile) {
 #pragma unroll
       for (int f = 0; f < 4; ++f) {
         const double2 b = r.at(f ^ 2, i), v = make_double2(-a.x * b.x, -a.y * b.y);
-        fx_put64(fr + 2 * f * C + i, v);
+        fx_put64(fr + 2 * f * L + i, v);
         mx[f] = fx_absmax(mx[f], v);
       }
     }
 #pragma unroll
     for (int f = 0; f < 4; ++f) fx_put_max(f, mx[f]);
-    const auto z = xf_c2c_staged<false, 4, 1, kFxOnly, true>(fr, r.z, FxLay{4, 2 * C, 0}, R.px);
+    const auto z = xf_c2c_staged<false, 4, 1, kFxOnly, true>(fr, r.z, FxLay{4, 2 * L, 0}, R.px);
     for (int f = 0; f < 4; ++f) put_row(z, f, A.mixB[f] + m.off_mix + (long long)j * Kx, Kx, 1.0, 2.0);
     __syncthreads();
   }
@@ -598,7 +597,7 @@ __global__ void __launch_bounds__(kKolThreads) closure_rows_kernel(const __grid_
   const int Kx = m.Kx;
   const int fs = 0;
   const double2* g = reinterpret_cast<const double2*>(grid + m.off_grid + (long long)j * m.M);
-  const auto z = xf_r2c<1, kFxOnly>(fs, fs + m.CL, FxLay{1, m.CL, 0}, R.px, [&](int, int i) { return ldg128(g + i); });
+  const auto z = xf_r2c<1, kFxOnly>(fs, fs + m.L, FxLay{1, m.L, 0}, R.px, [&](int, int i) { return ldg128(g + i); });
   if (mode == 0) {
     double2* dst = A.mixB[0] + m.off_mix + (long long)j * Kx;
     const double s = 1.0 / m.M;
@@ -708,7 +707,7 @@ struct Kol : EqImpl {
   int closure = 0;
   DevBuf gridW, gridG, corr, xq, hbuf[3], dact[3], dh, dz, dz2, pbuf, wq, bq, part, gp, chunkbuf;
   static constexpr int kWgradChunks = 8;
-  int CLmax = 0, CMmax = 0, Nmax = 0;
+  int Lmax = 0, Mmax = 0, Nmax = 0;
   double Re = 100.0, dt = 0;
   int forcing = 1, nonlinear = 1;
   int CW = 4, RW = 2, ctas_per_sm = 0, persistent = 1;
@@ -773,7 +772,6 @@ struct Kol : EqImpl {
       }
       KMember m{};
       m.N = N; m.Kx = N / 2; m.M = 3 * N / 2; m.L = m.M / 2; m.res = r;
-      m.CM = m.M; m.CL = m.L;
       m.off_state = offs; m.off_mix = offm; m.off_grid = offg;
       offs += (long long)m.Kx * N;
       offm += (long long)m.M * m.Kx;
@@ -781,7 +779,7 @@ struct Kol : EqImpl {
       if (closure && b > 0 && N != hm[0].N)
         return p->fail(SPADJ_ERR_UNSUPPORTED, "kolmogorov: the learned closure needs one resolution for the whole batch");
       hm.push_back(m);
-      CLmax = std::max(CLmax, m.CL); CMmax = std::max(CMmax, m.CM); Nmax = std::max(Nmax, N);
+      Lmax = std::max(Lmax, m.L); Mmax = std::max(Mmax, m.M); Nmax = std::max(Nmax, N);
     }
     state_size = offs;
     mix_size = offm;
@@ -897,12 +895,12 @@ struct Kol : EqImpl {
     }
     SPADJ_CUDA_TRY(p, ctr.ensure(sizeof(int) * (2 * (size_t)nmem + 2)));
     SPADJ_CUDA_TRY(p, tmp.ensure(sb));
-    // shared memory: max over tile kinds (B and B': 8 CL, four transform pairs; CA': 2 CM + 2 N, or 4 CM + N
+    // shared memory: max over tile kinds (B and B': 8 L, four transform pairs; CA': 2 M + 2 N, or 4 M + N
     // with its VJP transforms in pairs).  The paired form's
     // size is taken when it keeps as many CTAs resident per SM.
     {
-      const size_t base = sizeof(double2) * std::max<size_t>({8 * (size_t)CLmax, 4 * (size_t)CMmax, 2 * (size_t)CMmax + 2 * (size_t)Nmax});
-      const size_t ext = std::max<size_t>(base, sizeof(double2) * (4 * (size_t)CMmax + Nmax));
+      const size_t base = sizeof(double2) * std::max<size_t>({8 * (size_t)Lmax, 4 * (size_t)Mmax, 2 * (size_t)Mmax + 2 * (size_t)Nmax});
+      const size_t ext = std::max<size_t>(base, sizeof(double2) * (4 * (size_t)Mmax + Nmax));
       smem = base;
       if (ext > base && ext <= 227 * 1024) {
         int ob = 0, oe = 0;
@@ -954,17 +952,17 @@ struct Kol : EqImpl {
   }
 
   int nt_persistent = kKolThreads;
-  // Threads per CTA of kol_persistent.  The four row transforms of a tile have CL butterflies per radix-4 pass; with more
+  // Threads per CTA of kol_persistent.  The four row transforms of a tile have L butterflies per radix-4 pass; with more
   // of them than kKolThreads and too few tiles to fill the SMs, twice the threads finish a tile sooner (8-step
   // gradients, 128 against 256 threads: N = 192 3196 and 2504 us, 512 6551 and 4546, four of 256 3862 and 2954,
-  // 16 of 96 and 192 (3456 grid rows) 3949 and 3846); 12 of 256 (4608 rows) 5167 and 5274, 16 of 128 (CL = 96) 2677
+  // 16 of 96 and 192 (3456 grid rows) 3949 and 3846); 12 of 256 (4608 rows) 5167 and 5274, 16 of 128 (L = 96) 2677
   // and 3115, one of 96 1853 and 1936.
   int threads(int sms) const {
     long long rows = 0;
     int cl = 0;
     for (auto& m : hm) {
       rows += m.M;
-      cl = std::max(cl, m.CL);
+      cl = std::max(cl, m.L);
     }
     return !closure && cl > kKolThreads && rows <= 24LL * sms ? kKolThreadsFew : kKolThreads;
   }

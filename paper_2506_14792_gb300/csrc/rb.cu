@@ -81,7 +81,7 @@ struct RB : EqImpl {
   DevBuf tdx[4], tdv[4], tdf[4], axb[4], avb[4], afb[4], aacc, atmp, axs;
   WS ws[4];
   WS* w = &ws[0];
-  size_t zsmem = 0, xsmem = 0, ssmem = 0, csmem = 0, ctsmem = 0;
+  size_t zsmem = 0, ssmem = 0, csmem = 0, ctsmem = 0;
   bool fused = false;  // fused column stage (rb_colstep_kernel) usable for these sizes
   int xnb = 1;         // x-FFT launch variant, xvar(rows per CTA, threads) (tuned at creation)
   // internal streams (joined to the caller's stream by events) and captured step graphs
@@ -153,7 +153,6 @@ struct RB : EqImpl {
     npts = (size_t)Mz * Mx;
     xp.Kx = Kx; xp.Mx = Mx; xp.L = L; xp.kscale = 2.0 * M_PI / Lx;
     xp.plan = make_plan(L);
-    xp.C = L;
     if (xp.plan.nrad < 0) return p->fail(SPADJ_ERR_INVALID, "rb: 3*n[0]/4 must be of the form 2^a 3^b");
 
     // host operators and solution operators
@@ -244,7 +243,6 @@ struct RB : EqImpl {
     SPADJ_CUDA_TRY(p, errbuf.ensure(sizeof(int)));
     SPADJ_CUDA_TRY(p, cudaMemsetAsync(errbuf.ptr, 0, sizeof(int), p->stream));
     zsmem = zmm_smem(std::max(N, Mz / 2));
-    xsmem = sizeof(double2) * (4 * L + Kx);
     const int H = 3 * (N / 2);
     ssmem = sizeof(double2) * (H + 4 * solve_rows(H)) + sizeof(double) * (size_t)H * solve_rows(H);
     csmem = colstep_smem(N, Mz);

@@ -434,7 +434,6 @@ struct XJobs {
 
 struct XParams {
   int Kx, Mx, L;
-  int C;  // entries of one transform buffer
   double kscale;
   FFTPlan plan;
   const double2* WM;
@@ -453,13 +452,13 @@ __global__ void __launch_bounds__(kXThreadsMax) xfft_kernel(const __grid_constan
   pdl_wait();
   const XJob& J = js.j[blockIdx.y];
   const int row0 = blockIdx.x * NB;
-  const int L = P.L, Kx = P.Kx, Mx = P.Mx, C = P.C;
+  const int L = P.L, Kx = P.Kx, Mx = P.Mx;
   const int tid = threadIdx.x, nt = blockDim.x;
   const double2 zero = make_double2(0.0, 0.0);
-  const FxLay lay{NB, 2 * C, 0};  // row s in the buffers 2 s C and (2 s + 1) C
+  const FxLay lay{NB, 2 * L, 0};  // row s in the buffers 2 s L and (2 s + 1) L
   if (J.dir == 0) {
     const double2* src = J.cin + (size_t)row0 * Kx;
-    const auto z = xf_c2r<NB>(0, C, lay, P.plan, Kx, [&](int s, int k) {
+    const auto z = xf_c2r<NB>(0, L, lay, P.plan, Kx, [&](int s, int k) {
       if (row0 + s >= nrows) return zero;
       double2 v = ldg128(src + (size_t)s * Kx + k);
       if (J.cmul == 1) {  // i k v
@@ -496,7 +495,7 @@ __global__ void __launch_bounds__(kXThreadsMax) xfft_kernel(const __grid_constan
   };
   if (J.nprod > 0) {
     const double p0 = J.ps[0], p1 = J.ps[1];
-    store(xf_r2c<NB>(0, C, lay, P.plan, [&](int s, int j) {
+    store(xf_r2c<NB>(0, L, lay, P.plan, [&](int s, int j) {
       if (row0 + s >= nrows) return zero;
       const size_t ro = (size_t)(row0 + s) * Mx;
       auto at = [&](const double* base, int slot) {
@@ -514,18 +513,16 @@ __global__ void __launch_bounds__(kXThreadsMax) xfft_kernel(const __grid_constan
     const int t = s / NB, q = row0 + s - t * NB;
     return q < nrows ? ldg128(reinterpret_cast<const double2*>(J.rin[t] + (size_t)q * Mx) + j) : zero;
   };
-  if (J.nr > 1) store(xf_r2c<2 * NB>(0, C, FxLay{2 * NB, 2 * C, 0}, P.plan, row), 2);
-  else store(xf_r2c<NB>(0, C, lay, P.plan, row), 1);
+  if (J.nr > 1) store(xf_r2c<2 * NB>(0, L, FxLay{2 * NB, 2 * L, 0}, P.plan, row), 2);
+  else store(xf_r2c<NB>(0, L, lay, P.plan, row), 1);
 }
 
-inline size_t xfft_smem(int C, int nb) { return sizeof(double2) * (size_t)nb * 4 * C; }
+inline size_t xfft_smem(int L, int nb) { return sizeof(double2) * (size_t)nb * 4 * L; }
 constexpr int kXRowsMax = 4;
 
 // Launch variant of the x transforms: rows per CTA nb (low byte) and threads per CTA nt (the
 // bits above; 0 = 64).
-// Threads per CTA that are a multiple of the butterflies of a pass keep every lane busy in
-// it: for L = 192 (radix 4, 4, 4, 3: 48, 48, 48, 64 butterflies per row) that is 96 threads
-// on two rows or 192 on four.
+// The threads of a CTA share out over its sequences (two per row of a two-input job), so their number is a power of two.
 constexpr int xvar(int nb, int nt) { return nb | (nt << 8); }
 constexpr int xvar_rows(int xv) { return xv & 0xff; }
 constexpr int xvar_threads(int xv) { return (xv >> 8) ? (xv >> 8) : 64; }
@@ -534,7 +531,7 @@ constexpr int xvar_threads(int xv) { return (xv >> 8) ? (xv >> 8) : 64; }
 inline cudaError_t launch_xfft(bool pdl, int xv, const XJobs& js, const XParams& xp, int nrows, cudaStream_t st) {
   const int nb = xvar_rows(xv) < 1 ? 1 : xvar_rows(xv), nt = xvar_threads(xv);
   auto go = [&](auto kernel) {
-    return launch_kernel(pdl, kernel, dim3((nrows + nb - 1) / nb, js.n), dim3(nt), xfft_smem(xp.C, nb), st, js, xp, nrows);
+    return launch_kernel(pdl, kernel, dim3((nrows + nb - 1) / nb, js.n), dim3(nt), xfft_smem(xp.L, nb), st, js, xp, nrows);
   };
   return nb == 1 ? go(xfft_kernel<1>) : nb == 2 ? go(xfft_kernel<2>) : go(xfft_kernel<4>);
 }
@@ -549,7 +546,7 @@ inline int tune_xfft_rows(const XJobs& js, const XParams& xp, int nrows, cudaStr
   // row counts whose shared memory fits one CTA (raising the opt-in limit where needed)
   bool ok[kXRowsMax + 1] = {false, false, false, false, false};
   for (int nb : {1, 2, 4}) {
-    const size_t sm = xfft_smem(xp.C, nb), fix = sizeof(FxShared);
+    const size_t sm = xfft_smem(xp.L, nb), fix = sizeof(FxShared);
     if (sm + fix <= 48 * 1024) {
       ok[nb] = true;
     } else if (sm + fix <= 227 * 1024) {
