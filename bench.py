@@ -70,6 +70,17 @@ def bf16_peak_gflops():
         return 1.9e6, "fallback"
 
 
+# Kernel classes whose transforms and matrix products run in fixed point on the integer pipes: their rate of
+# algorithmic flops is no fraction of the FP64 pipe's.  The whole sweeps of the Fourier problems are such a class; the
+# Rayleigh-Benard column stages (the same class name) run on the FP64 pipe.
+INTEGER_CLASSES = ("x_fft", "y_fft", "z_transform")
+FOURIER_WORKLOADS = ("burgers", "kolmogorov", "closure")
+
+
+def on_integer_pipes(workload, kernel_class):
+    return kernel_class in INTEGER_CLASSES or (kernel_class == "fused_trajectory" and workload.startswith(FOURIER_WORKLOADS))
+
+
 def hbm_fraction(traffic, avg_launch_s):
     """DRAM bytes of one launch of the dominant kernel over its CUDA-event duration, against the
     measured HBM roof (the metric's "% HBM roofline"); None without an ncu traffic figure."""
@@ -83,22 +94,18 @@ def hbm_fraction(traffic, avg_launch_s):
 # DRAM traffic (bytes per launch) of the dominant kernel from an ncu capture, keyed by
 # (workload, kernel class); None until measured for the current kernels.
 TRAFFIC = {
-    # cou_solve_kernel: 81.66 MB read + 1.44 MB written per launch on the 64x32x32 capture (equal to
-    # the algorithmic operator + vector bytes); scaled to 128x64x64 by the operator bytes (16x) and
-    # the vector bytes (8x), averaged over the forward (5 vectors) and transposed (2) launches
-    ("couette3d_128x64x64_Re1000_sbdf2_4000steps_gain", "pencil_solve"): 1.252e9,
-    # xfft_kernel, one row per CTA (the setting the problem picks): dram read + write per launch on
-    # the RB capture (8-job 1.23 MB, 6-job 2.41 MB, 3-job 0.64 / 2.41 MB), weighted by the launch mix
-    # of the gradient (484 : 200 : 200 : 380); the working set is L2-resident, so this is the
-    # cold-cache fill ncu sees after its cache flush
-    ("rayleigh_benard2d_256x64_Ra1e6_rk222_2000steps", "x_fft"): 1.68e6,
-    # Burgers trajectory + adjoint kernels, captured at 50 steps (forward: 36 MB read + 1.650 GB of
-    # trajectory written; adjoint: 1.715 GB of trajectory read + 44 MB written), trajectory bytes
-    # scaled to 1000 steps by (1001 / 51), averaged over the two launches of a gradient
-    ("burgers1d_N256_sbdf2_1000steps", "fused_trajectory"): 3.31e10,
-    # kol_persistent: no capture of the gradient's own sweeps yet (the captured launches were the
-    # 5-step forward sweeps that generate the observations: 6.76 GB read + 4.88 GB written each,
-    # about 2.3 GB per step of the 64 members' mixed-space arrays)
+    # cou_band_kernel: 392.0 MB read + 0.3 MB written per launch (the factors and right-hand sides)
+    ("couette3d_128x64x64_Re1000_sbdf2_4000steps_gain", "pencil_solve"): 3.92e8,
+    # xfft_kernel (two rows per CTA): dram read + write per launch, averaged over the 44 launches of a
+    # 4-step gradient; the working set is L2-resident, so this is the cold-cache fill ncu sees after its
+    # cache flush
+    ("rayleigh_benard2d_256x64_Ra1e6_rk222_2000steps", "x_fft"): 1.69e6,
+    # Burgers trajectory + adjoint kernels, captured at 20 steps (forward: 35 MB read + 692 MB of
+    # trajectory written; adjoint: 705 MB of trajectory read + 29 MB written), trajectory bytes
+    # scaled to 1000 steps by (1001 / 21), averaged over the two launches of a gradient
+    ("burgers1d_N256_sbdf2_1000steps", "fused_trajectory"): 3.33e10,
+    # kol_persistent: not captured at the benchmark's horizon (a 4-step sweep and its adjoint: 8.7 GB read and
+    # 4.9 GB written each, about 3.4 GB per step of the 64 members' mixed-space arrays)
     ("kolmogorov2d_batch64_mixed128-512_Re100_sbdf2_2000steps_4dvar8", "fused_trajectory"): None,
 }
 
@@ -1146,21 +1153,26 @@ def run_gpu(args, wl):
                       "gflops": v[1] / (v[0] / 1e3) / 1e9 if v[0] > 0 else None} for k, v in rep.items()}
     # the FP64 classes only: a class on the BF16 tensor cores (the closure network) has its own roof
     total_flops = sum(v[1] for k, v in rep.items() if k != "cnn")
+    integer = sorted(k for k in rep if on_integer_pipes(wl.name, k))
     bound, dpeak, psrc = "alu", peak, "measured"
+    if on_integer_pipes(wl.name, dom):  # issue slots of the integer and FP64 pipes together: no single peak
+        bound, dpeak, psrc = "issue", None, None
     if dom == "cnn":  # BF16 operands on the tensor cores: the measured dense BF16 rate
         bound = "tensor"
         dpeak, psrc = bf16_peak_gflops()
     roof = {"kernel": dom, "bound": bound, "achieved": achieved, "peak": dpeak, "unit": "GFLOP/s",
-            "frac": achieved / dpeak, "traffic": traffic_for(wl, dom),
+            "frac": achieved / dpeak if dpeak else None, "traffic": traffic_for(wl, dom),
             "hbm": hbm_fraction(traffic_for(wl, dom), dms / dn / 1e3),
             "avg_launch_us": 1e3 * dms / dn, "flops_per_launch": dfl / dn, "per_kernel": per_kernel,
+            "integer_classes": integer,
             "whole_step": {"algorithmic_gflop": total_flops / 1e9,
                            "achieved": total_flops / (ms / args.steps / 1e3) / 1e9,
-                           "frac": total_flops / (ms / args.steps / 1e3) / 1e9 / peak,
-                           "note": "all FP64 kernel classes' algorithmic flops of one step over the timed step"
+                           "frac": None if integer else total_flops / (ms / args.steps / 1e3) / 1e9 / peak,
+                           "note": "all kernel classes' algorithmic flops of one step over the timed step"
+                                   + ("; no fraction of the FP64 peak: the integer classes' work runs beside it" if integer else "")
                                    + (" (the closure network's BF16 tensor-core class excluded)" if "cnn" in rep else "")},
-            "peak_source": psrc, "peak_measurement": fp64 if bound == "alu" else "MEASURED_PEAKS.json bf16_tflops",
-            "peak_note": "FP64 peak measured by the library's FMA-chain probe on this GPU (nominal %.0f GFLOP/s = "
+            "peak_source": psrc, "peak_measurement": "MEASURED_PEAKS.json bf16_tflops" if bound == "tensor" else fp64,
+            "peak_note": "Classes on the integer pipes (integer_classes) have no fraction. FP64 peak measured by the library's FMA-chain probe on this GPU (nominal %.0f GFLOP/s = "
                          "152 SM x 2 DFMA/clk x 2 flop x 2.07 GHz); no tensor-core FP64 path (GB300's FP64 "
                          "tensor rate is the same). Per-class times come from one instrumented step in which "
                          "the reverse sweep's lanes overlap, so each class's GFLOP/s is a lower bound"

@@ -1011,6 +1011,7 @@ struct ShearEvp : EqImpl {
     ia.XY = XY.as<double2>();
     ia.out = out;
     ia.n_iter = n_iter;
+    double dense_flops = 0.0;  // the operator's columns, and its two products per step (16 flops per entry)
     if (dense_iterations(P, n_iter)) {
       if (phi.ensure(sizeof(double2) * (size_t)P * H * H) == cudaSuccess) {
         const int blocks = (H + kPhiWarps - 1) / kPhiWarps;
@@ -1021,13 +1022,14 @@ struct ShearEvp : EqImpl {
         kEvpDense[(H + 31) / 32 - 1]<<<P, kEvpThreads, dsmem, p->stream>>>(da);
         if ((s = check_launch(p, "evp dense iterate")) != SPADJ_OK) return s;
         ia.n_iter = 0;
+        dense_flops = (8.0 * nv * (kl + ku + 1.0) + 16.0 * H * n_iter) * H * P;
       } else {
         cudaGetLastError();  // no memory for the operators: the banded iterations need none
       }
     }
     evp_iter_kernel<<<P, kIterThreads, iter_smem(N, kuf), p->stream>>>(ia);
     // two factorisations, and two banded solves per step and for the eigenvectors, 8 flops per factor entry
-    p->toc(t0, KC_SOLVE, 16.0 * nv * ((double)kl * (kl + ku) + (kl + ku + 1.0) * (n_iter + 1)) * P);
+    p->toc(t0, KC_SOLVE, 16.0 * nv * ((double)kl * (kl + ku) + (kl + ku + 1.0) * (ia.n_iter + 1)) * P + dense_flops);
     if ((s = check_launch(p, "evp iterate")) != SPADJ_OK) return s;
     EvpSensArgs sa{};
     sa.XY = XY.as<double2>();
