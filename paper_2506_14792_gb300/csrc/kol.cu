@@ -547,7 +547,11 @@ __device__ bool wait_ge(int* ctr, int target, int* err, unsigned limit) {
   return ok != 0;
 }
 
-__global__ void __launch_bounds__(kKolThreadsFew) kol_persistent(const __grid_constant__ KolArgs A) {
+// NT: most threads per CTA.  Bounded by 256 the compiler keeps 80 registers (and spills), bounded by 128 it takes 96: CTAs of
+// 128 threads run whichever keeps more of them resident, and the second where both keep the same number (64 members of 128^2 to
+// 512^2, whose buffers limit both: 44.8 and 44.1 ms; 128 closure windows of 64^2, 6 and 5 CTAs per SM: 21.6 and 22.2 ms).
+template <int NT>
+__global__ void __launch_bounds__(NT) kol_persistent(const __grid_constant__ KolArgs A) {
   __shared__ int item;
   const int per = A.nCAtot + A.nBtot;
   const int nrun = A.nrun > 0 ? A.nrun : A.nstage;
@@ -904,13 +908,14 @@ struct Kol : EqImpl {
       smem = base;
       if (ext > base && ext <= 227 * 1024) {
         int ob = 0, oe = 0;
-        SPADJ_CUDA_TRY(p, raise_smem(kol_persistent, ext));
-        SPADJ_CUDA_TRY(p, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ob, kol_persistent, kKolThreads, base));
-        SPADJ_CUDA_TRY(p, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&oe, kol_persistent, kKolThreads, ext));
+        SPADJ_CUDA_TRY(p, raise_smem(kol_persistent<kKolThreadsFew>, ext));
+        SPADJ_CUDA_TRY(p, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ob, kol_persistent<kKolThreadsFew>, kKolThreads, base));
+        SPADJ_CUDA_TRY(p, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&oe, kol_persistent<kKolThreadsFew>, kKolThreads, ext));
         if (oe >= ob) smem = ext;
       }
     }
-    SPADJ_CUDA_TRY(p, raise_smem(kol_persistent, smem));
+    SPADJ_CUDA_TRY(p, raise_smem(kol_persistent<kKolThreads>, smem));
+    SPADJ_CUDA_TRY(p, raise_smem(kol_persistent<kKolThreadsFew>, smem));
     SPADJ_CUDA_TRY(p, raise_smem(kol_phase, smem));
     layout();
     SPADJ_CUDA_TRY(p, dmem.ensure(sizeof(KMember) * nmem));
@@ -952,6 +957,7 @@ struct Kol : EqImpl {
   }
 
   int nt_persistent = kKolThreads;
+  void (*persistent_kernel)(const KolArgs) = kol_persistent<kKolThreadsFew>;
   // Threads per CTA of kol_persistent.  The four row transforms of a tile have L butterflies per radix-4 pass; with more
   // of them than kKolThreads and too few tiles to fill the SMs, twice the threads finish a tile sooner (8-step
   // gradients, 128 against 256 threads: N = 192 3196 and 2504 us, 512 6551 and 4546, four of 256 3862 and 2954,
@@ -976,14 +982,23 @@ struct Kol : EqImpl {
         int dev = 0, sms = 0, occ = 0;
         SPADJ_CUDA_TRY(p, cudaGetDevice(&dev));
         SPADJ_CUDA_TRY(p, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        SPADJ_CUDA_TRY(p, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kol_persistent, threads(sms), smem));
+        nt_persistent = threads(sms);
+        persistent_kernel = kol_persistent<kKolThreadsFew>;
+        SPADJ_CUDA_TRY(p, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, persistent_kernel, nt_persistent, smem));
+        if (nt_persistent == kKolThreads) {
+          int wide = 0;
+          SPADJ_CUDA_TRY(p, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&wide, kol_persistent<kKolThreads>, nt_persistent, smem));
+          if (wide >= occ) {
+            occ = wide;
+            persistent_kernel = kol_persistent<kKolThreads>;
+          }
+        }
         if (occ < 1) return p->fail(SPADJ_ERR_INVALID, "kolmogorov: kernel does not fit on an SM");
         const int per_sm = ctas_per_sm > 0 ? std::min(ctas_per_sm, occ) : occ;
         grid_persistent = sms * per_sm;
-        nt_persistent = threads(sms);
       }
       if (!closure) {
-        kol_persistent<<<grid_persistent, nt_persistent, smem, p->stream>>>(A);
+        persistent_kernel<<<grid_persistent, nt_persistent, smem, p->stream>>>(A);
         spadj_status s = check_launch(p, "kolmogorov persistent");
         p->toc(t, KC_FUSED, work_flops(A));
         return s;
@@ -996,7 +1011,7 @@ struct Kol : EqImpl {
         if (st > 0) SPADJ_CUDA_TRY(p, cudaMemsetAsync(ctr.ptr, 0, sizeof(int), p->stream));  // the item queue only
         A.stage0 = st;
         A.nrun = 1;
-        kol_persistent<<<grid_persistent, nt_persistent, smem, p->stream>>>(A);
+        persistent_kernel<<<grid_persistent, nt_persistent, smem, p->stream>>>(A);
         spadj_status s = check_launch(p, "kolmogorov persistent step");
         if (s != SPADJ_OK) return s;
         p->toc(ts, KC_FUSED, st + 1 < A.nstage ? per_stage : 0.0);
