@@ -104,7 +104,7 @@ TRAFFIC = {
     # trajectory written; adjoint: 705 MB of trajectory read + 29 MB written), trajectory bytes
     # scaled to 1000 steps by (1001 / 21), averaged over the two launches of a gradient
     ("burgers1d_N256_sbdf2_1000steps", "fused_trajectory"): 3.33e10,
-    # kol_persistent: not captured at the benchmark's horizon (a 4-step sweep and its adjoint: 8.7 GB read and
+    # kol_persistent: not captured at the benchmark's horizon (a 4-step sweep and its adjoint: 8.6 GB read and
     # 4.9 GB written each, about 3.4 GB per step of the 64 members' mixed-space arrays)
     ("kolmogorov2d_batch64_mixed128-512_Re100_sbdf2_2000steps_4dvar8", "fused_trajectory"): None,
 }
